@@ -99,6 +99,9 @@ struct ItGraph {
   int kind = 0;  // 0: `len` CG iterations; 1: one reliable update
   int len = 0, nrhs = 0;
   bool prof = false;
+  // operator state recorded in the kernels' arguments and choice
+  double kappa = 0;
+  int recon = 18;
   SolverFields f;
   cudaGraphExec_t exec = nullptr;
   long long kernels = 0;
@@ -220,6 +223,12 @@ qcd_status ws_get(qcd_ctx* c, int slot, size_t bytes, void** out) {
   }
   *out = b.ptr;
   return QCD_OK;
+}
+
+void destroy_graph(ItGraph* gph) {
+  if (gph->exec) cudaGraphExecDestroy(gph->exec);
+  for (auto e : gph->events) cudaEventDestroy(e);
+  delete gph;
 }
 
 // --------------------------------------------------------------- profiling --
@@ -582,11 +591,7 @@ qcd_status qcd_destroy(qcd_ctx* c) {
     cudaEventDestroy(p.b);
   }
   for (auto e : c->ev_free) cudaEventDestroy(e);
-  for (ItGraph* gph : c->graphs) {
-    if (gph->exec) cudaGraphExecDestroy(gph->exec);
-    for (auto e : gph->events) cudaEventDestroy(e);
-    delete gph;
-  }
+  for (ItGraph* gph : c->graphs) destroy_graph(gph);
   if (c->cap) cudaStreamDestroy(c->cap);
   delete c;
   return QCD_OK;
@@ -898,6 +903,17 @@ qcd_status capture_graph(qcd_ctx* c, ItGraph* gph) {
 
 // cached graph for (kind, len) on these fields, recorded on first use
 qcd_status get_graph(qcd_ctx* c, int kind, int len, const SolverFields& f, int nrhs, ItGraph** out) {
+  for (size_t i = 0; i < c->graphs.size();) {
+    // a graph of another kappa or link storage will not run again (its last launch has ended: the builds
+    // that change them synchronise)
+    ItGraph* gph = c->graphs[i];
+    if (gph->kappa == c->kappa && gph->recon == c->recon) {
+      i++;
+      continue;
+    }
+    destroy_graph(gph);
+    c->graphs.erase(c->graphs.begin() + i);
+  }
   for (ItGraph* gph : c->graphs) {
     if (gph->kind == kind && gph->len == len && gph->nrhs == nrhs && gph->prof == c->prof_on &&
         memcmp(&gph->f, &f, sizeof f) == 0) {
@@ -910,6 +926,8 @@ qcd_status get_graph(qcd_ctx* c, int kind, int len, const SolverFields& f, int n
   gph->len = len;
   gph->nrhs = nrhs;
   gph->prof = c->prof_on;
+  gph->kappa = c->kappa;
+  gph->recon = c->recon;
   gph->f = f;
   qcd_status s = capture_graph(c, gph);
   if (s) {

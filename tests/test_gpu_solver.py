@@ -146,3 +146,23 @@ def test_persistent_rounds_past_convergence(problem, inner):
     assert rows.get("dslash_p64_r18_cloverinv") == 2 * (n + 1)
     assert rows.get("dslash_p64_r18_xpay") == 2 * (n + 1)
     assert rows.get(f"cg_persistent_p{inner}") == n
+
+
+@pytest.mark.parametrize("nrhs", [1, 2])
+def test_second_kappa_and_link_storage_on_one_context(nrhs):
+    """A solve's recorded iterations hold kappa and the link storage: those of an earlier operator on the
+    same context are not run for a later one."""
+    require_gpu()
+    from paper_0910_0262_gb300.qcd import CloverWilson
+    dims = (6, 4, 4, 6)
+    U, b = synth.make_problem(dims, 0.2, 17, nrhs)
+    op = CloverWilson(dims, -1.0)
+    for kappa, recon12 in ((0.12, True), (0.1, True), (0.1, False)):
+        op.load_gauge(to_dev(U), recon12=recon12)
+        op.clover_build(kappa, 1.0)
+        ref = evenodd.SchurOperator(U, kappa, 1.0, -1.0)
+        x, _, ok = op.cg_solve(to_dev(b), tol=1e-9, inner_prec=32)
+        assert ok
+        for v, w in zip(to_np(x), b):
+            assert np.linalg.norm(ref.MdagM(v) - w) <= 1.001e-9 * np.linalg.norm(w)
+    op.close()
