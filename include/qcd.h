@@ -346,6 +346,14 @@ long long qcd_selftest_fastdiv(void);
 long long qcd_selftest_site_order(void);
 
 /*
+ * Host-only self-test of the block fixed-point arithmetic of the FP64 operators (the same functions,
+ * evaluated on the host): conversions of doubles of every size there and back, and sums of products of
+ * random and of extreme operands, up to the stated bounds, against exact integer arithmetic.  Returns the
+ * number of mismatches (0 on success); needs no GPU and no context.
+ */
+long long qcd_selftest_fixed(void);
+
+/*
  * Time decomposition over several GPUs (one process per GPU).  The paper runs its application as MPI
  * processes that each hold part of the lattice and exchange boundary data between kernels (Sec. 4);
  * here the global lattice X x Y x Z x T is cut into slabs of consecutive time slices, one per rank.

@@ -19,6 +19,7 @@
 
 #include "qcd.h"
 #include "qcd_dslash.cuh"
+#include "qcd_fixed.cuh"
 #include "qcd_kernels.h"
 #include "qcd_force.h"
 #include "qcd_api_scope.h"
@@ -52,6 +53,7 @@ qcd_status fail(qcd_status s, const char* fmt, ...) {
 
 enum Slot {
   S_IN, S_OUT, S_T, S_Y, S_IN_N, S_OUT_N, S_T_N, S_Y_N,   // qcd_dslash
+  S_AP_HI_N, S_T_HI_N, S_Y_HI_N,                         // exponents of FP64 solver fields in fixed point
   S_CANON,                                               // canonical staging
   S_B_HI, S_X_HI, S_AP_HI, S_T_HI, S_Y_HI,               // FP64 solver fields
   S_X_LO, S_R_LO, S_P, S_AP, S_TL, S_YL,                 // inner solver fields
@@ -81,9 +83,11 @@ struct ProfPending {
 
 struct SolverFields {
   int pr, pp;  // precision of x_lo/r_lo and of p/Ap/temporaries
+  int hp, pad;  // representation of the FP64 operator's fields: 64, or 60 (block fixed point)
   double2 *b_hi, *x_hi, *ap_hi, *t_hi, *y_hi;
   void *x_lo, *r_lo, *p, *ap, *t, *y;
   float *x_lo_n, *r_lo_n, *p_n, *ap_n, *t_n, *y_n;
+  float *ap_hi_n, *t_hi_n, *y_hi_n;  // exponents (hp = 60)
 };
 
 // one profiled launch inside a captured graph: an event pair recorded by the graph itself
@@ -127,6 +131,11 @@ struct qcd_ctx {
   void* g16 = nullptr;
   int recon = 18;
   bool have_gauge = false;
+  // the FP64 operators' operands in block fixed point (qcd_fixed.cuh), for near-unitary links: null where
+  // they could not be allocated or on t-slabs, which keep the FP64 kernels
+  void* gfx = nullptr;
+  FxClover cfx{};
+  bool fx_links = false;
   // clover
   void* A64 = nullptr;
   void* Ainv64 = nullptr;
@@ -199,8 +208,9 @@ const int MAX_RHS = 8;
 // rounds (persistent segment + gated reliable update) enqueued per look at the solver state
 const int PC_MAX_ROUNDS = 32;
 
+// precision 60: block fixed point (FP64 operators)
 size_t spinor_bytes(const Geom& g, int prec, int nrhs) {
-  const size_t per = prec == 64 ? 192 : (prec == 32 ? 96 : 48);
+  const size_t per = prec >= 60 ? 192 : (prec == 32 ? 96 : 48);
   return per * (size_t)g.Vh * nrhs;
 }
 
@@ -229,6 +239,14 @@ void destroy_graph(ItGraph* gph) {
   if (gph->exec) cudaGraphExecDestroy(gph->exec);
   for (auto e : gph->events) cudaEventDestroy(e);
   delete gph;
+}
+
+// device memory that the library can do without: false (and no error left behind) if there is none
+bool try_alloc(void** p, size_t bytes) {
+  if (cudaMalloc(p, bytes) == cudaSuccess) return true;
+  cudaGetLastError();
+  *p = nullptr;
+  return false;
 }
 
 // --------------------------------------------------------------- profiling --
@@ -304,19 +322,19 @@ void prof_collect(qcd_ctx* c) {
 }
 
 // ------------------------------------------------------ operator helpers --
-int real_bytes(int prec) { return prec == 64 ? 8 : (prec == 32 ? 4 : 2); }
+int real_bytes(int prec) { return prec >= 60 ? 8 : (prec == 32 ? 4 : 2); }
 
 void dslash_cost(const qcd_ctx* c, int prec, int epi, int nrhs, double* bytes, double* flops) {
   const double Vh = c->g.Vh;
-  const int R = prec == 64 ? 18 : c->recon;
+  const int R = prec >= 60 ? 18 : c->recon;
   const double bl = real_bytes(prec);
-  const double bc = prec == 64 ? 8 : (prec == 32 ? 4 : 2);
+  const double bc = prec >= 60 ? 8 : (prec == 32 ? 4 : 2);
   const double bs = 24.0 * real_bytes(prec) + (prec == 16 ? 4 : 0);
   double site = 8.0 * R * bl + (epi != EPI_NONE ? 72.0 * bc : 0.0);
   double rhs = bs * (epi == EPI_XPAY ? 3.0 : 2.0);
   if (epi == EPI_XPAY_CG) {
     // reads in, x, p; reads and writes x_lo, r_lo; writes nothing else
-    const double sr = 24.0 * (prec == 64 ? 8 : 4);
+    const double sr = 24.0 * (prec >= 60 ? 8 : 4);
     rhs = 3.0 * bs + 4.0 * sr;
   }
   *bytes = Vh * site + Vh * nrhs * rhs;
@@ -324,9 +342,14 @@ void dslash_cost(const qcd_ctx* c, int prec, int epi, int nrhs, double* bytes, d
                         (epi == EPI_XPAY_CG ? 96.0 : 0.0));
 }
 
-const void* gauge_ptr(const qcd_ctx* c, int prec) { return prec == 64 ? c->g64 : (prec == 32 ? c->g32 : c->g16); }
+const void* gauge_ptr(const qcd_ctx* c, int prec) {
+  if (prec == 60) return c->gfx;
+  return prec == 64 ? c->g64 : (prec == 32 ? c->g32 : c->g16);
+}
 
+// (precision 60 keeps A on even and A^-1 on odd sites only, the parities the operators use)
 const void* clover_ptr(const qcd_ctx* c, int prec, bool inverse, int parity) {
+  if (prec == 60) return inverse ? c->cfx.Ainv_odd : c->cfx.A_even;
   if (prec == 64) {
     const double2* base = static_cast<const double2*>(inverse ? c->Ainv64 : c->A64);
     return base + (size_t)parity * 36 * c->g.Vh;
@@ -339,6 +362,16 @@ const void* clover_ptr(const qcd_ctx* c, int prec, bool inverse, int parity) {
   return base + (size_t)parity * 18 * c->g.Vh;
 }
 
+const int* clover_exps(const qcd_ctx* c, bool inverse) { return inverse ? c->cfx.eAinv_odd : c->cfx.eA_even; }
+
+// The representation of FP64 operator fields: block fixed point (60) wherever its operands are there, at
+// every size (a hopping pass with the inverse clover block, FP64 pair units -> fixed point: 4^3 x 8
+// 27.3 -> 12.6 us, 16^4 78.3 -> 27.5 us, 32^4 1.07 ms -> 256 us, 4 RHS 4.3 -> 1.05 ms).  Links that are
+// not near-unitary (smeared or scaled ones) and t-slabs keep FP64.
+int fp64_rep(const qcd_ctx* c, bool with_clover) {
+  return c->gfx && c->fx_links && (!with_clover || c->cfx.A_even) ? 60 : 64;
+}
+
 DslashArgs base_args(const qcd_ctx* c, int prec, int parity, int nrhs) {
   DslashArgs a;
   memset(&a, 0, sizeof a);
@@ -346,6 +379,7 @@ DslashArgs base_args(const qcd_ctx* c, int prec, int parity, int nrhs) {
   a.p = parity;
   a.nrhs = nrhs;
   a.gauge = gauge_ptr(c, prec);
+  a.clover_e = clover_exps(c, parity == 1);  // A^-1 on odd, A on even output
   return a;
 }
 
@@ -353,10 +387,19 @@ void run_dslash(qcd_ctx* c, int prec, int epi, const DslashArgs& a) {
   double bytes, flops;
   dslash_cost(c, prec, epi, a.nrhs, &bytes, &flops);
   char name[40];
-  snprintf(name, sizeof name, "dslash_p%d_r%d_%s", prec, prec == 64 ? 18 : c->recon,
+  snprintf(name, sizeof name, "dslash_p%d_r%d_%s", prec >= 60 ? 64 : prec, prec >= 60 ? 18 : c->recon,
            epi == EPI_NONE ? "plain" : (epi == EPI_CLOVER_INV ? "cloverinv" : (epi == EPI_XPAY ? "xpay" : "xpaycg")));
   ProfScope ps(c, name, bytes, flops);
-  launch_dslash(prec, prec == 64 ? 18 : c->recon, epi, a, c->cur);
+  if (prec == 60) launch_dslash_fixed(epi, a, c->cur);
+  else launch_dslash(prec, prec == 64 ? 18 : c->recon, epi, a, c->cur);
+}
+
+// out = A in (even sites) or A^-1 in (odd sites)
+void run_clover(qcd_ctx* c, int prec, bool inverse, const void* in, const float* in_n, void* out, float* out_n,
+                int nrhs) {
+  const void* cl = clover_ptr(c, prec, inverse, inverse ? 1 : 0);
+  if (prec == 60) launch_clover_apply_fixed(c->g, cl, clover_exps(c, inverse), in, in_n, out, out_n, nrhs, c->st);
+  else launch_clover_apply(prec, c->g, cl, in, in_n, out, out_n, nrhs, c->st);
 }
 
 ReduceArgs reduce_args(qcd_ctx* c, int mode) {
@@ -372,10 +415,10 @@ ReduceArgs reduce_args(qcd_ctx* c, int mode) {
 }
 
 // out = Mhat in (dagger: Mhat^dag) on even sites, t: odd temporary.
-// red (may be null) reduces |out|^2 per RHS.
+// red (may be null) reduces |out|^2 per RHS.  out64 (precision 60): out is an FP64 field, not a fixed one.
 void apply_mhat(qcd_ctx* c, int prec, int nrhs, bool dagger, const void* in, const float* in_n, void* out,
                 float* out_n, void* t, float* t_n, const ReduceArgs* red, const int* halt,
-                const int* gate = nullptr) {
+                const int* gate = nullptr, bool out64 = false) {
   const double k2 = c->kappa * c->kappa;
   DslashArgs a = base_args(c, prec, 1, nrhs);
   a.in = in;
@@ -398,6 +441,7 @@ void apply_mhat(qcd_ctx* c, int prec, int nrhs, bool dagger, const void* in, con
   b.a = -k2;
   b.x_g5 = dagger;
   b.out_g5 = dagger;
+  b.out_f64 = out64;
   b.halt = halt;
   b.gate = gate;
   if (red) {
@@ -410,9 +454,9 @@ void apply_mhat(qcd_ctx* c, int prec, int nrhs, bool dagger, const void* in, con
 // out = Mhat^dag Mhat in; y: even temporary, t: odd temporary; pap reduces |Mhat in|^2
 void apply_mdagm(qcd_ctx* c, int prec, int nrhs, const void* in, const float* in_n, void* out, float* out_n, void* t,
                  float* t_n, void* y, float* y_n, const ReduceArgs* pap, const int* halt,
-                 const int* gate = nullptr) {
+                 const int* gate = nullptr, bool out64 = false) {
   apply_mhat(c, prec, nrhs, false, in, in_n, y, y_n, t, t_n, pap, halt, gate);
-  apply_mhat(c, prec, nrhs, true, y, y_n, out, out_n, t, t_n, nullptr, halt, gate);
+  apply_mhat(c, prec, nrhs, true, y, y_n, out, out_n, t, t_n, nullptr, halt, gate, out64);
 }
 
 qcd_status sync_and_check(qcd_ctx* c, const char* what) {
@@ -574,7 +618,7 @@ qcd_status qcd_destroy(qcd_ctx* c) {
   QCD_API_ENTER("qcd_destroy", c);
   if (c->st) cudaStreamSynchronize(c->st);
   else cudaDeviceSynchronize();
-  void* dev[] = {c->g64, c->g32, c->g16, c->A64, c->Ainv64, c->A32, c->Ainv32, c->A16, c->Ainv16, c->logdet, c->flags,
+  void* dev[] = {c->gfx, c->cfx.A_even, c->cfx.Ainv_odd, c->cfx.eA_even, c->cfx.eAinv_odd, c->g64, c->g32, c->g16, c->A64, c->Ainv64, c->A32, c->Ainv32, c->A16, c->Ainv16, c->logdet, c->flags,
                  c->pc_part, c->pc_bar, c->pc_rounds,
                  c->partials, c->counter, c->results, c->cg, c->ctl,
                  c->U_ext, c->ext_g64, c->ext_A64, c->ext_Ainv64, c->ext_A32, c->ext_Ainv32, c->ext_A16, c->ext_Ainv16,
@@ -610,6 +654,7 @@ qcd_status qcd_load_gauge(qcd_ctx* c, const double* U, int on_device, int flags)
     CUDA_TRY(cudaMalloc(&c->g64, canon_bytes));
     CUDA_TRY(cudaMalloc(&c->g32, n_links * 9 * sizeof(float2)));
     CUDA_TRY(cudaMalloc(&c->g16, n_links * 9 * sizeof(uint32_t)));
+    if (!c->slab) try_alloc(&c->gfx, n_links * 9 * sizeof(int4));
   }
   // a t-slab keeps the whole extended field (its clover build reads it); the slab's own links start
   // two time slices in
@@ -630,10 +675,11 @@ qcd_status qcd_load_gauge(qcd_ctx* c, const double* U, int on_device, int flags)
   CUDA_TRY(cudaMemsetAsync(c->flags, 0, 4 * sizeof(int), c->st));
   launch_check_finite(reinterpret_cast<const double*>(src), in_links * 18, c->flags + 1, c->st);
   launch_pack_gauge(g, src + (c->slab ? (size_t)2 * g.XYZ * 4 * 9 : 0), c->g64, c->g32, c->recon, c->g16, c->recon,
-                    c->st);
+                    c->gfx, c->flags + 2, c->st);
   CUDA_TRY(cudaMemcpyAsync(c->h_flags, c->flags, 4 * sizeof(int), cudaMemcpyDeviceToHost, c->st));
   if ((s = sync_and_check(c, "load_gauge"))) return s;
   c->have_clover = false;
+  c->fx_links = c->gfx && !c->h_flags[2];
   if (c->h_flags[1]) {
     c->have_gauge = false;
     return fail(QCD_ERR_NAN, "gauge field holds a non-finite value");
@@ -657,6 +703,15 @@ qcd_status qcd_clover_build(qcd_ctx* c, double kappa, double csw) {
     CUDA_TRY(cudaMalloc(&c->Ainv16, (size_t)2 * 9 * g.Vh * sizeof(uint4)));
     CUDA_TRY(cudaMalloc(&c->logdet, (size_t)2 * 2 * g.Vh * sizeof(double)));
   }
+  if (c->fx_links && !c->cfx.A_even) {
+    void *a = nullptr, *b = nullptr, *ea = nullptr, *eb = nullptr;
+    const size_t blocks = (size_t)36 * g.Vh * sizeof(int4), exps = (size_t)2 * g.Vh * sizeof(int);
+    if (try_alloc(&a, blocks) && try_alloc(&b, blocks) && try_alloc(&ea, exps) && try_alloc(&eb, exps)) {
+      c->cfx = FxClover{a, b, static_cast<int*>(ea), static_cast<int*>(eb)};
+    } else {
+      for (void* p : {a, b, ea, eb}) cudaFree(p);
+    }
+  }
   void* work;
   if ((s = ws_get(c, S_F_CL, force_clover_bytes(c->slab ? c->ge : g), &work))) return s;
   CUDA_TRY(cudaMemsetAsync(c->flags, 0, 4 * sizeof(int), c->st));
@@ -667,7 +722,7 @@ qcd_status qcd_clover_build(qcd_ctx* c, double kappa, double csw) {
     // the two inversions
     ProfScope ps(c, "clover_build", 0, 2.0 * g.Vh * (60 * 216.0 + 2 * 1000.0));
     launch_clover_build(g, c->g64, kappa, csw, c->A64, c->Ainv64, c->A32, c->Ainv32, c->A16, c->Ainv16, work,
-                        c->logdet, c->flags, c->st);
+                        c->logdet, c->flags, c->fx_links ? c->cfx : FxClover{}, c->st);
   }
   CUDA_TRY(cudaMemcpyAsync(c->h_flags, c->flags, 4 * sizeof(int), cudaMemcpyDeviceToHost, c->st));
   if ((s = sync_and_check(c, "clover_build"))) return s;
@@ -697,6 +752,7 @@ qcd_status qcd_dslash(qcd_ctx* c, double* out, const double* in, int op, int dag
   const size_t canon = (size_t)g.Vh * 12 * sizeof(double2);
   if ((const char*)out < (const char*)in + canon * nrhs && (const char*)in < (const char*)out + canon * nrhs)
     return fail(QCD_ERR_ARG, "in and out overlap");
+  if (prec == 64) prec = fp64_rep(c, needs_clover);
   int done = 0;
   while (done < nrhs) {
     const int nb = batch_of(nrhs - done);
@@ -707,7 +763,7 @@ qcd_status qcd_dslash(qcd_ctx* c, double* out, const double* in, int op, int dag
     if ((s = ws_get(c, S_IN, fb, &vin)) || (s = ws_get(c, S_OUT, fb, &vout)) || (s = ws_get(c, S_T, fb, &vt)) ||
         (s = ws_get(c, S_Y, fb, &vy)))
       return s;
-    if (prec == 16) {
+    if (prec == 16 || prec == 60) {
       if ((s = ws_get(c, S_IN_N, nbytes, &nin)) || (s = ws_get(c, S_OUT_N, nbytes, &nout)) ||
           (s = ws_get(c, S_T_N, nbytes, &nt)) || (s = ws_get(c, S_Y_N, nbytes, &ny)))
         return s;
@@ -733,10 +789,10 @@ qcd_status qcd_dslash(qcd_ctx* c, double* out, const double* in, int op, int dag
         apply_mdagm(c, prec, nb, vin, fin, vout, fout, vt, ft, vy, fy, nullptr, nullptr);
         break;
       case QCD_OP_CLOVER:
-        launch_clover_apply(prec, g, clover_ptr(c, prec, false, 0), vin, fin, vout, fout, nb, c->st);
+        run_clover(c, prec, false, vin, fin, vout, fout, nb);
         break;
       case QCD_OP_CLOVER_INV:
-        launch_clover_apply(prec, g, clover_ptr(c, prec, true, 1), vin, fin, vout, fout, nb, c->st);
+        run_clover(c, prec, true, vin, fin, vout, fout, nb);
         break;
     }
     launch_spinor_to_canon(prec, g, vout, fout, cout, nb, c->st);
@@ -756,7 +812,9 @@ namespace {
 
 qcd_status solver_fields(qcd_ctx* c, int inner, int nrhs, SolverFields* f) {
   const Geom& g = c->g;
-  f->pp = inner;
+  f->hp = fp64_rep(c, true);
+  f->pad = 0;
+  f->pp = inner == 64 ? f->hp : inner;
   f->pr = inner == 64 ? 64 : 32;
   qcd_status s;
   void* v;
@@ -776,8 +834,14 @@ qcd_status solver_fields(qcd_ctx* c, int inner, int nrhs, SolverFields* f) {
   GET(S_TL, lo_p, f->t, void*);
   GET(S_YL, lo_p, f->y, void*);
   f->x_lo_n = f->r_lo_n = f->p_n = f->ap_n = f->t_n = f->y_n = nullptr;
-  if (f->pp == 16) {
-    const size_t nb = sizeof(float) * (size_t)g.Vh * nrhs;
+  f->ap_hi_n = f->t_hi_n = f->y_hi_n = nullptr;
+  const size_t nb = sizeof(float) * (size_t)g.Vh * nrhs;
+  if (f->hp == 60) {
+    GET(S_AP_HI_N, nb, f->ap_hi_n, float*);
+    GET(S_T_HI_N, nb, f->t_hi_n, float*);
+    GET(S_Y_HI_N, nb, f->y_hi_n, float*);
+  }
+  if (f->pp == 16 || f->pp == 60) {
     GET(S_P_N, nb, f->p_n, float*);
     GET(S_AP_N, nb, f->ap_n, float*);
     GET(S_TL_N, nb, f->t_n, float*);
@@ -833,7 +897,8 @@ void enqueue_iteration(qcd_ctx* c, const SolverFields& f, int nrhs) {
   b.cg_p_norm = f.p_n;
   run_dslash(c, f.pp, EPI_XPAY_CG, b);
   {
-    const double pb = (double)g.Vh * nrhs * (24.0 * real_bytes(f.pr) + 2 * (24.0 * real_bytes(f.pp) + (f.pp == 16 ? 4 : 0)));
+    const double pb =
+        (double)g.Vh * nrhs * (24.0 * real_bytes(f.pr) + 2 * (24.0 * real_bytes(f.pp) + (f.p_n ? 4 : 0)));
     ProfScope ps(c, "p_update", pb, 0);
     launch_p_update(f.pr, f.pp, g, nrhs, f.r_lo, f.r_lo_n, f.p, f.p_n, c->cg, halt, c->cur);
   }
@@ -846,9 +911,12 @@ void enqueue_iteration(qcd_ctx* c, const SolverFields& f, int nrhs) {
 void enqueue_reliable(qcd_ctx* c, const SolverFields& f, int nrhs, bool gated) {
   const Geom& g = c->g;
   const int* gate = gated ? &c->ctl->rel_go : nullptr;
-  launch_accumulate_x(f.pr, g, nrhs, f.x_hi, f.x_lo, f.x_lo_n, c->cur, gate);
-  apply_mdagm(c, 64, nrhs, f.x_hi, nullptr, f.ap_hi, nullptr, f.t_hi, nullptr, f.y_hi, nullptr, nullptr, nullptr,
-              gate);
+  // in fixed point the operator's input is a copy of x_hi that is kept where its output goes (the last
+  // of the four passes, which writes ap_hi, does not read it any more)
+  void* x_fx = f.hp == 60 ? f.ap_hi : nullptr;
+  launch_accumulate_x(f.pr, g, nrhs, f.x_hi, f.x_lo, f.x_lo_n, c->cur, gate, x_fx, f.ap_hi_n);
+  apply_mdagm(c, f.hp, nrhs, x_fx ? x_fx : f.x_hi, f.ap_hi_n, f.ap_hi, nullptr, f.t_hi, f.t_hi_n, f.y_hi, f.y_hi_n,
+              nullptr, nullptr, gate, true);
   launch_true_residual(f.pr, g, nrhs, f.b_hi, f.ap_hi, f.r_lo, f.r_lo_n, reduce_args(c, FIN_CG_TRUE), c->cur, gate);
   launch_p_update(f.pr, f.pp, g, nrhs, f.r_lo, f.r_lo_n, f.p, f.p_n, c->cg, nullptr, c->cur, gate);
   if (gated) launch_gate_clear(&c->ctl->rel_go, c->cur);
@@ -1136,9 +1204,11 @@ qcd_status cg_batch(qcd_ctx* c, double2* x, const double2* b, int nrhs, const qc
   launch_zero(f.x_lo, spinor_bytes(g, f.pr, nrhs), c->st);
   launch_zero(f.p, spinor_bytes(g, f.pp, nrhs), c->st);
   if (f.p_n) launch_zero(f.p_n, sizeof(float) * (size_t)g.Vh * nrhs, c->st);
-  if (prm->use_x0)
-    apply_mdagm(c, 64, nrhs, f.x_hi, nullptr, f.ap_hi, nullptr, f.t_hi, nullptr, f.y_hi, nullptr, nullptr, nullptr);
-  else
+  if (prm->use_x0) {
+    if (f.hp == 60) launch_spinor_to_native(60, g, x, f.ap_hi, f.ap_hi_n, nrhs, c->st);
+    apply_mdagm(c, f.hp, nrhs, f.hp == 60 ? f.ap_hi : f.x_hi, f.ap_hi_n, f.ap_hi, nullptr, f.t_hi, f.t_hi_n, f.y_hi,
+                f.y_hi_n, nullptr, nullptr, nullptr, true);
+  } else
     launch_zero(f.ap_hi, spinor_bytes(g, 64, nrhs), c->st);
   launch_true_residual(f.pr, g, nrhs, f.b_hi, f.ap_hi, f.r_lo, f.r_lo_n, reduce_args(c, FIN_CG_TRUE), c->st);
   launch_p_update(f.pr, f.pp, g, nrhs, f.r_lo, f.r_lo_n, f.p, f.p_n, c->cg, nullptr, c->st);
@@ -1155,7 +1225,7 @@ qcd_status cg_batch(qcd_ctx* c, double2* x, const double2* b, int nrhs, const qc
   // one RHS: the persistent kernel runs each segment of iterations, and the rounds (segment, gated
   // reliable update) expected before convergence are enqueued together, with one look at the state
   // after them
-  const bool use_pc = c->persistent && nrhs == 1 && g.Vh <= PERSISTENT_MAX_VH;
+  const bool use_pc = c->persistent && nrhs == 1 && f.pp != 60 && g.Vh <= PERSISTENT_MAX_VH;
   qcd_status result = QCD_OK;
   bool after_reliable = true;
   int done_iters = 0;
@@ -1380,20 +1450,36 @@ qcd_status qcd_fermion_force(qcd_ctx* c, double* F, const double* phi_or_x, int 
     batches.push_back({(size_t)done * 12 * g.Vh, nb});
     done += nb;
   }
+  const int rep = fp64_rep(c, true);
   for (size_t k = 0; k < batches.size(); k++) {
     const size_t off = batches[k].first;
     const int nb = batches[k].second;
     launch_spinor_to_native(64, g, X + off, Xe + off, nullptr, nb, c->st);
+    void *x = Xe + off, *y = Ye + off, *t = Xo + off, *xn = nullptr, *yn = nullptr, *tn = nullptr;
+    if (rep == 60) {
+      // the operators' fields in fixed point; the FP64 copies that the kernels below read are made from them
+      const size_t fb = spinor_bytes(g, 60, nb), eb = sizeof(int) * (size_t)g.Vh * nb;
+      if ((s = ws_get(c, S_IN, fb, &x)) || (s = ws_get(c, S_Y, fb, &y)) || (s = ws_get(c, S_T, fb, &t)) ||
+          (s = ws_get(c, S_IN_N, eb, &xn)) || (s = ws_get(c, S_Y_N, eb, &yn)) || (s = ws_get(c, S_T_N, eb, &tn)))
+        return s;
+      launch_spinor_to_native(60, g, X + off, x, (float*)xn, nb, c->st);
+    }
     // Y_e = Mhat X_e with X_o = A_oo^-1 D_oe X_e left in the odd temporary
-    apply_mhat(c, 64, nb, false, Xe + off, nullptr, Ye + off, nullptr, Xo + off, nullptr, nullptr, nullptr);
+    apply_mhat(c, rep, nb, false, x, (float*)xn, y, (float*)yn, t, (float*)tn, nullptr, nullptr);
+    if (rep == 60) {
+      launch_fixed_to_double(g, y, (float*)yn, Ye + off, nb, c->st);
+      launch_fixed_to_double(g, t, (float*)tn, Xo + off, nb, c->st);
+    }
     // Y_o = A_oo^-1 D_eo^dag Y_e = g5 A_oo^-1 D_oe g5 Y_e
-    DslashArgs a = base_args(c, 64, 1, nb);
-    a.in = Ye + off;
+    DslashArgs a = base_args(c, rep, 1, nb);
+    a.in = y;
+    a.in_norm = (float*)yn;
     a.out = Yo + off;
-    a.clover = clover_ptr(c, 64, true, 1);
+    a.out_f64 = 1;
+    a.clover = clover_ptr(c, rep, true, 1);
     a.in_g5 = 1;
     a.out_g5 = 1;
-    run_dslash(c, 64, EPI_CLOVER_INV, a);
+    run_dslash(c, rep, EPI_CLOVER_INV, a);
     ProfScope ps(c, "force_clover_coeff", V * (nb * 2 * 192.0 + 6 * 144.0), V * force_coeff_flops(nb));
     launch_force_coeff(g, c->kappa, c->csw, nb, Xe + off, Xo + off, Ye + off, Yo + off, static_cast<double2*>(clf),
                        k > 0, c->st);
@@ -1444,6 +1530,7 @@ qcd_status qcd_debug_violations(qcd_ctx* c, unsigned* violations, int* is_debug)
   if (!violations) return fail(QCD_ERR_ARG, "null pointer");
   if ((s = sync_and_check(c, "debug_violations"))) return s;
   *violations = debug_take_blas() | debug_take_cg_persistent() | debug_take_clover() | debug_take_dslash() |
+                debug_take_dslash_fx() |
                 debug_take_force() | debug_take_halo() | debug_take_layout() | debug_take_md() |
                 debug_take_probe();
   if (is_debug) *is_debug = QCD_DEBUG;
@@ -1504,23 +1591,27 @@ qcd_status qcd_prepare_source(qcd_ctx* c, double* bhat_e, const double* b_e, con
   const Geom& g = c->g;
   const size_t n = (size_t)g.Vh * 12;
   for (int done = 0; done < nrhs;) {
-    const int nb = batch_of(nrhs - done);
+    const int nb = batch_of(nrhs - done), rep = fp64_rep(c, true);
     const double2* ce = reinterpret_cast<const double2*>(b_e) + done * n;
     double2* cout = reinterpret_cast<double2*>(bhat_e) + done * n;
     if (!b_o) {
       CUDA_TRY(cudaMemcpyAsync(cout, ce, n * nb * sizeof(double2), cudaMemcpyDeviceToDevice, c->st));
     } else {
-      void *u, *t;
-      const size_t fb = spinor_bytes(g, 64, nb);
-      if ((s = ws_get(c, S_IN, fb, &u)) || (s = ws_get(c, S_T, fb, &t))) return s;
+      void *u, *t, *un, *tn;
+      const size_t fb = spinor_bytes(g, rep, nb), eb = sizeof(int) * (size_t)g.Vh * nb;
+      if ((s = ws_get(c, S_IN, fb, &u)) || (s = ws_get(c, S_T, fb, &t)) || (s = ws_get(c, S_IN_N, eb, &un)) ||
+          (s = ws_get(c, S_T_N, eb, &tn)))
+        return s;
       // t = A_oo^-1 b_o, u = D_eo t (native), bhat_e = kappa u + b_e (canonical)
-      launch_spinor_to_native(64, g, reinterpret_cast<const double2*>(b_o) + done * n, u, nullptr, nb, c->st);
-      launch_clover_apply(64, g, clover_ptr(c, 64, true, 1), u, nullptr, t, nullptr, nb, c->st);
-      DslashArgs a = base_args(c, 64, 0, nb);
+      launch_spinor_to_native(rep, g, reinterpret_cast<const double2*>(b_o) + done * n, u, (float*)un, nb, c->st);
+      run_clover(c, rep, true, u, (float*)un, t, (float*)tn, nb);
+      DslashArgs a = base_args(c, rep, 0, nb);
       a.in = t;
+      a.in_norm = (float*)tn;
       a.out = u;
-      run_dslash(c, 64, EPI_NONE, a);
-      launch_spinor_to_canon(64, g, u, nullptr, cout, nb, c->st);
+      a.out_norm = (float*)un;
+      run_dslash(c, rep, EPI_NONE, a);
+      launch_spinor_to_canon(rep, g, u, (float*)un, cout, nb, c->st);
       launch_axpby(n * nb, 1.0, ce, c->kappa, cout, c->st);
     }
     done += nb;
@@ -1538,26 +1629,30 @@ qcd_status qcd_reconstruct_odd(qcd_ctx* c, double* x_o, const double* x_e, const
   const Geom& g = c->g;
   const size_t n = (size_t)g.Vh * 12;
   for (int done = 0; done < nrhs;) {
-    const int nb = batch_of(nrhs - done);
-    void *u, *t;
-    const size_t fb = spinor_bytes(g, 64, nb);
-    if ((s = ws_get(c, S_IN, fb, &u)) || (s = ws_get(c, S_T, fb, &t))) return s;
+    const int nb = batch_of(nrhs - done), rep = fp64_rep(c, true);
+    void *u, *t, *un, *tn;
+    const size_t fb = spinor_bytes(g, rep, nb), eb = sizeof(int) * (size_t)g.Vh * nb;
+    if ((s = ws_get(c, S_IN, fb, &u)) || (s = ws_get(c, S_T, fb, &t)) || (s = ws_get(c, S_IN_N, eb, &un)) ||
+        (s = ws_get(c, S_T_N, eb, &tn)))
+      return s;
     // t = A_oo^-1 D_oe x_e (one fused launch), then x_o = kappa t + A_oo^-1 b_o
-    launch_spinor_to_native(64, g, reinterpret_cast<const double2*>(x_e) + done * n, u, nullptr, nb, c->st);
-    DslashArgs a = base_args(c, 64, 1, nb);
+    launch_spinor_to_native(rep, g, reinterpret_cast<const double2*>(x_e) + done * n, u, (float*)un, nb, c->st);
+    DslashArgs a = base_args(c, rep, 1, nb);
     a.in = u;
+    a.in_norm = (float*)un;
     a.out = t;
-    a.clover = clover_ptr(c, 64, true, 1);
-    run_dslash(c, 64, EPI_CLOVER_INV, a);
+    a.out_norm = (float*)tn;
+    a.clover = clover_ptr(c, rep, true, 1);
+    run_dslash(c, rep, EPI_CLOVER_INV, a);
     double2* cout = reinterpret_cast<double2*>(x_o) + done * n;
-    launch_spinor_to_canon(64, g, t, nullptr, cout, nb, c->st);
+    launch_spinor_to_canon(rep, g, t, (float*)tn, cout, nb, c->st);
     if (b_o) {
-      launch_spinor_to_native(64, g, reinterpret_cast<const double2*>(b_o) + done * n, u, nullptr, nb, c->st);
-      launch_clover_apply(64, g, clover_ptr(c, 64, true, 1), u, nullptr, t, nullptr, nb, c->st);
+      launch_spinor_to_native(rep, g, reinterpret_cast<const double2*>(b_o) + done * n, u, (float*)un, nb, c->st);
+      run_clover(c, rep, true, u, (float*)un, t, (float*)tn, nb);
       // x_o = kappa x_o + (A_oo^-1 b_o): the native result goes through the canonical staging
       void* stage;
       if ((s = ws_get(c, S_CANON, n * nb * sizeof(double2), &stage))) return s;
-      launch_spinor_to_canon(64, g, t, nullptr, static_cast<double2*>(stage), nb, c->st);
+      launch_spinor_to_canon(rep, g, t, (float*)tn, static_cast<double2*>(stage), nb, c->st);
       launch_axpby(n * nb, 1.0, static_cast<const double2*>(stage), c->kappa, cout, c->st);
     } else {
       launch_axpby(n * nb, 0.0, cout, c->kappa, cout, c->st);

@@ -5,6 +5,7 @@
 // FP64 by block_partial / grid_finish (warp shuffles -> shared memory -> per-block partials ->
 // fixed-order sum in the last block), so the scalars of CG are produced on the device and the
 // iteration needs no host round trip.
+#include "qcd_fixed.cuh"
 #include "qcd_kernels.h"
 
 namespace qcd {
@@ -39,8 +40,8 @@ __global__ void __launch_bounds__(BB) p_update_kernel(Geom g, const void* r, con
 }
 
 template <int PR>
-__global__ void __launch_bounds__(BB) accumulate_x_kernel(Geom g, double2* x_hi, void* x_lo, float* xn,
-                                                          const int* gate) {
+__global__ void __launch_bounds__(BB) accumulate_x_kernel(Geom g, double2* x_hi, void* x_lo, float* xn, void* x_fx,
+                                                          float* x_fx_e, const int* gate) {
   using RR = typename Real<PR>::T;
   if (gate && !*gate) return;
   const int k = blockIdx.y;
@@ -58,6 +59,7 @@ __global__ void __launch_bounds__(BB) accumulate_x_kernel(Geom g, double2* x_hi,
   }
   SpinorIO<64>::store(x_hi, nullptr, g.Vh, k, h, hi);
   SpinorIO<PR>::store(x_lo, xn, g.Vh, k, h, lo);
+  if (x_fx) SpinorIO<60>::store(x_fx, x_fx_e, g.Vh, k, h, hi);
 }
 
 template <int PR>
@@ -200,16 +202,17 @@ __global__ void finalize_kernel(ReduceArgs red, const double* totals, int nrhs) 
 void launch_p_update(int prec_r, int prec_p, const Geom& g, int nrhs, const void* r, const float* rn, void* p,
                      float* pn, const CGState* cg, const int* halt, cudaStream_t st, const int* gate) {
   g_kernel_launches += 1;
-  if (prec_r == 64) p_update_kernel<64, 64><<<grid2(g, nrhs), BB, 0, st>>>(g, r, rn, p, pn, cg, halt, gate);
+  if (prec_p == 60) p_update_kernel<64, 60><<<grid2(g, nrhs), BB, 0, st>>>(g, r, rn, p, pn, cg, halt, gate);
+  else if (prec_r == 64) p_update_kernel<64, 64><<<grid2(g, nrhs), BB, 0, st>>>(g, r, rn, p, pn, cg, halt, gate);
   else if (prec_p == 32) p_update_kernel<32, 32><<<grid2(g, nrhs), BB, 0, st>>>(g, r, rn, p, pn, cg, halt, gate);
   else p_update_kernel<32, 16><<<grid2(g, nrhs), BB, 0, st>>>(g, r, rn, p, pn, cg, halt, gate);
 }
 
 void launch_accumulate_x(int prec_r, const Geom& g, int nrhs, double2* x_hi, void* x_lo, float* x_lon,
-                         cudaStream_t st, const int* gate) {
+                         cudaStream_t st, const int* gate, void* x_fx, float* x_fx_e) {
   g_kernel_launches += 1;
-  if (prec_r == 64) accumulate_x_kernel<64><<<grid2(g, nrhs), BB, 0, st>>>(g, x_hi, x_lo, x_lon, gate);
-  else accumulate_x_kernel<32><<<grid2(g, nrhs), BB, 0, st>>>(g, x_hi, x_lo, x_lon, gate);
+  if (prec_r == 64) accumulate_x_kernel<64><<<grid2(g, nrhs), BB, 0, st>>>(g, x_hi, x_lo, x_lon, x_fx, x_fx_e, gate);
+  else accumulate_x_kernel<32><<<grid2(g, nrhs), BB, 0, st>>>(g, x_hi, x_lo, x_lon, x_fx, x_fx_e, gate);
 }
 
 void launch_debug_index_probe(const Geom& g, const double2* buf, double* out, cudaStream_t st) {

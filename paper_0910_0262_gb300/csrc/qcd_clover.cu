@@ -11,6 +11,7 @@
 //   b = 1: B1 = F_yz + F_xt, B2 = F_xz - F_yt, B3 = F_xy + F_zt.
 // The inverse is formed once per gauge field in FP64 by a Cholesky factorisation
 // A_b = L L^dag and A_b^-1 = L^-dag L^-1; a non-positive pivot raises a flag.
+#include "qcd_fixed.cuh"
 #include "qcd_kernels.h"
 #include "qcd_su3.cuh"
 
@@ -192,7 +193,7 @@ __global__ void __launch_bounds__(128) field_strength_kernel(Geom g, const doubl
 __global__ void __launch_bounds__(128) clover_assemble_kernel(Geom g, const double2* __restrict__ Fbuf, double kappa,
                                                               double csw, double2* A64, double2* Ainv64, float4* A32,
                                                               float4* Ainv32, uint4* A16, uint4* Ainv16,
-                                                              double* logdet, int* notposdef) {
+                                                              double* logdet, int* notposdef, FxClover fx) {
   const int V = 2 * g.Vh;
   const int tid = blockIdx.x * blockDim.x + threadIdx.x;
   if (tid >= 2 * V) return;
@@ -243,6 +244,11 @@ __global__ void __launch_bounds__(128) clover_assemble_kernel(Geom g, const doub
   logdet[((size_t)p * 2 + b) * g.Vh + h] = ld;
   store_block64(A64 + (size_t)p * 36 * g.Vh, g.Vh, h, b, d, L);
   store_block64(Ainv64 + (size_t)p * 36 * g.Vh, g.Vh, h, b, di, Li);
+  if (fx.A_even) {
+    const size_t at = (size_t)b * 18 * g.Vh + h;
+    if (p == 0) fx.eA_even[(size_t)b * g.Vh + h] = fx_store_clover(static_cast<int4*>(fx.A_even) + at, g.Vh, d, L);
+    else fx.eAinv_odd[(size_t)b * g.Vh + h] = fx_store_clover(static_cast<int4*>(fx.Ainv_odd) + at, g.Vh, di, Li);
+  }
   if (A32) store_block32(A32 + (size_t)p * 18 * g.Vh, g.Vh, h, b, d, L);
   if (Ainv32) store_block32(Ainv32 + (size_t)p * 18 * g.Vh, g.Vh, h, b, di, Li);
   if (A16) store_block16(A16 + (size_t)p * 9 * g.Vh, g.Vh, h, b, d, L);
@@ -268,7 +274,7 @@ __global__ void clover_apply_kernel(Geom g, const void* clov, const void* in, co
 
 void launch_clover_build(const Geom& g, const void* g64, double kappa, double csw, void* A64, void* Ainv64, void* A32,
                          void* Ainv32, void* A16, void* Ainv16, void* work, double* logdet, int* notposdef,
-                         cudaStream_t st) {
+                         const FxClover& fx, cudaStream_t st) {
   const int B = 128;
   const long long V = 2LL * g.Vh;
   // F per (site, plane), then one chiral block per thread
@@ -278,7 +284,7 @@ void launch_clover_build(const Geom& g, const void* g64, double kappa, double cs
   clover_assemble_kernel<<<(int)((2 * V + B - 1) / B), B, 0, st>>>(
       g, static_cast<const double2*>(work), kappa, csw, static_cast<double2*>(A64), static_cast<double2*>(Ainv64),
       static_cast<float4*>(A32), static_cast<float4*>(Ainv32), static_cast<uint4*>(A16), static_cast<uint4*>(Ainv16),
-      logdet, notposdef);
+      logdet, notposdef, fx);
 }
 
 void launch_clover_apply(int prec, const Geom& g, const void* clover, const void* in, const float* in_norm, void* out,

@@ -36,6 +36,8 @@ struct DslashArgs {
   const void* x;           // EPI_XPAY local term (parity p)
   const float* x_norm;
   const void* clover;      // clover block field of parity p (A or A^-1)
+  const int* clover_e;     // fixed-point kernels: its exponents [2][Vh]
+  int out_f64;             // fixed-point kernels: out is an FP64 field (else block fixed point)
   double a;                // EPI_XPAY coefficient on the hopping sum
   int in_g5;               // apply gamma_5 to the input before hopping
   int x_g5;                // apply gamma_5 to x before the clover multiply

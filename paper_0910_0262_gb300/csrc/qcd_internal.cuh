@@ -18,6 +18,7 @@
 #include <cuda_fp16.h>
 #include <cuda_runtime.h>
 #include <stdint.h>
+#include <string.h>
 
 namespace qcd {
 
@@ -839,10 +840,12 @@ __device__ __forceinline__ void block_partial(double v, int r, int blk, int nblk
   __syncthreads();
 }
 
+// BLOCK 0: a block size known at run time.
 template <int BLOCK>
 __device__ __forceinline__ void grid_finish(int nrhs, long long blk_total, int nblk, const ReduceArgs& ra) {
-  __shared__ double sm[BLOCK / 32];
+  __shared__ double sm[BLOCK ? BLOCK / 32 : 32];
   __shared__ bool is_last;
+  const int threads = BLOCK ? BLOCK : (int)blockDim.x;
   const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
   __threadfence();
   __syncthreads();
@@ -858,11 +861,11 @@ __device__ __forceinline__ void grid_finish(int nrhs, long long blk_total, int n
     // issued together (a grid of 32768 blocks leaves 256 partials per thread of a 128-thread block)
     constexpr int U = 16;
     double s = 0.0;
-    for (int j0 = threadIdx.x; j0 < nblk; j0 += U * BLOCK) {
+    for (int j0 = threadIdx.x; j0 < nblk; j0 += U * threads) {
       double v[U];
 #pragma unroll
       for (int u = 0; u < U; u++) {
-        const int j = j0 + u * BLOCK;
+        const int j = j0 + u * threads;
         const long long slot = (long long)r * nblk + j;
         v[u] = (j < nblk && slot < ra.capacity) ? __ldcg(ra.partials + slot) : 0.0;
       }
@@ -875,7 +878,7 @@ __device__ __forceinline__ void grid_finish(int nrhs, long long blk_total, int n
     __syncthreads();
     if (threadIdx.x == 0) {
       double tot = 0.0;
-      for (int w = 0; w < BLOCK / 32; w++) tot += sm[w];
+      for (int w = 0; w < threads / 32; w++) tot += sm[w];
       finalize_total(ra, r, tot);
     }
   }

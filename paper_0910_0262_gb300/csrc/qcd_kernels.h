@@ -54,22 +54,34 @@ cudaError_t launch_cg_persistent(int prec, int recon, const PersistentCGArgs& q,
 // one grid barrier that a block never reaches (the wait must give up and set *err)
 cudaError_t launch_barrier_probe(unsigned* count, int* err, cudaStream_t st);
 
-// ---- layout (qcd_layout.cu)
+// ---- layout (qcd_layout.cu); prec 60 names block fixed point (qcd_fixed.cuh) with norm its exponents
+// gfx (may be null): the block fixed-point links; *not_unitary is set if a link is not near-unitary
 void launch_pack_gauge(const Geom& g, const double2* canon, void* g64, void* g32, int recon32, void* g16,
-                       int recon16, cudaStream_t st);
+                       int recon16, void* gfx, int* not_unitary, cudaStream_t st);
 void launch_spinor_to_native(int prec, const Geom& g, const double2* canon, void* nat, float* norm, int nrhs,
                              cudaStream_t st);
 void launch_spinor_to_canon(int prec, const Geom& g, const void* nat, const float* norm, double2* canon, int nrhs,
                             cudaStream_t st);
+// an FP64 native field from a block fixed-point one
+void launch_fixed_to_double(const Geom& g, const void* in, const float* ex, void* out, int nrhs, cudaStream_t st);
 void launch_check_finite(const double* data, size_t n, int* flag, cudaStream_t st);
 
 // ---- clover (qcd_clover.cu)
+// the block fixed-point copies the operators read: A on even sites, A^-1 on odd sites, [36][Vh] int4 each
+// with exponents [2][Vh] (null: not kept)
+struct FxClover {
+  void *A_even, *Ainv_odd;
+  int *eA_even, *eAinv_odd;
+};
 // A (both parities) and A^-1 (both parities) in FP64, FP32 and FP16; flag set if a block is not positive definite.
 // work: 6 * 9 * V double2 for the field strengths (two kernels: F per site and plane, then one chiral
 // block per thread); logdet: [parity][block][Vh] log det of each 6x6 block.
 void launch_clover_build(const Geom& g, const void* g64, double kappa, double csw, void* A64, void* Ainv64,
                          void* A32, void* Ainv32, void* A16, void* Ainv16, void* work, double* logdet,
-                         int* notposdef, cudaStream_t st);
+                         int* notposdef, const FxClover& fx, cudaStream_t st);
+// the same for block fixed-point fields and blocks (clover_e: their exponents [2][Vh])
+void launch_clover_apply_fixed(const Geom& g, const void* clover, const int* clover_e, const void* in,
+                               const float* in_e, void* out, float* out_e, int nrhs, cudaStream_t st);
 // out = C in for a site-local clover field C of parity-matched fields
 void launch_clover_apply(int prec, const Geom& g, const void* clover, const void* in, const float* in_norm,
                          void* out, float* out_norm, int nrhs, cudaStream_t st);
@@ -79,6 +91,7 @@ unsigned debug_take_blas();
 unsigned debug_take_cg_persistent();
 unsigned debug_take_clover();
 unsigned debug_take_dslash();
+unsigned debug_take_dslash_fx();
 unsigned debug_take_force();
 unsigned debug_take_halo();
 unsigned debug_take_layout();
@@ -91,6 +104,8 @@ void launch_debug_index_probe(const Geom& g, const double2* buf, double* out, cu
 // ---- hopping term (qcd_dslash.cu)
 struct DslashArgs;
 void launch_dslash(int prec, int recon, int epi, const DslashArgs& a, cudaStream_t st);
+// the FP64 operators on block fixed-point fields (in, x, cg_p; out unless out_f64) and links, any epi
+void launch_dslash_fixed(int epi, const DslashArgs& a, cudaStream_t st);
 // the same operators on the sites of a t-slab, time hops that leave the slab taken from a.halo_lo /
 // a.halo_hi (epi: EPI_NONE, EPI_CLOVER_INV or EPI_XPAY)
 void launch_dslash_halo(int prec, int recon, int epi, const DslashArgs& a, cudaStream_t st);
@@ -107,9 +122,9 @@ void launch_halo_pack(int prec, int recon, const Geom& g, const void* gauge, con
 // p = r + beta p
 void launch_p_update(int prec_r, int prec_p, const Geom& g, int nrhs, const void* r, const float* rn, void* p,
                      float* pn, const CGState* cg, const int* halt, cudaStream_t st, const int* gate = nullptr);
-// x_hi += x_lo ; x_lo = 0
+// x_hi += x_lo ; x_lo = 0 ; x_fx (if given) = x_hi in block fixed point
 void launch_accumulate_x(int prec_r, const Geom& g, int nrhs, double2* x_hi, void* x_lo, float* x_lon,
-                         cudaStream_t st, const int* gate = nullptr);
+                         cudaStream_t st, const int* gate = nullptr, void* x_fx = nullptr, float* x_fx_e = nullptr);
 // r_lo = b - Ap_hi ; |b - Ap_hi|^2 -> reduction (FIN_CG_TRUE)
 void launch_true_residual(int prec_r, const Geom& g, int nrhs, const double2* b, const double2* Ap, void* r_lo,
                           float* r_lon, const ReduceArgs& red, cudaStream_t st, const int* gate = nullptr);

@@ -5,6 +5,7 @@
 // the equivalent goal -- every byte fetched is a byte used -- is met by a
 // component-major, site-minor layout per parity: consecutive threads (sites)
 // read consecutive 8/16-byte words, so no padding is transferred at all.
+#include "qcd_fixed.cuh"
 #include "qcd_kernels.h"
 
 namespace qcd {
@@ -24,9 +25,32 @@ __device__ __forceinline__ void coords_of(const Geom& g, int i, int& x, int& y, 
   t = c[3];
 }
 
-// canonical gauge U[i][mu][3][3] complex128 -> per-parity, per-direction SoA copies
+// whether U U^dag = 1 to 1e-5 (rows 0, 1, 2 of u), in FP32
+__device__ __forceinline__ bool near_unitary(const double2 u[9]) {
+  float2 v[9];
+#pragma unroll
+  for (int k = 0; k < 9; k++) v[k] = make_float2((float)u[k].x, (float)u[k].y);
+  float worst = 0.f;
+#pragma unroll
+  for (int a = 0; a < 3; a++)
+#pragma unroll
+    for (int b = 0; b <= a; b++) {
+      float re = a == b ? -1.f : 0.f, im = 0.f;
+#pragma unroll
+      for (int k = 0; k < 3; k++) {
+        const float2 x = v[3 * a + k], y = v[3 * b + k];
+        re += x.x * y.x + x.y * y.y;
+        im += x.y * y.x - x.x * y.y;
+      }
+      worst = fmaxf(worst, fmaxf(fabsf(re), fabsf(im)));
+    }
+  return worst < 1e-5f;
+}
+
+// canonical gauge U[i][mu][3][3] complex128 -> per-parity, per-direction SoA copies.  gfx: the block
+// fixed-point copy, which serves near-unitary links only; *not_unitary is set if one is not.
 __global__ void pack_gauge_kernel(Geom g, const double2* __restrict__ U, double2* g64, void* g32, int recon32,
-                                  void* g16, int recon16) {
+                                  void* g16, int recon16, int4* gfx, int* not_unitary) {
   const int tid = blockIdx.x * blockDim.x + threadIdx.x;
   const int V = 2 * g.Vh;
   if (tid >= V * 4) return;
@@ -42,6 +66,10 @@ __global__ void pack_gauge_kernel(Geom g, const double2* __restrict__ U, double2
   const size_t base = (size_t)(p * 4 + mu);
 #pragma unroll
   for (int k = 0; k < 9; k++) g64[(base * 9 + k) * g.Vh + h] = u[k];
+  if (gfx) {
+    fx_store_link(gfx + base * 9 * g.Vh + h, g.Vh, u);
+    if (!near_unitary(u)) *not_unitary = 1;
+  }
   if (g32) {
     if (recon32 == 12) {
       float4* q = static_cast<float4*>(g32);
@@ -102,6 +130,15 @@ __global__ void spinor_to_canon_kernel(Geom g, const void* nat, const float* nor
   for (int c = 0; c < 12; c++) dst[c] = make_double2(double(s[c].re), double(s[c].im));
 }
 
+__global__ void fixed_to_double_kernel(Geom g, const void* in, const float* ex, void* out, int nrhs) {
+  const int tid = blockIdx.x * blockDim.x + threadIdx.x;
+  if (tid >= g.Vh * nrhs) return;
+  const int r = tid / g.Vh, h = tid - r * g.Vh;
+  cx<double> s[12];
+  SpinorIO<60>::load(in, ex, g.Vh, r, h, s);
+  SpinorIO<64>::store(out, nullptr, g.Vh, r, h, s);
+}
+
 __global__ void check_finite_kernel(const double* __restrict__ d, size_t n, int* flag) {
   size_t i = blockIdx.x * (size_t)blockDim.x + threadIdx.x;
   const size_t stride = (size_t)gridDim.x * blockDim.x;
@@ -115,11 +152,11 @@ inline int nblocks(long long n, int b) { return (int)((n + b - 1) / b); }
 }  // namespace
 
 void launch_pack_gauge(const Geom& g, const double2* canon, void* g64, void* g32, int recon32, void* g16,
-                       int recon16, cudaStream_t st) {
+                       int recon16, void* gfx, int* not_unitary, cudaStream_t st) {
   g_kernel_launches += 1;
   const int B = 128;
   pack_gauge_kernel<<<nblocks(8LL * g.Vh, B), B, 0, st>>>(g, canon, static_cast<double2*>(g64), g32, recon32, g16,
-                                                          recon16);
+                                                          recon16, static_cast<int4*>(gfx), not_unitary);
 }
 
 void launch_spinor_to_native(int prec, const Geom& g, const double2* canon, void* nat, float* norm, int nrhs,
@@ -127,7 +164,8 @@ void launch_spinor_to_native(int prec, const Geom& g, const double2* canon, void
   g_kernel_launches += 1;
   const int B = 128;
   const int nb = nblocks((long long)g.Vh * nrhs, B);
-  if (prec == 64) spinor_to_native_kernel<64><<<nb, B, 0, st>>>(g, canon, nat, norm, nrhs);
+  if (prec == 60) spinor_to_native_kernel<60><<<nb, B, 0, st>>>(g, canon, nat, norm, nrhs);
+  else if (prec == 64) spinor_to_native_kernel<64><<<nb, B, 0, st>>>(g, canon, nat, norm, nrhs);
   else if (prec == 32) spinor_to_native_kernel<32><<<nb, B, 0, st>>>(g, canon, nat, norm, nrhs);
   else spinor_to_native_kernel<16><<<nb, B, 0, st>>>(g, canon, nat, norm, nrhs);
 }
@@ -137,9 +175,16 @@ void launch_spinor_to_canon(int prec, const Geom& g, const void* nat, const floa
   g_kernel_launches += 1;
   const int B = 128;
   const int nb = nblocks((long long)g.Vh * nrhs, B);
-  if (prec == 64) spinor_to_canon_kernel<64><<<nb, B, 0, st>>>(g, nat, norm, canon, nrhs);
+  if (prec == 60) spinor_to_canon_kernel<60><<<nb, B, 0, st>>>(g, nat, norm, canon, nrhs);
+  else if (prec == 64) spinor_to_canon_kernel<64><<<nb, B, 0, st>>>(g, nat, norm, canon, nrhs);
   else if (prec == 32) spinor_to_canon_kernel<32><<<nb, B, 0, st>>>(g, nat, norm, canon, nrhs);
   else spinor_to_canon_kernel<16><<<nb, B, 0, st>>>(g, nat, norm, canon, nrhs);
+}
+
+void launch_fixed_to_double(const Geom& g, const void* in, const float* ex, void* out, int nrhs, cudaStream_t st) {
+  g_kernel_launches += 1;
+  const int B = 128;
+  fixed_to_double_kernel<<<nblocks((long long)g.Vh * nrhs, B), B, 0, st>>>(g, in, ex, out, nrhs);
 }
 
 void launch_check_finite(const double* data, size_t n, int* flag, cudaStream_t st) {

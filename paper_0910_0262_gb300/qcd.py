@@ -89,6 +89,7 @@ _SIGNATURES = {
     "qcd_selftest_barrier_timeout": (ctypes.c_int, [_P]),
     "qcd_selftest_fastdiv": (ctypes.c_longlong, []),
     "qcd_selftest_site_order": (ctypes.c_longlong, []),
+    "qcd_selftest_fixed": (ctypes.c_longlong, []),
     "qcd_clover_logdet": (ctypes.c_int, [_P, ctypes.POINTER(ctypes.c_double)]),
     "qcd_prepare_source": (ctypes.c_int, [_P, _P, _P, _P, ctypes.c_int]),
     "qcd_reconstruct_odd": (ctypes.c_int, [_P, _P, _P, _P, ctypes.c_int]),
@@ -304,6 +305,11 @@ def qcd_selftest_fastdiv():
 def qcd_selftest_site_order():
     """Lattices on which the staged FP32 kernel's block order is not a permutation (host only)."""
     return lib().qcd_selftest_site_order()
+
+
+def qcd_selftest_fixed():
+    """Mismatches of the FP64 operators' block fixed-point arithmetic against exact integers (host only)."""
+    return lib().qcd_selftest_fixed()
 
 
 def qcd_probe_fma_peak(precision=64, stream=None):

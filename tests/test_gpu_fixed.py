@@ -1,0 +1,131 @@
+"""The FP64 operators on block fixed-point integers (near-unitary links) and the FP64 kernels they stand
+beside (other links), against the oracle.
+
+Sizes at the edges of the kernels' blocks of 32 sites: 8 and 24 sites per parity (part of one block), 32
+and 96 (whole blocks), 40, 72, 120 and 1080 (a ragged last block), with 1, 2, 3, 4 and 5 right-hand sides
+(pairs of warps per block: 1, 2, 4; batches 2 + 1 and 4 + 1).  Tolerances: a row of an operator sums at most
+8 x 6 products of a link and 11 of a clover block, each rounded to 2^-53 in FP64, so 1e-15 in the norm; of
+one hopping term, site by site, 16 x 2^-53 of the neighbours' largest values.
+"""
+
+import numpy as np
+import pytest
+
+from oracle import evenodd
+from oracle.lattice import join_eo, split_eo
+from paper_0910_0262_gb300 import synth
+from gpu_util import require_gpu, to_dev, to_np, rel_l2, rand_eo
+
+gpu = pytest.mark.gpu
+DIMS = [(2, 2, 2, 2), (2, 2, 6, 2), (6, 2, 10, 2), (4, 4, 2, 2), (4, 4, 2, 6), (10, 2, 2, 2), (18, 2, 2, 2), (6, 10, 2, 18)]
+KAPPA, CSW = 0.12, 1.0
+
+
+def test_fixed_point_arithmetic():
+    """Conversions, limbs and sums of products against exact integers (host evaluation)."""
+    from paper_0910_0262_gb300 import build, qcd
+    build.build()
+    assert qcd.qcd_selftest_fixed() == 0
+
+
+def _context(dims, t_bc=-1.0, scale=1.0, seed=3, clover=True):
+    from paper_0910_0262_gb300.qcd import CloverWilson
+    U = synth.make_problem(dims, 0.2, seed)[0] * scale
+    op = CloverWilson(dims, t_bc)
+    op.load_gauge(to_dev(U))
+    if clover:
+        op.clover_build(KAPPA, CSW)
+    return U, op
+
+
+@gpu
+@pytest.mark.parametrize("t_bc", [-1.0, 1.0])
+@pytest.mark.parametrize("dims", DIMS, ids=["x".join(map(str, d)) for d in DIMS])
+@pytest.mark.parametrize("scale", [1.0, 1.0 - 4e-6, 1.25], ids=["su3", "near", "far"])
+def test_operators(dims, t_bc, scale):
+    """scale 1 and 1 - 4e-6: fixed point (links unitary to 1e-5); 1.25: the FP64 kernels."""
+    require_gpu()
+    U, op = _context(dims, t_bc, scale)
+    ref = evenodd.SchurOperator(U, KAPPA, CSW, t_bc)
+    rng = np.random.default_rng(11)
+    vh = ref.A_ee.shape[0]
+    table = {(0, 0): ref.D_eo, (0, 1): ref.D_oe_dag, (1, 0): ref.D_oe, (1, 1): ref.D_eo_dag, (2, 0): ref.Mhat,
+             (2, 1): ref.Mhat_dag, (3, 0): ref.MdagM, (4, 0): lambda v: ref.site(ref.A_ee, v),
+             (5, 0): lambda v: ref.site(ref.A_oo_inv, v)}
+    for n in (1, 2, 3, 4, 5):
+        x = rand_eo(n, vh, rng)
+        for (o, dag), f in table.items():
+            got = to_np(op.dslash(to_dev(x), o, dagger=bool(dag), precision=64))
+            assert rel_l2(got, np.stack([f(v) for v in x])) < 1e-15, (n, o, dag)
+    op.close()
+
+
+@gpu
+def test_sites_of_very_different_size():
+    """Each site keeps its own exponent: sites 2^-300 .. 2^300 apart, zero sites, subnormal ones."""
+    require_gpu()
+    dims = (6, 4, 4, 6)
+    U, op = _context(dims, clover=False)
+    ref = evenodd.SchurOperator(U, KAPPA, CSW, -1.0)
+    rng = np.random.default_rng(7)
+    vh = ref.A_ee.shape[0]
+    x = rand_eo(1, vh, rng)
+    x *= (2.0 ** rng.integers(-300, 300, vh))[None, :, None, None]
+    x[0, ::7] = 0.0
+    x[0, 3] = 5e-324
+    x[0, 5] *= 1e-290 / np.abs(x[0, 5]).max()
+    got = to_np(op.dslash(to_dev(x), 0, precision=64))[0]
+    want = ref.D_eo(x[0])
+    big = np.abs(x[0]).max(axis=(1, 2))  # per odd site
+    full = join_eo(None, np.broadcast_to(big[:, None, None], (vh, 4, 3)).astype(complex), dims)
+    near = sum(np.roll(full, s, ax) for ax in range(4) for s in (1, -1))
+    near = split_eo(near, dims)[0].real[:, 0, 0]
+    err = np.abs(got - want).max(axis=(1, 2))
+    assert np.all(err <= 16 * 2.0 ** -53 * np.sqrt(6) * near + 5e-324)
+    # a field of zeros gives zeros
+    assert not np.any(to_np(op.dslash(to_dev(0 * x), 0, precision=64)))
+    op.close()
+
+
+@gpu
+@pytest.mark.parametrize("value", [np.nan, np.inf, -np.inf])
+def test_non_finite_sites_reach_their_neighbours_only(value):
+    require_gpu()
+    dims = (6, 4, 4, 6)
+    U, op = _context(dims)
+    x = rand_eo(1, U.size // 72, np.random.default_rng(9))
+    clean = to_np(op.dslash(to_dev(x), 2, precision=64))[0]
+    mark = np.zeros_like(x[0])
+    mark[17] = 1.0
+    around = lambda f: sum(np.roll(f, s, ax) for ax in range(4) for s in (1, -1))
+    full = join_eo(mark, None, dims)
+    reach = split_eo(full + around(around(full)), dims)[0].real[:, 0, 0] > 0  # two hops, and the site itself
+    x[0, 17, 2, 1] = value
+    got = to_np(op.dslash(to_dev(x), 2, precision=64))[0]
+    finite = np.isfinite(got).all(axis=(1, 2))
+    assert np.array_equal(finite[~reach], np.ones((~reach).sum(), bool)) and not finite[17]
+    assert np.array_equal(got[~reach], clean[~reach])
+    op.close()
+
+
+@gpu
+@pytest.mark.parametrize("nrhs", [1, 2, 3, 8])
+def test_fp64_solve(nrhs):
+    """Plain FP64 conjugate gradients with the search direction in fixed point, and a second kappa on the
+    same context (whose recorded iterations must not be those of the first)."""
+    require_gpu()
+    dims = (6, 4, 4, 6)
+    U, op = _context(dims)
+    vh = U.size // 72
+    b = rand_eo(nrhs, vh, np.random.default_rng(13))
+    for kappa in (KAPPA, 0.11):
+        op.clover_build(kappa, CSW)
+        ref = evenodd.SchurOperator(U, kappa, CSW, -1.0)
+        for prec in (64, 32, 16):
+            x, st, ok = op.cg_solve(to_dev(b), tol=1e-11, inner_prec=prec)
+            assert ok
+            r = np.stack([ref.MdagM(v) for v in to_np(x)]) - b
+            for k in range(nrhs):
+                rel = np.linalg.norm(r[k]) / np.linalg.norm(b[k])
+                assert rel < 1.01e-11 and abs(rel - st[k]["true_rel_resid"]) < 1e-13
+    op.close()
