@@ -128,9 +128,9 @@ qcd_status qcd_destroy(qcd_ctx* ctx);
 qcd_status qcd_load_gauge(qcd_ctx* ctx, const double* U, int on_device, int flags);
 
 /*
- * Build the clover term A (both parities) from the loaded links and invert it
- * on every site in FP64 (Cholesky of each 6x6 chiral block); keeps FP64 and FP32
- * copies.  Returns QCD_ERR_STATE without links, QCD_ERR_NOT_POSDEF if a block
+ * Build the clover term A from the loaded links and factorise it on every site in
+ * FP64 (Cholesky of each 6x6 chiral block); keeps A on even and A^-1 on odd sites,
+ * the ones the operators use.  Returns QCD_ERR_STATE without links, QCD_ERR_NOT_POSDEF if a block
  * is not positive definite.
  */
 qcd_status qcd_clover_build(qcd_ctx* ctx, double kappa, double csw);

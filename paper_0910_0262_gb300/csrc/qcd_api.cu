@@ -58,7 +58,7 @@ enum Slot {
   S_B_HI, S_X_HI, S_AP_HI, S_T_HI, S_Y_HI,               // FP64 solver fields
   S_X_LO, S_R_LO, S_P, S_AP, S_TL, S_YL,                 // inner solver fields
   S_X_LO_N, S_R_LO_N, S_P_N, S_AP_N, S_TL_N, S_YL_N,
-  S_F_X, S_F_Y, S_F_CL, S_F_E,                           // force work fields
+  S_F_X, S_F_Y, S_F_CL, S_F_E, S_F_XN, S_F_YN, S_F_CX,   // force work fields
   S_MD_F, S_MD_PHI,                                      // R-algorithm step
   S_PBP,                                                 // psi-bar psi estimate
   S_COUNT
@@ -721,7 +721,7 @@ qcd_status qcd_clover_build(qcd_ctx* c, double kappa, double csw) {
     // 6 planes x 10 products of 3x3 complex matrices per site (two leaves share a product), plus
     // the two inversions
     ProfScope ps(c, "clover_build", 0, 2.0 * g.Vh * (60 * 216.0 + 2 * 1000.0));
-    launch_clover_build(g, c->g64, kappa, csw, c->A64, c->Ainv64, c->A32, c->Ainv32, c->A16, c->Ainv16, work,
+    launch_clover_build(g, c->g64, c->fx_links ? c->gfx : nullptr, kappa, csw, c->A64, c->Ainv64, c->A32, c->Ainv32, c->A16, c->Ainv16, work,
                         c->logdet, c->flags, c->fx_links ? c->cfx : FxClover{}, c->st);
   }
   CUDA_TRY(cudaMemcpyAsync(c->h_flags, c->flags, 4 * sizeof(int), cudaMemcpyDeviceToHost, c->st));
@@ -1354,6 +1354,67 @@ qcd_status check_params(const qcd_solver_params* p) {
 
 }  // namespace
 
+namespace {
+
+// The force or gradient from the solutions X (canonical, nrhs of them, may be 0 with det) on block fixed-point
+// fields.  *ran = false (and QCD_OK): there was no memory for its work space, and nothing was done.
+qcd_status force_fixed(qcd_ctx* c, double2* F, const double2* X, int nrhs, bool gradient, bool det, bool* ran) {
+  const Geom& g = c->g;
+  qcd_status s = QCD_OK;
+  void *xf = nullptr, *yf = nullptr, *xn = nullptr, *yn = nullptr, *clf, *cxf, *ef;
+  const size_t half = (size_t)nrhs * 12 * g.Vh, hn = (size_t)nrhs * g.Vh;
+  *ran = false;
+  if ((nrhs > 0 && (ws_get(c, S_F_X, 2 * half * sizeof(double2), &xf) || ws_get(c, S_F_Y, 2 * half * sizeof(double2), &yf) ||
+                    ws_get(c, S_F_XN, 2 * hn * sizeof(int), &xn) || ws_get(c, S_F_YN, 2 * hn * sizeof(int), &yn))) ||
+      ws_get(c, S_F_CL, force_clover_bytes(g), &clf) || ws_get(c, S_F_CX, fixed_matrix_bytes(g, 6), &cxf) ||
+      ws_get(c, S_F_E, fixed_matrix_bytes(g, 12), &ef))
+    return QCD_OK;
+  *ran = true;
+  double2 *Xe = static_cast<double2*>(xf), *Xo = Xe + half, *Ye = static_cast<double2*>(yf), *Yo = Ye + half;
+  float *xe = static_cast<float*>(xn), *xo = xe + hn, *ye = static_cast<float*>(yn), *yo = ye + hn;
+  double2* C = static_cast<double2*>(clf);
+  for (int done = 0; done < nrhs;) {
+    const int nb = batch_of(nrhs - done);
+    const size_t off = (size_t)done * 12 * g.Vh, on = (size_t)done * g.Vh;
+    launch_spinor_to_native(60, g, X + off, Xe + off, xe + on, nb, c->st);
+    // Y_e = Mhat X_e with X_o = A_oo^-1 D_oe X_e left in the odd temporary
+    apply_mhat(c, 60, nb, false, Xe + off, xe + on, Ye + off, ye + on, Xo + off, xo + on, nullptr, nullptr);
+    // Y_o = A_oo^-1 D_eo^dag Y_e = g5 A_oo^-1 D_oe g5 Y_e
+    DslashArgs a = base_args(c, 60, 1, nb);
+    a.in = Ye + off;
+    a.in_norm = ye + on;
+    a.out = Yo + off;
+    a.out_norm = yo + on;
+    a.clover = clover_ptr(c, 60, true, 1);
+    a.in_g5 = 1;
+    a.out_g5 = 1;
+    run_dslash(c, 60, EPI_CLOVER_INV, a);
+    done += nb;
+  }
+  const double V = 2.0 * g.Vh;
+  if (nrhs > 0) {
+    ProfScope ps(c, "force_clover_coeff", V * (nrhs * 2 * 192.0 + 6 * 144.0), V * force_coeff_flops(nrhs));
+    launch_force_coeff_fixed(g, c->kappa, c->csw, nrhs, Xe, Xo, Ye, Yo, xe, xo, ye, yo, C, c->st);
+  } else {
+    CUDA_TRY(cudaMemsetAsync(C, 0, force_clover_bytes(g), c->st));
+  }
+  if (det) {
+    ProfScope ps(c, "force_det_coeff", g.Vh * (72 * 16.0) + V * 6 * 144.0 * 2, 0.0);
+    launch_force_det_coeff(g, c->kappa, c->csw, static_cast<const double2*>(clover_ptr(c, 64, true, 1)), C, true, c->st);
+  }
+  {
+    ProfScope ps(c, "force_edges", V * (6 + 4 + 12) * 144.0, V * force_edge_flops());
+    launch_force_edges_fixed(g, c->gfx, C, cxf, ef, c->st);
+  }
+  {
+    ProfScope ps(c, "force_links", 4 * V * (144.0 + 3 * 144.0 + 144.0 + 192.0 * nrhs), 4 * V * force_link_flops(nrhs, true));
+    launch_force_links_fixed(g, c->kappa, nrhs, c->gfx, Xe, Xo, Ye, Yo, xe, xo, ye, yo, ef, F, gradient, c->st);
+  }
+  return sync_and_check(c, "fermion_force");
+}
+
+}  // namespace
+
 extern "C" {
 
 qcd_status qcd_cg_solve(qcd_ctx* c, double* x, const double* b, int nrhs, const qcd_solver_params* prm,
@@ -1395,6 +1456,25 @@ qcd_status qcd_fermion_force(qcd_ctx* c, double* F, const double* phi_or_x, int 
     return fail(QCD_ERR_ARG, "unknown force flags");
   if (!c->have_clover) return fail(QCD_ERR_STATE, "fermion_force before clover_build");
   const Geom& g = c->g;
+  const size_t fs = (size_t)g.Vh * 12;
+  // X (canonical, FP64) for all RHS
+  const double2* X = reinterpret_cast<const double2*>(phi_or_x);
+  if (nrhs > 0 && !(flags & QCD_FORCE_INPUT_IS_SOLUTION)) {
+    if ((s = check_params(prm))) return s;
+    void* v;
+    if ((s = ws_get(c, S_CANON, fs * nrhs * sizeof(double2), &v))) return s;
+    CUDA_TRY(cudaMemsetAsync(v, 0, fs * nrhs * sizeof(double2), c->st));
+    qcd_solver_params p2 = *prm;
+    p2.use_x0 = 0;
+    s = qcd_cg_solve(c, static_cast<double*>(v), phi_or_x, nrhs, &p2, stats);
+    if (s && s != QCD_ERR_NOT_CONVERGED) return s;
+    X = static_cast<const double2*>(v);
+  }
+  if (fp64_rep(c, true) == 60) {
+    bool ran = false;
+    if ((s = force_fixed(c, reinterpret_cast<double2*>(F), X, nrhs, (flags & QCD_FORCE_GRADIENT) != 0, det, &ran)) || ran)
+      return s;
+  }
   if (nrhs == 0) {
     // the determinant term alone: its coefficients into a zeroed buffer, then the leaves
     void* clf;
@@ -1404,7 +1484,7 @@ qcd_status qcd_fermion_force(qcd_ctx* c, double* F, const double* phi_or_x, int 
     {
       ProfScope ps(c, "force_det_coeff", g.Vh * (72 * 16.0) + V * 6 * 144.0 * 2, 0.0);
       launch_force_det_coeff(g, c->kappa, c->csw, static_cast<const double2*>(clover_ptr(c, 64, true, 1)),
-                             static_cast<double2*>(clf), c->st);
+                             static_cast<double2*>(clf), false, c->st);
     }
     void* ef;
     if ((s = ws_get(c, S_F_E, force_edge_bytes(g), &ef))) return s;
@@ -1416,20 +1496,6 @@ qcd_status qcd_fermion_force(qcd_ctx* c, double* F, const double* phi_or_x, int 
     launch_force_links(g, c->kappa, 0, c->g64, nullptr, nullptr, nullptr, nullptr, static_cast<const double2*>(ef),
                        reinterpret_cast<double2*>(F), (flags & QCD_FORCE_GRADIENT) != 0, true, false, c->st);
     return sync_and_check(c, "fermion_force");
-  }
-  const size_t fs = (size_t)g.Vh * 12;
-  // X (canonical, FP64) for all RHS
-  const double2* X = reinterpret_cast<const double2*>(phi_or_x);
-  if (!(flags & QCD_FORCE_INPUT_IS_SOLUTION)) {
-    if ((s = check_params(prm))) return s;
-    void* v;
-    if ((s = ws_get(c, S_CANON, fs * nrhs * sizeof(double2), &v))) return s;
-    CUDA_TRY(cudaMemsetAsync(v, 0, fs * nrhs * sizeof(double2), c->st));
-    qcd_solver_params p2 = *prm;
-    p2.use_x0 = 0;
-    s = qcd_cg_solve(c, static_cast<double*>(v), phi_or_x, nrhs, &p2, stats);
-    if (s && s != QCD_ERR_NOT_CONVERGED) return s;
-    X = static_cast<const double2*>(v);
   }
   // native FP64 X_e, Y_e = Mhat X_e, X_o = A^-1 D_oe X_e, Y_o = g5 A^-1 D_oe g5 Y_e; batches of <= 8 RHS
   const size_t hi1 = spinor_bytes(g, 64, 1);
@@ -1450,36 +1516,20 @@ qcd_status qcd_fermion_force(qcd_ctx* c, double* F, const double* phi_or_x, int 
     batches.push_back({(size_t)done * 12 * g.Vh, nb});
     done += nb;
   }
-  const int rep = fp64_rep(c, true);
   for (size_t k = 0; k < batches.size(); k++) {
     const size_t off = batches[k].first;
     const int nb = batches[k].second;
     launch_spinor_to_native(64, g, X + off, Xe + off, nullptr, nb, c->st);
-    void *x = Xe + off, *y = Ye + off, *t = Xo + off, *xn = nullptr, *yn = nullptr, *tn = nullptr;
-    if (rep == 60) {
-      // the operators' fields in fixed point; the FP64 copies that the kernels below read are made from them
-      const size_t fb = spinor_bytes(g, 60, nb), eb = sizeof(int) * (size_t)g.Vh * nb;
-      if ((s = ws_get(c, S_IN, fb, &x)) || (s = ws_get(c, S_Y, fb, &y)) || (s = ws_get(c, S_T, fb, &t)) ||
-          (s = ws_get(c, S_IN_N, eb, &xn)) || (s = ws_get(c, S_Y_N, eb, &yn)) || (s = ws_get(c, S_T_N, eb, &tn)))
-        return s;
-      launch_spinor_to_native(60, g, X + off, x, (float*)xn, nb, c->st);
-    }
     // Y_e = Mhat X_e with X_o = A_oo^-1 D_oe X_e left in the odd temporary
-    apply_mhat(c, rep, nb, false, x, (float*)xn, y, (float*)yn, t, (float*)tn, nullptr, nullptr);
-    if (rep == 60) {
-      launch_fixed_to_double(g, y, (float*)yn, Ye + off, nb, c->st);
-      launch_fixed_to_double(g, t, (float*)tn, Xo + off, nb, c->st);
-    }
+    apply_mhat(c, 64, nb, false, Xe + off, nullptr, Ye + off, nullptr, Xo + off, nullptr, nullptr, nullptr);
     // Y_o = A_oo^-1 D_eo^dag Y_e = g5 A_oo^-1 D_oe g5 Y_e
-    DslashArgs a = base_args(c, rep, 1, nb);
-    a.in = y;
-    a.in_norm = (float*)yn;
+    DslashArgs a = base_args(c, 64, 1, nb);
+    a.in = Ye + off;
     a.out = Yo + off;
-    a.out_f64 = 1;
-    a.clover = clover_ptr(c, rep, true, 1);
+    a.clover = clover_ptr(c, 64, true, 1);
     a.in_g5 = 1;
     a.out_g5 = 1;
-    run_dslash(c, rep, EPI_CLOVER_INV, a);
+    run_dslash(c, 64, EPI_CLOVER_INV, a);
     ProfScope ps(c, "force_clover_coeff", V * (nb * 2 * 192.0 + 6 * 144.0), V * force_coeff_flops(nb));
     launch_force_coeff(g, c->kappa, c->csw, nb, Xe + off, Xo + off, Ye + off, Yo + off, static_cast<double2*>(clf),
                        k > 0, c->st);
@@ -1487,7 +1537,7 @@ qcd_status qcd_fermion_force(qcd_ctx* c, double* F, const double* phi_or_x, int 
   if (det) {
     ProfScope ps(c, "force_det_coeff", g.Vh * (72 * 16.0) + V * 6 * 144.0 * 2, 0.0);
     launch_force_det_coeff(g, c->kappa, c->csw, static_cast<const double2*>(clover_ptr(c, 64, true, 1)),
-                           static_cast<double2*>(clf), c->st);
+                           static_cast<double2*>(clf), false, c->st);
   }
   {
     ProfScope ps(c, "force_edges", V * (6 + 4 + 12) * 144.0, V * force_edge_flops());
@@ -1531,7 +1581,7 @@ qcd_status qcd_debug_violations(qcd_ctx* c, unsigned* violations, int* is_debug)
   if ((s = sync_and_check(c, "debug_violations"))) return s;
   *violations = debug_take_blas() | debug_take_cg_persistent() | debug_take_clover() | debug_take_dslash() |
                 debug_take_dslash_fx() |
-                debug_take_force() | debug_take_halo() | debug_take_layout() | debug_take_md() |
+                debug_take_force() | debug_take_force_fx() | debug_take_halo() | debug_take_layout() | debug_take_md() |
                 debug_take_probe();
   if (is_debug) *is_debug = QCD_DEBUG;
   cudaError_t e = cudaGetLastError();
@@ -1675,8 +1725,9 @@ qcd_status qcd_gauge_force(qcd_ctx* c, double* F, double beta, int flags) {
     const double V = 2.0 * c->g.Vh;
     ProfScope ps(c, "gauge_force", 4 * V * (18 * 144.0 + 144.0 * ((flags & QCD_FORCE_ACCUMULATE) ? 2 : 1)),
                  4 * V * 13 * 198.0);
-    launch_gauge_force(c->g, beta, c->g64, reinterpret_cast<double2*>(F), (flags & QCD_FORCE_GRADIENT) != 0,
-                       (flags & QCD_FORCE_ACCUMULATE) != 0, c->st);
+    const bool grad = (flags & QCD_FORCE_GRADIENT) != 0, add = (flags & QCD_FORCE_ACCUMULATE) != 0;
+    if (c->fx_links) launch_gauge_force_fixed(c->g, beta, c->gfx, reinterpret_cast<double2*>(F), grad, add, c->st);
+    else launch_gauge_force(c->g, beta, c->g64, reinterpret_cast<double2*>(F), grad, add, c->st);
   }
   cudaError_t e = cudaGetLastError();
   if (e != cudaSuccess) return fail(QCD_ERR_CUDA, "gauge_force launch: %s", cudaGetErrorString(e));
@@ -1689,7 +1740,8 @@ qcd_status qcd_plaquette(qcd_ctx* c, double* mean) {
   qcd_status s = QCD_OK;
   if (!mean) return fail(QCD_ERR_ARG, "null pointer");
   if (!c->have_gauge) return fail(QCD_ERR_STATE, "plaquette before load_gauge");
-  launch_plaquette(c->g, c->g64, reduce_args(c, FIN_STORE), c->st);
+  if (c->fx_links) launch_plaquette_fixed(c->g, c->gfx, reduce_args(c, FIN_STORE), c->st);
+  else launch_plaquette(c->g, c->g64, reduce_args(c, FIN_STORE), c->st);
   CUDA_TRY(cudaMemcpyAsync(c->h_results, c->results, sizeof(double), cudaMemcpyDeviceToHost, c->st));
   if ((s = sync_and_check(c, "plaquette"))) return s;
   *mean = c->h_results[0] / (6.0 * 2.0 * c->g.Vh);

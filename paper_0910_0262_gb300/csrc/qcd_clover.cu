@@ -11,7 +11,7 @@
 //   b = 1: B1 = F_yz + F_xt, B2 = F_xz - F_yt, B3 = F_xy + F_zt.
 // The inverse is formed once per gauge field in FP64 by a Cholesky factorisation
 // A_b = L L^dag and A_b^-1 = L^-dag L^-1; a non-positive pivot raises a flag.
-#include "qcd_fixed.cuh"
+#include "qcd_fxmat.cuh"
 #include "qcd_kernels.h"
 #include "qcd_su3.cuh"
 
@@ -78,8 +78,9 @@ __host__ __device__ constexpr int tri(int i, int j) { return i * (i - 1) / 2 + j
 // Cholesky-based inverse of a Hermitian positive definite 6x6 matrix given as (diag d,
 // strictly-lower L), and log det = sum_j log L_jj^2.  Returns false on a non-positive pivot.  All
 // loops are unrolled, so the packed triangles stay in registers: A = l l^dag (l lower, diagonal ld),
-// m = l^-1 (lower), A^-1 = m^dag m.
-__device__ __forceinline__ bool invert6(const double d[6], const C L[15], double di[6], C Li[15], double* logdet) {
+// m = l^-1 (lower), A^-1 = m^dag m.  inverse false: the factorisation and log det only.
+__device__ __forceinline__ bool invert6(const double d[6], const C L[15], bool inverse, double di[6], C Li[15],
+                                        double* logdet) {
   double ild[6];  // 1 / l_jj: one division per pivot, multiplications elsewhere
   C lo[15];       // strictly-lower part of l
   double ldet = 0.0;
@@ -102,6 +103,8 @@ __device__ __forceinline__ bool invert6(const double d[6], const C L[15], double
     }
   }
   if (!ok) return false;
+  *logdet = ldet;
+  if (!inverse) return true;
   // m = l^-1: m_jj = 1 / l_jj, m_ij = -(sum_{k=j}^{i-1} l_ik m_kj) / l_ii for i > j
   C mo[15];
 #pragma unroll
@@ -128,7 +131,6 @@ __device__ __forceinline__ bool invert6(const double d[6], const C L[15], double
       Li[tri(i, j)] = s;
     }
   }
-  *logdet = ldet;
   return true;
 }
 
@@ -174,7 +176,76 @@ __device__ __forceinline__ void store_block16(uint4* base, int Vh, int h, int b,
   else store_block16_b<1>(base, Vh, h, d, L);
 }
 
-// F_{mu nu} for one (site, plane) per thread into Fbuf[plane][9][V] (V = all sites, lexicographic)
+// Fbuf[plane][9][V]: F_{mu nu} of the site of half index h and parity p at p Vh + h
+
+__device__ __forceinline__ void plane_of(int pl, int& mu, int& nu) {
+  mu = pl < 3 ? 0 : (pl < 5 ? 1 : 2);
+  nu = pl < 3 ? pl + 1 : (pl < 5 ? pl - 1 : 3);
+}
+
+// F_{mu nu} from the block fixed-point links (the expressions of field_strength, leaf by leaf along a row:
+// 11 products of a row instead of 10 of matrices).  Three warps per 32 sites of one parity, a row of F each;
+// blockIdx.y is the plane.
+__global__ void __launch_bounds__(96) field_strength_fixed_kernel(Geom g, const int4* __restrict__ gfx, double2* Fbuf) {
+  __shared__ i64 sm[3][6][32];
+  const int lane = threadIdx.x & 31, row = threadIdx.x >> 5;
+  const int nb = (g.Vh + 31) / 32, p = (int)blockIdx.x / nb, h = ((int)blockIdx.x - p * nb) * 32 + lane;
+  const bool valid = h < g.Vh;
+  const int Vh = g.Vh;
+  const size_t V = 2 * (size_t)Vh;
+  int mu, nu;
+  plane_of(blockIdx.y, mu, nu);
+  cx<i64> M[3] = {};
+  if (valid && dbg_link(Vh, p, mu, h)) {
+    const Site s = site_of(g, p, h);
+    const FxSites f = {gfx, Vh, g.X, g.Y, g.Z, g.T, {s.x, s.y, s.z, s.t}, p};
+    auto at = [&](int sm_, int sn, int dir) { return fx_link_at(f, mu, sm_, nu, sn, dir); };
+    cx<i64> t[3];
+    {  // U_mu(x) [U_nu(x+mu) U_mu(x+nu)^dag U_nu(x)^dag - U_nu(x+mu-nu)^dag U_mu(x-nu)^dag U_nu(x-nu)]
+      const FxRow r = fx_load_row<false>(at(0, 0, mu), Vh, row);
+      fx_row_mul<true>(fx_row_times<true>(fx_row_times<false>(r, at(1, 0, nu), Vh), at(0, 1, mu), Vh), at(0, 0, nu), Vh, M);
+      fx_row_mul<false>(fx_row_times<true>(fx_row_times<true>(r, at(1, -1, nu), Vh), at(0, -1, mu), Vh), at(0, -1, nu), Vh,
+                        t);
+#pragma unroll
+      for (int j = 0; j < 3; j++) M[j] = M[j] - t[j];
+    }
+    {  // [U_nu(x) U_mu(x-mu+nu)^dag U_nu(x-mu)^dag - U_nu(x-nu)^dag U_mu(x-mu-nu)^dag U_nu(x-mu-nu)] U_mu(x-mu)
+      cx<i64> u[3];
+      fx_row_mul<true>(fx_row_times<true>(fx_load_row<false>(at(0, 0, nu), Vh, row), at(-1, 1, mu), Vh), at(-1, 0, nu), Vh,
+                       t);
+      fx_row_mul<false>(fx_row_times<true>(fx_load_row<true>(at(0, -1, nu), Vh, row), at(-1, -1, mu), Vh), at(-1, -1, nu),
+                        Vh, u);
+#pragma unroll
+      for (int j = 0; j < 3; j++) t[j] = t[j] - u[j];
+      fx_row_mul<false>(fx_row(t), at(-1, 0, mu), Vh, u);
+#pragma unroll
+      for (int j = 0; j < 3; j++) M[j] = M[j] + u[j];
+    }
+  }
+#pragma unroll
+  for (int j = 0; j < 3; j++) {
+    sm[row][2 * j][lane] = M[j].re;
+    sm[row][2 * j + 1][lane] = M[j].im;
+  }
+  __syncthreads();
+  if (!valid) return;
+  // F = traceless part of (M - M^dag) / (8 i): the diagonal of M - M^dag is 2 i Im M
+  const i64 tr = sm[0][1][lane] + sm[1][3][lane] + sm[2][5][lane];
+  double2* q = Fbuf + ((size_t)blockIdx.y * 9 + 3 * row) * V + (size_t)p * Vh + h;
+#pragma unroll
+  for (int j = 0; j < 3; j++) {
+    double re, im = 0.0;
+    if (j == row) {
+      re = fx_to_double_in_range(3 * M[j].im - tr, -FX_LINK - 2) * (1.0 / 3.0);
+    } else {
+      re = fx_to_double_in_range(M[j].im + sm[j][2 * row + 1][lane], -FX_LINK - 3);
+      im = fx_to_double_in_range(sm[j][2 * row][lane] - M[j].re, -FX_LINK - 3);
+    }
+    q[(size_t)j * V] = make_double2(re, im);
+  }
+}
+
+// the same from the FP64 links (not near-unitary ones, t-slabs), one (site, plane) per thread
 __global__ void __launch_bounds__(128) field_strength_kernel(Geom g, const double2* __restrict__ g64, double2* Fbuf) {
   const int V = 2 * g.Vh;
   const long long tid = (long long)blockIdx.x * blockDim.x + threadIdx.x;
@@ -184,12 +255,14 @@ __global__ void __launch_bounds__(128) field_strength_kernel(Geom g, const doubl
   int c[4];
   lattice_coords(g, i, c);
   const M3 F = field_strength(g, g64, c, PM[pl], PN[pl]);
-  double2* q = Fbuf + (size_t)pl * 9 * V + i;
+  const int p = (c[0] + c[1] + c[2] + c[3]) & 1;
+  double2* q = Fbuf + (size_t)pl * 9 * V + (size_t)p * g.Vh + (i >> 1);
 #pragma unroll
   for (int k = 0; k < 9; k++) q[(size_t)k * V] = make_double2(F.e[k].re, F.e[k].im);
 }
 
-// A's chiral block b and its inverse for one (site, block) per thread, from the six F_{mu nu}
+// A's chiral block b (even sites) or its inverse (odd sites), the ones the operators read, and log det, for
+// one (site, block) per thread, from the six F_{mu nu}
 __global__ void __launch_bounds__(128) clover_assemble_kernel(Geom g, const double2* __restrict__ Fbuf, double kappa,
                                                               double csw, double2* A64, double2* Ainv64, float4* A32,
                                                               float4* Ainv32, uint4* A16, uint4* Ainv16,
@@ -197,11 +270,8 @@ __global__ void __launch_bounds__(128) clover_assemble_kernel(Geom g, const doub
   const int V = 2 * g.Vh;
   const int tid = blockIdx.x * blockDim.x + threadIdx.x;
   if (tid >= 2 * V) return;
-  const int b = tid / V, i = tid - b * V;  // block b of lexicographic site i
-  int c[4];
-  lattice_coords(g, i, c);
-  const int p = (c[0] + c[1] + c[2] + c[3]) & 1;
-  const int h = i >> 1;
+  const int b = tid / V, i = tid - b * V;  // block b of the site of parity p, half index h
+  const int p = i >= g.Vh, h = i - p * g.Vh;
   auto Fe = [&](int pl, int e) {
     const double2 v = __ldg(Fbuf + ((size_t)pl * 9 + e) * V + i);
     return cmk(v.x, v.y);
@@ -235,26 +305,23 @@ __global__ void __launch_bounds__(128) clover_assemble_kernel(Geom g, const doub
   double di[6];
   C Li[15];
   double ld = 0.0;
-  if (!invert6(d, L, di, Li, &ld)) {
+  if (!invert6(d, L, p == 1, di, Li, &ld)) {
     *notposdef = 1;
     ld = 0.0;
     for (int k = 0; k < 6; k++) di[k] = 0.0;
     for (int k = 0; k < 15; k++) Li[k] = cmk(0.0, 0.0);
   }
   logdet[((size_t)p * 2 + b) * g.Vh + h] = ld;
-  store_block64(A64 + (size_t)p * 36 * g.Vh, g.Vh, h, b, d, L);
-  store_block64(Ainv64 + (size_t)p * 36 * g.Vh, g.Vh, h, b, di, Li);
-  if (fx.A_even) {
-    const size_t at = (size_t)b * 18 * g.Vh + h;
-    if (p == 0) fx.eA_even[(size_t)b * g.Vh + h] = fx_store_clover(static_cast<int4*>(fx.A_even) + at, g.Vh, d, L);
-    else fx.eAinv_odd[(size_t)b * g.Vh + h] = fx_store_clover(static_cast<int4*>(fx.Ainv_odd) + at, g.Vh, di, Li);
-  }
-  if (A32) store_block32(A32 + (size_t)p * 18 * g.Vh, g.Vh, h, b, d, L);
-  if (Ainv32) store_block32(Ainv32 + (size_t)p * 18 * g.Vh, g.Vh, h, b, di, Li);
-  if (A16) store_block16(A16 + (size_t)p * 9 * g.Vh, g.Vh, h, b, d, L);
-  if (Ainv16) store_block16(Ainv16 + (size_t)p * 9 * g.Vh, g.Vh, h, b, di, Li);
+  auto store = [&](const double* dd, const C* LL, double2* c64, float4* c32, uint4* c16, void* cfx, int* efx) {
+    store_block64(c64 + (size_t)p * 36 * g.Vh, g.Vh, h, b, dd, LL);
+    store_block32(c32 + (size_t)p * 18 * g.Vh, g.Vh, h, b, dd, LL);
+    store_block16(c16 + (size_t)p * 9 * g.Vh, g.Vh, h, b, dd, LL);
+    if (cfx)
+      efx[(size_t)b * g.Vh + h] = fx_store_clover(static_cast<int4*>(cfx) + (size_t)b * 18 * g.Vh + h, g.Vh, dd, LL);
+  };
+  if (p == 0) store(d, L, A64, A32, A16, fx.A_even, fx.eA_even);
+  else store(di, Li, Ainv64, Ainv32, Ainv16, fx.Ainv_odd, fx.eAinv_odd);
 }
-
 template <int P>
 __global__ void clover_apply_kernel(Geom g, const void* clov, const void* in, const float* in_norm, void* out,
                                     float* out_norm, int nrhs) {
@@ -272,15 +339,21 @@ __global__ void clover_apply_kernel(Geom g, const void* clov, const void* in, co
 
 }  // namespace
 
-void launch_clover_build(const Geom& g, const void* g64, double kappa, double csw, void* A64, void* Ainv64, void* A32,
+void launch_clover_build(const Geom& g, const void* g64, const void* gfx, double kappa, double csw, void* A64, void* Ainv64, void* A32,
                          void* Ainv32, void* A16, void* Ainv16, void* work, double* logdet, int* notposdef,
                          const FxClover& fx, cudaStream_t st) {
   const int B = 128;
   const long long V = 2LL * g.Vh;
   // F per (site, plane), then one chiral block per thread
   g_kernel_launches += 2;
-  field_strength_kernel<<<(int)((6 * V + B - 1) / B), B, 0, st>>>(g, static_cast<const double2*>(g64),
-                                                                    static_cast<double2*>(work));
+  // (block fixed point against FP64: 24^3 x 32 5.23 -> 1.33 ms, 16^4 805 -> 200 us; 7 or 8 blocks per SM in
+  // place of 6 change nothing)
+  if (gfx)
+    field_strength_fixed_kernel<<<dim3(2 * ((g.Vh + 31) / 32), 6), 96, 0, st>>>(g, static_cast<const int4*>(gfx),
+                                                                                static_cast<double2*>(work));
+  else
+    field_strength_kernel<<<(int)((6 * V + B - 1) / B), B, 0, st>>>(g, static_cast<const double2*>(g64),
+                                                                      static_cast<double2*>(work));
   clover_assemble_kernel<<<(int)((2 * V + B - 1) / B), B, 0, st>>>(
       g, static_cast<const double2*>(work), kappa, csw, static_cast<double2*>(A64), static_cast<double2*>(Ainv64),
       static_cast<float4*>(A32), static_cast<float4*>(Ainv32), static_cast<uint4*>(A16), static_cast<uint4*>(Ainv16),

@@ -189,14 +189,15 @@ __device__ __forceinline__ void hop_terms(const C Xy[12], const C Yy[12], const 
 // F the traceless part of (Q - Q^dag)/(8i), its leaf coefficient at an odd site is
 //   C_{mu nu} = -i (kappa c_sw / 4)(B + B^dag),  B the traceless part of
 //   B_ac = sum_t sigma_{mu nu}[t][s] (A^-1)_{(s a),(t c)}  (s = the one spin sigma couples to t),
-// the same form as the pseudofermion's clover coefficient; it is added to Cbuf.  One thread per odd
+// the same form as the pseudofermion's clover coefficient; it is added to Cbuf (sites in lexicographic
+// order, or by_parity: even sites first).  One thread per odd
 // site reads the two 6x6 blocks of A_oo^-1 (diagonal, then strictly-lower entries).
 __global__ void __launch_bounds__(FB) det_coeff_kernel(Geom g, double kappa, double csw, const double2* Ainv_odd,
-                                                       double2* Cbuf) {
+                                                       double2* Cbuf, int by_parity) {
   const int h = blockIdx.x * FB + threadIdx.x;
   if (h >= g.Vh) return;
   const int V = 2 * g.Vh;
-  const Site st = site_of(g, 1, h);
+  const int at = by_parity ? g.Vh + h : site_of(g, 1, h).i;
   double d[2][6];
   C L[2][15];
 #pragma unroll
@@ -241,7 +242,7 @@ __global__ void __launch_bounds__(FB) det_coeff_kernel(Geom g, double kappa, dou
     B.e[0] = B.e[0] - cmk(tr, ti);
     B.e[4] = B.e[4] - cmk(tr, ti);
     B.e[8] = B.e[8] - cmk(tr, ti);
-    M3 Cm = load_m3(Cbuf, pl, V, st.i);
+    M3 Cm = load_m3(Cbuf, pl, V, at);
 #pragma unroll
     for (int a = 0; a < 3; a++)
 #pragma unroll
@@ -249,7 +250,7 @@ __global__ void __launch_bounds__(FB) det_coeff_kernel(Geom g, double kappa, dou
         const C h2 = B.e[3 * a + c] + conj(B.e[3 * c + a]);
         Cm.e[3 * a + c] = Cm.e[3 * a + c] + cmk(f * h2.im, -f * h2.re);  // -i f h2
       }
-    store_m3(Cbuf, pl, V, st.i, Cm);
+    store_m3(Cbuf, pl, V, at, Cm);
   }
 }
 
@@ -432,9 +433,9 @@ void launch_force_links(const Geom& g, double kappa, int nrhs, const void* g64, 
 }
 
 void launch_force_det_coeff(const Geom& g, double kappa, double csw, const double2* Ainv_odd, double2* Cbuf,
-                            cudaStream_t st) {
+                            bool by_parity, cudaStream_t st) {
   g_kernel_launches += 1;
-  det_coeff_kernel<<<(g.Vh + FB - 1) / FB, FB, 0, st>>>(g, kappa, csw, Ainv_odd, Cbuf);
+  det_coeff_kernel<<<(g.Vh + FB - 1) / FB, FB, 0, st>>>(g, kappa, csw, Ainv_odd, Cbuf, by_parity ? 1 : 0);
 }
 
 // clover part per link: 6 plaquettes x (4 products of 198 flops + 36 adds); per site of kernel 2:

@@ -32,9 +32,22 @@ void launch_force_links(const Geom& g, double kappa, int nrhs, const void* g64, 
                         const double2* Ye, const double2* Yo, const double2* Ebuf, double2* out, bool gradient,
                         bool with_clover, bool accumulate, cudaStream_t st);
 // 4. add to Cbuf the coefficients of the clover determinant term S_det = -2 sum_{x odd} log det A(x)
-// (at odd sites), from the FP64 A_oo^-1 blocks ([36][Vh] double2 of the odd parity).
+// (at odd sites), from the FP64 A_oo^-1 blocks ([36][Vh] double2 of the odd parity).  by_parity: Cbuf is
+// the block fixed-point path's, its sites even ones first, else in lexicographic order.
 void launch_force_det_coeff(const Geom& g, double kappa, double csw, const double2* Ainv_odd, double2* Cbuf,
-                            cudaStream_t st);
+                            bool by_parity, cudaStream_t st);
+// The same from block fixed-point links and fields (qcd_fixed.cuh; near-unitary links): X_e, X_o, Y_e, Y_o
+// hold all nrhs right-hand sides, xe .. yo their exponents.  Cbuf is FP64, the site of parity p and half index
+// h at p Vh + h (the determinant's coefficients are added to it); Cfx and Efx are work space of fixed_matrix_bytes(g, 6) and (g, 12); nrhs 0 in
+// launch_force_links_fixed leaves the clover part alone.
+size_t fixed_matrix_bytes(const Geom& g, int n);
+void launch_force_coeff_fixed(const Geom& g, double kappa, double csw, int nrhs, const void* Xe, const void* Xo,
+                              const void* Ye, const void* Yo, const float* xe, const float* xo, const float* ye,
+                              const float* yo, double2* Cbuf, cudaStream_t st);
+void launch_force_edges_fixed(const Geom& g, const void* gfx, const double2* Cbuf, void* Cfx, void* Efx, cudaStream_t st);
+void launch_force_links_fixed(const Geom& g, double kappa, int nrhs, const void* gfx, const void* Xe, const void* Xo,
+                              const void* Ye, const void* Yo, const float* xe, const float* xo, const float* ye,
+                              const float* yo, const void* Efx, double2* out, bool gradient, cudaStream_t st);
 // conventional FP64 flop counts: per link of kernel 2, per site of kernel 1
 double force_link_flops(int nrhs, bool with_clover);
 double force_edge_flops();

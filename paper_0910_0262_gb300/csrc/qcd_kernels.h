@@ -62,8 +62,6 @@ void launch_spinor_to_native(int prec, const Geom& g, const double2* canon, void
                              cudaStream_t st);
 void launch_spinor_to_canon(int prec, const Geom& g, const void* nat, const float* norm, double2* canon, int nrhs,
                             cudaStream_t st);
-// an FP64 native field from a block fixed-point one
-void launch_fixed_to_double(const Geom& g, const void* in, const float* ex, void* out, int nrhs, cudaStream_t st);
 void launch_check_finite(const double* data, size_t n, int* flag, cudaStream_t st);
 
 // ---- clover (qcd_clover.cu)
@@ -73,10 +71,12 @@ struct FxClover {
   void *A_even, *Ainv_odd;
   int *eA_even, *eAinv_odd;
 };
-// A (both parities) and A^-1 (both parities) in FP64, FP32 and FP16; flag set if a block is not positive definite.
+// A (even sites) and A^-1 (odd sites) in FP64, FP32 and FP16; flag set if a block is not positive definite.
 // work: 6 * 9 * V double2 for the field strengths (two kernels: F per site and plane, then one chiral
 // block per thread); logdet: [parity][block][Vh] log det of each 6x6 block.
-void launch_clover_build(const Geom& g, const void* g64, double kappa, double csw, void* A64, void* Ainv64,
+// gfx (may be null): the near-unitary links in block fixed point, from which F is then formed.  A is stored on
+// even, A^-1 on odd sites.
+void launch_clover_build(const Geom& g, const void* g64, const void* gfx, double kappa, double csw, void* A64, void* Ainv64,
                          void* A32, void* Ainv32, void* A16, void* Ainv16, void* work, double* logdet,
                          int* notposdef, const FxClover& fx, cudaStream_t st);
 // the same for block fixed-point fields and blocks (clover_e: their exponents [2][Vh])
@@ -93,6 +93,7 @@ unsigned debug_take_clover();
 unsigned debug_take_dslash();
 unsigned debug_take_dslash_fx();
 unsigned debug_take_force();
+unsigned debug_take_force_fx();
 unsigned debug_take_halo();
 unsigned debug_take_layout();
 unsigned debug_take_md();
@@ -143,6 +144,10 @@ void launch_norm2(const Geom& g, int nrhs, const double2* v, const ReduceArgs& r
 // to or added to out
 void launch_gauge_force(const Geom& g, double beta, const void* g64, double2* out, bool gradient, bool accumulate,
                         cudaStream_t st);
+// the same from the block fixed-point links, and the plaquette sum below
+void launch_gauge_force_fixed(const Geom& g, double beta, const void* gfx, double2* out, bool gradient, bool accumulate,
+                              cudaStream_t st);
+void launch_plaquette_fixed(const Geom& g, const void* gfx, const ReduceArgs& red, cudaStream_t st);
 // result[0] = sum over sites and planes of Re tr P_{mu nu}(x) / 3 (FIN_STORE)
 void launch_plaquette(const Geom& g, const void* g64, const ReduceArgs& red, cudaStream_t st);
 // result[0] = sum of |v_j|^2 over n complex numbers (FIN_STORE)

@@ -130,15 +130,6 @@ __global__ void spinor_to_canon_kernel(Geom g, const void* nat, const float* nor
   for (int c = 0; c < 12; c++) dst[c] = make_double2(double(s[c].re), double(s[c].im));
 }
 
-__global__ void fixed_to_double_kernel(Geom g, const void* in, const float* ex, void* out, int nrhs) {
-  const int tid = blockIdx.x * blockDim.x + threadIdx.x;
-  if (tid >= g.Vh * nrhs) return;
-  const int r = tid / g.Vh, h = tid - r * g.Vh;
-  cx<double> s[12];
-  SpinorIO<60>::load(in, ex, g.Vh, r, h, s);
-  SpinorIO<64>::store(out, nullptr, g.Vh, r, h, s);
-}
-
 __global__ void check_finite_kernel(const double* __restrict__ d, size_t n, int* flag) {
   size_t i = blockIdx.x * (size_t)blockDim.x + threadIdx.x;
   const size_t stride = (size_t)gridDim.x * blockDim.x;
@@ -179,12 +170,6 @@ void launch_spinor_to_canon(int prec, const Geom& g, const void* nat, const floa
   else if (prec == 64) spinor_to_canon_kernel<64><<<nb, B, 0, st>>>(g, nat, norm, canon, nrhs);
   else if (prec == 32) spinor_to_canon_kernel<32><<<nb, B, 0, st>>>(g, nat, norm, canon, nrhs);
   else spinor_to_canon_kernel<16><<<nb, B, 0, st>>>(g, nat, norm, canon, nrhs);
-}
-
-void launch_fixed_to_double(const Geom& g, const void* in, const float* ex, void* out, int nrhs, cudaStream_t st) {
-  g_kernel_launches += 1;
-  const int B = 128;
-  fixed_to_double_kernel<<<nblocks((long long)g.Vh * nrhs, B), B, 0, st>>>(g, in, ex, out, nrhs);
 }
 
 void launch_check_finite(const double* data, size_t n, int* flag, cudaStream_t st) {

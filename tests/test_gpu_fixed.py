@@ -129,3 +129,60 @@ def test_fp64_solve(nrhs):
                 rel = np.linalg.norm(r[k]) / np.linalg.norm(b[k])
                 assert rel < 1.01e-11 and abs(rel - st[k]["true_rel_resid"]) < 1e-13
     op.close()
+
+
+@gpu
+@pytest.mark.parametrize("dims", [(2, 2, 2, 2), (4, 4, 2, 2), (4, 2, 6, 4), (6, 10, 2, 4)], ids=lambda d: "x".join(map(str, d)))
+@pytest.mark.parametrize("scale,t_bc", [(1.0, -1.0), (1.0, 1.0), (1.25, -1.0)], ids=["su3", "su3_periodic", "far"])
+def test_matrix_fields(dims, scale, t_bc):
+    """Clover blocks and log det, fermion and determinant force, gauge force and plaquette on partial, whole
+    and ragged blocks of sites, with 0, 1, 2 and 5 right-hand sides (sums over several exponents).  Sums of
+    at most 12 triple products of matrices per link beside the fields' own 1e-15."""
+    require_gpu()
+    from oracle import cloverdet, force as oforce, md as omd
+    U, op = _context(dims, t_bc, scale)
+    ref = evenodd.SchurOperator(U, KAPPA, CSW, t_bc)
+    vh = ref.A_ee.shape[0]
+    rng = np.random.default_rng(19)
+    for p, A in enumerate((ref.A_ee, ref.A_oo)):
+        want = np.linalg.slogdet(A)[1].sum()
+        assert abs(op.clover_logdet()[p] - want) < 1e-13 * vh
+    if t_bc == -1.0:  # (the oracle's gradient helpers take the antiperiodic operator)
+        Gdet = cloverdet.gradient(ref)
+        for n in (1, 2, 5):
+            x = rand_eo(n, vh, rng) * np.array([1.0, 2.0 ** -20, 3.0, 0.0, 2.0 ** 9])[:n, None, None, None]
+            G = oforce.gradient(ref, x)
+            for det in (False, True):
+                want = G + Gdet if det else G
+                got, _ = op.fermion_force(to_dev(x), input_is_solution=True, gradient=True, clover_det=det)
+                assert rel_l2(to_np(got), want) < 2e-15
+                got, _ = op.fermion_force(to_dev(x), input_is_solution=True, clover_det=det)
+                assert rel_l2(to_np(got), oforce.lie_force(U, want)) < 4e-15
+        got, _ = op.fermion_force(None, clover_det=True)
+        assert rel_l2(to_np(got), oforce.lie_force(U, Gdet)) < 1e-14  # (small beside the blocks it comes from)
+    want = omd.gauge_force(U, 5.6)
+    F = op.gauge_force(5.6)
+    assert rel_l2(to_np(F), want) < 4e-15
+    op.gauge_force(5.6, out=F)
+    assert rel_l2(to_np(F), 2 * want) < 4e-15
+    assert rel_l2(to_np(op.gauge_force(5.6, gradient=True)), omd.gauge_gradient(U, 5.6)) < 2e-15
+    assert abs(op.plaquette() - omd.mean_plaquette(U)) < 4e-15 * scale ** 4
+    op.close()
+
+
+@gpu
+def test_force_of_fields_with_marked_and_empty_sites():
+    """A non-finite solution gives non-finite links around it; one that meets zeros elsewhere stays marked."""
+    require_gpu()
+    dims = (4, 4, 4, 6)
+    U, op = _context(dims)
+    x = np.zeros((1, U.size // 72, 4, 3), complex)
+    x[0, 40, 1, 1] = np.nan
+    F, _ = op.fermion_force(to_dev(x), input_is_solution=True)
+    bad = ~np.isfinite(to_np(F)).all(axis=(-1, -2, -3))
+    full = join_eo(np.isnan(x[0]).astype(complex), None, dims)
+    assert bad[np.abs(full).max(axis=(-1, -2)) > 0].all()  # the site itself
+    x[:] = 0
+    F, _ = op.fermion_force(to_dev(x), input_is_solution=True)
+    assert not np.any(to_np(F))
+    op.close()
