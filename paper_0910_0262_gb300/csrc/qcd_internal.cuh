@@ -152,6 +152,34 @@ __device__ __forceinline__ int neighbor_bwd(const Geom& g, const Site& s, int mu
   }
 }
 
+// ---------------------------------------------------- float <-> double ----
+// The conversion instructions run on the FP64 pipe (two a clock and SM); these give the same values with
+// integer operations, and leave the ends of the float range to them.
+__device__ __forceinline__ double widen(float f) {
+  const unsigned u = __float_as_uint(f), m = u & 0x7fffffffu;
+  if (m - 0x00800000u < 0x7f000000u)  // normal
+    return __hiloint2double((int)((u & 0x80000000u) | ((m >> 3) + 0x38000000u)), (int)(u << 29));
+  return m == 0 ? __hiloint2double((int)u, 0) : (double)f;
+}
+// rounded to nearest even
+__device__ __forceinline__ float narrow(double x) {
+  const unsigned long long b = (unsigned long long)__double_as_longlong(x), m = b & 0x7fffffffffffffffULL;
+  // magnitudes from the smallest normal float to below the largest one's upper neighbour's half way
+  if (m - 0x3810000000000000ULL < 0x47efffffe0000000ULL - 0x3810000000000000ULL) {
+    const unsigned long long r = (m + 0x0fffffffULL + ((m >> 29) & 1ULL)) >> 29;
+    return __uint_as_float((unsigned)(b >> 32 & 0x80000000u) | (unsigned)(r - (896ULL << 23)));
+  }
+  return m == 0 ? __uint_as_float((unsigned)(b >> 32)) : (float)x;
+}
+template <typename R>
+__device__ __forceinline__ R to_real(double x);
+template <>
+__device__ __forceinline__ double to_real<double>(double x) { return x; }
+template <>
+__device__ __forceinline__ float to_real<float>(double x) { return narrow(x); }
+__device__ __forceinline__ double to_double(double x) { return x; }
+__device__ __forceinline__ double to_double(float x) { return widen(x); }
+
 // ------------------------------------------------------------ debug checks ----
 // Builds with QCD_DEBUG=1 (libqcd_debug.so) check the indices every field accessor below is given: the
 // site (0 <= h < Vh, or the face index against its face), the RHS (r >= 0), the link's parity and

@@ -55,9 +55,10 @@ cudaError_t launch_cg_persistent(int prec, int recon, const PersistentCGArgs& q,
 cudaError_t launch_barrier_probe(unsigned* count, int* err, cudaStream_t st);
 
 // ---- layout (qcd_layout.cu); prec 60 names block fixed point (qcd_fixed.cuh) with norm its exponents
-// gfx (may be null): the block fixed-point links; *not_unitary is set if a link is not near-unitary
+// gfx (may be null): the block fixed-point links; *not_unitary is set if a link is not near-unitary,
+// *non_finite (may be null) if one holds a non-finite value
 void launch_pack_gauge(const Geom& g, const double2* canon, void* g64, void* g32, int recon32, void* g16,
-                       int recon16, void* gfx, int* not_unitary, cudaStream_t st);
+                       int recon16, void* gfx, int* not_unitary, int* non_finite, cudaStream_t st);
 void launch_spinor_to_native(int prec, const Geom& g, const double2* canon, void* nat, float* norm, int nrhs,
                              cudaStream_t st);
 void launch_spinor_to_canon(int prec, const Geom& g, const void* nat, const float* norm, double2* canon, int nrhs,

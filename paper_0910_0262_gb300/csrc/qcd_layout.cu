@@ -25,11 +25,8 @@ __device__ __forceinline__ void coords_of(const Geom& g, int i, int& x, int& y, 
   t = c[3];
 }
 
-// whether U U^dag = 1 to 1e-5 (rows 0, 1, 2 of u), in FP32
-__device__ __forceinline__ bool near_unitary(const double2 u[9]) {
-  float2 v[9];
-#pragma unroll
-  for (int k = 0; k < 9; k++) v[k] = make_float2((float)u[k].x, (float)u[k].y);
+// whether U U^dag = 1 to 1e-5 (rows 0, 1, 2 of v), in FP32
+__device__ __forceinline__ bool near_unitary(const float2 v[9]) {
   float worst = 0.f;
 #pragma unroll
   for (int a = 0; a < 3; a++)
@@ -48,9 +45,10 @@ __device__ __forceinline__ bool near_unitary(const double2 u[9]) {
 }
 
 // canonical gauge U[i][mu][3][3] complex128 -> per-parity, per-direction SoA copies.  gfx: the block
-// fixed-point copy, which serves near-unitary links only; *not_unitary is set if one is not.
+// fixed-point copy, which serves near-unitary links only; *not_unitary is set if one is not.  *non_finite
+// (may be null) is set if a link holds a non-finite value.
 __global__ void pack_gauge_kernel(Geom g, const double2* __restrict__ U, double2* g64, void* g32, int recon32,
-                                  void* g16, int recon16, int4* gfx, int* not_unitary) {
+                                  void* g16, int recon16, int4* gfx, int* not_unitary, int* non_finite) {
   const int tid = blockIdx.x * blockDim.x + threadIdx.x;
   const int V = 2 * g.Vh;
   if (tid >= V * 4) return;
@@ -63,24 +61,31 @@ __global__ void pack_gauge_kernel(Geom g, const double2* __restrict__ U, double2
   double2 u[9];
 #pragma unroll
   for (int k = 0; k < 9; k++) u[k] = src[k];
+  bool bad = false;
+  float2 v[9];
+#pragma unroll
+  for (int k = 0; k < 9; k++) {
+    bad |= !isfinite(u[k].x) || !isfinite(u[k].y);
+    v[k] = make_float2(narrow(u[k].x), narrow(u[k].y));
+  }
+  if (bad && non_finite) *non_finite = 1;
   const size_t base = (size_t)(p * 4 + mu);
 #pragma unroll
   for (int k = 0; k < 9; k++) g64[(base * 9 + k) * g.Vh + h] = u[k];
   if (gfx) {
     fx_store_link(gfx + base * 9 * g.Vh + h, g.Vh, u);
-    if (!near_unitary(u)) *not_unitary = 1;
+    if (!near_unitary(v)) *not_unitary = 1;
   }
   if (g32) {
     if (recon32 == 12) {
       float4* q = static_cast<float4*>(g32);
 #pragma unroll
       for (int k = 0; k < 3; k++)
-        q[(base * 3 + k) * g.Vh + h] = make_float4((float)u[2 * k].x, (float)u[2 * k].y, (float)u[2 * k + 1].x,
-                                                   (float)u[2 * k + 1].y);
+        q[(base * 3 + k) * g.Vh + h] = make_float4(v[2 * k].x, v[2 * k].y, v[2 * k + 1].x, v[2 * k + 1].y);
     } else {
       float2* q = static_cast<float2*>(g32);
 #pragma unroll
-      for (int k = 0; k < 9; k++) q[(base * 9 + k) * g.Vh + h] = make_float2((float)u[k].x, (float)u[k].y);
+      for (int k = 0; k < 9; k++) q[(base * 9 + k) * g.Vh + h] = v[k];
     }
   }
   if (g16) {
@@ -88,18 +93,24 @@ __global__ void pack_gauge_kernel(Geom g, const double2* __restrict__ U, double2
       uint2* q = static_cast<uint2*>(g16);
 #pragma unroll
       for (int k = 0; k < 3; k++) {
-        uint2 v;
-        v.x = f2h((float)u[2 * k].x, (float)u[2 * k].y);
-        v.y = f2h((float)u[2 * k + 1].x, (float)u[2 * k + 1].y);
-        q[(base * 3 + k) * g.Vh + h] = v;
+        q[(base * 3 + k) * g.Vh + h] =
+            make_uint2(f2h(v[2 * k].x, v[2 * k].y), f2h(v[2 * k + 1].x, v[2 * k + 1].y));
       }
     } else {
       uint32_t* q = static_cast<uint32_t*>(g16);
 #pragma unroll
-      for (int k = 0; k < 9; k++) q[(base * 9 + k) * g.Vh + h] = f2h((float)u[k].x, (float)u[k].y);
+      for (int k = 0; k < 9; k++) q[(base * 9 + k) * g.Vh + h] = f2h(v[k].x, v[k].y);
     }
   }
 }
+
+// Canonical sites are 12 consecutive complex128.  Reading them site by site is fine (a site's lines stay in
+// L1 between its 12 loads), but a site's store instruction touches half of 32 sectors, so the way back moves a
+// block's sites through shared memory and its lanes write consecutive 16-byte words: 32^3 x 64, 8 RHS, FP16
+// to canonical 1037 -> 300 us, the time its bytes take (reads staged the same way: 328 -> 410 us).  Sites in
+// shared memory are 13 words apart, so that eight lanes' 16-byte accesses hit distinct banks.
+constexpr int LB = 128;         // sites of a block
+constexpr int SITE_WORDS = 13;  // double2 words between sites in shared memory
 
 template <int P>
 __global__ void spinor_to_native_kernel(Geom g, const double2* __restrict__ canon, void* nat, float* norm, int nrhs) {
@@ -112,22 +123,33 @@ __global__ void spinor_to_native_kernel(Geom g, const double2* __restrict__ cano
 #pragma unroll
   for (int c = 0; c < 12; c++) {
     double2 v = src[c];
-    s[c] = cmk(R(v.x), R(v.y));
+    s[c] = cmk(to_real<R>(v.x), to_real<R>(v.y));
   }
   SpinorIO<P>::store(nat, norm, g.Vh, r, h, s);
 }
 
 template <int P>
-__global__ void spinor_to_canon_kernel(Geom g, const void* nat, const float* norm, double2* canon, int nrhs) {
+__global__ void __launch_bounds__(LB) spinor_to_canon_kernel(Geom g, const void* nat, const float* norm,
+                                                             double2* canon, int nrhs) {
   using R = typename Real<P>::T;
-  const int tid = blockIdx.x * blockDim.x + threadIdx.x;
-  if (tid >= g.Vh * nrhs) return;
-  const int r = tid / g.Vh, h = tid - r * g.Vh;
-  cx<R> s[12];
-  SpinorIO<P>::load(nat, norm, g.Vh, r, h, s);
-  double2* dst = canon + (size_t)tid * 12;
+  __shared__ double2 buf[LB * SITE_WORDS];
+  const long long first = (long long)blockIdx.x * LB, n = (long long)g.Vh * nrhs;
+  const int here = (int)min((long long)LB, n - first);
+  if ((int)threadIdx.x < here) {
+    const int tid = (int)(first + threadIdx.x), r = tid / g.Vh, h = tid - r * g.Vh;
+    cx<R> s[12];
+    SpinorIO<P>::load(nat, norm, g.Vh, r, h, s);
 #pragma unroll
-  for (int c = 0; c < 12; c++) dst[c] = make_double2(double(s[c].re), double(s[c].im));
+    for (int c = 0; c < 12; c++)
+      buf[threadIdx.x * SITE_WORDS + c] = make_double2(to_double(s[c].re), to_double(s[c].im));
+  }
+  __syncthreads();
+  double2* dst = canon + first * 12;
+#pragma unroll
+  for (int k = 0; k < 12; k++) {
+    const int j = k * LB + threadIdx.x, site = j / 12;
+    if (site < here) dst[j] = buf[site * SITE_WORDS + (j - 12 * site)];
+  }
 }
 
 __global__ void check_finite_kernel(const double* __restrict__ d, size_t n, int* flag) {
@@ -143,11 +165,12 @@ inline int nblocks(long long n, int b) { return (int)((n + b - 1) / b); }
 }  // namespace
 
 void launch_pack_gauge(const Geom& g, const double2* canon, void* g64, void* g32, int recon32, void* g16,
-                       int recon16, void* gfx, int* not_unitary, cudaStream_t st) {
+                       int recon16, void* gfx, int* not_unitary, int* non_finite, cudaStream_t st) {
   g_kernel_launches += 1;
   const int B = 128;
   pack_gauge_kernel<<<nblocks(8LL * g.Vh, B), B, 0, st>>>(g, canon, static_cast<double2*>(g64), g32, recon32, g16,
-                                                          recon16, static_cast<int4*>(gfx), not_unitary);
+                                                          recon16, static_cast<int4*>(gfx), not_unitary,
+                                                          non_finite);
 }
 
 void launch_spinor_to_native(int prec, const Geom& g, const double2* canon, void* nat, float* norm, int nrhs,
@@ -164,7 +187,7 @@ void launch_spinor_to_native(int prec, const Geom& g, const double2* canon, void
 void launch_spinor_to_canon(int prec, const Geom& g, const void* nat, const float* norm, double2* canon, int nrhs,
                             cudaStream_t st) {
   g_kernel_launches += 1;
-  const int B = 128;
+  const int B = LB;
   const int nb = nblocks((long long)g.Vh * nrhs, B);
   if (prec == 60) spinor_to_canon_kernel<60><<<nb, B, 0, st>>>(g, nat, norm, canon, nrhs);
   else if (prec == 64) spinor_to_canon_kernel<64><<<nb, B, 0, st>>>(g, nat, norm, canon, nrhs);
