@@ -100,7 +100,7 @@ struct ProfSlot {
 
 // an instantiated CUDA graph of CG work for one set of solver fields
 struct ItGraph {
-  int kind = 0;  // 0: `len` CG iterations; 1: one reliable update
+  int kind = 0;  // 0: `len` CG iterations; 1: one reliable update; 2: one without its p update
   int len = 0, nrhs = 0;
   bool prof = false;
   // operator state recorded in the kernels' arguments and choice
@@ -331,13 +331,14 @@ void dslash_cost(const qcd_ctx* c, int prec, int epi, int nrhs, double* bytes, d
   const double bc = prec >= 60 ? 8 : (prec == 32 ? 4 : 2);
   const double bs = 24.0 * real_bytes(prec) + (prec == 16 ? 4 : 0);
   double site = 8.0 * R * bl + (epi != EPI_NONE ? 72.0 * bc : 0.0);
-  double rhs = bs * (epi == EPI_XPAY ? 3.0 : 2.0);
+  double rhs = bs * (epi == EPI_XPAY ? 3.0 : (epi == EPI_RESID ? 4.0 : 2.0));
   if (epi == EPI_XPAY_CG) {
     // reads in, x, p; reads and writes x_lo, r_lo; writes nothing else
     const double sr = 24.0 * (prec >= 60 ? 8 : 4);
     rhs = 3.0 * bs + 4.0 * sr;
   }
   *bytes = Vh * site + Vh * nrhs * rhs;
+  // (EPI_RESID reads in, x and b and writes r_lo, counted as a field of this precision)
   *flops = Vh * nrhs * (1320.0 + (epi != EPI_NONE ? 504.0 : 0.0) + (epi >= EPI_XPAY ? 48.0 : 0.0) +
                         (epi == EPI_XPAY_CG ? 96.0 : 0.0));
 }
@@ -388,7 +389,7 @@ void run_dslash(qcd_ctx* c, int prec, int epi, const DslashArgs& a) {
   dslash_cost(c, prec, epi, a.nrhs, &bytes, &flops);
   char name[40];
   snprintf(name, sizeof name, "dslash_p%d_r%d_%s", prec >= 60 ? 64 : prec, prec >= 60 ? 18 : c->recon,
-           epi == EPI_NONE ? "plain" : (epi == EPI_CLOVER_INV ? "cloverinv" : (epi == EPI_XPAY ? "xpay" : "xpaycg")));
+           epi == EPI_NONE ? "plain" : (epi == EPI_CLOVER_INV ? "cloverinv" : (epi == EPI_XPAY_CG ? "xpaycg" : "xpay")));
   ProfScope ps(c, name, bytes, flops);
   if (prec == 60) launch_dslash_fixed(epi, a, c->cur);
   else launch_dslash(prec, prec == 64 ? 18 : c->recon, epi, a, c->cur);
@@ -411,6 +412,7 @@ ReduceArgs reduce_args(qcd_ctx* c, int mode) {
   r.mode = mode;
   r.cg = c->cg;
   r.ctl = c->ctl;
+  r.lower_gate = 0;
   return r;
 }
 
@@ -465,6 +467,38 @@ qcd_status sync_and_check(qcd_ctx* c, const char* what) {
   if (e != cudaSuccess) return fail(QCD_ERR_CUDA, "%s: %s", what, cudaGetErrorString(e));
   if (c->prof_on) prof_collect(c);
   return QCD_OK;
+}
+
+// r_lo = b - Mhat^dag Mhat x for the fixed-point field x and its |.|^2 -> red: the true residual of the CG, formed
+// in the epilogue of the last pass (a pass of its own over b and the operator's result took 15 us beside the
+// passes' 27 at 16^4, 471 us at 24^3 x 48 with 8 RHS)
+void apply_mdagm_resid(qcd_ctx* c, int nrhs, const SolverFields& f, const void* x, const ReduceArgs& red,
+                       const int* gate) {
+  apply_mhat(c, 60, nrhs, false, x, f.ap_hi_n, f.y_hi, f.y_hi_n, f.t_hi, f.t_hi_n, nullptr, nullptr, gate);
+  DslashArgs a = base_args(c, 60, 1, nrhs);
+  a.in = f.y_hi;
+  a.in_norm = f.y_hi_n;
+  a.out = f.t_hi;
+  a.out_norm = f.t_hi_n;
+  a.clover = clover_ptr(c, 60, true, 1);
+  a.in_g5 = 1;
+  a.gate = gate;
+  run_dslash(c, 60, EPI_CLOVER_INV, a);
+  DslashArgs b = base_args(c, 60, 0, nrhs);
+  b.in = f.t_hi;
+  b.in_norm = f.t_hi_n;
+  b.x = f.y_hi;
+  b.x_norm = f.y_hi_n;
+  b.clover = clover_ptr(c, 60, false, 0);
+  b.a = -c->kappa * c->kappa;
+  b.x_g5 = 1;
+  b.out_g5 = 1;
+  b.gate = gate;
+  b.cg_p = f.b_hi;
+  b.cg_r = f.r_lo;
+  b.r_f64 = f.pr == 64;
+  b.red = red;
+  run_dslash(c, 60, EPI_RESID, b);
 }
 
 bool valid_prec(int p) { return p == 64 || p == 32 || p == 16; }
@@ -907,19 +941,25 @@ void enqueue_iteration(qcd_ctx* c, const SolverFields& f, int nrhs) {
 }
 
 // x_hi += x_lo, r = b - Mhat^dag Mhat x_hi in FP64 (true residual, convergence test, halt cleared
-// unless every RHS is done), p = r + beta p.  gated: every step returns at once unless a trigger
-// raised ctl->rel_go, which the last step lowers (so the update can be enqueued before it is known
-// to be due).
-void enqueue_reliable(qcd_ctx* c, const SolverFields& f, int nrhs, bool gated) {
+// unless every RHS is done), p = r + beta p (with_p false: left to the persistent kernel's first
+// iteration).  gated: every step returns at once unless a trigger raised ctl->rel_go, which the last step
+// lowers (so the update can be enqueued before it is known to be due).
+void enqueue_reliable(qcd_ctx* c, const SolverFields& f, int nrhs, bool gated, bool with_p = true) {
   const Geom& g = c->g;
   const int* gate = gated ? &c->ctl->rel_go : nullptr;
-  // in fixed point the operator's input is a copy of x_hi that is kept where its output goes (the last
-  // of the four passes, which writes ap_hi, does not read it any more)
-  void* x_fx = f.hp == 60 ? f.ap_hi : nullptr;
-  launch_accumulate_x(f.pr, g, nrhs, f.x_hi, f.x_lo, f.x_lo_n, c->cur, gate, x_fx, f.ap_hi_n);
-  apply_mdagm(c, f.hp, nrhs, x_fx ? x_fx : f.x_hi, f.ap_hi_n, f.ap_hi, nullptr, f.t_hi, f.t_hi_n, f.y_hi, f.y_hi_n,
-              nullptr, nullptr, gate, true);
-  launch_true_residual(f.pr, g, nrhs, f.b_hi, f.ap_hi, f.r_lo, f.r_lo_n, reduce_args(c, FIN_CG_TRUE), c->cur, gate);
+  ReduceArgs red = reduce_args(c, FIN_CG_TRUE);
+  red.lower_gate = gated && !with_p;
+  if (f.hp == 60) {
+    // in fixed point the operator's input is a copy of x_hi, and its last pass forms the residual
+    void* x_fx = f.ap_hi;
+    launch_accumulate_x(f.pr, g, nrhs, f.x_hi, f.x_lo, f.x_lo_n, c->cur, gate, x_fx, f.ap_hi_n);
+    apply_mdagm_resid(c, nrhs, f, x_fx, red, gate);
+  } else {
+    launch_accumulate_x(f.pr, g, nrhs, f.x_hi, f.x_lo, f.x_lo_n, c->cur, gate);
+    apply_mdagm(c, 64, nrhs, f.x_hi, nullptr, f.ap_hi, nullptr, f.t_hi, nullptr, f.y_hi, nullptr, nullptr, nullptr, gate);
+    launch_true_residual(f.pr, g, nrhs, f.b_hi, f.ap_hi, f.r_lo, f.r_lo_n, red, c->cur, gate);
+  }
+  if (!with_p) return;
   launch_p_update(f.pr, f.pp, g, nrhs, f.r_lo, f.r_lo_n, f.p, f.p_n, c->cg, nullptr, c->cur, gate);
   if (gated) launch_gate_clear(&c->ctl->rel_go, c->cur);
 }
@@ -950,7 +990,7 @@ qcd_status capture_graph(qcd_ctx* c, ItGraph* gph) {
         enqueue_iteration(c, gph->f, gph->nrhs);
       }
     } else {
-      enqueue_reliable(c, gph->f, gph->nrhs, true);
+      enqueue_reliable(c, gph->f, gph->nrhs, true, gph->kind == 1);
     }
     cudaGraph_t graph = nullptr;
     e = cudaStreamEndCapture(c->cap, &graph);
@@ -1198,6 +1238,11 @@ qcd_status cg_batch(qcd_ctx* c, double2* x, const double2* b, int nrhs, const qc
   *c->h_ctl = ctl;
   CUDA_TRY(cudaMemcpyAsync(c->cg, c->h_cg, sizeof(CGState) * nrhs, cudaMemcpyHostToDevice, c->st));
   CUDA_TRY(cudaMemcpyAsync(c->ctl, c->h_ctl, sizeof(CGControl), cudaMemcpyHostToDevice, c->st));
+  // one RHS: the persistent kernel runs each segment of iterations.  Its FP32 iterations form p = r + beta p
+  // where they read p, also in a segment's first iteration, so nothing else updates p then.
+  const bool use_pc = c->persistent && nrhs == 1 && f.pp != 60 && g.Vh <= PERSISTENT_MAX_VH;
+  const bool pc_p = use_pc && f.pp == 32;
+  const int rel_kind = pc_p ? 2 : 1;
   // b_hi, |b|^2 (tolerance, zero sources), x_hi = x0 or 0, x_lo = 0, p = 0, r = b - A x_hi, p = r
   launch_spinor_to_native(64, g, b, f.b_hi, nullptr, nrhs, c->st);
   launch_norm2(g, nrhs, f.b_hi, reduce_args(c, FIN_CG_BNORM), c->st);
@@ -1209,11 +1254,11 @@ qcd_status cg_batch(qcd_ctx* c, double2* x, const double2* b, int nrhs, const qc
   if (prm->use_x0) {
     if (f.hp == 60) launch_spinor_to_native(60, g, x, f.ap_hi, f.ap_hi_n, nrhs, c->st);
     apply_mdagm(c, f.hp, nrhs, f.hp == 60 ? f.ap_hi : f.x_hi, f.ap_hi_n, f.ap_hi, nullptr, f.t_hi, f.t_hi_n, f.y_hi,
-                f.y_hi_n, nullptr, nullptr, nullptr, true);
+                f.y_hi_n, nullptr, nullptr, nullptr, true);  // (its result in FP64)
   } else
     launch_zero(f.ap_hi, spinor_bytes(g, 64, nrhs), c->st);
   launch_true_residual(f.pr, g, nrhs, f.b_hi, f.ap_hi, f.r_lo, f.r_lo_n, reduce_args(c, FIN_CG_TRUE), c->st);
-  launch_p_update(f.pr, f.pp, g, nrhs, f.r_lo, f.r_lo_n, f.p, f.p_n, c->cg, nullptr, c->st);
+  if (!pc_p) launch_p_update(f.pr, f.pp, g, nrhs, f.r_lo, f.r_lo_n, f.p, f.p_n, c->cg, nullptr, c->st);
 
   std::vector<double> rho(nrhs, c->last_rho);
   // event pairs of persistent launches and graphs left by a solve that returned early (an error)
@@ -1224,10 +1269,8 @@ qcd_status cg_batch(qcd_ctx* c, double2* x, const double2* b, int nrhs, const qc
   }
   c->pc_pending.clear();
   c->launched.clear();
-  // one RHS: the persistent kernel runs each segment of iterations, and the rounds (segment, gated
-  // reliable update) expected before convergence are enqueued together, with one look at the state
-  // after them
-  const bool use_pc = c->persistent && nrhs == 1 && f.pp != 60 && g.Vh <= PERSISTENT_MAX_VH;
+  // one RHS: the rounds (persistent segment, gated reliable update) expected before convergence are enqueued
+  // together, with one look at the state after them
   qcd_status result = QCD_OK;
   bool after_reliable = true;
   int done_iters = 0;
@@ -1242,7 +1285,7 @@ qcd_status cg_batch(qcd_ctx* c, double2* x, const double2* b, int nrhs, const qc
       for (int k = 0; k < rounds; k++) {
         if ((s = launch_persistent(c, f, prm->max_iter, k))) return s;
         ItGraph* rk;
-        if ((s = get_graph(c, 1, k, f, nrhs, &rk))) return s;
+        if ((s = get_graph(c, rel_kind, k, f, nrhs, &rk))) return s;
         if ((s = launch_graph(c, rk, 0, k))) return s;
       }
       CUDA_TRY(cudaMemcpyAsync(c->h_pc_rounds, c->pc_rounds, sizeof(int) * rounds, cudaMemcpyDeviceToHost, c->st));
@@ -1305,7 +1348,7 @@ qcd_status cg_batch(qcd_ctx* c, double2* x, const double2* b, int nrhs, const qc
     }
     after_reliable = false;
     if (c->h_ctl->halt) {
-      if (!rel && (s = get_graph(c, 1, 0, f, nrhs, &rel))) return s;
+      if (!rel && (s = get_graph(c, rel_kind, 0, f, nrhs, &rel))) return s;
       if ((s = launch_graph(c, rel, 0))) return s;
       after_reliable = true;
       if (candidate) {
@@ -1325,7 +1368,7 @@ qcd_status cg_batch(qcd_ctx* c, double2* x, const double2* b, int nrhs, const qc
   for (int r = 0; r < nrhs; r++)
     if (rho[r] > 0.0 && rho[r] < 1.0) c->last_rho = rho[r];
   // not converged: fold the progress into x and recompute the true residual for the stats
-  if (result == QCD_ERR_NOT_CONVERGED) enqueue_reliable(c, f, nrhs, false);
+  if (result == QCD_ERR_NOT_CONVERGED) enqueue_reliable(c, f, nrhs, false, !pc_p);
   // fold the last low-precision increment into x and write out
   launch_accumulate_x(f.pr, g, nrhs, f.x_hi, f.x_lo, f.x_lo_n, c->st);
   launch_spinor_to_canon(64, g, f.x_hi, nullptr, x, nrhs, c->st);

@@ -270,10 +270,10 @@ __global__ void __launch_bounds__(PcShape<P>::THREADS, PcShape<P>::MIN_BLOCKS)
 
   // FP32: the p update p = r + beta p of iteration k is formed where p is read in phases 1 and 2 of
   // iteration k+1 (phase 2 writes it back), so phase 5 and its grid barrier are not needed; the first
-  // iteration of a launch finds p already updated (coefficients 0, 1)
+  // iteration of a launch takes beta from the state (the reliable update or the set-up before it left p as it
+  // was; a p update and a kernel lowering the gate, each 5 us of launch and latency a round at 16^4)
   constexpr bool LAZY = P == 32;
-  bool first = true;
-  double alpha = 0.0, beta = 0.0, pAp = 0.0;
+  double alpha = 0.0, beta = st0.beta, pAp = 0.0;
   unsigned bar_target = 0;
   while (true) {
     // phase 1
@@ -281,8 +281,8 @@ __global__ void __launch_bounds__(PcShape<P>::THREADS, PcShape<P>::MIN_BLOCKS)
     a1.in_norm = Q.p_n;
     a1.in_g5 = 0;
     a1.lz_r = Q.r;
-    a1.lz_a = first ? 0.f : 1.f;
-    a1.lz_b = first ? 1.f : float(beta);
+    a1.lz_a = 1.f;
+    a1.lz_b = float(beta);
     run_phase<P, RECON, EPI_CLOVER_INV, LAZY>(a1, part, xch, stage, 0.0);
     if (!grid_barrier(Q.bar_count, bar_target, Q.bar_err)) return;
     // phase 2
@@ -346,11 +346,8 @@ __global__ void __launch_bounds__(PcShape<P>::THREADS, PcShape<P>::MIN_BLOCKS)
     iters += 1;
     since += 1;
     const bool want = rr_new <= st0.tol2 || since >= every || rr_new < delta2 * st0.rr_reliable;
-    first = false;
-    // phase 5 (with LAZY only when the launch ends without a reliable update, so that the next launch
-    // finds p updated; at a reliable update the update's own p = r + beta p follows)
-    if (!want && (!LAZY || iters >= Q.iter_limit)) {
-      // phase 5
+    // phase 5 (at a reliable update the update's own p = r + beta p follows; LAZY: the next iteration's)
+    if (!want && !LAZY) {
       for (int h = blockIdx.x * BLOCK + threadIdx.x; h < Vh; h += gridDim.x * BLOCK) {
         cx<RR> rs[12];
         cx<R> ps[12], out[12];

@@ -21,6 +21,7 @@ enum Epilogue {
   EPI_NONE = 0,        // out = D in
   EPI_CLOVER_INV = 1,  // out = C (D in)            (C = A^-1 of the output parity)
   EPI_XPAY = 2,        // out = C x + a (D in)      (C = A of the output parity)
+  EPI_RESID = 4,       // fixed-point kernels: r_lo = b - (C x + a (D in)), |b - ...|^2 (the true residual of the CG)
   EPI_XPAY_CG = 3,     // Ap = C x + a (D in), not stored: x_lo += alpha p, r_lo -= alpha Ap, |r_lo|^2
 };
 
@@ -51,6 +52,8 @@ struct DslashArgs {
   void* cg_r;
   const void* cg_p;
   const float* cg_p_norm;
+  // EPI_RESID: b (FP64) in cg_p, r_lo (FP32, or FP64 where r_f64) in cg_r
+  int r_f64;
   // t-slab halos (hopping kernels instantiated with HALO): the neighbouring slabs' contributions to
   // the time hops that leave this slab, one entry per site of a t-face (XYZ/2 per parity), layout of
   // HaloIO.  halo_hi: (1 - g_t) psi of the upper slab's t = 0 sites, multiplied here by U_t(x);

@@ -331,7 +331,7 @@ __device__ __forceinline__ double pair_fx(const DslashArgs& A, const FxScalar& s
       for (int k = 0; k < 6; k++) t[k] = -t[k];
     }
   }
-  if (EPI == EPI_XPAY_CG || A.out_f64) {
+  if (EPI == EPI_XPAY_CG || EPI == EPI_RESID || A.out_f64) {
     if (valid) {
       cx<double> res[6];
       const int e = bad ? FX_NAN : unit;
@@ -355,6 +355,23 @@ __device__ __forceinline__ double pair_fx(const DslashArgs& A, const FxScalar& s
           }
           SpinorIO<64>::store_block(A.cg_x, nullptr, Vh, r, hh, B, xs);
           SpinorIO<64>::store_block(A.cg_r, nullptr, Vh, r, hh, B, rs);
+        }
+      } else if (EPI == EPI_RESID) {
+        cx<double> bs[6];
+        SpinorIO<64>::load_block(A.cg_p, nullptr, Vh, r, hh, B, bs);
+#pragma unroll
+        for (int k = 0; k < 6; k++) {
+          res[k] = bs[k] - res[k];
+          nrm = fma(res[k].re, res[k].re, nrm);
+          nrm = fma(res[k].im, res[k].im, nrm);
+        }
+        if (A.r_f64) {
+          SpinorIO<64>::store_block(A.cg_r, nullptr, Vh, r, hh, B, res);
+        } else {
+          cx<float> lo[6];
+#pragma unroll
+          for (int k = 0; k < 6; k++) lo[k] = cmk(narrow(res[k].re), narrow(res[k].im));
+          SpinorIO<32>::store_block(A.cg_r, nullptr, Vh, r, hh, B, lo);
         }
       } else {
         SpinorIO<64>::store_block(A.out, nullptr, Vh, r, hh, B, res);
@@ -423,7 +440,7 @@ __global__ void __launch_bounds__(64 * PAIRS, 8 / PAIRS) dslash_fixed_kernel(Dsl
     }
   }
   __syncthreads();
-  const bool reduce = A.do_norm || EPI == EPI_XPAY_CG;
+  const bool reduce = A.do_norm || EPI == EPI_XPAY_CG || EPI == EPI_RESID;
 #pragma unroll 1
   for (int r0 = 0; r0 < A.nrhs; r0 += PAIRS) {
     const int r = r0 + q;
@@ -512,6 +529,7 @@ void launch_dslash_fixed(int epi, const DslashArgs& a, cudaStream_t st) {
     case EPI_NONE: launch_fx<EPI_NONE>(a, sc, st); break;
     case EPI_CLOVER_INV: launch_fx<EPI_CLOVER_INV>(a, sc, st); break;
     case EPI_XPAY_CG: launch_fx<EPI_XPAY_CG>(a, sc, st); break;
+    case EPI_RESID: launch_fx<EPI_RESID>(a, sc, st); break;
     default: launch_fx<EPI_XPAY>(a, sc, st); break;
   }
 }

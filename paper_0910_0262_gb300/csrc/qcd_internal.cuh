@@ -766,6 +766,7 @@ struct ReduceArgs {
   int mode;
   CGState* cg;
   CGControl* ctl;
+  int lower_gate;          // FIN_CG_TRUE: also lower ctl->rel_go (no later kernel of the update is gated by it)
 };
 
 // Per-RHS action of the last block once the grid-wide total is known.
@@ -917,6 +918,7 @@ __device__ __forceinline__ void grid_finish(int nrhs, long long blk_total, int n
       int any = 0;
       for (int r = 0; r < nrhs; r++) any |= ra.cg[r].active;
       ra.ctl->halt = (any && !ra.ctl->nan) ? 0 : 1;
+      if (ra.lower_gate) ra.ctl->rel_go = 0;
     }
     *ra.counter = 0u;
   }
