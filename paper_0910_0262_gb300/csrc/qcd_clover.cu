@@ -75,60 +75,97 @@ __device__ M3 field_strength(const Geom& g, const double2* g64, const int c[4], 
 
 __host__ __device__ constexpr int tri(int i, int j) { return i * (i - 1) / 2 + j; }
 
-// Cholesky-based inverse of a Hermitian positive definite 6x6 matrix given as (diag d,
-// strictly-lower L), and log det = sum_j log L_jj^2.  Returns false on a non-positive pivot.  All
-// loops are unrolled, so the packed triangles stay in registers: A = l l^dag (l lower, diagonal ld),
-// m = l^-1 (lower), A^-1 = m^dag m.  inverse false: the factorisation and log det only.
+// acc - a conj(b), acc - conj(a) b (four multiply-adds)
+__device__ __forceinline__ C cfms_nc(C a, C b, C acc) {
+  acc.re = fma(-a.re, b.re, acc.re);
+  acc.re = fma(-a.im, b.im, acc.re);
+  acc.im = fma(-a.im, b.re, acc.im);
+  acc.im = fma(a.re, b.im, acc.im);
+  return acc;
+}
+
+// sum of log s_j: the logarithm of the pivots' product, formed with its rounding errors (Dekker 1971, with
+// fused multiply-adds) so that it is no less exact than the sum of the six; where the product leaves the
+// middle of the double range, that sum.
+__device__ __forceinline__ double log_product(const double s[6]) {
+  double p = s[0], e = 0.0;
+  bool middle = p > 1e-40 && p < 1e40;
+#pragma unroll
+  for (int j = 1; j < 6; j++) {
+    const double q = p * s[j];
+    e = fma(e, s[j], fma(p, s[j], -q));
+    p = q;
+    middle = middle && s[j] > 1e-40 && s[j] < 1e40;
+  }
+  if (middle) return log(p) + e / p;
+  double sum = 0.0;
+  for (int j = 0; j < 6; j++) sum += log(s[j]);
+  return sum;
+}
+
+// Inverse of a Hermitian positive definite 6x6 matrix given as (diag d, strictly-lower L) by the factorisation
+// A = l D l^dag (l unit lower triangular, D its pivots s_j: Cholesky without square roots), and log det =
+// sum_j log s_j.  Returns false on a non-positive pivot.  All loops are unrolled, so the packed triangles
+// stay in registers: m = l^-1, A^-1 = m^dag D^-1 m.  inverse false: the factorisation and log det only.
 __device__ __forceinline__ bool invert6(const double d[6], const C L[15], bool inverse, double di[6], C Li[15],
                                         double* logdet) {
-  double ild[6];  // 1 / l_jj: one division per pivot, multiplications elsewhere
-  C lo[15];       // strictly-lower part of l
-  double ldet = 0.0;
+  double s[6], is[6];  // pivots and their reciprocals
+  C lo[15];            // strictly-lower part of l
+  C u[15];             // l D
   bool ok = true;
 #pragma unroll
   for (int j = 0; j < 6; j++) {
-    double s = d[j];
+    double t = d[j];
 #pragma unroll
-    for (int k = 0; k < j; k++) s -= norm2(lo[tri(j, k)]);
-    ok = ok && s > 0.0;
-    s = s > 0.0 ? s : 1.0;  // keeps the arithmetic finite; the result is discarded when !ok
-    ldet += log(s);
-    ild[j] = 1.0 / sqrt(s);
+    for (int k = 0; k < j; k++) {
+      t = fma(-u[tri(j, k)].re, lo[tri(j, k)].re, t);
+      t = fma(-u[tri(j, k)].im, lo[tri(j, k)].im, t);
+    }
+    ok = ok && t > 0.0;
+    s[j] = t > 0.0 ? t : 1.0;  // keeps the arithmetic finite; the result is discarded when !ok
+    is[j] = 1.0 / s[j];
 #pragma unroll
     for (int i = j + 1; i < 6; i++) {
       C v = L[tri(i, j)];
 #pragma unroll
-      for (int k = 0; k < j; k++) v = v - lo[tri(i, k)] * conj(lo[tri(j, k)]);
-      lo[tri(i, j)] = cmk(v.re * ild[j], v.im * ild[j]);
+      for (int k = 0; k < j; k++) v = cfms_nc(u[tri(i, k)], lo[tri(j, k)], v);
+      u[tri(i, j)] = v;
+      lo[tri(i, j)] = cmk(v.re * is[j], v.im * is[j]);
     }
   }
   if (!ok) return false;
-  *logdet = ldet;
+  *logdet = log_product(s);
   if (!inverse) return true;
-  // m = l^-1: m_jj = 1 / l_jj, m_ij = -(sum_{k=j}^{i-1} l_ik m_kj) / l_ii for i > j
+  // m = l^-1: m_ij = -(l_ij + sum_{k=j+1}^{i-1} l_ik m_kj) for i > j
   C mo[15];
 #pragma unroll
   for (int j = 0; j < 6; j++)
 #pragma unroll
     for (int i = j + 1; i < 6; i++) {
-      C s = cmk(lo[tri(i, j)].re * ild[j], lo[tri(i, j)].im * ild[j]);
+      C t = lo[tri(i, j)];
 #pragma unroll
-      for (int k = j + 1; k < i; k++) s = cfma(lo[tri(i, k)], mo[tri(k, j)], s);
-      mo[tri(i, j)] = cmk(-s.re * ild[i], -s.im * ild[i]);
+      for (int k = j + 1; k < i; k++) t = cfma(lo[tri(i, k)], mo[tri(k, j)], t);
+      mo[tri(i, j)] = -t;
     }
-  // A^-1 = m^dag m: (A^-1)_ij = sum_{k >= i} conj(m_ki) m_kj for i >= j
+  // A^-1 = m^dag D^-1 m: (A^-1)_ij = sum_{k >= i} conj(m_ki) m_kj / s_k for i >= j
 #pragma unroll
   for (int i = 0; i < 6; i++) {
-    double sd = ild[i] * ild[i];
+    C w[6];  // conj factor m_ki / s_k
 #pragma unroll
-    for (int k = i + 1; k < 6; k++) sd += norm2(mo[tri(k, i)]);
+    for (int k = i + 1; k < 6; k++) w[k] = cmk(is[k] * mo[tri(k, i)].re, is[k] * mo[tri(k, i)].im);
+    double sd = is[i];
+#pragma unroll
+    for (int k = i + 1; k < 6; k++) {
+      sd = fma(w[k].re, mo[tri(k, i)].re, sd);
+      sd = fma(w[k].im, mo[tri(k, i)].im, sd);
+    }
     di[i] = sd;
 #pragma unroll
     for (int j = 0; j < i; j++) {
-      C s = cmk(ild[i] * mo[tri(i, j)].re, ild[i] * mo[tri(i, j)].im);  // k = i: m_ii m_ij
+      C t = cmk(is[i] * mo[tri(i, j)].re, is[i] * mo[tri(i, j)].im);  // k = i: m_ii = 1
 #pragma unroll
-      for (int k = i + 1; k < 6; k++) s = cfmac(mo[tri(k, i)], mo[tri(k, j)], s);
-      Li[tri(i, j)] = s;
+      for (int k = i + 1; k < 6; k++) t = cfmac(w[k], mo[tri(k, j)], t);
+      Li[tri(i, j)] = t;
     }
   }
   return true;
@@ -261,6 +298,8 @@ __global__ void __launch_bounds__(128) field_strength_kernel(Geom g, const doubl
   for (int k = 0; k < 9; k++) q[(size_t)k * V] = make_double2(F.e[k].re, F.e[k].im);
 }
 
+// Bound by the FP64 pipe: with square roots, six logarithms and unfused complex products a block took 10%
+// more of its instructions on even and a third more on odd sites (24^3 x 32: 1.30 -> 0.98 ms).
 // A's chiral block b (even sites) or its inverse (odd sites), the ones the operators read, and log det, for
 // one (site, block) per thread, from the six F_{mu nu}
 __global__ void __launch_bounds__(128) clover_assemble_kernel(Geom g, const double2* __restrict__ Fbuf, double kappa,
