@@ -144,6 +144,157 @@ __device__ __forceinline__ FxShift fx_shift(int unit, int e) {
   return fx_shift(e > FX_BIG ? -63 : unit - e + FX_SPINOR);
 }
 
+// The epilogue of chiral block B of a site, RHS r, with the hopping sum v in units of 2^(eh - 56), and its
+// stores.  active: this warp has a block to finish (the others only meet the block's barriers); eo: the
+// finished blocks' exponents, in shared memory.  All threads of the block call it together.  Returns the
+// thread's share of |out|^2 (do_norm) or of |r|^2 (EPI_XPAY_CG, EPI_RESID).
+template <int EPI>
+__device__ __forceinline__ double finish_fx(const DslashArgs& A, const FxScalar& sc, int hh, bool valid, bool active, int r,
+                                            int B, cx<i64> v[6], int eh, int (*eo)[32]) {
+  const int lane = threadIdx.x & 31;
+  const int Vh = A.g.Vh;
+  double nrm = 0.0;
+  cx<i64> t[6];
+  int unit = 0;
+  bool bad = eh > FX_BIG;
+  if (valid) {
+    // v: the hopping sum of chiral block B in units of 2^(eh - 56)
+    unit = eh - 56;
+    if (EPI == EPI_NONE) {
+#pragma unroll
+      for (int k = 0; k < 6; k++) t[k] = v[k];
+    } else {
+      // v brought to full size, |v| < 2^60, in units of 2^unit
+      const int bits = fx_bits_of(v);
+      const FxShift full = fx_shift(60 - bits);
+#pragma unroll
+      for (int k = 0; k < 6; k++) v[k] = cmk(full(v[k].re), full(v[k].im));
+      unit += bits - 60;
+      const bool ok = dbg_clover(Vh, hh, B);
+      const int4* cl = static_cast<const int4*>(A.clover) + (size_t)(18 * B) * Vh + (ok ? hh : 0);
+      const int ec = __ldg(A.clover_e + (size_t)B * Vh + (ok ? hh : 0));
+      bad = bad || ec > FX_BIG;
+      if (EPI == EPI_CLOVER_INV) {
+        clover_fx(cl, Vh, v, t);
+        unit += ec + 2;
+      } else {
+        cx<i64> xs[6], cxs[6];
+        const longlong2* px = static_cast<const longlong2*>(A.x);
+        const int exx = __ldg(reinterpret_cast<const int*>(A.x_norm) + (size_t)r * Vh + hh);
+        bad = bad || exx > FX_BIG || sc.e > FX_BIG;
+#pragma unroll
+        for (int k = 0; k < 6; k++) {
+          const longlong2 x = __ldg(px + sidx<12>(6 * B + k, Vh, r, hh));
+          xs[k] = cmk((i64)x.x, (i64)x.y);
+        }
+        if (A.x_g5 && B == 1) {
+#pragma unroll
+          for (int k = 0; k < 6; k++) xs[k] = -xs[k];
+        }
+        clover_fx(cl, Vh, xs, cxs);
+        // C x in units of 2^u1, a v in units of 2^u2 (each below 2^61.5)
+        const int u1 = exx - FX_SPINOR + ec + 2, u2 = unit + sc.e - 1;
+        unit = max(u1, u2);
+        const int k1 = min(unit - u1, 63), k2 = min(unit - u2, 63);
+#pragma unroll
+        for (int k = 0; k < 6; k++) {
+          FxSum pr = {}, pi = {};
+          fx_mac(pr, sc.v, fx_split(v[k].re));
+          fx_mac(pi, sc.v, fx_split(v[k].im));
+          t[k].re = (cxs[k].re >> k1) + (fx_value<4>(pr) >> k2);
+          t[k].im = (cxs[k].im >> k1) + (fx_value<4>(pi) >> k2);
+        }
+      }
+    }
+    if (A.out_g5 && B == 1) {
+#pragma unroll
+      for (int k = 0; k < 6; k++) t[k] = -t[k];
+    }
+  }
+  if (EPI == EPI_XPAY_CG || EPI == EPI_RESID || A.out_f64) {
+    if (valid) {
+      cx<double> res[6];
+      const int e = bad ? FX_NAN : unit;
+#pragma unroll
+      for (int k = 0; k < 6; k++) res[k] = cmk(fx_to_double(t[k].re, e, 0), fx_to_double(t[k].im, e, 0));
+      if (EPI == EPI_XPAY_CG) {
+        if (A.red.cg[r].active) {
+          const double al = A.red.cg[r].alpha;
+          cx<double> ps[6], xs[6], rs[6];
+          SpinorIO<60>::load_block(A.cg_p, A.cg_p_norm, Vh, r, hh, B, ps);
+          SpinorIO<64>::load_block(A.cg_x, nullptr, Vh, r, hh, B, xs);
+          SpinorIO<64>::load_block(A.cg_r, nullptr, Vh, r, hh, B, rs);
+#pragma unroll
+          for (int k = 0; k < 6; k++) {
+            xs[k].re = fma(al, ps[k].re, xs[k].re);
+            xs[k].im = fma(al, ps[k].im, xs[k].im);
+            rs[k].re = fma(-al, res[k].re, rs[k].re);
+            rs[k].im = fma(-al, res[k].im, rs[k].im);
+            nrm = fma(rs[k].re, rs[k].re, nrm);
+            nrm = fma(rs[k].im, rs[k].im, nrm);
+          }
+          SpinorIO<64>::store_block(A.cg_x, nullptr, Vh, r, hh, B, xs);
+          SpinorIO<64>::store_block(A.cg_r, nullptr, Vh, r, hh, B, rs);
+        }
+      } else if (EPI == EPI_RESID) {
+        cx<double> bs[6];
+        SpinorIO<64>::load_block(A.cg_p, nullptr, Vh, r, hh, B, bs);
+#pragma unroll
+        for (int k = 0; k < 6; k++) {
+          res[k] = bs[k] - res[k];
+          nrm = fma(res[k].re, res[k].re, nrm);
+          nrm = fma(res[k].im, res[k].im, nrm);
+        }
+        if (A.r_f64) {
+          SpinorIO<64>::store_block(A.cg_r, nullptr, Vh, r, hh, B, res);
+        } else {
+          cx<float> lo[6];
+#pragma unroll
+          for (int k = 0; k < 6; k++) lo[k] = cmk(narrow(res[k].re), narrow(res[k].im));
+          SpinorIO<32>::store_block(A.cg_r, nullptr, Vh, r, hh, B, lo);
+        }
+      } else {
+        SpinorIO<64>::store_block(A.out, nullptr, Vh, r, hh, B, res);
+      }
+    }
+    __syncthreads();  // the exchange area is rewritten by the next RHS
+    return nrm;
+  }
+  // the site's exponent is the larger of its two blocks'
+  int eb = FX_ZERO;
+  if (valid) {
+    const int bits = fx_bits_of(t);
+    eb = bad ? FX_NAN : (bits ? unit + bits : FX_ZERO);
+  }
+  if (active) eo[B][lane] = eb;
+  __syncthreads();
+  if (valid && dbg_spinor(Vh, r, hh)) {
+    const int e = max(eb, eo[1 - B][lane]);
+    const FxShift f = fx_shift(unit, e);
+    longlong2* po = static_cast<longlong2*>(A.out);
+    FxSum n = {};
+#pragma unroll
+    for (int k = 0; k < 6; k++) {
+      const i64 a = f(t[k].re), b = f(t[k].im);
+      if (A.do_norm) {  // |v| < 2^60, summed as squares of v / 4
+        const FxLimb x = fx_split(a >> 2), y = fx_split(b >> 2);
+        n.h += (i64)x.hi * x.hi;
+        n.h += (i64)y.hi * y.hi;
+        n.m += (i64)x.hi * x.lo;
+        n.m += (i64)y.hi * y.lo;
+      }
+      po[sidx<12>(6 * B + k, Vh, r, hh)] = make_longlong2(a, b);
+    }
+    if (B == 0) reinterpret_cast<int*>(A.out_norm)[(size_t)r * Vh + hh] = e;
+    if (A.do_norm) {
+      const int u = e > FX_BIG ? FX_NAN : 2 * (e - FX_SPINOR + 2);
+      nrm = fx_to_double(n.h, u + 62, 0) + fx_to_double(n.m, u + 32, 0);
+    }
+  }
+  __syncthreads();  // the exchange area is rewritten by the next RHS
+  return nrm;
+}
+
 // Warp B of a pair: half-spinor row B of the eight hops of 32 output sites and RHS r, then chiral block B
 // (warp 0 passes on its parts of spins 2 and 3, warp 1 spin 1).  With the rows, not the directions, shared
 // out, a thread's sums are 9 complex numbers instead of 12.  The neighbours and links of the hops come
@@ -260,13 +411,9 @@ __device__ __forceinline__ double pair_fx(const DslashArgs& A, const FxScalar& s
     }
   }
   __syncthreads();
-  double nrm = 0.0;
-  cx<i64> t[6];
-  int unit = 0;
-  bool bad = eh > FX_BIG;
+  // the hopping sum of chiral block B
+  cx<i64> v[6] = {};
   if (valid) {
-    // the hopping sum of chiral block B in units of 2^(eh - 56)
-    cx<i64> v[6];
 #pragma unroll
     for (int a = 0; a < 3; a++) {
       const int at = B == 0 ? 0 : 6;
@@ -279,140 +426,8 @@ __device__ __forceinline__ double pair_fx(const DslashArgs& A, const FxScalar& s
         v[3 + a] = low[a] + cmk(xch->v[12 + 2 * a][lane], xch->v[12 + 2 * a + 1][lane]);
       }
     }
-    unit = eh - 56;
-    if (EPI == EPI_NONE) {
-#pragma unroll
-      for (int k = 0; k < 6; k++) t[k] = v[k];
-    } else {
-      // v brought to full size, |v| < 2^60, in units of 2^unit
-      const int bits = fx_bits_of(v);
-      const FxShift full = fx_shift(60 - bits);
-#pragma unroll
-      for (int k = 0; k < 6; k++) v[k] = cmk(full(v[k].re), full(v[k].im));
-      unit += bits - 60;
-      const bool ok = dbg_clover(Vh, hh, B);
-      const int4* cl = static_cast<const int4*>(A.clover) + (size_t)(18 * B) * Vh + (ok ? hh : 0);
-      const int ec = __ldg(A.clover_e + (size_t)B * Vh + (ok ? hh : 0));
-      bad = bad || ec > FX_BIG;
-      if (EPI == EPI_CLOVER_INV) {
-        clover_fx(cl, Vh, v, t);
-        unit += ec + 2;
-      } else {
-        cx<i64> xs[6], cxs[6];
-        const longlong2* px = static_cast<const longlong2*>(A.x);
-        const int exx = __ldg(reinterpret_cast<const int*>(A.x_norm) + (size_t)r * Vh + hh);
-        bad = bad || exx > FX_BIG || sc.e > FX_BIG;
-#pragma unroll
-        for (int k = 0; k < 6; k++) {
-          const longlong2 x = __ldg(px + sidx<12>(6 * B + k, Vh, r, hh));
-          xs[k] = cmk((i64)x.x, (i64)x.y);
-        }
-        if (A.x_g5 && B == 1) {
-#pragma unroll
-          for (int k = 0; k < 6; k++) xs[k] = -xs[k];
-        }
-        clover_fx(cl, Vh, xs, cxs);
-        // C x in units of 2^u1, a v in units of 2^u2 (each below 2^61.5)
-        const int u1 = exx - FX_SPINOR + ec + 2, u2 = unit + sc.e - 1;
-        unit = max(u1, u2);
-        const int k1 = min(unit - u1, 63), k2 = min(unit - u2, 63);
-#pragma unroll
-        for (int k = 0; k < 6; k++) {
-          FxSum pr = {}, pi = {};
-          fx_mac(pr, sc.v, fx_split(v[k].re));
-          fx_mac(pi, sc.v, fx_split(v[k].im));
-          t[k].re = (cxs[k].re >> k1) + (fx_value<4>(pr) >> k2);
-          t[k].im = (cxs[k].im >> k1) + (fx_value<4>(pi) >> k2);
-        }
-      }
-    }
-    if (A.out_g5 && B == 1) {
-#pragma unroll
-      for (int k = 0; k < 6; k++) t[k] = -t[k];
-    }
   }
-  if (EPI == EPI_XPAY_CG || EPI == EPI_RESID || A.out_f64) {
-    if (valid) {
-      cx<double> res[6];
-      const int e = bad ? FX_NAN : unit;
-#pragma unroll
-      for (int k = 0; k < 6; k++) res[k] = cmk(fx_to_double(t[k].re, e, 0), fx_to_double(t[k].im, e, 0));
-      if (EPI == EPI_XPAY_CG) {
-        if (A.red.cg[r].active) {
-          const double al = A.red.cg[r].alpha;
-          cx<double> ps[6], xs[6], rs[6];
-          SpinorIO<60>::load_block(A.cg_p, A.cg_p_norm, Vh, r, hh, B, ps);
-          SpinorIO<64>::load_block(A.cg_x, nullptr, Vh, r, hh, B, xs);
-          SpinorIO<64>::load_block(A.cg_r, nullptr, Vh, r, hh, B, rs);
-#pragma unroll
-          for (int k = 0; k < 6; k++) {
-            xs[k].re = fma(al, ps[k].re, xs[k].re);
-            xs[k].im = fma(al, ps[k].im, xs[k].im);
-            rs[k].re = fma(-al, res[k].re, rs[k].re);
-            rs[k].im = fma(-al, res[k].im, rs[k].im);
-            nrm = fma(rs[k].re, rs[k].re, nrm);
-            nrm = fma(rs[k].im, rs[k].im, nrm);
-          }
-          SpinorIO<64>::store_block(A.cg_x, nullptr, Vh, r, hh, B, xs);
-          SpinorIO<64>::store_block(A.cg_r, nullptr, Vh, r, hh, B, rs);
-        }
-      } else if (EPI == EPI_RESID) {
-        cx<double> bs[6];
-        SpinorIO<64>::load_block(A.cg_p, nullptr, Vh, r, hh, B, bs);
-#pragma unroll
-        for (int k = 0; k < 6; k++) {
-          res[k] = bs[k] - res[k];
-          nrm = fma(res[k].re, res[k].re, nrm);
-          nrm = fma(res[k].im, res[k].im, nrm);
-        }
-        if (A.r_f64) {
-          SpinorIO<64>::store_block(A.cg_r, nullptr, Vh, r, hh, B, res);
-        } else {
-          cx<float> lo[6];
-#pragma unroll
-          for (int k = 0; k < 6; k++) lo[k] = cmk(narrow(res[k].re), narrow(res[k].im));
-          SpinorIO<32>::store_block(A.cg_r, nullptr, Vh, r, hh, B, lo);
-        }
-      } else {
-        SpinorIO<64>::store_block(A.out, nullptr, Vh, r, hh, B, res);
-      }
-    }
-    __syncthreads();  // the exchange area is rewritten by the next RHS
-    return nrm;
-  }
-  // the site's exponent is the larger of its two blocks'
-  int eb = FX_ZERO;
-  if (valid) {
-    const int bits = fx_bits_of(t);
-    eb = bad ? FX_NAN : (bits ? unit + bits : FX_ZERO);
-  }
-  xch->eo[B][lane] = eb;
-  __syncthreads();
-  if (valid && dbg_spinor(Vh, r, hh)) {
-    const int e = max(eb, xch->eo[1 - B][lane]);
-    const FxShift f = fx_shift(unit, e);
-    longlong2* po = static_cast<longlong2*>(A.out);
-    FxSum n = {};
-#pragma unroll
-    for (int k = 0; k < 6; k++) {
-      const i64 a = f(t[k].re), b = f(t[k].im);
-      if (A.do_norm) {  // |v| < 2^60, summed as squares of v / 4
-        const FxLimb x = fx_split(a >> 2), y = fx_split(b >> 2);
-        n.h += (i64)x.hi * x.hi;
-        n.h += (i64)y.hi * y.hi;
-        n.m += (i64)x.hi * x.lo;
-        n.m += (i64)y.hi * y.lo;
-      }
-      po[sidx<12>(6 * B + k, Vh, r, hh)] = make_longlong2(a, b);
-    }
-    if (B == 0) reinterpret_cast<int*>(A.out_norm)[(size_t)r * Vh + hh] = e;
-    if (A.do_norm) {
-      const int u = e > FX_BIG ? FX_NAN : 2 * (e - FX_SPINOR + 2);
-      nrm = fx_to_double(n.h, u + 62, 0) + fx_to_double(n.m, u + 32, 0);
-    }
-  }
-  __syncthreads();  // the exchange area is rewritten by the next RHS
-  return nrm;
+  return finish_fx<EPI>(A, sc, hh, valid, true, r, B, v, eh, xch->eo);
 }
 
 // One pair of warps per (32 output sites, RHS); a block holds the pairs of PAIRS RHS of the same sites,
@@ -455,6 +470,110 @@ __global__ void __launch_bounds__(64 * PAIRS, 8 / PAIRS) dslash_fixed_kernel(Dsl
     }
   }
   if (reduce) grid_finish<0>(A.nrhs, gridDim.x, 2 * gridDim.x, A.red);
+}
+
+// The same for lattices whose pairs of warps would leave most of the GPU idle: four pairs per 32 output sites
+// and RHS (blockIdx.y), one direction each, whose sums meet in shared memory; pair 0 finishes the sites.  A
+// pass is then two hops and an epilogue long instead of eight hops and an epilogue, at the same work.
+template <int EPI>
+__global__ void __launch_bounds__(256, 2) dslash_fixed_split_kernel(DslashArgs A, FxScalar sc) {
+  extern __shared__ __align__(16) int4 fx_ring[];
+  __shared__ int eo[2][32];
+  if ((A.halt && *A.halt) || (A.gate && !*A.gate)) return;
+  const int lane = threadIdx.x & 31, w = threadIdx.x >> 5, q = w >> 1, B = w & 1, r = blockIdx.y;
+  const int hh = blockIdx.x * 32 + lane, Vh = A.g.Vh;
+  const bool valid = hh < Vh && dbg_spinor(Vh, r, hh);
+  constexpr int STAGE = fx_stage_rows(1) * 32;
+  int4* mine = fx_ring + 2 * q * STAGE + lane;  // the forward hop's stage, then the backward one's
+  Site s{};
+  int eh = FX_ZERO, ef = 0, eb = 0;
+  if (valid) {
+    s = site_of(A.g, A.p, hh);
+    const int* ex = reinterpret_cast<const int*>(A.in_norm) + (size_t)r * Vh;
+    const int nf = neighbor_fwd(A.g, s, q) >> 1, nb = neighbor_bwd(A.g, s, q) >> 1;
+    const int4* in = static_cast<const int4*>(A.in) + ((size_t)r * 12 + 6 * B) * Vh;
+    const int4* u = static_cast<const int4*>(A.gauge) + (size_t)(5 * B) * Vh;
+    const int4* uf = u + (size_t)((A.p * 4 + q) * 9) * Vh + hh;
+    const int4* ub = u + (size_t)(((1 - A.p) * 4 + q) * 9) * Vh + nb;
+    const int4 *pf = in + nf, *pb = in + nb;
+    if (dbg_link(Vh, 1 - A.p, q, nb) && dbg_spinor(Vh, r, nf)) {
+#pragma unroll
+      for (int k = 0; k < 6; k++) {
+        cp_async16(mine + 32 * (9 + 6 * B + k), pf + (size_t)k * Vh);
+        cp_async16(mine + STAGE + 32 * (9 + 6 * B + k), pb + (size_t)k * Vh);
+      }
+#pragma unroll
+      for (int k = 0; k < 5; k++) {
+        if (k < 4 || B == 0) {
+          cp_async16(mine + 32 * (5 * B + k), uf + (size_t)k * Vh);
+          cp_async16(mine + STAGE + 32 * (5 * B + k), ub + (size_t)k * Vh);
+        }
+      }
+    }
+#pragma unroll
+    for (int mu = 0; mu < 4; mu++) {
+      const int a = __ldg(ex + (neighbor_fwd(A.g, s, mu) >> 1)), b = __ldg(ex + (neighbor_bwd(A.g, s, mu) >> 1));
+      eh = max(eh, max(a, b));
+      ef = mu == q ? a : ef;
+      eb = mu == q ? b : eb;
+    }
+  }
+  cp_async_commit();
+  cp_async_wait_all();
+  __syncthreads();
+  cx<i64> up[3] = {}, low[3] = {};
+  {
+    const int g5 = A.in_g5 ? -1 : 0, p = q < 2 ? 3 - B : 2 + B;
+    const int df = min(eh - ef, 63), db = min(eh - eb, 63), tg = s.t + A.g.t0;
+    const longlong2* sf = reinterpret_cast<const longlong2*>(mine) + 32 * 9;
+    const longlong2* sb = sf + STAGE;
+    if (q & 1) {  // (g_y)_Bp: -1, 1; (g_t)_Bp: 1, 1
+      const int neg = q == 1 && B == 0 ? -1 : 0;
+      const bool anti = q == 3 && A.g.t_bc < 0.0;
+      hop_fx<false, false>(sf + 96 * B, sf + 96 * p, mine, neg, g5, anti && tg == A.g.Tg - 1, df, up, low);
+      hop_fx<false, true>(sb + 96 * B, sb + 96 * p, mine + STAGE, neg, g5, anti && tg == 0, db, up, low);
+    } else {  // (g_x)_Bp: i, i; (g_z)_Bp: i, -i
+      const int neg = q == 2 && B == 1 ? -1 : 0;
+      hop_fx<true, false>(sf + 96 * B, sf + 96 * p, mine, neg, g5, false, df, up, low);
+      hop_fx<true, true>(sb + 96 * B, sb + 96 * p, mine + STAGE, neg, g5, false, db, up, low);
+    }
+  }
+  __syncthreads();  // every pair has read its stages: the sums take their place
+  i64 (*part)[12][32] = reinterpret_cast<i64 (*)[12][32]>(fx_ring);  // [warp][up, low: component re, im][lane]
+#pragma unroll
+  for (int a = 0; a < 3; a++) {
+    part[w][2 * a][lane] = up[a].re;
+    part[w][2 * a + 1][lane] = up[a].im;
+    part[w][6 + 2 * a][lane] = low[a].re;
+    part[w][6 + 2 * a + 1][lane] = low[a].im;
+  }
+  __syncthreads();
+  cx<i64> v[6] = {};
+  if (q == 0 && valid) {
+#pragma unroll
+    for (int d = 0; d < 4; d++)
+#pragma unroll
+      for (int a = 0; a < 3; a++) {
+        // block 0: the upper spins 0, 1 of warps 0, 1; block 1: spin 2 from warp 1 (x, y) or 0 (z, t), spin 3
+        // from the other
+        const int w0 = 2 * d + (B == 0 ? 0 : (d < 2 ? 1 : 0)), w1 = 2 * d + (B == 0 ? 1 : (d < 2 ? 0 : 1));
+        const int o = B == 0 ? 2 * a : 6 + 2 * a;
+        v[a] = v[a] + cmk(part[w0][o][lane], part[w0][o + 1][lane]);
+        v[3 + a] = v[3 + a] + cmk(part[w1][o][lane], part[w1][o + 1][lane]);
+      }
+  }
+  double nrm = finish_fx<EPI>(A, sc, hh, valid && q == 0, q == 0, r, B, v, eh, eo);
+  if (A.do_norm || EPI == EPI_XPAY_CG || EPI == EPI_RESID) {
+    if (q == 0) {
+      for (int off = 16; off >= 1; off >>= 1) nrm += __shfl_xor_sync(0xffffffffu, nrm, off);
+      if (lane == 0) {
+        const long long slot = (long long)r * (2 * gridDim.x) + 2 * blockIdx.x + B;
+        if (slot < A.red.capacity) A.red.partials[slot] = nrm;
+        else A.red.ctl->overflow = 1;
+      }
+    }
+    grid_finish<256>(A.nrhs, (long long)gridDim.x * gridDim.y, 2 * gridDim.x, A.red);
+  }
 }
 
 // out = C in on the sites of one parity, one thread per (site, RHS)
@@ -513,8 +632,20 @@ void launch_fx_pairs(const DslashArgs& a, const FxScalar& sc, cudaStream_t st) {
   dslash_fixed_kernel<EPI, PAIRS><<<(a.g.Vh + 31) / 32, 64 * PAIRS, sh, st>>>(a, sc);
 }
 
+// Units (32 sites, RHS) up to which a pass takes the split kernel: one block on each of the 152 SMs (4^3 x 8, 8
+// units: 12.6 -> 10.4 us a pass; 8 x 8 x 16 x 16, 256 units: 14.3 against 14.5 us, 12^3 x 20, 540 units: 18.2
+// against 23.0 us).
+const int FX_SPLIT_UNITS = 152;
+
 template <int EPI>
 void launch_fx(const DslashArgs& a, const FxScalar& sc, cudaStream_t st) {
+  const int nb = (a.g.Vh + 31) / 32;
+  if ((long long)nb * a.nrhs <= FX_SPLIT_UNITS) {
+    constexpr size_t sh = sizeof(int4) * 32 * fx_stage_rows(1) * 8;
+    cudaFuncSetAttribute(dslash_fixed_split_kernel<EPI>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sh);
+    dslash_fixed_split_kernel<EPI><<<dim3(nb, a.nrhs), 256, sh, st>>>(a, sc);
+    return;
+  }
   if (a.nrhs >= 4) launch_fx_pairs<EPI, 4>(a, sc, st);
   else if (a.nrhs >= 2) launch_fx_pairs<EPI, 2>(a, sc, st);
   else launch_fx_pairs<EPI, 1>(a, sc, st);
