@@ -1258,7 +1258,7 @@ __device__ __forceinline__ void dslash_site_body(const DslashArgs& A) {
       act = A.red.cg[r].active != 0;
       al = A.red.cg[r].alpha;
     }
-    double nrm = 0.0;
+    RR nb[2] = {RR(0), RR(0)};  // |.|^2 of the two chiral blocks in the precision of r (FP32 below FP64)
     if (valid) {
       cx<R> acc[12];
       if constexpr (P == 16) {
@@ -1333,7 +1333,7 @@ __device__ __forceinline__ void dslash_site_body(const DslashArgs& A) {
               n6 = fma(rs[j].re, rs[j].re, n6);
               n6 = fma(rs[j].im, rs[j].im, n6);
             }
-            nrm += double(n6);
+            nb[b] = n6;
             SpinorIO<PR>::store_block(A.cg_x, nullptr, Vh, r, hh, b, xs);
             SpinorIO<PR>::store_block(A.cg_r, nullptr, Vh, r, hh, b, rs);
           }
@@ -1345,7 +1345,7 @@ __device__ __forceinline__ void dslash_site_body(const DslashArgs& A) {
               n6 = fma(o[j].re, o[j].re, n6);
               n6 = fma(o[j].im, o[j].im, n6);
             }
-            nrm += double(n6);
+            nb[b] = n6;
           }
 #pragma unroll
           for (int j = 0; j < 6; j++) res[6 * b + j] = o[j];
@@ -1363,7 +1363,7 @@ __device__ __forceinline__ void dslash_site_body(const DslashArgs& A) {
       }
     }
     if (reduce) {
-      for (int off = 16; off >= 1; off >>= 1) nrm += __shfl_xor_sync(0xffffffffu, nrm, off);
+      const double nrm = warp_sum_nonneg(nb[0], nb[1]);
       if (lane == 0) {
         const long long slot = (long long)r * (gridDim.x * G) + blockIdx.x * G + grp;
         if (slot < A.red.capacity) A.red.partials[slot] = nrm;

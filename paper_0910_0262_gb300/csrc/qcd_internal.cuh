@@ -846,6 +846,37 @@ __device__ __forceinline__ void finalize_total(const ReduceArgs& ra, int r, doub
   }
 }
 
+// v 2^p as a double, rounded to nearest, with integer operations, for results well inside the double range
+// (no subnormals, no overflow: -900 < p < 900)
+__device__ __forceinline__ double scaled_to_double(unsigned long long m, int p) {
+  const int n = __clzll((long long)m);  // 64 for zero
+  const unsigned long long t = m << (n & 63);
+  const unsigned long long r = (t >> 11) + ((t >> 10) & 1);
+  return m ? __longlong_as_double((long long)(((unsigned long long)(p + 63 - n + 1022) << 52) + r)) : 0.0;
+}
+
+// The sum over the warp's lanes of a + b for FP32 a, b >= 0, rounded once to double, on every lane.  The
+// values' mantissas are added as integers in units of 2^-57 of the largest one's power of two: a shuffle
+// tree of FP64 adds takes 16 clocks of the SM's FP64 pipe an add and conversion, 144 for each 32 sites and
+// right-hand side (32^3 x 64, 8 RHS FP16, the pass that forms |Mhat p|^2: TBD us).
+__device__ __forceinline__ double warp_sum_nonneg(float a, float b) {
+  const unsigned ua = __float_as_uint(a), ub = __float_as_uint(b);
+  const unsigned mx = __reduce_max_sync(0xffffffffu, max(ua & 0x7fffffffu, ub & 0x7fffffffu));
+  if (mx >= 0x7f800000u) return (double)__uint_as_float(mx);  // a non-finite value
+  const int e = max((int)(mx >> 23), 1);
+  auto fixed = [&](unsigned u) {
+    const int x = max((int)(u >> 23), 1);
+    const unsigned long long m = (u & 0x7fffffu) | (u >= 0x00800000u ? 0x800000u : 0u);
+    return (m << 33) >> min(e - x, 63);
+  };
+  const unsigned long long v = fixed(ua & 0x7fffffffu) + fixed(ub & 0x7fffffffu);  // < 2^58; 32 of them < 2^63
+  const unsigned s0 = __reduce_add_sync(0xffffffffu, (unsigned)v & 0xfffffu);
+  const unsigned s1 = __reduce_add_sync(0xffffffffu, (unsigned)(v >> 20) & 0xfffffu);
+  const unsigned s2 = __reduce_add_sync(0xffffffffu, (unsigned)(v >> 40));
+  const unsigned long long t = ((unsigned long long)s2 << 40) + ((unsigned long long)s1 << 20) + s0;
+  return scaled_to_double(t, e - 127 - 23 - 33);
+}
+
 // Grid-wide deterministic sums, one per right-hand side, in two parts.  block_partial: the block's
 // sum of one double per thread for RHS r (warp shuffles, then shared memory) into slot
 // r * nblk + blk of the partials.  grid_finish: after all of a block's partials are written, the
