@@ -152,7 +152,9 @@ struct qcd_ctx {
   int* h_flags = nullptr;
   // reductions and CG state
   double* partials = nullptr;
-  unsigned* counter = nullptr;
+  unsigned* counter = nullptr;   // [1 + group_cap]
+  double* group_sums = nullptr;  // [MAX_RHS][group_cap]
+  int group_cap = 0;
   double* results = nullptr;
   CGState* cg = nullptr;
   CGControl* ctl = nullptr;
@@ -408,6 +410,8 @@ ReduceArgs reduce_args(qcd_ctx* c, int mode) {
   r.partials = c->partials;
   r.capacity = c->max_partials;
   r.counter = c->counter;
+  r.group_sums = c->group_sums;
+  r.group_cap = c->group_cap;
   r.result = c->results;
   r.mode = mode;
   r.cg = c->cg;
@@ -594,9 +598,13 @@ static qcd_status create_ctx(qcd_ctx** out, const int dims[4], double t_bc, void
   // (site, RHS) pairs per block, the fewest of all reducing kernels, so nrhs <= MAX_RHS needs
   // at most MAX_RHS * ceil(Vh * MAX_RHS / 32) slots
   c->max_partials = (long long)MAX_RHS * ((c->g.Vh * (long long)MAX_RHS + 31) / 32) + 64;
+  // groups of 64 blocks of a two-step sum: the hopping kernels' one block per 32 sites is the largest grid of
+  // those with several RHS; larger ones (flat sums over the links) take one step
+  c->group_cap = (c->g.Vh / 32 + 1 + 63) / 64;
   bool ok = cudaMalloc(&c->flags, 4 * sizeof(int)) == cudaSuccess &&
             cudaMalloc(&c->partials, sizeof(double) * (size_t)c->max_partials) == cudaSuccess &&
-            cudaMalloc(&c->counter, sizeof(unsigned)) == cudaSuccess &&
+            cudaMalloc(&c->counter, sizeof(unsigned) * (1 + (size_t)c->group_cap)) == cudaSuccess &&
+            cudaMalloc(&c->group_sums, sizeof(double) * MAX_RHS * (size_t)c->group_cap) == cudaSuccess &&
             cudaMalloc(&c->results, sizeof(double) * MAX_RHS) == cudaSuccess &&
             cudaMalloc(&c->cg, sizeof(CGState) * MAX_RHS) == cudaSuccess &&
             cudaMalloc(&c->ctl, sizeof(CGControl)) == cudaSuccess &&
@@ -611,7 +619,7 @@ static qcd_status create_ctx(qcd_ctx** out, const int dims[4], double t_bc, void
     qcd_destroy(c);
     return fail(QCD_ERR_NOMEM, "context allocation failed");
   }
-  cudaMemset(c->counter, 0, sizeof(unsigned));
+  cudaMemset(c->counter, 0, sizeof(unsigned) * (1 + (size_t)c->group_cap));
   cudaMemset(c->flags, 0, 4 * sizeof(int));
   cudaMemset(c->ctl, 0, sizeof(CGControl));
   {
@@ -622,8 +630,8 @@ static qcd_status create_ctx(qcd_ctx** out, const int dims[4], double t_bc, void
     c->persistent = coop != 0;
     const char* e = getenv("QCD_CG_PERSISTENT");
     if (e && e[0] == '0') c->persistent = false;
-    // two sets of per-block partials, then the two grid totals
-    if (cudaMalloc(&c->pc_part, sizeof(double) * (2 * c->pc_slots + 2)) != cudaSuccess ||
+    // two sets of per-block partials, then the two results of the summing barriers
+    if (cudaMalloc(&c->pc_part, sizeof(double) * (2 * c->pc_slots) + 2 * sizeof(PcTotal)) != cudaSuccess ||
         cudaMalloc(&c->pc_bar, 4 * sizeof(unsigned)) != cudaSuccess) {
       cudaGetLastError();
       qcd_destroy(c);
@@ -654,7 +662,7 @@ qcd_status qcd_destroy(qcd_ctx* c) {
   else cudaDeviceSynchronize();
   void* dev[] = {c->gfx, c->cfx.A_even, c->cfx.Ainv_odd, c->cfx.eA_even, c->cfx.eAinv_odd, c->g64, c->g32, c->g16, c->A64, c->Ainv64, c->A32, c->Ainv32, c->A16, c->Ainv16, c->logdet, c->flags,
                  c->pc_part, c->pc_bar, c->pc_rounds,
-                 c->partials, c->counter, c->results, c->cg, c->ctl,
+                 c->partials, c->counter, c->group_sums, c->results, c->cg, c->ctl,
                  c->U_ext, c->ext_g64, c->ext_A64, c->ext_Ainv64, c->ext_A32, c->ext_Ainv32, c->ext_A16, c->ext_Ainv16,
                  c->ext_logdet};
   for (void* p : dev)
@@ -1135,7 +1143,7 @@ qcd_status launch_persistent(qcd_ctx* c, const SolverFields& f, int iter_limit, 
   q.slots = c->pc_slots;
   q.bar_count = c->pc_bar;
   q.bar_flag = c->pc_bar + 1;
-  q.totals = c->pc_part + 2 * c->pc_slots;
+  q.totals = reinterpret_cast<PcTotal*>(c->pc_part + 2 * c->pc_slots);
   q.bar_err = reinterpret_cast<int*>(c->pc_bar + 2);
   q.iter_limit = iter_limit;
   q.round_out = c->pc_rounds + round;

@@ -25,7 +25,7 @@ __global__ void __launch_bounds__(BB) p_update_kernel(Geom g, const void* r, con
   const int k = blockIdx.y;
   const int h = blockIdx.x * BB + threadIdx.x;
   if (h >= g.Vh || !cg[k].active) return;
-  const RR beta = RR(cg[k].beta);
+  const RR beta = to_real<RR>(cg[k].beta);
   cx<RR> rs[12];
   cx<RP> ps[12];
   SpinorIO<PR>::load(r, rn, g.Vh, k, h, rs);
@@ -159,7 +159,7 @@ __global__ void __launch_bounds__(BB) xr_update_kernel(Geom g, int nrhs, void* x
   const int h = blockIdx.x * BB + threadIdx.x;
   double v = 0.0;
   if (h < g.Vh && cg[k].active) {
-    const RR al = RR(cg[k].alpha);
+    const RR al = to_real<RR>(cg[k].alpha);
     cx<RR> xs[12], rs[12];
     cx<RP> ps[12], as[12];
     SpinorIO<PR>::load(x_lo, nullptr, g.Vh, k, h, xs);

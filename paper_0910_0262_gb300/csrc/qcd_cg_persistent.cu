@@ -96,14 +96,17 @@ __device__ __forceinline__ double grid_total(const double* part);
 // Grid-wide barrier that also sums one double per block (`mine`, thread 0's value): every block
 // writes its partial and arrives on the counter with an acquire-release add; the block whose arrival
 // completes the count reads all partials (the add's acquire makes them visible), sums them in block
-// order -- the same bits whichever block arrives last -- publishes the total and releases the others
-// through *flag.  The total comes out of the barrier instead of after it (at 16^4 the separate sum of
-// 512 partials after a barrier took 2.5 us).  Returns false as grid_barrier does; *total: the sum.
-template <int BLOCK>
+// order -- the same bits whichever block arrives last -- derives from the total what every block needs next
+// (result(total): the step's coefficient and status, by its thread 0 alone), publishes it and releases the
+// others through *flag.  The total comes out of the barrier instead of after it (at 16^4 the separate sum of
+// 512 partials after a barrier took 2.5 us), and its consequences too: a division or comparison in FP64 that
+// every warp repeats for itself takes a sub-partition's FP64 pipe 64 clocks an instruction and warp (16^4:
+// 259 -> 251 us a launch).  Returns false as grid_barrier does; *out: the published result.
+template <int BLOCK, typename F>
 __device__ __forceinline__ bool grid_barrier_sum(unsigned* count, unsigned* flag, unsigned& target, int* err,
-                                                 double* part, double* slot, double mine, double* total) {
+                                                 double* part, PcTotal* slot, double mine, F result, PcTotal* out) {
   __shared__ int ok, last;
-  __shared__ double tot;
+  __shared__ PcTotal tot;
   target += gridDim.x;
   __syncthreads();
   if (threadIdx.x == 0) {
@@ -117,24 +120,30 @@ __device__ __forceinline__ bool grid_barrier_sum(unsigned* count, unsigned* flag
   if (last) {
     const double t = grid_total<BLOCK>(part);
     if (threadIdx.x == 0) {
-      *slot = t;
+      *slot = result(t);
       asm volatile("st.release.gpu.global.u32 [%0], %1;" ::"l"(flag), "r"(target) : "memory");
     }
   }
   if (threadIdx.x == 0) {
     ok = wait_word(flag, target, err) ? 1 : 0;
-    if (ok) tot = __ldcg(slot);
+    if (ok) {
+      const double2 d = __ldcg(reinterpret_cast<const double2*>(slot));
+      const int2 i = __ldcg(reinterpret_cast<const int2*>(slot) + 2);
+      tot = PcTotal{d.x, d.y, __int_as_float(i.x), i.y};
+    }
   }
   __syncthreads();
-  *total = tot;
+  *out = tot;
   return ok != 0;
 }
 
-// sum of one double per thread over the BLOCK threads of the block (thread 0 gets it)
-template <int BLOCK>
+// sum of one double per thread over the BLOCK threads of the block, or per warp where its lanes hold one value
+// already (thread 0 gets it)
+template <int BLOCK, bool PER_WARP>
 __device__ __forceinline__ double block_sum(double v) {
   __shared__ double sm[BLOCK / 32];
-  for (int off = 16; off >= 1; off >>= 1) v += __shfl_xor_sync(0xffffffffu, v, off);
+  if (!PER_WARP)
+    for (int off = 16; off >= 1; off >>= 1) v += __shfl_xor_sync(0xffffffffu, v, off);
   if ((threadIdx.x & 31) == 0) sm[threadIdx.x >> 5] = v;
   __syncthreads();
   double s = 0.0;
@@ -146,12 +155,65 @@ __device__ __forceinline__ double block_sum(double v) {
   return s;
 }
 
-// sum of the gridDim.x per-block partials, on every thread: each thread adds a fixed strided
-// subset (its loads issued together), then a fixed shuffle / shared-memory tree, so every block
-// gets the same bits
+// Sum of the gridDim.x per-block partials (each >= 0), on every thread.  The partials' mantissas are added as
+// integers in units of 2^-64 of the largest one's power of two (three limbs over the block), rounded once;
+// partials at the ends of the double range, or more of them than 8 a thread, go through a fixed tree of FP64
+// adds.
 template <int BLOCK>
 __device__ __forceinline__ double grid_total(const double* part) {
   __shared__ double sm[BLOCK / 32];
+  if (gridDim.x <= 8 * BLOCK && gridDim.x <= 1000) {
+    __shared__ unsigned su[4][BLOCK / 32];
+    const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+    unsigned long long v[8];
+    unsigned mx = 0;
+#pragma unroll
+    for (int i = 0; i < 8; i++) {
+      const int j = (int)threadIdx.x + BLOCK * i;
+      v[i] = j < (int)gridDim.x ? (unsigned long long)__double_as_longlong(__ldcg(part + j)) & 0x7fffffffffffffffULL : 0ULL;
+    }
+#pragma unroll
+    for (int i = 0; i < 8; i++) mx = max(mx, (unsigned)(v[i] >> 32));
+    mx = __reduce_max_sync(0xffffffffu, mx);
+    if (lane == 0) su[3][warp] = mx;
+    __syncthreads();
+#pragma unroll
+    for (int w = 0; w < BLOCK / 32; w++) mx = max(mx, su[3][w]);
+    const int e = (int)(mx >> 20);  // (the same on every thread)
+    if (e == 0x7ff) return __longlong_as_double(0x7ff8000000000000LL);
+    if (e > 200 && e < 1800) {
+      unsigned l0 = 0, l1 = 0, l2 = 0;
+#pragma unroll
+      for (int i = 0; i < 8; i++) {
+        const int x = (int)(v[i] >> 52);
+        const unsigned long long m = x > 0 ? (v[i] & 0xfffffffffffffULL) | 0x10000000000000ULL : 0ULL;
+        const unsigned long long t = (m << 11) >> min(e - x, 63);
+        l0 += (unsigned)t & 0x1fffffu;
+        l1 += (unsigned)(t >> 21) & 0x1fffffu;
+        l2 += (unsigned)(t >> 42);  // 22 bits; at most 1000 values in all: the sum below stays under 2^64
+      }
+      l0 = __reduce_add_sync(0xffffffffu, l0);
+      l1 = __reduce_add_sync(0xffffffffu, l1);
+      l2 = __reduce_add_sync(0xffffffffu, l2);
+      if (lane == 0) {
+        su[0][warp] = l0;
+        su[1][warp] = l1;
+        su[2][warp] = l2;
+      }
+      __syncthreads();
+      unsigned long long s0 = 0, s1 = 0, s2 = 0;
+#pragma unroll
+      for (int w = 0; w < BLOCK / 32; w++) {
+        s0 += su[0][w];
+        s1 += su[1][w];
+        s2 += su[2][w];
+      }
+      __syncthreads();
+      const unsigned long long low = s0 + (s1 << 21) + (1ULL << 9);
+      return scaled_to_double((s2 << 32) + (low >> 10), e - 1075 - 1);
+    }
+    __syncthreads();
+  }
   double s = 0.0;
   for (int base = 0; base < (int)gridDim.x; base += 8 * BLOCK) {
     double v[8];
@@ -194,7 +256,8 @@ struct PcShape {
                                      : 0;
 };
 
-// one phase over the site blocks this block owns; returns the thread's share of the phase's sum
+// one phase over the site blocks this block owns; returns the thread's share of the phase's sum (pair units:
+// the warp's, on each of its lanes)
 template <int P, int RECON, int EPI, bool LAZY = false>
 __device__ __forceinline__ double run_phase(const DslashArgs& A, cx<typename Real<P>::T> (*part)[12][32],
                                             PairXch<float> (*xch)[2], uint4* stage, double alpha) {
@@ -204,14 +267,20 @@ __device__ __forceinline__ double run_phase(const DslashArgs& A, cx<typename Rea
     constexpr int NP = PcShape<P>::PAIRS;
     const int w = threadIdx.x >> 5, q = w >> 1, d = w & 1;
     int slot = 0;
+    bool first = true;
     // site block sb goes to block sb mod grid, pair sb / grid: every SM gets a share of the phase
     for (int sb = q * gridDim.x + blockIdx.x; sb < nsb; sb += NP * gridDim.x) {
       int hh;
       bool valid;
       Site s;
       split_prologue(A, sb, hh, valid, s);
-      v += pair_unit<P, RECON, EPI, LDM, LAZY>(A, hh, valid, s, d, q, true, alpha, &xch[q][slot],
-                                               stage + w * PcShape<P>::PAIR_STAGE);
+      const float n = pair_unit<P, RECON, EPI, LDM, LAZY>(A, hh, valid, s, d, q, true, alpha, &xch[q][slot],
+                                                          stage + w * PcShape<P>::PAIR_STAGE);
+      if (EPI == EPI_XPAY || EPI == EPI_XPAY_CG) {
+        const double t = warp_sum_nonneg(n, 0.f);
+        v = first ? t : v + t;
+        first = false;
+      }
       slot ^= 1;
     }
   } else {
@@ -273,7 +342,9 @@ __global__ void __launch_bounds__(PcShape<P>::THREADS, PcShape<P>::MIN_BLOCKS)
   // iteration of a launch takes beta from the state (the reliable update or the set-up before it left p as it
   // was; a p update and a kernel lowering the gate, each 5 us of launch and latency a round at 16^4)
   constexpr bool LAZY = P == 32;
+  PcTotal res{};  // of the last summing barrier
   double alpha = 0.0, beta = st0.beta, pAp = 0.0;
+  float beta32 = narrow(beta);
   unsigned bar_target = 0;
   while (true) {
     // phase 1
@@ -282,7 +353,7 @@ __global__ void __launch_bounds__(PcShape<P>::THREADS, PcShape<P>::MIN_BLOCKS)
     a1.in_g5 = 0;
     a1.lz_r = Q.r;
     a1.lz_a = 1.f;
-    a1.lz_b = float(beta);
+    a1.lz_b = beta32;
     run_phase<P, RECON, EPI_CLOVER_INV, LAZY>(a1, part, xch, stage, 0.0);
     if (!grid_barrier(Q.bar_count, bar_target, Q.bar_err)) return;
     // phase 2
@@ -296,11 +367,17 @@ __global__ void __launch_bounds__(PcShape<P>::THREADS, PcShape<P>::MIN_BLOCKS)
       a.lz_r = a1.lz_r;
       a.lz_a = a1.lz_a;
       a.lz_b = a1.lz_b;
-      const double v = block_sum<BLOCK>(run_phase<P, RECON, EPI_XPAY, LAZY>(a, part, xch, stage, 0.0));
-      if (!grid_barrier_sum<BLOCK>(Q.bar_count, Q.bar_flag, bar_target, Q.bar_err, Q.part_pap, Q.totals, v, &pAp))
+      const double v = block_sum<BLOCK, PAIR>(run_phase<P, RECON, EPI_XPAY, LAZY>(a, part, xch, stage, 0.0));
+      auto next = [&](double t) {
+        const double q = rr / t;
+        return PcTotal{t, q, narrow(q), t > 0.0 && isfinite(t) ? 0 : PC_BAD};
+      };
+      if (!grid_barrier_sum<BLOCK>(Q.bar_count, Q.bar_flag, bar_target, Q.bar_err, Q.part_pap, Q.totals, v, next, &res))
         return;
     }
-    if (!(pAp > 0.0) || !isfinite(pAp)) {
+    pAp = res.total;
+    alpha = res.coef;
+    if (res.status & PC_BAD) {
       if (blockIdx.x == 0 && threadIdx.x == 0) {
         Q.ctl->nan = 1;
         Q.ctl->halt = 1;
@@ -308,7 +385,6 @@ __global__ void __launch_bounds__(PcShape<P>::THREADS, PcShape<P>::MIN_BLOCKS)
       }
       return;
     }
-    alpha = rr / pAp;
     // phase 3
     a1.in = Q.y;
     a1.in_norm = Q.y_n;
@@ -316,7 +392,6 @@ __global__ void __launch_bounds__(PcShape<P>::THREADS, PcShape<P>::MIN_BLOCKS)
     run_phase<P, RECON, EPI_CLOVER_INV>(a1, part, xch, stage, 0.0);
     if (!grid_barrier(Q.bar_count, bar_target, Q.bar_err)) return;
     // phase 4
-    double rr_new;
     {
       DslashArgs a = a2;
       a.x = Q.y;
@@ -327,12 +402,16 @@ __global__ void __launch_bounds__(PcShape<P>::THREADS, PcShape<P>::MIN_BLOCKS)
       a.cg_r = Q.r;
       a.cg_p = Q.p;
       a.cg_p_norm = Q.p_n;
-      const double v = block_sum<BLOCK>(run_phase<P, RECON, EPI_XPAY_CG>(a, part, xch, stage, alpha));
-      if (!grid_barrier_sum<BLOCK>(Q.bar_count, Q.bar_flag, bar_target, Q.bar_err, Q.part_rr, Q.totals + 1, v,
-                                   &rr_new))
+      const double v = block_sum<BLOCK, PAIR>(run_phase<P, RECON, EPI_XPAY_CG>(a, part, xch, stage, alpha));
+      auto next = [&](double t) {
+        const double q = t / rr;
+        const bool want = t <= st0.tol2 || since + 1 >= every || t < delta2 * st0.rr_reliable;
+        return PcTotal{t, q, narrow(q), (isfinite(t) ? 0 : PC_BAD) | (want ? PC_WANT : 0)};
+      };
+      if (!grid_barrier_sum<BLOCK>(Q.bar_count, Q.bar_flag, bar_target, Q.bar_err, Q.part_rr, Q.totals + 1, v, next, &res))
         return;
     }
-    if (!isfinite(rr_new)) {
+    if (res.status & PC_BAD) {
       if (blockIdx.x == 0 && threadIdx.x == 0) {
         Q.ctl->nan = 1;
         Q.ctl->halt = 1;
@@ -340,12 +419,13 @@ __global__ void __launch_bounds__(PcShape<P>::THREADS, PcShape<P>::MIN_BLOCKS)
       }
       return;
     }
-    beta = rr_new / rr;
+    beta = res.coef;
+    beta32 = res.coef32;
     rr_prev = rr;
-    rr = rr_new;
+    rr = res.total;
     iters += 1;
     since += 1;
-    const bool want = rr_new <= st0.tol2 || since >= every || rr_new < delta2 * st0.rr_reliable;
+    const bool want = (res.status & PC_WANT) != 0;
     // phase 5 (at a reliable update the update's own p = r + beta p follows; LAZY: the next iteration's)
     if (!want && !LAZY) {
       for (int h = blockIdx.x * BLOCK + threadIdx.x; h < Vh; h += gridDim.x * BLOCK) {
@@ -353,7 +433,7 @@ __global__ void __launch_bounds__(PcShape<P>::THREADS, PcShape<P>::MIN_BLOCKS)
         cx<R> ps[12], out[12];
         SpinorIO<PR>::template load<LDM>(Q.r, nullptr, Vh, 0, h, rs);
         SpinorIO<P>::template load<LDM>(Q.p, Q.p_n, Vh, 0, h, ps);
-        const RR b = RR(beta);
+        const RR b = to_real<RR>(beta);
 #pragma unroll
         for (int c = 0; c < 12; c++) {
           out[c].re = R(fma(b, RR(ps[c].re), rs[c].re));

@@ -50,7 +50,10 @@ void launch_site_k(int epi, const DslashArgs& a, int nb, cudaStream_t st) {
       case EPI_NONE: dslash_site_fp16_kernel<RECON, EPI_NONE, STAGED><<<nb, 128, 0, st>>>(a); break;
       case EPI_CLOVER_INV: dslash_site_fp16_kernel<RECON, EPI_CLOVER_INV, STAGED><<<nb, 128, 0, st>>>(a); break;
       case EPI_XPAY_CG: dslash_site_fp16_kernel<RECON, EPI_XPAY_CG, STAGED><<<nb, 128, 0, st>>>(a); break;
-      default: dslash_site_fp16_kernel<RECON, EPI_XPAY, STAGED><<<nb, 128, 0, st>>>(a); break;
+      default:
+        if (a.do_norm) dslash_site_fp16_kernel<RECON, EPI_XPAY, STAGED, true><<<nb, 128, 0, st>>>(a);
+        else dslash_site_fp16_kernel<RECON, EPI_XPAY, STAGED><<<nb, 128, 0, st>>>(a);
+        break;
     }
   } else {
     switch (epi) {
@@ -63,7 +66,9 @@ void launch_site_k(int epi, const DslashArgs& a, int nb, cudaStream_t st) {
 }
 
 template <int P, int RECON>
-void launch_site(int epi, const DslashArgs& a, cudaStream_t st) {
+void launch_site(int epi, const DslashArgs& args, cudaStream_t st) {
+  DslashArgs a = args;
+  a.af = (float)a.a;
   const int G = a.nrhs == 1 ? 4 : (a.nrhs == 2 ? 2 : 1);
   const int nb = (a.g.Vh + 32 * G - 1) / (32 * G);
   // staging pays once its cost is spread over enough RHS: FP32 from 4 RHS (32^3 x 64, 8 RHS: 857 ->

@@ -40,6 +40,7 @@ struct DslashArgs {
   const int* clover_e;     // fixed-point kernels: its exponents [2][Vh]
   int out_f64;             // fixed-point kernels: out is an FP64 field (else block fixed point)
   double a;                // EPI_XPAY coefficient on the hopping sum
+  float af;                // the same in FP32 (set by the launcher of the site kernels)
   int in_g5;               // apply gamma_5 to the input before hopping
   int x_g5;                // apply gamma_5 to x before the clover multiply
   int out_g5;              // apply gamma_5 to the result
@@ -274,8 +275,9 @@ __device__ __forceinline__ void dir_index(const Geom& g, const Site& s, DirLinks
   L.nbf = neighbor_fwd(g, s, MU) >> 1;
   L.nbb = neighbor_bwd(g, s, MU) >> 1;
   const int tg = s.t + g.t0;
-  L.sf = (MU == 3 && tg == g.Tg - 1) ? R(g.t_bc) : R(1);
-  L.sb = (MU == 3 && tg == 0) ? R(g.t_bc) : R(1);
+  const R bc = __double2hiint(g.t_bc) < 0 ? R(-1) : R(1);  // t_bc is 1 or -1
+  L.sf = (MU == 3 && tg == g.Tg - 1) ? bc : R(1);
+  L.sb = (MU == 3 && tg == 0) ? bc : R(1);
   L.hf = L.hb = -1;
 }
 
@@ -542,7 +544,7 @@ __device__ __forceinline__ double split_unit(const DslashArgs& A, int hh, bool v
       }
       if (ST::ON) CloverIO<CloverPrec<P>::CP>::template apply<LD_SM>(stage, 32, lane, b, xs, cxs);
       else CloverIO<CloverPrec<P>::CP>::apply(A.clover, A.g.Vh, hh, b, xs, cxs);
-      const R a = R(A.a);
+      const R a = to_real<R>(A.a);
 #pragma unroll
       for (int k = 0; k < 6; k++) {
         res[k].re = fma(a, v[k].re, cxs[k].re);
@@ -558,7 +560,7 @@ __device__ __forceinline__ double split_unit(const DslashArgs& A, int hh, bool v
       constexpr int PR = P == 64 ? 64 : 32;
       using RR = typename Real<PR>::T;
       if (cg_active) {
-        const RR al = RR(cg_alpha);
+        const RR al = to_real<RR>(cg_alpha);
         cx<R> ps[6];
         cx<RR> xs[6], rs[6];
         if (ST::ON) {
@@ -816,7 +818,7 @@ __device__ __forceinline__ float pair_unit_b(const DslashArgs& A, int hh, bool v
         for (int k = 0; k < 6; k++) xs[k] = -xs[k];
       }
       staged_clover_block<P>(stage, lane, b, xs, cxs);
-      const float a = float(A.a);
+      const float a = narrow(A.a);
 #pragma unroll
       for (int k = 0; k < 6; k++) {
         res[k].re = fmaf(a, v[k].re, cxs[k].re);
@@ -830,7 +832,7 @@ __device__ __forceinline__ float pair_unit_b(const DslashArgs& A, int hh, bool v
     if (EPI == EPI_XPAY_CG) {
       // res = (A p)_b: advance x and r (FP32) of this RHS with alpha from the <p, A p> reduction
       if (cg_active) {
-        const float al = float(cg_alpha);
+        const float al = narrow(cg_alpha);
         cx<float> ps[6], xs[6], rs[6];
         staged_spinor_block<P>(stage + ST::OFF_P, lane, b, ps);
         SpinorIO<32>::template load_block<COH>(A.cg_x, nullptr, Vh, 0, hh, b, xs);
@@ -1175,8 +1177,9 @@ __device__ __forceinline__ void hops_fp16_sp(const DslashArgs& A, const Site& s,
 // epilogue of its RHS, with no block barrier.  The links and the clover pair of the block's sites
 // are the same for every RHS: with STAGED (nrhs >= 3, one site group) the block decodes them once
 // (12-real links reconstructed, FP16 converted) into shared memory; otherwise every warp reads them
-// through L1.  Sums are reduced per warp into the partial slot of (RHS, site group).
-template <int P, int RECON, int EPI, bool STAGED>
+// through L1.  Sums are reduced per warp into the partial slot of (RHS, site group).  NORM: the code of the
+// sum of |out|^2 (do_norm).
+template <int P, int RECON, int EPI, bool STAGED, bool NORM>
 __device__ __forceinline__ void dslash_site_body(const DslashArgs& A) {
   using R = typename Real<P>::T;
   constexpr int CP = CloverPrec<P>::CP;
@@ -1246,7 +1249,10 @@ __device__ __forceinline__ void dslash_site_body(const DslashArgs& A) {
   }
   Site s;
   if (valid) s = site_of(A.g, A.p, hh);
-  const bool reduce = A.do_norm || EPI == EPI_XPAY_CG;
+  // FP16: the code of the sums costs a pass without them registers (32^3 x 64, 8 RHS, xpay 627 us without it, 703
+  // us with it).  FP32, at 80 registers, is the other way round (8 RHS: xpay 731 us without the code, 713 us with
+  // it; 1 RHS 163.5 and 161.9 us), so its one instance tests do_norm
+  const bool reduce = EPI == EPI_XPAY_CG || (NORM && A.do_norm);
   auto apply_cl = [&](int b, const cx<R> x[6], cx<R> y[6]) {
     if (SCL) clover_apply_smem(scl, lane, b, x, y);
     else CloverIO<CP>::apply(A.clover, Vh, hh, b, x, y);
@@ -1304,11 +1310,10 @@ __device__ __forceinline__ void dslash_site_body(const DslashArgs& A) {
             for (int j = 0; j < 6; j++) xs[j] = -xs[j];
           }
           apply_cl(b, xs, cxs);
-          const R a = R(A.a);
 #pragma unroll
           for (int j = 0; j < 6; j++) {
-            o[j].re = fma(a, v[j].re, cxs[j].re);
-            o[j].im = fma(a, v[j].im, cxs[j].im);
+            o[j].re = fma(A.af, v[j].re, cxs[j].re);
+            o[j].im = fma(A.af, v[j].im, cxs[j].im);
           }
         }
         if (A.out_g5 && b == 1) {
@@ -1317,7 +1322,7 @@ __device__ __forceinline__ void dslash_site_body(const DslashArgs& A) {
         }
         if (EPI == EPI_XPAY_CG) {
           if (act) {
-            const RR alr = RR(al);
+            const RR alr = to_real<RR>(al);
             cx<R> ps[6];
             cx<RR> xs[6], rs[6];
             SpinorIO<P>::load_block(A.cg_p, A.cg_p_norm, Vh, r, hh, b, ps);
@@ -1338,7 +1343,7 @@ __device__ __forceinline__ void dslash_site_body(const DslashArgs& A) {
             SpinorIO<PR>::store_block(A.cg_r, nullptr, Vh, r, hh, b, rs);
           }
         } else {
-          if (A.do_norm) {
+          if (NORM && A.do_norm) {
             R n6 = R(0);
 #pragma unroll
             for (int j = 0; j < 6; j++) {
@@ -1377,9 +1382,9 @@ __device__ __forceinline__ void dslash_site_body(const DslashArgs& A) {
 // FP32: 6 blocks per SM (80 registers).  32^3 x 64 against the compiler's own choice (96 registers
 // unstaged, 5 blocks): 1 RHS 159 -> 153.5 us, 4 RHS 418 -> 413 us, 8 RHS 698 -> 688 us; 48^3 x 96,
 // 1 RHS 782 -> 744 us.  7 blocks spill (1 RHS 170 us), 5 staged blocks are slower (8 RHS 715 us).
-template <int P, int RECON, int EPI, bool STAGED>
+template <int P, int RECON, int EPI, bool STAGED, bool NORM = true>
 __global__ void __launch_bounds__(128, 6) dslash_site_kernel(DslashArgs A) {
-  dslash_site_body<P, RECON, EPI, STAGED>(A);
+  dslash_site_body<P, RECON, EPI, STAGED, NORM>(A);
 }
 
 // FP16: 4 blocks per SM of up to 128 registers.  Unstaged, the registers hold the links and
@@ -1387,9 +1392,9 @@ __global__ void __launch_bounds__(128, 6) dslash_site_kernel(DslashArgs A) {
 // 1 RHS; 6 of 80: 108 us); staged, the 47 KB of shared memory (links as broadcast pairs, clover pair)
 // allow 4 blocks (5 blocks of 96 registers with the clover read through L1 instead: 32^3 x 64, 8 RHS
 // 631 -> 658 us)
-template <int RECON, int EPI, bool STAGED>
+template <int RECON, int EPI, bool STAGED, bool NORM = false>
 __global__ void __launch_bounds__(128, 4) dslash_site_fp16_kernel(DslashArgs A) {
-  dslash_site_body<16, RECON, EPI, STAGED>(A);
+  dslash_site_body<16, RECON, EPI, STAGED, NORM>(A);
 }
 
 // The single-RHS FP16 operator is bound by latency: it is held to 64 registers, so that 8 blocks

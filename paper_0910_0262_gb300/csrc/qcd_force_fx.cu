@@ -580,7 +580,7 @@ __global__ void __launch_bounds__(96) plaquette_fixed_kernel(Geom g, const int4*
     v = fx_to_double_in_range(fx_value<2>(t), -56) / 3.0;
   }
   const int nblk = gridDim.x * gridDim.y;
-  block_partial<96>(v, 0, blockIdx.y * gridDim.x + blockIdx.x, nblk, red);
+  block_partial<96>(v, 0, blockIdx.x * gridDim.y + blockIdx.y, nblk, red);
   grid_finish<96>(1, nblk, nblk, red);
 }
 

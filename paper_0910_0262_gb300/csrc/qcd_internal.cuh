@@ -762,6 +762,8 @@ struct ReduceArgs {
   double* partials;        // [nrhs][gridDim.x]
   long long capacity;      // slots in partials; a launch needing more records ctl->overflow
   unsigned int* counter;   // zero before the launch; the last block resets it
+  double* group_sums;      // [nrhs][groups] of a two-step sum, with counters [1 + group_cap]
+  int group_cap;           // most groups of blocks that these hold
   double* result;          // [nrhs], FIN_STORE
   int mode;
   CGState* cg;
@@ -858,7 +860,7 @@ __device__ __forceinline__ double scaled_to_double(unsigned long long m, int p) 
 // The sum over the warp's lanes of a + b for FP32 a, b >= 0, rounded once to double, on every lane.  The
 // values' mantissas are added as integers in units of 2^-57 of the largest one's power of two: a shuffle
 // tree of FP64 adds takes 16 clocks of the SM's FP64 pipe an add and conversion, 144 for each 32 sites and
-// right-hand side (32^3 x 64, 8 RHS FP16, the pass that forms |Mhat p|^2: TBD us).
+// right-hand side (24^3 x 48, 8 RHS FP16, the pass that forms |Mhat p|^2: 302 -> 248 us).
 __device__ __forceinline__ double warp_sum_nonneg(float a, float b) {
   const unsigned ua = __float_as_uint(a), ub = __float_as_uint(b);
   const unsigned mx = __reduce_max_sync(0xffffffffu, max(ua & 0x7fffffffu, ub & 0x7fffffffu));
@@ -901,45 +903,83 @@ __device__ __forceinline__ void block_partial(double v, int r, int blk, int nblk
 }
 
 // BLOCK 0: a block size known at run time.
+//
+// A launch of many blocks sums in two steps: the last of each 64 consecutive blockIdx.x (over blockIdx.y) adds
+// its group's partials, the last group's block adds the groups' sums.  (One block adding all of them runs on
+// one SM's FP64 units, two adds a clock: 83 thousand partials of 8 RHS at 24^3 x 48 took it 20 us at the end
+// of a 200 us pass.)  The slots of RHS r are r * nblk + blockIdx.x * (nblk / gridDim.x) + j.
 template <int BLOCK>
 __device__ __forceinline__ void grid_finish(int nrhs, long long blk_total, int nblk, const ReduceArgs& ra) {
   __shared__ double sm[BLOCK ? BLOCK / 32 : 32];
   __shared__ bool is_last;
   const int threads = BLOCK ? BLOCK : (int)blockDim.x;
-  const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+  const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5, warps = threads >> 5;
+  constexpr int GROUP = 64;
+  const int gx = (int)gridDim.x, groups = (gx + GROUP - 1) / GROUP;
+  const bool two = groups >= 8 && groups <= ra.group_cap;
+  const double* src = ra.partials;
+  long long cap = ra.capacity;
+  int n = nblk;
   __threadfence();
   __syncthreads();
-  if (threadIdx.x == 0) {
-    const unsigned int ticket = atomicAdd(ra.counter, 1u);
-    is_last = (ticket == blk_total - 1);
+  if (two) {
+    const int grp = (int)blockIdx.x / GROUP, wide = min(GROUP, gx - grp * GROUP), per = nblk / gx;
+    if (threadIdx.x == 0) is_last = atomicAdd(ra.counter + 1 + grp, 1u) == (unsigned)wide * gridDim.y - 1;
+    __syncthreads();
+    if (!is_last) return;
+    __threadfence();
+    for (int r = warp; r < nrhs; r += warps) {
+      const long long at = (long long)r * nblk + (long long)grp * GROUP * per;
+      double s = 0.0;
+      for (int j = lane; j < wide * per; j += 32) s += at + j < cap ? __ldcg(src + at + j) : 0.0;
+      for (int off = 16; off >= 1; off >>= 1) s += __shfl_xor_sync(0xffffffffu, s, off);
+      if (lane == 0) ra.group_sums[(long long)r * groups + grp] = s;
+    }
+    if (threadIdx.x == 0) ra.counter[1 + grp] = 0u;
+    src = ra.group_sums;
+    cap = (long long)nrhs * groups;
+    n = groups;
+    blk_total = groups;
+    __threadfence();
+    __syncthreads();
   }
+  if (threadIdx.x == 0) is_last = (atomicAdd(ra.counter, 1u) == (unsigned)(blk_total - 1));
   __syncthreads();
   if (!is_last) return;
   __threadfence();
-  for (int r = 0; r < nrhs; r++) {
-    // thread t adds partials t, t + BLOCK, t + 2 BLOCK, ... in that order; the loads of U terms are
-    // issued together (a grid of 32768 blocks leaves 256 partials per thread of a 128-thread block)
-    constexpr int U = 16;
+  // thread t of a team adds slots t, t + TEAM, t + 2 TEAM, ... in that order; the loads of U terms are issued
+  // together.  Several RHS: a team is a warp, and the warps share out the RHS.
+  constexpr int U = 16;
+  auto part_sum = [&](int r, int t, int team) {
     double s = 0.0;
-    for (int j0 = threadIdx.x; j0 < nblk; j0 += U * threads) {
+    for (int j0 = t; j0 < n; j0 += U * team) {
       double v[U];
 #pragma unroll
       for (int u = 0; u < U; u++) {
-        const int j = j0 + u * threads;
-        const long long slot = (long long)r * nblk + j;
-        v[u] = (j < nblk && slot < ra.capacity) ? __ldcg(ra.partials + slot) : 0.0;
+        const int j = j0 + u * team;
+        const long long slot = (long long)r * n + j;
+        v[u] = (j < n && slot < cap) ? __ldcg(src + slot) : 0.0;
       }
 #pragma unroll
       for (int u = 0; u < U; u++) s += v[u];
     }
     for (int off = 16; off >= 1; off >>= 1) s += __shfl_xor_sync(0xffffffffu, s, off);
+    return s;
+  };
+  if (nrhs > 1) {
+    for (int r = warp; r < nrhs; r += warps) {
+      const double s = part_sum(r, lane, 32);
+      if (lane == 0) finalize_total(ra, r, s);
+    }
     __syncthreads();
+  } else {
+    const double s = part_sum(0, threadIdx.x, threads);
     if (lane == 0) sm[warp] = s;
     __syncthreads();
     if (threadIdx.x == 0) {
       double tot = 0.0;
-      for (int w = 0; w < threads / 32; w++) tot += sm[w];
-      finalize_total(ra, r, tot);
+      for (int w = 0; w < warps; w++) tot += sm[w];
+      finalize_total(ra, 0, tot);
     }
   }
   if (threadIdx.x == 0) {

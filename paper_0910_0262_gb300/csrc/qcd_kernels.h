@@ -29,6 +29,14 @@ bool ctx_view(const qcd_ctx* c, CtxView* v);
 extern std::atomic<long long> g_kernel_launches;
 
 // ---- persistent single-RHS CG iteration (qcd_cg_persistent.cu)
+// what a summing barrier publishes: the total, the coefficient it gives (alpha, beta; also in FP32) and whether
+// the iteration broke down (PC_BAD) or a reliable update or the convergence test is due (PC_WANT)
+struct __align__(16) PcTotal {
+  double total, coef;
+  float coef32;
+  int status;
+};
+enum { PC_BAD = 1, PC_WANT = 2 };
 struct PersistentCGArgs {
   Geom g;
   const void* gauge;           // links of the inner precision
@@ -44,7 +52,7 @@ struct PersistentCGArgs {
   int slots;                   // slots in each; the grid never exceeds it
   unsigned* bar_count;         // barrier arrivals, zeroed before the launch
   unsigned* bar_flag;          // release word of the summing barriers, zeroed before the launch
-  double* totals;              // [2]: the grid totals the summing barriers publish (pAp, |r|^2)
+  PcTotal* totals;             // [2]: what the summing barriers publish (of pAp, |r|^2)
   int* bar_err;                // set when a barrier wait gave up
   int iter_limit;              // total iterations of the RHS (over all launches) at which to stop
   int* round_out;              // non-null: 2 x iterations this launch ran, + 1 if it raised a reliable
