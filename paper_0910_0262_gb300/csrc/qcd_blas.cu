@@ -39,6 +39,42 @@ __global__ void __launch_bounds__(BB) p_update_kernel(Geom g, const void* r, con
   SpinorIO<PP>::store(p, pn, g.Vh, k, h, out);
 }
 
+// p = r + beta p for FP64 r and p in block fixed point: two warps per 32 sites, a chiral block each (a thread's
+// conversions of a whole site, a thousand instructions, set the kernel's time, 9.0 us at 10 x 12 x 14 x 18, 2 RHS:
+// 7.89 -> 7.84 ms a solve there)
+__global__ void __launch_bounds__(64) p_update_fixed_kernel(Geom g, const double2* r, longlong2* p, int* pe,
+                                                            const CGState* cg, const int* halt, const int* gate) {
+  __shared__ unsigned long long sm[2][32];
+  if ((halt && *halt) || (gate && !*gate)) return;
+  const int k = blockIdx.y, lane = threadIdx.x & 31, b = threadIdx.x >> 5, Vh = g.Vh;
+  if (!cg[k].active) return;
+  const int h = blockIdx.x * 32 + lane;
+  const bool valid = h < Vh && dbg_spinor(Vh, k, h);
+  const double beta = cg[k].beta;
+  cx<double> o[6];
+  u64 mx = 0;
+  if (valid) {
+    cx<double> rs[6];
+    SpinorIO<64>::load_block(r, nullptr, Vh, k, h, b, rs);
+    SpinorIO<60>::load_block(p, reinterpret_cast<const float*>(pe), Vh, k, h, b, o);
+#pragma unroll
+    for (int c = 0; c < 6; c++) {
+      o[c].re = fma(beta, o[c].re, rs[c].re);
+      o[c].im = fma(beta, o[c].im, rs[c].im);
+      mx = max(mx, max(fx_mag(o[c].re), fx_mag(o[c].im)));
+    }
+  }
+  sm[b][lane] = mx;
+  __syncthreads();  // (also: both blocks have read the site's exponent)
+  if (!valid) return;
+  const int e = fx_exponent(max(mx, sm[1 - b][lane]));
+#pragma unroll
+  for (int c = 0; c < 6; c++)
+    p[sidx<12>(6 * b + c, Vh, k, h)] =
+        make_longlong2(fx_of_double<FX_SPINOR>(o[c].re, e), fx_of_double<FX_SPINOR>(o[c].im, e));
+  if (b == 0) pe[(size_t)k * Vh + h] = e;
+}
+
 template <int PR>
 __global__ void __launch_bounds__(BB) accumulate_x_kernel(Geom g, double2* x_hi, void* x_lo, float* xn, void* x_fx,
                                                           float* x_fx_e, const int* gate) {
@@ -202,7 +238,10 @@ __global__ void finalize_kernel(ReduceArgs red, const double* totals, int nrhs) 
 void launch_p_update(int prec_r, int prec_p, const Geom& g, int nrhs, const void* r, const float* rn, void* p,
                      float* pn, const CGState* cg, const int* halt, cudaStream_t st, const int* gate) {
   g_kernel_launches += 1;
-  if (prec_p == 60) p_update_kernel<64, 60><<<grid2(g, nrhs), BB, 0, st>>>(g, r, rn, p, pn, cg, halt, gate);
+  if (prec_p == 60)
+    p_update_fixed_kernel<<<dim3((g.Vh + 31) / 32, nrhs), 64, 0, st>>>(g, static_cast<const double2*>(r),
+                                                                       static_cast<longlong2*>(p),
+                                                                       reinterpret_cast<int*>(pn), cg, halt, gate);
   else if (prec_r == 64) p_update_kernel<64, 64><<<grid2(g, nrhs), BB, 0, st>>>(g, r, rn, p, pn, cg, halt, gate);
   else if (prec_p == 32) p_update_kernel<32, 32><<<grid2(g, nrhs), BB, 0, st>>>(g, r, rn, p, pn, cg, halt, gate);
   else p_update_kernel<32, 16><<<grid2(g, nrhs), BB, 0, st>>>(g, r, rn, p, pn, cg, halt, gate);
