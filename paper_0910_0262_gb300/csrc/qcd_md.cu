@@ -181,32 +181,47 @@ __global__ void __launch_bounds__(MB) flat_redot_kernel(size_t n, int nrhs, cons
 // eps |P| of a molecular-dynamics step), then s squarings (Moler and Van Loan, "Nineteen dubious ways
 // to compute the exponential of a matrix", 2003).  The truncated series is summed in the basis
 // I, M, M^2: by the Cayley-Hamilton theorem M^3 = tr(M) M^2 - c M + det(M) I with
-// c = (tr(M)^2 - tr(M^2)) / 2, so M^k / k! = a_k I + b_k M + c_k M^2 with
-//   (a, b, c)_{k+1} = (c_k det M, a_k - c_k c, b_k + c_k tr M) / (k + 1),
-// the same sum as the matrix series, for one matrix product (M^2) instead of one per term.
-// 1 / (k + 1): each a quotient rounded once, as the division gives it (an FP64 division is a score of
-// instructions on a pipe that takes two a clock: with the 17 of them the link update of 16^4 took 458 us)
-__device__ const double INVERSE[20] = {1.0 / 1,  1.0 / 2,  1.0 / 3,  1.0 / 4,  1.0 / 5,  1.0 / 6,  1.0 / 7,
-                                       1.0 / 8,  1.0 / 9,  1.0 / 10, 1.0 / 11, 1.0 / 12, 1.0 / 13, 1.0 / 14,
-                                       1.0 / 15, 1.0 / 16, 1.0 / 17, 1.0 / 18, 1.0 / 19, 1.0 / 20};
+// c = (tr(M)^2 - tr(M^2)) / 2, so M^k = a_k I + b_k M + c_k M^2 with
+//   (a, b, c)_{k+1} = (c_k det M, a_k - c_k c, b_k + c_k tr M),
+// the same sum as the matrix series, for one matrix product (M^2) instead of one per term.  s and n
+// are chosen in FP32 (r rounded up): on the FP64 pipe, two instructions a clock and SM, the norms'
+// comparisons and divisions of the series took as long as its terms (16^4: 458 us with the divisions,
+// 330 with stored reciprocals, 270 as it stands).
+__device__ const double INVERSE_FACTORIAL[21] = {
+    1.0, 1.0, 1.0 / 2, 1.0 / 6, 1.0 / 24, 1.0 / 120, 1.0 / 720, 1.0 / 5040, 1.0 / 40320, 1.0 / 362880, 1.0 / 3628800,
+    1.0 / 39916800, 1.0 / 479001600, 1.0 / 6227020800.0, 1.0 / 87178291200.0, 1.0 / 1307674368000.0,
+    1.0 / 20922789888000.0, 1.0 / 355687428096000.0, 1.0 / 6402373705728000.0, 1.0 / 121645100408832000.0,
+    1.0 / 2432902008176640000.0};
 
 __device__ M3 expm3(M3 m) {
-  double nrm = 0.0;
+  double n2 = 0.0;
 #pragma unroll
-  for (int k = 0; k < 9; k++) nrm += norm2(m.e[k]);
-  nrm = sqrt(nrm);
-  int s = 0;
-  while (nrm > 0.25 && s < 60) {
-    nrm *= 0.5;
-    s++;
+  for (int k = 0; k < 9; k++) {
+    n2 = fma(m.e[k].re, m.e[k].re, n2);
+    n2 = fma(m.e[k].im, m.e[k].im, n2);
   }
-  const double sc = ldexp(1.0, -s);
+  const int x = (int)((unsigned)__double2hiint(n2) >> 20) - 1022;  // r^2 < 2^x
+  int s = 0;
+  float nrm = 0.f;
+  if (x >= -120 && x <= 120) {
+    nrm = sqrtf(__double2float_ru(n2)) * 1.000001f;
+    while (nrm > 0.25f) {
+      nrm *= 0.5f;
+      s++;
+    }
+  } else if (x > 120) {  // r < 2^(x / 2): halved x / 2 + 2 times, at most 60
+    s = 60;
+    nrm = 0.25f;
+  }
+  if (s > 0) {
+    const double sc = __hiloint2double((1023 - s) << 20, 0);  // 2^-s
 #pragma unroll
-  for (int k = 0; k < 9; k++) m.e[k] = cmk(sc * m.e[k].re, sc * m.e[k].im);
+    for (int k = 0; k < 9; k++) m.e[k] = cmk(sc * m.e[k].re, sc * m.e[k].im);
+  }
   int order = 0;
-  for (double t = 1.0; order < 20; order++) {
-    t *= nrm * __ldg(INVERSE + order);  // r^(order+1) / (order+1)!
-    if (t <= 1e-17) break;
+  for (float t = 1.f; order < 20; order++) {
+    t *= __fdividef(nrm, (float)(order + 1));  // r^(order+1) / (order+1)!
+    if (t <= 1e-17f) break;
   }
   const M3 m2 = mul(m, m);
   const C tr1 = m.e[0] + m.e[4] + m.e[8];
@@ -214,21 +229,22 @@ __device__ M3 expm3(M3 m) {
   const C cc = 0.5 * (tr1 * tr1 - tr2);
   const C det = m.e[0] * (m.e[4] * m.e[8] - m.e[5] * m.e[7]) - m.e[1] * (m.e[3] * m.e[8] - m.e[5] * m.e[6]) +
                 m.e[2] * (m.e[3] * m.e[7] - m.e[4] * m.e[6]);
-  C a = cmk(1.0, 0.0), b = cmk(0.0, 0.0), c = cmk(0.0, 0.0);  // M^k / k! in the basis I, M, M^2
-  C sa = a, sb = b, scm = c;                                    // their sums over k <= order
-  for (int k = 0; k < order; k++) {
-    const double f = __ldg(INVERSE + k);
-    const C na = f * (c * det), nb = f * (a - c * cc), nc = f * (b + c * tr1);
+  const C ncc = -cc;
+  C a = cmk(1.0, 0.0), b = cmk(0.0, 0.0), c = cmk(0.0, 0.0);  // M^k in the basis I, M, M^2
+  C sa = a, sb = b, scm = c;                                    // their sums over k <= order, over k!
+  for (int k = 1; k <= order; k++) {
+    const C na = c * det, nb = cfma(c, ncc, a), nc = cfma(c, tr1, b);
     a = na;
     b = nb;
     c = nc;
-    sa = sa + a;
-    sb = sb + b;
-    scm = scm + c;
+    const double f = __ldg(INVERSE_FACTORIAL + k);
+    sa = cmk(fma(f, a.re, sa.re), fma(f, a.im, sa.im));
+    sb = cmk(fma(f, b.re, sb.re), fma(f, b.im, sb.im));
+    scm = cmk(fma(f, c.re, scm.re), fma(f, c.im, scm.im));
   }
   M3 e;
 #pragma unroll
-  for (int k = 0; k < 9; k++) e.e[k] = sb * m.e[k] + scm * m2.e[k];
+  for (int k = 0; k < 9; k++) e.e[k] = cfma(scm, m2.e[k], sb * m.e[k]);
   e.e[0] = e.e[0] + sa;
   e.e[4] = e.e[4] + sa;
   e.e[8] = e.e[8] + sa;
@@ -240,8 +256,8 @@ __device__ M3 expm3(M3 m) {
 __device__ __forceinline__ M3 reunitarise(M3 u) {
   double n0 = 0.0;
 #pragma unroll
-  for (int j = 0; j < 3; j++) n0 += norm2(u.e[j]);
-  const double i0 = 1.0 / sqrt(n0);
+  for (int j = 0; j < 3; j++) n0 = fma(u.e[j].im, u.e[j].im, fma(u.e[j].re, u.e[j].re, n0));
+  const double i0 = rsqrt(n0);
 #pragma unroll
   for (int j = 0; j < 3; j++) u.e[j] = cmk(i0 * u.e[j].re, i0 * u.e[j].im);
   C d = cmk(0.0, 0.0);  // <row 0, row 1>
@@ -251,8 +267,8 @@ __device__ __forceinline__ M3 reunitarise(M3 u) {
   for (int j = 0; j < 3; j++) u.e[3 + j] = u.e[3 + j] - d * u.e[j];
   double n1 = 0.0;
 #pragma unroll
-  for (int j = 0; j < 3; j++) n1 += norm2(u.e[3 + j]);
-  const double i1 = 1.0 / sqrt(n1);
+  for (int j = 0; j < 3; j++) n1 = fma(u.e[3 + j].im, u.e[3 + j].im, fma(u.e[3 + j].re, u.e[3 + j].re, n1));
+  const double i1 = rsqrt(n1);
 #pragma unroll
   for (int j = 0; j < 3; j++) u.e[3 + j] = cmk(i1 * u.e[3 + j].re, i1 * u.e[3 + j].im);
   u.e[6] = conj(u.e[1] * u.e[5] - u.e[2] * u.e[4]);
