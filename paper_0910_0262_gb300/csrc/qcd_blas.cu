@@ -76,8 +76,8 @@ __global__ void __launch_bounds__(64) p_update_fixed_kernel(Geom g, const double
 }
 
 template <int PR>
-__global__ void __launch_bounds__(BB) accumulate_x_kernel(Geom g, double2* x_hi, void* x_lo, float* xn, void* x_fx,
-                                                          float* x_fx_e, const int* gate) {
+__global__ void __launch_bounds__(BB) accumulate_x_kernel(Geom g, double2* x_hi, void* x_lo, float* xn,
+                                                          const int* gate) {
   using RR = typename Real<PR>::T;
   if (gate && !*gate) return;
   const int k = blockIdx.y;
@@ -95,7 +95,44 @@ __global__ void __launch_bounds__(BB) accumulate_x_kernel(Geom g, double2* x_hi,
   }
   SpinorIO<64>::store(x_hi, nullptr, g.Vh, k, h, hi);
   SpinorIO<PR>::store(x_lo, xn, g.Vh, k, h, lo);
-  if (x_fx) SpinorIO<60>::store(x_fx, x_fx_e, g.Vh, k, h, hi);
+}
+
+// the same with a copy of x_hi in block fixed point: two warps per 32 sites, a chiral block each (one thread per
+// site: 16^4 10.1 -> 9.0 us)
+template <int PR>
+__global__ void __launch_bounds__(64) accumulate_x_fixed_kernel(Geom g, double2* x_hi, void* x_lo, longlong2* x_fx,
+                                                                int* x_fx_e, const int* gate) {
+  using RR = typename Real<PR>::T;
+  __shared__ u64 sm[2][32];
+  if (gate && !*gate) return;
+  const int k = blockIdx.y, lane = threadIdx.x & 31, b = threadIdx.x >> 5, Vh = g.Vh;
+  const int h = blockIdx.x * 32 + lane;
+  const bool valid = h < Vh && dbg_spinor(Vh, k, h);
+  cx<double> hi[6];
+  u64 mx = 0;
+  if (valid) {
+    cx<RR> lo[6];
+    SpinorIO<PR>::load_block(x_lo, nullptr, Vh, k, h, b, lo);
+    SpinorIO<64>::load_block(x_hi, nullptr, Vh, k, h, b, hi);
+#pragma unroll
+    for (int c = 0; c < 6; c++) {
+      hi[c].re += to_double(lo[c].re);
+      hi[c].im += to_double(lo[c].im);
+      lo[c] = cmk(RR(0), RR(0));
+      mx = max(mx, max(fx_mag(hi[c].re), fx_mag(hi[c].im)));
+    }
+    SpinorIO<64>::store_block(x_hi, nullptr, Vh, k, h, b, hi);
+    SpinorIO<PR>::store_block(x_lo, nullptr, Vh, k, h, b, lo);
+  }
+  sm[b][lane] = mx;
+  __syncthreads();
+  if (!valid) return;
+  const int e = fx_exponent(max(mx, sm[1 - b][lane]));
+#pragma unroll
+  for (int c = 0; c < 6; c++)
+    x_fx[sidx<12>(6 * b + c, Vh, k, h)] =
+        make_longlong2(fx_of_double<FX_SPINOR>(hi[c].re, e), fx_of_double<FX_SPINOR>(hi[c].im, e));
+  if (b == 0) x_fx_e[(size_t)k * Vh + h] = e;
 }
 
 template <int PR>
@@ -250,8 +287,17 @@ void launch_p_update(int prec_r, int prec_p, const Geom& g, int nrhs, const void
 void launch_accumulate_x(int prec_r, const Geom& g, int nrhs, double2* x_hi, void* x_lo, float* x_lon,
                          cudaStream_t st, const int* gate, void* x_fx, float* x_fx_e) {
   g_kernel_launches += 1;
-  if (prec_r == 64) accumulate_x_kernel<64><<<grid2(g, nrhs), BB, 0, st>>>(g, x_hi, x_lo, x_lon, x_fx, x_fx_e, gate);
-  else accumulate_x_kernel<32><<<grid2(g, nrhs), BB, 0, st>>>(g, x_hi, x_lo, x_lon, x_fx, x_fx_e, gate);
+  if (x_fx) {
+    const dim3 grid((g.Vh + 31) / 32, nrhs);
+    longlong2* fx = static_cast<longlong2*>(x_fx);
+    int* e = reinterpret_cast<int*>(x_fx_e);
+    if (prec_r == 64) accumulate_x_fixed_kernel<64><<<grid, 64, 0, st>>>(g, x_hi, x_lo, fx, e, gate);
+    else accumulate_x_fixed_kernel<32><<<grid, 64, 0, st>>>(g, x_hi, x_lo, fx, e, gate);
+  } else if (prec_r == 64) {
+    accumulate_x_kernel<64><<<grid2(g, nrhs), BB, 0, st>>>(g, x_hi, x_lo, x_lon, gate);
+  } else {
+    accumulate_x_kernel<32><<<grid2(g, nrhs), BB, 0, st>>>(g, x_hi, x_lo, x_lon, gate);
+  }
 }
 
 void launch_debug_index_probe(const Geom& g, const double2* buf, double* out, cudaStream_t st) {

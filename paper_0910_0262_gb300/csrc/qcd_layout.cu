@@ -108,7 +108,10 @@ __global__ void pack_gauge_kernel(Geom g, const double2* __restrict__ U, double2
 // L1 between its 12 loads), but a site's store instruction touches half of 32 sectors, so the way back moves a
 // block's sites through shared memory and its lanes write consecutive 16-byte words: 32^3 x 64, 8 RHS, FP16
 // to canonical 1037 -> 300 us, the time its bytes take (reads staged the same way: 328 -> 410 us).  Sites in
-// shared memory are 13 words apart, so that eight lanes' 16-byte accesses hit distinct banks.
+// shared memory are 13 words apart, so that eight lanes' 16-byte accesses hit distinct banks.  Three threads
+// share a site, four components each: the conversions of block fixed point, some 25 instructions a number,
+// are long chains on a small lattice (4^3 x 8, one thread per site: 10.7 us to canonical, 5.7 us from it; three: 5.9
+// and 4.8 us).
 constexpr int LB = 128;         // sites of a block
 constexpr int SITE_WORDS = 13;  // double2 words between sites in shared memory
 
@@ -128,26 +131,92 @@ __global__ void spinor_to_native_kernel(Geom g, const double2* __restrict__ cano
   SpinorIO<P>::store(nat, norm, g.Vh, r, h, s);
 }
 
+// the same to block fixed point
+__global__ void __launch_bounds__(3 * LB) spinor_to_fixed_kernel(Geom g, const double2* __restrict__ canon, longlong2* nat,
+                                                                 int* ex, int nrhs) {
+  __shared__ u64 sm[3][LB];
+  const int site = threadIdx.x % LB, part = threadIdx.x / LB;
+  const int tid = blockIdx.x * LB + site;  // (eight right-hand sides at most: below 2^31)
+  const bool valid = tid < g.Vh * nrhs;
+  const int r = tid / g.Vh, h = tid - r * g.Vh;
+  double2 v[4];
+  u64 mx = 0;
+  if (valid) {
+    const double2* src = canon + (size_t)tid * 12 + 4 * part;
+#pragma unroll
+    for (int c = 0; c < 4; c++) {
+      v[c] = src[c];
+      mx = max(mx, max(fx_mag(v[c].x), fx_mag(v[c].y)));
+    }
+  }
+  sm[part][site] = mx;
+  __syncthreads();
+  if (!valid || !dbg_spinor(g.Vh, r, h)) return;
+  const int e = fx_exponent(max(sm[0][site], max(sm[1][site], sm[2][site])));
+#pragma unroll
+  for (int c = 0; c < 4; c++)
+    nat[sidx<12>(4 * part + c, g.Vh, r, h)] =
+        make_longlong2(fx_of_double<FX_SPINOR>(v[c].x, e), fx_of_double<FX_SPINOR>(v[c].y, e));
+  if (part == 0) ex[(size_t)r * g.Vh + h] = e;
+}
+
+// components 4 part .. 4 part + 3 of a site as doubles
 template <int P>
-__global__ void __launch_bounds__(LB) spinor_to_canon_kernel(Geom g, const void* nat, const float* norm,
-                                                             double2* canon, int nrhs) {
-  using R = typename Real<P>::T;
+__device__ __forceinline__ void load_part(const void* nat, const float* norm, int Vh, int r, int h, int part, double2 o[4]) {
+  if (!dbg_spinor(Vh, r, h)) {
+    for (int c = 0; c < 4; c++) o[c] = {};
+    return;
+  }
+  if constexpr (P == 60) {
+    const longlong2* p = static_cast<const longlong2*>(nat);
+    const int e = __ldg(reinterpret_cast<const int*>(norm) + (size_t)r * Vh + h);
+#pragma unroll
+    for (int c = 0; c < 4; c++) {
+      const longlong2 v = __ldg(p + sidx<12>(4 * part + c, Vh, r, h));
+      o[c] = make_double2(fx_to_double(v.x, e, FX_SPINOR), fx_to_double(v.y, e, FX_SPINOR));
+    }
+  } else if constexpr (P == 64) {
+    const double2* p = static_cast<const double2*>(nat);
+#pragma unroll
+    for (int c = 0; c < 4; c++) o[c] = __ldg(p + sidx<12>(4 * part + c, Vh, r, h));
+  } else if constexpr (P == 32) {
+    const float4* p = static_cast<const float4*>(nat);
+#pragma unroll
+    for (int k = 0; k < 2; k++) {
+      const float4 v = __ldg(p + sidx<6>(2 * part + k, Vh, r, h));
+      o[2 * k] = make_double2(widen(v.x), widen(v.y));
+      o[2 * k + 1] = make_double2(widen(v.z), widen(v.w));
+    }
+  } else {
+    const float n = __ldg(norm + (size_t)r * Vh + h);
+    const uint4 v = __ldg(static_cast<const uint4*>(nat) + sidx<3>(part, Vh, r, h));
+    const float2 a = h2f(v.x), b = h2f(v.y), c = h2f(v.z), d = h2f(v.w);
+    o[0] = make_double2(widen(a.x * n), widen(a.y * n));
+    o[1] = make_double2(widen(b.x * n), widen(b.y * n));
+    o[2] = make_double2(widen(c.x * n), widen(c.y * n));
+    o[3] = make_double2(widen(d.x * n), widen(d.y * n));
+  }
+}
+
+template <int P>
+__global__ void __launch_bounds__(3 * LB) spinor_to_canon_kernel(Geom g, const void* nat, const float* norm,
+                                                                 double2* canon, int nrhs) {
   __shared__ double2 buf[LB * SITE_WORDS];
   const long long first = (long long)blockIdx.x * LB, n = (long long)g.Vh * nrhs;
   const int here = (int)min((long long)LB, n - first);
-  if ((int)threadIdx.x < here) {
-    const int tid = (int)(first + threadIdx.x), r = tid / g.Vh, h = tid - r * g.Vh;
-    cx<R> s[12];
-    SpinorIO<P>::load(nat, norm, g.Vh, r, h, s);
+  const int mine = threadIdx.x % LB, part = threadIdx.x / LB;
+  if (mine < here) {
+    const int tid = (int)first + mine, r = tid / g.Vh, h = tid - r * g.Vh;
+    double2 o[4];
+    load_part<P>(nat, norm, g.Vh, r, h, part, o);
 #pragma unroll
-    for (int c = 0; c < 12; c++)
-      buf[threadIdx.x * SITE_WORDS + c] = make_double2(to_double(s[c].re), to_double(s[c].im));
+    for (int c = 0; c < 4; c++) buf[mine * SITE_WORDS + 4 * part + c] = o[c];
   }
   __syncthreads();
   double2* dst = canon + first * 12;
 #pragma unroll
-  for (int k = 0; k < 12; k++) {
-    const int j = k * LB + threadIdx.x, site = j / 12;
+  for (int k = 0; k < 4; k++) {
+    const int j = k * 3 * LB + threadIdx.x, site = j / 12;
     if (site < here) dst[j] = buf[site * SITE_WORDS + (j - 12 * site)];
   }
 }
@@ -178,7 +247,9 @@ void launch_spinor_to_native(int prec, const Geom& g, const double2* canon, void
   g_kernel_launches += 1;
   const int B = 128;
   const int nb = nblocks((long long)g.Vh * nrhs, B);
-  if (prec == 60) spinor_to_native_kernel<60><<<nb, B, 0, st>>>(g, canon, nat, norm, nrhs);
+  if (prec == 60)
+    spinor_to_fixed_kernel<<<nblocks((long long)g.Vh * nrhs, LB), 3 * LB, 0, st>>>(
+        g, canon, static_cast<longlong2*>(nat), reinterpret_cast<int*>(norm), nrhs);
   else if (prec == 64) spinor_to_native_kernel<64><<<nb, B, 0, st>>>(g, canon, nat, norm, nrhs);
   else if (prec == 32) spinor_to_native_kernel<32><<<nb, B, 0, st>>>(g, canon, nat, norm, nrhs);
   else spinor_to_native_kernel<16><<<nb, B, 0, st>>>(g, canon, nat, norm, nrhs);
@@ -187,8 +258,8 @@ void launch_spinor_to_native(int prec, const Geom& g, const double2* canon, void
 void launch_spinor_to_canon(int prec, const Geom& g, const void* nat, const float* norm, double2* canon, int nrhs,
                             cudaStream_t st) {
   g_kernel_launches += 1;
-  const int B = LB;
-  const int nb = nblocks((long long)g.Vh * nrhs, B);
+  const int B = 3 * LB;
+  const int nb = nblocks((long long)g.Vh * nrhs, LB);
   if (prec == 60) spinor_to_canon_kernel<60><<<nb, B, 0, st>>>(g, nat, norm, canon, nrhs);
   else if (prec == 64) spinor_to_canon_kernel<64><<<nb, B, 0, st>>>(g, nat, norm, canon, nrhs);
   else if (prec == 32) spinor_to_canon_kernel<32><<<nb, B, 0, st>>>(g, nat, norm, canon, nrhs);

@@ -132,6 +132,25 @@ def test_fp64_solve(nrhs):
 
 
 @gpu
+@pytest.mark.parametrize("prec", [64, 32, 16])
+@pytest.mark.parametrize("nrhs", [1, 2, 5])
+@pytest.mark.parametrize("dims", [(2, 2, 10, 2), (6, 10, 2, 18), (10, 8, 8, 10)], ids=["40", "1080", "3200"])
+def test_solves_on_ragged_blocks(dims, nrhs, prec):
+    """40 and 1080 sites per parity: a ragged last block of 32; 3200: grid sums over two groups of 64 blocks, the
+    second one ragged.  The true residual, formed by the FP64 operator, differs
+    between two evaluations by its rounding, below 1e-13."""
+    require_gpu()
+    U, op = _context(dims)
+    b = rand_eo(nrhs, int(np.prod(dims)) // 2, np.random.default_rng(19))
+    x, stats, ok = op.cg_solve(to_dev(b), tol=1e-10, inner_prec=prec)
+    assert ok
+    r = b - to_np(op.dslash(x, 3, precision=64))
+    for i in range(nrhs):
+        assert np.linalg.norm(r[i]) <= (1e-10 + 1e-13) * np.linalg.norm(b[i])
+    op.close()
+
+
+@gpu
 @pytest.mark.parametrize("dims", [(2, 2, 2, 2), (4, 4, 2, 2), (4, 2, 6, 4), (6, 10, 2, 4)], ids=lambda d: "x".join(map(str, d)))
 @pytest.mark.parametrize("scale,t_bc", [(1.0, -1.0), (1.0, 1.0), (1.25, -1.0)], ids=["su3", "su3_periodic", "far"])
 def test_matrix_fields(dims, scale, t_bc):
