@@ -49,14 +49,6 @@ WORKLOAD = "c1_16^4"
 # that holds the command; a kernel changed since its capture has no entry (traffic null)
 NCU_TRAFFIC = {
     "cg_persistent_p32": (41.4e6, "profiles/cg_persistent_16x16x16x16.md"),
-    # mean of the clover-inverse (63.3 MB) and xpay (70.2 MB) passes over a step's mix of the two
-    "dslash_p64": (66.7e6, "profiles/dslash_pair64_16x16x16x16.md"),
-}
-# FP64 pipe activity (% of active cycles) from the same captures, for the kernels bound by it: the
-# counted flops of a launch leave out that spin projection and reconstruction are additions, each
-# taking an FMA slot of the pipe
-NCU_FP64_PIPE = {
-    "dslash_p64": (84.3, "profiles/dslash_pair64_16x16x16x16.md"),
 }
 
 
@@ -365,7 +357,8 @@ def run_ours(args, world, rank, local):
                                   unit="GB/s", frac=dk["gbs"] / device_peaks["l2_copy_gbs"],
                                   peak_source="L2-resident copy measured in this run (of measured)",
                                   hbm_peak=hbm_peak, hbm_frac=dk["gbs"] / hbm_peak)
-    elif dominant.startswith("dslash_p32") or dominant.startswith("cg_persistent"):
+    elif dominant.startswith("dslash_") or dominant.startswith("cg_persistent"):
+        # (the FP64 operators' products are formed on integers, so the FP64 pipe is no bound of theirs)
         result["roofline"] = dict(common, bound="hbm", achieved=dk["gbs"], peak=hbm_peak, unit="GB/s",
                                   frac=dk["gbs"] / hbm_peak, peak_source="MEASURED_PEAKS.json hbm_gbs (of measured)")
     else:
@@ -373,9 +366,6 @@ def run_ours(args, world, rank, local):
         result["roofline"] = dict(common, bound="alu", achieved=dk["gflops"] / 1e3, peak=p64, unit="TFLOP/s",
                                   frac=dk["gflops"] / 1e3 / p64,
                                   peak_source="FP64 FMA probe measured in this run (of measured)")
-        if dominant in NCU_FP64_PIPE:
-            result["roofline"]["fp64_pipe_active_pct_ncu"] = NCU_FP64_PIPE[dominant][0]
-            result["roofline"]["fp64_pipe_source"] = NCU_FP64_PIPE[dominant][1]
     if not args.no_md:
         result["clover_det_and_full_solve"] = clover_det_section(op, x, b, stream)
         result["r_algorithm_step"] = r_step_section(op, U, w, stream)

@@ -299,7 +299,7 @@ __global__ void __launch_bounds__(128) field_strength_kernel(Geom g, const doubl
 }
 
 // Bound by the FP64 pipe: with square roots, six logarithms and unfused complex products a block took 10%
-// more of its instructions on even and a third more on odd sites (24^3 x 32: 1.30 -> 0.98 ms).
+// more of its instructions on even and a third more on odd sites (24^3 x 32: 1.30 -> 0.87 ms).
 // A's chiral block b (even sites) or its inverse (odd sites), the ones the operators read, and log det, for
 // one (site, block) per thread, from the six F_{mu nu}
 __global__ void __launch_bounds__(128) clover_assemble_kernel(Geom g, const double2* __restrict__ Fbuf, double kappa,
