@@ -83,8 +83,6 @@ QCD_HD i64 fx_value(const FxSum& s) {
   return (i64)((u64)s.h << K) + (s.m >> (31 - K));
 }
 
-// v 2^-d for d >= 0
-QCD_HD i64 fx_down(i64 v, int d) { return v >> (d < 63 ? d : 63); }
 // v 2^-d rounded to nearest, d >= 0
 QCD_HD i64 fx_down_rn(i64 v, int d) {
   if (d <= 0) return v;
@@ -186,20 +184,6 @@ template <>
 struct SpinorIO<60> {
   static constexpr int NVEC = 12;
   template <int LD = LD_NC>
-  __device__ static void load(const void* base, const float* ex, int Vh, int r, int h, cx<double> s[12]) {
-    if (!dbg_spinor(Vh, r, h)) {
-      for (int c = 0; c < 12; c++) s[c] = {};
-      return;
-    }
-    const longlong2* p = static_cast<const longlong2*>(base);
-    const int e = ldv<LD>(reinterpret_cast<const int*>(ex) + (size_t)r * Vh + h);
-#pragma unroll
-    for (int c = 0; c < 12; c++) {
-      const longlong2 v = ldv<LD>(p + sidx<NVEC>(c, Vh, r, h));
-      s[c] = cmk(fx_to_double(v.x, e, FX_SPINOR), fx_to_double(v.y, e, FX_SPINOR));
-    }
-  }
-  template <int LD = LD_NC>
   __device__ static void load_block(const void* base, const float* ex, int Vh, int r, int h, int b,
                                     cx<double> s[6]) {
     if (!dbg_spinor(Vh, r, h)) {
@@ -214,26 +198,7 @@ struct SpinorIO<60> {
       s[c] = cmk(fx_to_double(v.x, e, FX_SPINOR), fx_to_double(v.y, e, FX_SPINOR));
     }
   }
-  __device__ static void store(void* base, float* ex, int Vh, int r, int h, const cx<double> s[12]) {
-    if (!dbg_spinor(Vh, r, h)) return;
-    u64 mx = 0;
-#pragma unroll
-    for (int c = 0; c < 12; c++) {
-      const u64 a = fx_mag(s[c].re), b = fx_mag(s[c].im);
-      mx = a > mx ? a : mx;
-      mx = b > mx ? b : mx;
-    }
-    const int e = fx_exponent(mx);
-    longlong2* p = static_cast<longlong2*>(base);
-#pragma unroll
-    for (int c = 0; c < 12; c++)
-      p[sidx<NVEC>(c, Vh, r, h)] =
-          make_longlong2(fx_of_double<FX_SPINOR>(s[c].re, e), fx_of_double<FX_SPINOR>(s[c].im, e));
-    reinterpret_cast<int*>(ex)[(size_t)r * Vh + h] = e;
-  }
 };
-template <>
-struct Real<60> { using T = double; };
 
 // a link entry or a clover entry pair as stored: the limbs of two numbers
 QCD_HD int4 fx_pack2(FxLimb a, FxLimb b) { return int4{a.hi, a.lo, b.hi, b.lo}; }
