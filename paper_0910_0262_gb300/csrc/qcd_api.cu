@@ -216,6 +216,9 @@ size_t spinor_bytes(const Geom& g, int prec, int nrhs) {
   return per * (size_t)g.Vh * nrhs;
 }
 
+// FP16's norm of a site, block fixed point's exponents of its two chiral blocks
+size_t norm_bytes(const Geom& g, int prec, int nrhs) { return (prec == 60 ? 8 : 4) * (size_t)g.Vh * nrhs; }
+
 qcd_status ws_get(qcd_ctx* c, int slot, size_t bytes, void** out) {
   Buf& b = c->ws[slot];
   if (b.bytes < bytes) {
@@ -803,7 +806,7 @@ qcd_status qcd_dslash(qcd_ctx* c, double* out, const double* in, int op, int dag
     const double2* cin = reinterpret_cast<const double2*>(in) + (size_t)done * g.Vh * 12;
     double2* cout = reinterpret_cast<double2*>(out) + (size_t)done * g.Vh * 12;
     void *vin, *vout, *vt, *vy, *nin = nullptr, *nout = nullptr, *nt = nullptr, *ny = nullptr;
-    const size_t fb = spinor_bytes(g, prec, nb), nbytes = sizeof(float) * (size_t)g.Vh * nb;
+    const size_t fb = spinor_bytes(g, prec, nb), nbytes = norm_bytes(g, prec, nb);
     if ((s = ws_get(c, S_IN, fb, &vin)) || (s = ws_get(c, S_OUT, fb, &vout)) || (s = ws_get(c, S_T, fb, &vt)) ||
         (s = ws_get(c, S_Y, fb, &vy)))
       return s;
@@ -879,12 +882,13 @@ qcd_status solver_fields(qcd_ctx* c, int inner, int nrhs, SolverFields* f) {
   GET(S_YL, lo_p, f->y, void*);
   f->x_lo_n = f->r_lo_n = f->p_n = f->ap_n = f->t_n = f->y_n = nullptr;
   f->ap_hi_n = f->t_hi_n = f->y_hi_n = nullptr;
-  const size_t nb = sizeof(float) * (size_t)g.Vh * nrhs;
   if (f->hp == 60) {
-    GET(S_AP_HI_N, nb, f->ap_hi_n, float*);
-    GET(S_T_HI_N, nb, f->t_hi_n, float*);
-    GET(S_Y_HI_N, nb, f->y_hi_n, float*);
+    const size_t eb = norm_bytes(g, 60, nrhs);
+    GET(S_AP_HI_N, eb, f->ap_hi_n, float*);
+    GET(S_T_HI_N, eb, f->t_hi_n, float*);
+    GET(S_Y_HI_N, eb, f->y_hi_n, float*);
   }
+  const size_t nb = norm_bytes(g, f->pp, nrhs);
   if (f->pp == 16 || f->pp == 60) {
     GET(S_P_N, nb, f->p_n, float*);
     GET(S_AP_N, nb, f->ap_n, float*);
@@ -942,7 +946,7 @@ void enqueue_iteration(qcd_ctx* c, const SolverFields& f, int nrhs) {
   run_dslash(c, f.pp, EPI_XPAY_CG, b);
   {
     const double pb =
-        (double)g.Vh * nrhs * (24.0 * real_bytes(f.pr) + 2 * (24.0 * real_bytes(f.pp) + (f.p_n ? 4 : 0)));
+        (double)g.Vh * nrhs * (24.0 * real_bytes(f.pr) + 2 * (24.0 * real_bytes(f.pp) + (f.pp == 60 ? 8 : (f.p_n ? 4 : 0))));
     ProfScope ps(c, "p_update", pb, 0);
     launch_p_update(f.pr, f.pp, g, nrhs, f.r_lo, f.r_lo_n, f.p, f.p_n, c->cg, halt, c->cur);
   }
@@ -1258,7 +1262,7 @@ qcd_status cg_batch(qcd_ctx* c, double2* x, const double2* b, int nrhs, const qc
   else launch_zero(f.x_hi, spinor_bytes(g, 64, nrhs), c->st);
   launch_zero(f.x_lo, spinor_bytes(g, f.pr, nrhs), c->st);
   launch_zero(f.p, spinor_bytes(g, f.pp, nrhs), c->st);
-  if (f.p_n) launch_zero(f.p_n, sizeof(float) * (size_t)g.Vh * nrhs, c->st);
+  if (f.p_n) launch_zero(f.p_n, norm_bytes(g, f.pp, nrhs), c->st);
   if (prm->use_x0) {
     if (f.hp == 60) launch_spinor_to_native(60, g, x, f.ap_hi, f.ap_hi_n, nrhs, c->st);
     apply_mdagm(c, f.hp, nrhs, f.hp == 60 ? f.ap_hi : f.x_hi, f.ap_hi_n, f.ap_hi, nullptr, f.t_hi, f.t_hi_n, f.y_hi,
@@ -1415,7 +1419,7 @@ qcd_status force_fixed(qcd_ctx* c, double2* F, const double2* X, int nrhs, bool 
   const Geom& g = c->g;
   qcd_status s = QCD_OK;
   void *xf = nullptr, *yf = nullptr, *xn = nullptr, *yn = nullptr, *clf, *cxf, *ef;
-  const size_t half = (size_t)nrhs * 12 * g.Vh, hn = (size_t)nrhs * g.Vh;
+  const size_t half = (size_t)nrhs * 12 * g.Vh, hn = (size_t)nrhs * 2 * g.Vh;
   *ran = false;
   if ((nrhs > 0 && (ws_get(c, S_F_X, 2 * half * sizeof(double2), &xf) || ws_get(c, S_F_Y, 2 * half * sizeof(double2), &yf) ||
                     ws_get(c, S_F_XN, 2 * hn * sizeof(int), &xn) || ws_get(c, S_F_YN, 2 * hn * sizeof(int), &yn))) ||
@@ -1428,7 +1432,7 @@ qcd_status force_fixed(qcd_ctx* c, double2* F, const double2* X, int nrhs, bool 
   double2* C = static_cast<double2*>(clf);
   for (int done = 0; done < nrhs;) {
     const int nb = batch_of(nrhs - done);
-    const size_t off = (size_t)done * 12 * g.Vh, on = (size_t)done * g.Vh;
+    const size_t off = (size_t)done * 12 * g.Vh, on = (size_t)done * 2 * g.Vh;
     launch_spinor_to_native(60, g, X + off, Xe + off, xe + on, nb, c->st);
     // Y_e = Mhat X_e with X_o = A_oo^-1 D_oe X_e left in the odd temporary
     apply_mhat(c, 60, nb, false, Xe + off, xe + on, Ye + off, ye + on, Xo + off, xo + on, nullptr, nullptr);
@@ -1701,7 +1705,7 @@ qcd_status qcd_prepare_source(qcd_ctx* c, double* bhat_e, const double* b_e, con
       CUDA_TRY(cudaMemcpyAsync(cout, ce, n * nb * sizeof(double2), cudaMemcpyDeviceToDevice, c->st));
     } else {
       void *u, *t, *un, *tn;
-      const size_t fb = spinor_bytes(g, rep, nb), eb = sizeof(int) * (size_t)g.Vh * nb;
+      const size_t fb = spinor_bytes(g, rep, nb), eb = norm_bytes(g, 60, nb);
       if ((s = ws_get(c, S_IN, fb, &u)) || (s = ws_get(c, S_T, fb, &t)) || (s = ws_get(c, S_IN_N, eb, &un)) ||
           (s = ws_get(c, S_T_N, eb, &tn)))
         return s;
@@ -1734,7 +1738,7 @@ qcd_status qcd_reconstruct_odd(qcd_ctx* c, double* x_o, const double* x_e, const
   for (int done = 0; done < nrhs;) {
     const int nb = batch_of(nrhs - done), rep = fp64_rep(c, true);
     void *u, *t, *un, *tn;
-    const size_t fb = spinor_bytes(g, rep, nb), eb = sizeof(int) * (size_t)g.Vh * nb;
+    const size_t fb = spinor_bytes(g, rep, nb), eb = norm_bytes(g, 60, nb);
     if ((s = ws_get(c, S_IN, fb, &u)) || (s = ws_get(c, S_T, fb, &t)) || (s = ws_get(c, S_IN_N, eb, &un)) ||
         (s = ws_get(c, S_T_N, eb, &tn)))
       return s;

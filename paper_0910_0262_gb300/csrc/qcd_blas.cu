@@ -44,35 +44,27 @@ __global__ void __launch_bounds__(BB) p_update_kernel(Geom g, const void* r, con
 // 7.89 -> 7.84 ms a solve there)
 __global__ void __launch_bounds__(64) p_update_fixed_kernel(Geom g, const double2* r, longlong2* p, int* pe,
                                                             const CGState* cg, const int* halt, const int* gate) {
-  __shared__ unsigned long long sm[2][32];
   if ((halt && *halt) || (gate && !*gate)) return;
   const int k = blockIdx.y, lane = threadIdx.x & 31, b = threadIdx.x >> 5, Vh = g.Vh;
-  if (!cg[k].active) return;
   const int h = blockIdx.x * 32 + lane;
-  const bool valid = h < Vh && dbg_spinor(Vh, k, h);
+  if (!cg[k].active || h >= Vh || !dbg_spinor(Vh, k, h)) return;
   const double beta = cg[k].beta;
-  cx<double> o[6];
+  cx<double> o[6], rs[6];
   u64 mx = 0;
-  if (valid) {
-    cx<double> rs[6];
-    SpinorIO<64>::load_block(r, nullptr, Vh, k, h, b, rs);
-    SpinorIO<60>::load_block(p, reinterpret_cast<const float*>(pe), Vh, k, h, b, o);
+  SpinorIO<64>::load_block(r, nullptr, Vh, k, h, b, rs);
+  SpinorIO<60>::load_block(p, reinterpret_cast<const float*>(pe), Vh, k, h, b, o);
 #pragma unroll
-    for (int c = 0; c < 6; c++) {
-      o[c].re = fma(beta, o[c].re, rs[c].re);
-      o[c].im = fma(beta, o[c].im, rs[c].im);
-      mx = max(mx, max(fx_mag(o[c].re), fx_mag(o[c].im)));
-    }
+  for (int c = 0; c < 6; c++) {
+    o[c].re = fma(beta, o[c].re, rs[c].re);
+    o[c].im = fma(beta, o[c].im, rs[c].im);
+    mx = max(mx, max(fx_mag(o[c].re), fx_mag(o[c].im)));
   }
-  sm[b][lane] = mx;
-  __syncthreads();  // (also: both blocks have read the site's exponent)
-  if (!valid) return;
-  const int e = fx_exponent(max(mx, sm[1 - b][lane]));
+  const int e = fx_exponent(mx);
 #pragma unroll
   for (int c = 0; c < 6; c++)
     p[sidx<12>(6 * b + c, Vh, k, h)] =
         make_longlong2(fx_of_double<FX_SPINOR>(o[c].re, e), fx_of_double<FX_SPINOR>(o[c].im, e));
-  if (b == 0) pe[(size_t)k * Vh + h] = e;
+  pe[eidx(b, Vh, k, h)] = e;
 }
 
 template <int PR>
@@ -103,36 +95,30 @@ template <int PR>
 __global__ void __launch_bounds__(64) accumulate_x_fixed_kernel(Geom g, double2* x_hi, void* x_lo, longlong2* x_fx,
                                                                 int* x_fx_e, const int* gate) {
   using RR = typename Real<PR>::T;
-  __shared__ u64 sm[2][32];
   if (gate && !*gate) return;
   const int k = blockIdx.y, lane = threadIdx.x & 31, b = threadIdx.x >> 5, Vh = g.Vh;
   const int h = blockIdx.x * 32 + lane;
-  const bool valid = h < Vh && dbg_spinor(Vh, k, h);
+  if (h >= Vh || !dbg_spinor(Vh, k, h)) return;
   cx<double> hi[6];
+  cx<RR> lo[6];
   u64 mx = 0;
-  if (valid) {
-    cx<RR> lo[6];
-    SpinorIO<PR>::load_block(x_lo, nullptr, Vh, k, h, b, lo);
-    SpinorIO<64>::load_block(x_hi, nullptr, Vh, k, h, b, hi);
+  SpinorIO<PR>::load_block(x_lo, nullptr, Vh, k, h, b, lo);
+  SpinorIO<64>::load_block(x_hi, nullptr, Vh, k, h, b, hi);
 #pragma unroll
-    for (int c = 0; c < 6; c++) {
-      hi[c].re += to_double(lo[c].re);
-      hi[c].im += to_double(lo[c].im);
-      lo[c] = cmk(RR(0), RR(0));
-      mx = max(mx, max(fx_mag(hi[c].re), fx_mag(hi[c].im)));
-    }
-    SpinorIO<64>::store_block(x_hi, nullptr, Vh, k, h, b, hi);
-    SpinorIO<PR>::store_block(x_lo, nullptr, Vh, k, h, b, lo);
+  for (int c = 0; c < 6; c++) {
+    hi[c].re += to_double(lo[c].re);
+    hi[c].im += to_double(lo[c].im);
+    lo[c] = cmk(RR(0), RR(0));
+    mx = max(mx, max(fx_mag(hi[c].re), fx_mag(hi[c].im)));
   }
-  sm[b][lane] = mx;
-  __syncthreads();
-  if (!valid) return;
-  const int e = fx_exponent(max(mx, sm[1 - b][lane]));
+  SpinorIO<64>::store_block(x_hi, nullptr, Vh, k, h, b, hi);
+  SpinorIO<PR>::store_block(x_lo, nullptr, Vh, k, h, b, lo);
+  const int e = fx_exponent(mx);
 #pragma unroll
   for (int c = 0; c < 6; c++)
     x_fx[sidx<12>(6 * b + c, Vh, k, h)] =
         make_longlong2(fx_of_double<FX_SPINOR>(hi[c].re, e), fx_of_double<FX_SPINOR>(hi[c].im, e));
-  if (b == 0) x_fx_e[(size_t)k * Vh + h] = e;
+  x_fx_e[eidx(b, Vh, k, h)] = e;
 }
 
 template <int PR>

@@ -20,11 +20,9 @@ constexpr int FX_STAGES = 2;
 __host__ __device__ constexpr int fx_stage_rows(int pairs) { return 9 + 12 * pairs; }
 
 // exchange area of one pair of warps: the components a warp passes to its partner (rows 0-5 to warp 0, 6-17
-// to warp 1) and the exponents of the finished blocks; it takes the place of the pair's spinor rows of stage
-// 0, which the last hop does not use
+// to warp 1); it takes the place of the pair's spinor rows of stage 0, which the last hop does not use
 struct FxXch {
   i64 v[18][32];  // [component re, im][lane]
-  int eo[2][32];
 };
 static_assert(sizeof(FxXch) <= 12 * 32 * sizeof(int4), "the exchange area fits a pair's spinor rows");
 
@@ -33,17 +31,21 @@ static_assert(sizeof(FxXch) <= 12 * 32 * sizeof(int4), "the exchange area fits a
 // false: mu = y, t) or +-i (IMAG: mu = x, z); w = U h is added to the sum of spin k (up), and conj(c) w to
 // that of spin p (low).  BWD: the backward hop (sgn = +1), which takes U^dag.  sk, sp, u: the staged rows of
 // the neighbour's spins k and p and of the link; neg = -1: (g_mu)_kp is -1 or -i (0: 1 or i); g5 = -1: gamma_5 psi in
-// place of psi, which changes the sign of psi_p (0: psi itself); flip: -w in place of w; the contribution is
-// brought down by d powers of two.
+// place of psi, which changes the sign of psi_p (0: psi itself); flip: -w in place of w; psi_k and psi_p are
+// brought down by dk and dp powers of two, from their blocks' units to the sum's.
 template <bool IMAG, bool BWD>
 __device__ __forceinline__ void hop_fx(const longlong2* sk, const longlong2* sp, const int4* u, int neg, int g5,
-                                       bool flip, int d, cx<i64> up[3], cx<i64> low[3]) {
+                                       bool flip, int dk, int dp, cx<i64> up[3], cx<i64> low[3]) {
   if (!BWD) neg = ~neg;  // c = -+1, -+i
   const int f = neg ^ g5;
   FxLimb re[3], im[3];
 #pragma unroll
   for (int b = 0; b < 3; b++) {
-    const longlong2 x = sk[32 * b], y = sp[32 * b];
+    longlong2 x = sk[32 * b], y = sp[32 * b];
+    x.x >>= dk;
+    x.y >>= dk;
+    y.x >>= dp;
+    y.y >>= dp;
     const i64 hr = x.x + (IMAG ? fx_sign(y.y, ~f) : fx_sign(y.x, f));
     const i64 hi = x.y + (IMAG ? fx_sign(y.x, f) : fx_sign(y.y, f));
     re[b] = fx_split(hr);
@@ -67,8 +69,6 @@ __device__ __forceinline__ void hop_fx(const longlong2* sk, const longlong2* sp,
       x = -x;
       y = -y;
     }
-    x >>= d;
-    y >>= d;
     up[a].re += x;
     up[a].im += y;
     // conj(c) w: c = +-1: +-w; c = +-i: -+i w
@@ -145,13 +145,10 @@ __device__ __forceinline__ FxShift fx_shift(int unit, int e) {
 }
 
 // The epilogue of chiral block B of a site, RHS r, with the hopping sum v in units of 2^(eh - 56), and its
-// stores.  active: this warp has a block to finish (the others only meet the block's barriers); eo: the
-// finished blocks' exponents, in shared memory.  All threads of the block call it together.  Returns the
-// thread's share of |out|^2 (do_norm) or of |r|^2 (EPI_XPAY_CG, EPI_RESID).
+// stores.  Returns the thread's share of |out|^2 (do_norm) or of |r|^2 (EPI_XPAY_CG, EPI_RESID).
 template <int EPI>
-__device__ __forceinline__ double finish_fx(const DslashArgs& A, const FxScalar& sc, int hh, bool valid, bool active, int r,
-                                            int B, cx<i64> v[6], int eh, int (*eo)[32]) {
-  const int lane = threadIdx.x & 31;
+__device__ __forceinline__ double finish_fx(const DslashArgs& A, const FxScalar& sc, int hh, bool valid, int r, int B,
+                                            cx<i64> v[6], int eh) {
   const int Vh = A.g.Vh;
   double nrm = 0.0;
   cx<i64> t[6];
@@ -180,7 +177,7 @@ __device__ __forceinline__ double finish_fx(const DslashArgs& A, const FxScalar&
       } else {
         cx<i64> xs[6], cxs[6];
         const longlong2* px = static_cast<const longlong2*>(A.x);
-        const int exx = __ldg(reinterpret_cast<const int*>(A.x_norm) + (size_t)r * Vh + hh);
+        const int exx = __ldg(reinterpret_cast<const int*>(A.x_norm) + eidx(B, Vh, r, hh));
         bad = bad || exx > FX_BIG || sc.e > FX_BIG;
 #pragma unroll
         for (int k = 0; k < 6; k++) {
@@ -257,19 +254,11 @@ __device__ __forceinline__ double finish_fx(const DslashArgs& A, const FxScalar&
         SpinorIO<64>::store_block(A.out, nullptr, Vh, r, hh, B, res);
       }
     }
-    __syncthreads();  // the exchange area is rewritten by the next RHS
     return nrm;
   }
-  // the site's exponent is the larger of its two blocks'
-  int eb = FX_ZERO;
-  if (valid) {
-    const int bits = fx_bits_of(t);
-    eb = bad ? FX_NAN : (bits ? unit + bits : FX_ZERO);
-  }
-  if (active) eo[B][lane] = eb;
-  __syncthreads();
   if (valid && dbg_spinor(Vh, r, hh)) {
-    const int e = max(eb, eo[1 - B][lane]);
+    const int bits = fx_bits_of(t);
+    const int e = bad ? FX_NAN : (bits ? unit + bits : FX_ZERO);
     const FxShift f = fx_shift(unit, e);
     longlong2* po = static_cast<longlong2*>(A.out);
     FxSum n = {};
@@ -285,13 +274,12 @@ __device__ __forceinline__ double finish_fx(const DslashArgs& A, const FxScalar&
       }
       po[sidx<12>(6 * B + k, Vh, r, hh)] = make_longlong2(a, b);
     }
-    if (B == 0) reinterpret_cast<int*>(A.out_norm)[(size_t)r * Vh + hh] = e;
+    reinterpret_cast<int*>(A.out_norm)[eidx(B, Vh, r, hh)] = e;
     if (A.do_norm) {
       const int u = e > FX_BIG ? FX_NAN : 2 * (e - FX_SPINOR + 2);
       nrm = fx_to_double(n.h, u + 62, 0) + fx_to_double(n.m, u + 32, 0);
     }
   }
-  __syncthreads();  // the exchange area is rewritten by the next RHS
   return nrm;
 }
 
@@ -345,18 +333,24 @@ __device__ __forceinline__ double pair_fx(const DslashArgs& A, const FxScalar& s
   static_assert(FX_STAGES == 2, "the loop below fetches one hop ahead");
   fetch(0, 0, 0);
   int eh = FX_ZERO;
-  unsigned dw[2] = {0, 0};
+  unsigned dwk[2] = {0, 0}, dwp[2] = {0, 0};
   if (valid) {
-    const int* ex = reinterpret_cast<const int*>(A.in_norm) + (size_t)r * Vh;
-    int e8[8];
+    const int* ex = reinterpret_cast<const int*>(A.in_norm) + eidx(0, Vh, r, 0);
+    int ek[8], ep[8];  // of the neighbours' blocks 0 (spin k) and 1 (spin p)
 #pragma unroll
-    for (int k = 0; k < 8; k++) e8[k] = __ldg(ex + nbs[k >> 1][k & 1][lane]);
+    for (int k = 0; k < 8; k++) {
+      const int nb = nbs[k >> 1][k & 1][lane];
+      ek[k] = __ldg(ex + nb);
+      ep[k] = __ldg(ex + Vh + nb);
+    }
 #pragma unroll
-    for (int k = 0; k < 8; k++) eh = max(eh, e8[k]);
+    for (int k = 0; k < 8; k++) eh = max(eh, max(ek[k], ep[k]));
     // the neighbours' shifts, eight bits each: byte 2 (mu >> 1) + bwd of word mu & 1
 #pragma unroll
-    for (int k = 0; k < 8; k++)
-      dw[(k >> 1) & 1] |= (unsigned)min(eh - e8[k], 63) << (8 * (2 * (k >> 2) + (k & 1)));
+    for (int k = 0; k < 8; k++) {
+      dwk[(k >> 1) & 1] |= (unsigned)min(eh - ek[k], 63) << (8 * (2 * (k >> 2) + (k & 1)));
+      dwp[(k >> 1) & 1] |= (unsigned)min(eh - ep[k], 63) << (8 * (2 * (k >> 2) + (k & 1)));
+    }
   }
   {
     const int g5 = A.in_g5 ? -1 : 0;
@@ -388,8 +382,9 @@ __device__ __forceinline__ double pair_fx(const DslashArgs& A, const FxScalar& s
         // (g_mu)_Bp: x i, i; y -1, 1; z i, -i; t 1, 1 (B = 0, 1)
         const int neg = ODD ? (!z && B == 0 ? -1 : 0) : (z && B == 1 ? -1 : 0);
         const bool flip = ODD && z && anti && tg == (BWD ? 0 : A.g.Tg - 1);
-        const int d = (dw[ODD ? 1 : 0] >> (16 * z + (BWD ? 8 : 0))) & 63;
-        hop_fx<!ODD, BWD>(sp + 96 * B, sp + 96 * p, buf, neg, g5, flip, d, up, low);
+        const int sh = 16 * z + (BWD ? 8 : 0);
+        const int dk = (dwk[ODD ? 1 : 0] >> sh) & 63, dp = (dwp[ODD ? 1 : 0] >> sh) & 63;
+        hop_fx<!ODD, BWD>(sp + 96 * B, sp + 96 * p, buf, neg, g5, flip, dk, dp, up, low);
       };
       hop(F(), F());
       hop(F(), T());
@@ -427,7 +422,7 @@ __device__ __forceinline__ double pair_fx(const DslashArgs& A, const FxScalar& s
       }
     }
   }
-  return finish_fx<EPI>(A, sc, hh, valid, true, r, B, v, eh, xch->eo);
+  return finish_fx<EPI>(A, sc, hh, valid, r, B, v, eh);
 }
 
 // One pair of warps per (32 output sites, RHS); a block holds the pairs of PAIRS RHS of the same sites,
@@ -459,6 +454,7 @@ __global__ void __launch_bounds__(64 * PAIRS, 8 / PAIRS) dslash_fixed_kernel(Dsl
 #pragma unroll 1
   for (int r0 = 0; r0 < A.nrhs; r0 += PAIRS) {
     const int r = r0 + q;
+    if (r0 > 0) __syncthreads();  // the exchange area of the last RHS has been read
     double nrm = pair_fx<EPI, PAIRS>(A, sc, hh, site && r < A.nrhs, s.t, r, q, w & 1, nbs, fx_ring);
     if (reduce && r < A.nrhs) {
       for (int off = 16; off >= 1; off >>= 1) nrm += __shfl_xor_sync(0xffffffffu, nrm, off);
@@ -478,7 +474,6 @@ __global__ void __launch_bounds__(64 * PAIRS, 8 / PAIRS) dslash_fixed_kernel(Dsl
 template <int EPI>
 __global__ void __launch_bounds__(256, 2) dslash_fixed_split_kernel(DslashArgs A, FxScalar sc) {
   extern __shared__ __align__(16) int4 fx_ring[];
-  __shared__ int eo[2][32];
   if ((A.halt && *A.halt) || (A.gate && !*A.gate)) return;
   const int lane = threadIdx.x & 31, w = threadIdx.x >> 5, q = w >> 1, B = w & 1, r = blockIdx.y;
   const int hh = blockIdx.x * 32 + lane, Vh = A.g.Vh;
@@ -486,10 +481,10 @@ __global__ void __launch_bounds__(256, 2) dslash_fixed_split_kernel(DslashArgs A
   constexpr int STAGE = fx_stage_rows(1) * 32;
   int4* mine = fx_ring + 2 * q * STAGE + lane;  // the forward hop's stage, then the backward one's
   Site s{};
-  int eh = FX_ZERO, ef = 0, eb = 0;
+  int eh = FX_ZERO, ef[2] = {0, 0}, eb[2] = {0, 0};  // [chiral block]
   if (valid) {
     s = site_of(A.g, A.p, hh);
-    const int* ex = reinterpret_cast<const int*>(A.in_norm) + (size_t)r * Vh;
+    const int* ex = reinterpret_cast<const int*>(A.in_norm) + eidx(0, Vh, r, 0);
     const int nf = neighbor_fwd(A.g, s, q) >> 1, nb = neighbor_bwd(A.g, s, q) >> 1;
     const int4* in = static_cast<const int4*>(A.in) + ((size_t)r * 12 + 6 * B) * Vh;
     const int4* u = static_cast<const int4*>(A.gauge) + (size_t)(5 * B) * Vh;
@@ -512,10 +507,14 @@ __global__ void __launch_bounds__(256, 2) dslash_fixed_split_kernel(DslashArgs A
     }
 #pragma unroll
     for (int mu = 0; mu < 4; mu++) {
-      const int a = __ldg(ex + (neighbor_fwd(A.g, s, mu) >> 1)), b = __ldg(ex + (neighbor_bwd(A.g, s, mu) >> 1));
-      eh = max(eh, max(a, b));
-      ef = mu == q ? a : ef;
-      eb = mu == q ? b : eb;
+      const int hf = neighbor_fwd(A.g, s, mu) >> 1, hb = neighbor_bwd(A.g, s, mu) >> 1;
+#pragma unroll
+      for (int k = 0; k < 2; k++) {
+        const int a = __ldg(ex + (size_t)k * Vh + hf), b = __ldg(ex + (size_t)k * Vh + hb);
+        eh = max(eh, max(a, b));
+        ef[k] = mu == q ? a : ef[k];
+        eb[k] = mu == q ? b : eb[k];
+      }
     }
   }
   cp_async_commit();
@@ -524,18 +523,19 @@ __global__ void __launch_bounds__(256, 2) dslash_fixed_split_kernel(DslashArgs A
   cx<i64> up[3] = {}, low[3] = {};
   {
     const int g5 = A.in_g5 ? -1 : 0, p = q < 2 ? 3 - B : 2 + B;
-    const int df = min(eh - ef, 63), db = min(eh - eb, 63), tg = s.t + A.g.t0;
+    const int fk = min(eh - ef[0], 63), fp = min(eh - ef[1], 63), bk = min(eh - eb[0], 63), bp = min(eh - eb[1], 63);
+    const int tg = s.t + A.g.t0;
     const longlong2* sf = reinterpret_cast<const longlong2*>(mine) + 32 * 9;
     const longlong2* sb = sf + STAGE;
     if (q & 1) {  // (g_y)_Bp: -1, 1; (g_t)_Bp: 1, 1
       const int neg = q == 1 && B == 0 ? -1 : 0;
       const bool anti = q == 3 && A.g.t_bc < 0.0;
-      hop_fx<false, false>(sf + 96 * B, sf + 96 * p, mine, neg, g5, anti && tg == A.g.Tg - 1, df, up, low);
-      hop_fx<false, true>(sb + 96 * B, sb + 96 * p, mine + STAGE, neg, g5, anti && tg == 0, db, up, low);
+      hop_fx<false, false>(sf + 96 * B, sf + 96 * p, mine, neg, g5, anti && tg == A.g.Tg - 1, fk, fp, up, low);
+      hop_fx<false, true>(sb + 96 * B, sb + 96 * p, mine + STAGE, neg, g5, anti && tg == 0, bk, bp, up, low);
     } else {  // (g_x)_Bp: i, i; (g_z)_Bp: i, -i
       const int neg = q == 2 && B == 1 ? -1 : 0;
-      hop_fx<true, false>(sf + 96 * B, sf + 96 * p, mine, neg, g5, false, df, up, low);
-      hop_fx<true, true>(sb + 96 * B, sb + 96 * p, mine + STAGE, neg, g5, false, db, up, low);
+      hop_fx<true, false>(sf + 96 * B, sf + 96 * p, mine, neg, g5, false, fk, fp, up, low);
+      hop_fx<true, true>(sb + 96 * B, sb + 96 * p, mine + STAGE, neg, g5, false, bk, bp, up, low);
     }
   }
   __syncthreads();  // every pair has read its stages: the sums take their place
@@ -562,7 +562,7 @@ __global__ void __launch_bounds__(256, 2) dslash_fixed_split_kernel(DslashArgs A
         v[3 + a] = v[3 + a] + cmk(part[w1][o][lane], part[w1][o + 1][lane]);
       }
   }
-  double nrm = finish_fx<EPI>(A, sc, hh, valid && q == 0, q == 0, r, B, v, eh, eo);
+  double nrm = finish_fx<EPI>(A, sc, hh, valid && q == 0, r, B, v, eh);
   if (A.do_norm || EPI == EPI_XPAY_CG || EPI == EPI_RESID) {
     if (q == 0) {
       for (int off = 16; off >= 1; off >>= 1) nrm += __shfl_xor_sync(0xffffffffu, nrm, off);
@@ -584,31 +584,25 @@ __global__ void __launch_bounds__(128) clover_fixed_kernel(Geom g, const int4* c
   if (tid >= Vh * nrhs) return;
   const int r = tid / Vh, h = tid - r * Vh;
   if (!dbg_spinor(Vh, r, h) || !dbg_clover(Vh, h, 0)) return;
-  const int ex = in_e[(size_t)r * Vh + h];
-  cx<i64> t[2][6];
-  int unit[2], e = FX_ZERO;
 #pragma unroll
   for (int b = 0; b < 2; b++) {
-    cx<i64> x[6];
+    const int ex = in_e[eidx(b, Vh, r, h)];
+    cx<i64> x[6], t[6];
 #pragma unroll
     for (int k = 0; k < 6; k++) {
       const longlong2 v = in[sidx<12>(6 * b + k, Vh, r, h)];
       x[k] = cmk((i64)v.x, (i64)v.y);
     }
     const int ec = clover_e[(size_t)b * Vh + h];
-    clover_fx(clover + (size_t)(18 * b) * Vh + h, Vh, x, t[b]);
-    unit[b] = ex - FX_SPINOR + ec + 2;
-    const int bits = fx_bits_of(t[b]);
-    e = max(e, ex > FX_BIG || ec > FX_BIG ? FX_NAN : (bits ? unit[b] + bits : FX_ZERO));
-  }
-#pragma unroll
-  for (int b = 0; b < 2; b++) {
-    const FxShift f = fx_shift(unit[b], e);
+    clover_fx(clover + (size_t)(18 * b) * Vh + h, Vh, x, t);
+    const int unit = ex - FX_SPINOR + ec + 2, bits = fx_bits_of(t);
+    const int e = ex > FX_BIG || ec > FX_BIG ? FX_NAN : (bits ? unit + bits : FX_ZERO);
+    const FxShift f = fx_shift(unit, e);
 #pragma unroll
     for (int k = 0; k < 6; k++)
-      out[sidx<12>(6 * b + k, Vh, r, h)] = make_longlong2(f(t[b][k].re), f(t[b][k].im));
+      out[sidx<12>(6 * b + k, Vh, r, h)] = make_longlong2(f(t[k].re), f(t[k].im));
+    out_e[eidx(b, Vh, r, h)] = e;
   }
-  out_e[(size_t)r * Vh + h] = e;
 }
 
 }  // namespace

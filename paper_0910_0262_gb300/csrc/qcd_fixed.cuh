@@ -3,7 +3,8 @@
 // GB300 issues two FP64 fused multiply-adds per clock and SM, and 61 integer multiply-adds of 32 x 32
 // into 64 bits (both measured), so the products of the hopping term and the clover blocks are formed on
 // integers.  A number is an integer v of at most 60 bits with a power-of-two unit shared by its group:
-//   spinor site   24 reals, |x| < 2^e for all of them, x = v 2^(e-60); e is stored per (RHS, site)
+//   spinor site   12 reals of each chiral block, |x| < 2^e for all of them, x = v 2^(e-60); e is stored per
+//                 (RHS, block, site): the site operators do not mix the blocks, and one may be much the smaller
 //   link          near-unitary, entries of magnitude <= 1 + 1e-5, x = v 2^-58 (no exponent)
 //   clover block  36 reals of one 6x6 block, |x| <= 2^e, x = v 2^(e-58); e per (block, site)
 // For a product both factors are split as v = hi 2^31 + lo, and
@@ -22,7 +23,7 @@
 //   clover: |hi| <= 2^27, |lo| <= 2^30 against |x| < 2^60 with hi <= 2^29, |lo| <= 2^30; eleven products:
 //     |sum ah bl + al bh| <= 11 (2^57 + 2^59) < 2^62.8, and their value in units of 2^60 is below 2^61.5
 //
-// A site whose reals are not all finite carries the exponent FX_NAN: the largest exponent of its
+// A block whose reals are not all finite carries the exponent FX_NAN: the largest exponent of its
 // neighbours is what a result takes its unit from, so the mark spreads as a NaN does, and the
 // conversion to double gives NaN.
 #pragma once
@@ -178,8 +179,10 @@ inline FxScalar fx_scalar(double a) {
 QCD_HD u64 fx_mag(double x) { return fx_bits(x) & ~(1ULL << 63); }
 
 // ------------------------------------------------------------- field access ----
-// Spinor sites in block fixed point ([rhs][12][Vh] pairs of 64-bit integers, exponents [rhs][Vh] in
+// Spinor sites in block fixed point ([rhs][12][Vh] pairs of 64-bit integers, exponents [rhs][2][Vh] in
 // place of the FP16 norms), seen as doubles: for the kernels that convert fields or update vectors.
+QCD_HD size_t eidx(int b, int Vh, int r, int h) { return ((size_t)2 * r + b) * Vh + h; }
+
 template <>
 struct SpinorIO<60> {
   static constexpr int NVEC = 12;
@@ -191,7 +194,7 @@ struct SpinorIO<60> {
       return;
     }
     const longlong2* p = static_cast<const longlong2*>(base);
-    const int e = ldv<LD>(reinterpret_cast<const int*>(ex) + (size_t)r * Vh + h);
+    const int e = ldv<LD>(reinterpret_cast<const int*>(ex) + eidx(b, Vh, r, h));
 #pragma unroll
     for (int c = 0; c < 6; c++) {
       const longlong2 v = ldv<LD>(p + sidx<NVEC>(6 * b + c, Vh, r, h));

@@ -83,7 +83,7 @@ __device__ __forceinline__ FxLimb limb58(i64 v, int down) { return fx_split_bala
 // D_b = T_00 - T_11, P_b = T_10 + T_01, Q_b = i (T_01 - T_10),
 //   xy = D_0 + D_1, xz = Q_0 + Q_1, xt = P_1 - P_0, yz = P_0 + P_1, yt = Q_0 - Q_1, zt = D_1 - D_0,
 // 18 complex products a row and right-hand side instead of 72.
-struct FieldPair {  // a field on even and odd sites in block fixed point
+struct FieldPair {  // a field on even and odd sites in block fixed point, exponents [rhs][2][Vh]
   const longlong2* v[2];
   const int* e[2];
 };
@@ -98,12 +98,17 @@ __global__ void __launch_bounds__(96, 4) clover_coeff_fixed_kernel(Geom g, doubl
   int ex = FX_ZERO;
   if (w.valid) {
     const int *eX = X.e[w.p] + w.h, *eY = Y.e[w.p] + w.h;
-    for (int r = 0; r < nrhs; r++)
-      ex = max(ex, fx_exp_sum(__ldg(eX + (size_t)r * Vh), __ldg(eY + (size_t)r * Vh)));
+    for (int k = 0; k < 2 * nrhs; k++)  // (right-hand side, chiral block)
+      ex = max(ex, fx_exp_sum(__ldg(eX + (size_t)k * Vh), __ldg(eY + (size_t)k * Vh)));
 #pragma unroll 1
     for (int r = 0; r < nrhs; r++) {
-      // units of 2^(eX + eY - 56), brought to the largest and down by lg for the sum over many
-      const int d = min(ex - fx_exp_sum(__ldg(eX + (size_t)r * Vh), __ldg(eY + (size_t)r * Vh)) + lg, 62);
+      // units of 2^(eX + eY - 56) of a block, brought to the largest and down by lg for the sum over many
+      int d[2];
+#pragma unroll
+      for (int b = 0; b < 2; b++) {
+        const size_t o = eidx(b, Vh, r, 0);
+        d[b] = min(ex - fx_exp_sum(__ldg(eX + o), __ldg(eY + o)) + lg, 62);
+      }
       cx<i64> xs[4];
       load_colour(X.v[w.p], Vh, r, w.h, w.row, xs);
       FxLimb xr[4], xi[4], nxr[4];
@@ -123,13 +128,13 @@ __global__ void __launch_bounds__(96, 4) clover_coeff_fixed_kernel(Geom g, doubl
           wr[s] = limb58(ws[s].re, 2);
           wi[s] = limb58(ws[s].im, 2);
         }
-        auto outer = [&](int s, int t) {  // X_s conj(W_t)
+        auto outer = [&](int s, int t) {  // X_s conj(W_t), s and t of one block
           FxSum re = {0, 1LL << 28}, im = {0, 1LL << 28};  // half of fx_value<2>'s unit
           fx_mac(re, xr[s], wr[t]);
           fx_mac(re, xi[s], wi[t]);
           fx_mac(im, xi[s], wr[t]);
           fx_mac(im, nxr[s], wi[t]);
-          return cmk(fx_round_down(fx_value<2>(re), d), fx_round_down(fx_value<2>(im), d));
+          return cmk(fx_round_down(fx_value<2>(re), d[s >> 1]), fx_round_down(fx_value<2>(im), d[s >> 1]));
         };
         cx<i64> D[2], P[2], Q[2];
 #pragma unroll
@@ -326,30 +331,34 @@ template <int MU>
 __device__ __forceinline__ void hop_force_fx(const Geom& g, const Where& w, int j, int nrhs, int lg, const FieldPair& X,
                                              const FieldPair& Y, cx<i64> t[3], int& unit, bool& bad) {
   const int Vh = g.Vh, p = w.p, n = 1 - w.p;
+  // a site's exponent, the larger of its blocks' (the projections add one to the other)
+  auto site_exp = [&](const int* e, int r, int h) { return max(__ldg(e + eidx(0, Vh, r, h)), __ldg(e + eidx(1, Vh, r, h))); };
   int em = FX_ZERO;
-  for (int r = 0; r < nrhs; r++) {
-    const size_t o = (size_t)r * Vh;
-    em = max(em, max(fx_exp_sum(__ldg(X.e[n] + o + j), __ldg(Y.e[p] + o + w.h)),
-                     fx_exp_sum(__ldg(X.e[p] + o + w.h), __ldg(Y.e[n] + o + j))));
-  }
+  for (int r = 0; r < nrhs; r++)
+    em = max(em, max(fx_exp_sum(site_exp(X.e[n], r, j), site_exp(Y.e[p], r, w.h)),
+                     fx_exp_sum(site_exp(X.e[p], r, w.h), site_exp(Y.e[n], r, j))));
 #pragma unroll
   for (int b = 0; b < 3; b++) t[b] = {};
 #pragma unroll 1
   for (int r = 0; r < nrhs; r++) {
-    const size_t o = (size_t)r * Vh;
-    const int dA = min(em - fx_exp_sum(__ldg(X.e[n] + o + j), __ldg(Y.e[p] + o + w.h)) + lg, 62);
-    const int dB = min(em - fx_exp_sum(__ldg(X.e[p] + o + w.h), __ldg(Y.e[n] + o + j)) + lg, 62);
+    const int dA = min(em - fx_exp_sum(site_exp(X.e[n], r, j), site_exp(Y.e[p], r, w.h)) + lg, 62);
+    const int dB = min(em - fx_exp_sum(site_exp(X.e[p], r, w.h), site_exp(Y.e[n], r, j)) + lg, 62);
     // colour `row` of the projected Y(y) and X(y)
     cx<i64> s[12] = {}, hy[6], hx[6];
-    auto colour = [&](const longlong2* f, int h, int a, cx<i64> q[12]) {
+    auto colour = [&](const FieldPair& F, int par, int h, int a, cx<i64> q[12]) {  // in units of the site's exponent
       cx<i64> c4[4];
-      load_colour(f, Vh, r, h, a, c4);
+      load_colour(F.v[par], Vh, r, h, a, c4);
+      const int e0 = __ldg(F.e[par] + eidx(0, Vh, r, h)), e1 = __ldg(F.e[par] + eidx(1, Vh, r, h));
+      const int d0 = min(max(e1 - e0, 0), 63), d1 = min(max(e0 - e1, 0), 63);
 #pragma unroll
-      for (int k = 0; k < 4; k++) q[3 * k] = c4[k];
+      for (int k = 0; k < 4; k++) {
+        const int d = k < 2 ? d0 : d1;
+        q[3 * k] = cmk(c4[k].re >> d, c4[k].im >> d);
+      }
     };
-    colour(Y.v[p], w.h, w.row, s);
+    colour(Y, p, w.h, w.row, s);
     project<MU, -1>(s, hy);
-    colour(X.v[p], w.h, w.row, s);
+    colour(X, p, w.h, w.row, s);
     project<MU, +1>(s, hx);
     FxLimb yr[2], yi[2], xr[2], xi[2];
 #pragma unroll
@@ -362,7 +371,7 @@ __device__ __forceinline__ void hop_force_fx(const Geom& g, const Where& w, int 
 #pragma unroll
     for (int b = 0; b < 3; b++) {
       cx<i64> h[6];
-      colour(X.v[n], j, b, s);
+      colour(X, n, j, b, s);
       project<MU, -1>(s, h);
       FxSum re = {0, 1LL << 28}, im = {0, 1LL << 28};
 #pragma unroll
@@ -375,7 +384,7 @@ __device__ __forceinline__ void hop_force_fx(const Geom& g, const Where& w, int 
       }
       t[b].re += fx_round_down(fx_value<2>(re), dA);
       t[b].im += fx_round_down(fx_value<2>(im), dA);
-      colour(Y.v[n], j, b, s);
+      colour(Y, n, j, b, s);
       project<MU, +1>(s, h);
       re = {0, 1LL << 28};
       im = {0, 1LL << 28};

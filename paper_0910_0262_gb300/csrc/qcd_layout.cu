@@ -109,9 +109,9 @@ __global__ void pack_gauge_kernel(Geom g, const double2* __restrict__ U, double2
 // block's sites through shared memory and its lanes write consecutive 16-byte words: 32^3 x 64, 8 RHS, FP16
 // to canonical 1037 -> 300 us, the time its bytes take (reads staged the same way: 328 -> 410 us).  Sites in
 // shared memory are 13 words apart, so that eight lanes' 16-byte accesses hit distinct banks.  Three threads
-// share a site, four components each: the conversions of block fixed point, some 25 instructions a number,
-// are long chains on a small lattice (4^3 x 8, one thread per site: 10.7 us to canonical, 5.7 us from it; three: 5.9
-// and 4.8 us).
+// share a site, four components each (four threads, to block fixed point: two a chiral block): the conversions of
+// block fixed point, some 25 instructions a number, are long chains on a small lattice (4^3 x 8, one thread per
+// site: 10.7 us to canonical, 5.7 us from it; three: 5.9 and 4.8 us).
 constexpr int LB = 128;         // sites of a block
 constexpr int SITE_WORDS = 13;  // double2 words between sites in shared memory
 
@@ -132,19 +132,19 @@ __global__ void spinor_to_native_kernel(Geom g, const double2* __restrict__ cano
 }
 
 // the same to block fixed point
-__global__ void __launch_bounds__(3 * LB) spinor_to_fixed_kernel(Geom g, const double2* __restrict__ canon, longlong2* nat,
+__global__ void __launch_bounds__(4 * LB) spinor_to_fixed_kernel(Geom g, const double2* __restrict__ canon, longlong2* nat,
                                                                  int* ex, int nrhs) {
-  __shared__ u64 sm[3][LB];
+  __shared__ u64 sm[4][LB];
   const int site = threadIdx.x % LB, part = threadIdx.x / LB;
   const int tid = blockIdx.x * LB + site;  // (eight right-hand sides at most: below 2^31)
   const bool valid = tid < g.Vh * nrhs;
   const int r = tid / g.Vh, h = tid - r * g.Vh;
-  double2 v[4];
+  double2 v[3];
   u64 mx = 0;
   if (valid) {
-    const double2* src = canon + (size_t)tid * 12 + 4 * part;
+    const double2* src = canon + (size_t)tid * 12 + 3 * part;
 #pragma unroll
-    for (int c = 0; c < 4; c++) {
+    for (int c = 0; c < 3; c++) {
       v[c] = src[c];
       mx = max(mx, max(fx_mag(v[c].x), fx_mag(v[c].y)));
     }
@@ -152,12 +152,12 @@ __global__ void __launch_bounds__(3 * LB) spinor_to_fixed_kernel(Geom g, const d
   sm[part][site] = mx;
   __syncthreads();
   if (!valid || !dbg_spinor(g.Vh, r, h)) return;
-  const int e = fx_exponent(max(sm[0][site], max(sm[1][site], sm[2][site])));
+  const int e = fx_exponent(max(mx, sm[part ^ 1][site]));
 #pragma unroll
-  for (int c = 0; c < 4; c++)
-    nat[sidx<12>(4 * part + c, g.Vh, r, h)] =
+  for (int c = 0; c < 3; c++)
+    nat[sidx<12>(3 * part + c, g.Vh, r, h)] =
         make_longlong2(fx_of_double<FX_SPINOR>(v[c].x, e), fx_of_double<FX_SPINOR>(v[c].y, e));
-  if (part == 0) ex[(size_t)r * g.Vh + h] = e;
+  if ((part & 1) == 0) ex[eidx(part >> 1, g.Vh, r, h)] = e;
 }
 
 // components 4 part .. 4 part + 3 of a site as doubles
@@ -169,10 +169,13 @@ __device__ __forceinline__ void load_part(const void* nat, const float* norm, in
   }
   if constexpr (P == 60) {
     const longlong2* p = static_cast<const longlong2*>(nat);
-    const int e = __ldg(reinterpret_cast<const int*>(norm) + (size_t)r * Vh + h);
+    // components 0-5 are those of block 0: part 1 holds two of each block
+    const int* ex = reinterpret_cast<const int*>(norm);
+    const int e0 = __ldg(ex + eidx(part == 2, Vh, r, h)), e1 = __ldg(ex + eidx(part > 0, Vh, r, h));
 #pragma unroll
     for (int c = 0; c < 4; c++) {
       const longlong2 v = __ldg(p + sidx<12>(4 * part + c, Vh, r, h));
+      const int e = c < 2 ? e0 : e1;
       o[c] = make_double2(fx_to_double(v.x, e, FX_SPINOR), fx_to_double(v.y, e, FX_SPINOR));
     }
   } else if constexpr (P == 64) {
@@ -248,7 +251,7 @@ void launch_spinor_to_native(int prec, const Geom& g, const double2* canon, void
   const int B = 128;
   const int nb = nblocks((long long)g.Vh * nrhs, B);
   if (prec == 60)
-    spinor_to_fixed_kernel<<<nblocks((long long)g.Vh * nrhs, LB), 3 * LB, 0, st>>>(
+    spinor_to_fixed_kernel<<<nblocks((long long)g.Vh * nrhs, LB), 4 * LB, 0, st>>>(
         g, canon, static_cast<longlong2*>(nat), reinterpret_cast<int*>(norm), nrhs);
   else if (prec == 64) spinor_to_native_kernel<64><<<nb, B, 0, st>>>(g, canon, nat, norm, nrhs);
   else if (prec == 32) spinor_to_native_kernel<32><<<nb, B, 0, st>>>(g, canon, nat, norm, nrhs);

@@ -1,0 +1,44 @@
+"""Accuracy of the block fixed-point kernels away from links and fields of order one."""
+
+import numpy as np
+import pytest
+
+from oracle import evenodd
+from paper_0910_0262_gb300 import synth
+from gpu_util import require_gpu, to_dev, to_np, rel_l2, rand_eo
+
+pytestmark = pytest.mark.gpu
+KAPPA, CSW = 0.12, 1.0
+
+
+def _context(dims, eps=0.2, seed=3):
+    from paper_0910_0262_gb300.qcd import CloverWilson
+    U = synth.make_problem(dims, eps, seed)[0]
+    op = CloverWilson(dims, -1.0)
+    op.load_gauge(to_dev(U))
+    op.clover_build(KAPPA, CSW)
+    return U, op
+
+
+def chiral_errors(dims=(6, 4, 4, 6), ratio=2.0 ** -20, small=1, n=3):
+    """Relative 2-norm errors of (A x, A^-1 x) per chiral block where one block of x is `ratio` times the other."""
+    U, op = _context(dims)
+    ref = evenodd.SchurOperator(U, KAPPA, CSW, -1.0)
+    x = rand_eo(n, ref.A_ee.shape[0], np.random.default_rng(5))
+    x[:, :, 2 * small:2 * small + 2] *= ratio
+    out = []
+    for o, A in ((4, ref.A_ee), (5, ref.A_oo_inv)):
+        got = to_np(op.dslash(to_dev(x), o, precision=64))
+        want = np.stack([ref.site(A, v) for v in x])
+        out += [rel_l2(got[:, :, 2 * b:2 * b + 2], want[:, :, 2 * b:2 * b + 2]) for b in range(2)]
+    op.close()
+    return out
+
+
+@pytest.mark.parametrize("small", [0, 1])
+@pytest.mark.parametrize("bits", [20, 70])
+def test_chiral_blocks_of_very_different_size(bits, small):
+    """A and A^-1 do not mix the two chiral blocks of a site: each block of the result is right to its own size
+    (a row sums 6 products, as test_operators states for blocks of like size: 1e-15)."""
+    require_gpu()
+    assert max(chiral_errors(ratio=2.0 ** -bits, small=small)) < 1e-15
