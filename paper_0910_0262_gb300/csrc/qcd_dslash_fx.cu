@@ -33,6 +33,9 @@ static_assert(sizeof(FxXch) <= 12 * 32 * sizeof(int4), "the exchange area fits a
 // the neighbour's spins k and p and of the link; neg = -1: (g_mu)_kp is -1 or -i (0: 1 or i); g5 = -1: gamma_5 psi in
 // place of psi, which changes the sign of psi_p (0: psi itself); flip: -w in place of w; psi_k and psi_p are
 // brought down by dk and dp powers of two, from their blocks' units to the sum's.
+// What is cut off to the unit is low by half a unit in the mean (with all hops cut off alike, every component
+// was by up to 2^-54 of its site's bound).  So the hops of y and t form -w and subtract it: in up their halves
+// cancel those of x and z, in low the forward hop's cancel the backward one's.  Exact values stay exact.
 template <bool IMAG, bool BWD>
 __device__ __forceinline__ void hop_fx(const longlong2* sk, const longlong2* sp, const int4* u, int neg, int g5,
                                        bool flip, int dk, int dp, cx<i64> up[3], cx<i64> low[3]) {
@@ -46,8 +49,8 @@ __device__ __forceinline__ void hop_fx(const longlong2* sk, const longlong2* sp,
     x.y >>= dk;
     y.x >>= dp;
     y.y >>= dp;
-    const i64 hr = x.x + (IMAG ? fx_sign(y.y, ~f) : fx_sign(y.x, f));
-    const i64 hi = x.y + (IMAG ? fx_sign(y.x, f) : fx_sign(y.y, f));
+    const i64 hr = IMAG ? x.x + fx_sign(y.y, ~f) : fx_sign(y.x, ~f) - x.x;  // h, or -h of y and t
+    const i64 hi = IMAG ? x.y + fx_sign(y.x, f) : fx_sign(y.y, ~f) - x.y;
     re[b] = fx_split(hr);
     im[b] = fx_split(hi);
   }
@@ -69,11 +72,11 @@ __device__ __forceinline__ void hop_fx(const longlong2* sk, const longlong2* sp,
       x = -x;
       y = -y;
     }
-    up[a].re += x;
-    up[a].im += y;
+    up[a].re += IMAG ? x : -x;
+    up[a].im += IMAG ? y : -y;
     // conj(c) w: c = +-1: +-w; c = +-i: -+i w
-    low[a].re += IMAG ? fx_sign(y, neg) : fx_sign(x, neg);
-    low[a].im += IMAG ? fx_sign(x, ~neg) : fx_sign(y, neg);
+    low[a].re += IMAG ? fx_sign(y, neg) : fx_sign(x, ~neg);
+    low[a].im += IMAG ? fx_sign(x, ~neg) : fx_sign(y, ~neg);
   }
 }
 

@@ -72,13 +72,16 @@ QCD_HD i64 fx_sign(i64 v, int f) { return (v ^ (i64)f) - (i64)f; }
 struct FxSum {
   i64 h, m;
 };
+// an empty sum whose fx_value<K> is rounded to nearest: cut off, values are low by half a unit in the mean
+template <int K>
+QCD_HD FxSum fx_sum() { return FxSum{0, 1LL << (30 - K)}; }
 QCD_HD i64 fx_mad(int a, int b, i64 c) { return c + (i64)a * b; }
 QCD_HD void fx_mac(FxSum& s, FxLimb a, FxLimb b) {
   s.h = fx_mad(a.hi, b.hi, s.h);
   s.m = fx_mad(a.hi, b.lo, s.m);
   s.m = fx_mad(a.lo, b.hi, s.m);
 }
-// the sum in units of 2^(62 - K)
+// the sum in units of 2^(62 - K), rounded if it began as fx_sum<K>
 template <int K>
 QCD_HD i64 fx_value(const FxSum& s) {
   return (i64)((u64)s.h << K) + (s.m >> (31 - K));

@@ -42,7 +42,7 @@ __device__ __forceinline__ i64 fx_scaled(i64 t, int sh) {
 // exponent of a product of members of two groups (marked if either is, whatever the other)
 __device__ __forceinline__ int fx_exp_sum(int a, int b) { return max(a, b) > FX_BIG ? FX_NAN : a + b; }
 
-// t 2^-d, 0 <= d <= 63, rounded to nearest: many such terms are added, and cut off they would add up to a bias
+// t 2^-d, 0 <= d <= 62, rounded to nearest: many such terms are added, and cut off they would add up to a bias
 __device__ __forceinline__ i64 fx_round_down(i64 t, int d) { return (t + ((1LL << d) >> 1)) >> d; }
 
 // exponent of a matrix whose entries are below 2^bits units of 2^unit
@@ -129,7 +129,7 @@ __global__ void __launch_bounds__(96, 4) clover_coeff_fixed_kernel(Geom g, doubl
           wi[s] = limb58(ws[s].im, 2);
         }
         auto outer = [&](int s, int t) {  // X_s conj(W_t), s and t of one block
-          FxSum re = {0, 1LL << 28}, im = {0, 1LL << 28};  // half of fx_value<2>'s unit
+          FxSum re = fx_sum<2>(), im = fx_sum<2>();
           fx_mac(re, xr[s], wr[t]);
           fx_mac(re, xi[s], wi[t]);
           fx_mac(im, xi[s], wr[t]);
@@ -233,11 +233,13 @@ __global__ void __launch_bounds__(96, 7) edge_fixed_kernel(Geom g, const int4* _
     const int4* c = Cfx + (size_t)pl * 9 * V;
     const int e0 = __ldg(eC + pl * V + at), e1 = __ldg(eC + pl * V + next), em = max(e0, e1);
     cx<i64> o[3];
-    fx_row_mul<false, 2>(fx_load_row<false>(c + at, V, w.row), u, Vh, t);
-    fx_row_mul<false, 2>(fx_load_row<false>(u, Vh, w.row), c + next, V, o);
-    const int d0 = min(em - e0, 63), d1 = min(em - e1, 63);
+    fx_row_mul<false, 2, true>(fx_load_row<false>(c + at, V, w.row), u, Vh, t);
+    fx_row_mul<false, 2, true>(fx_load_row<false>(u, Vh, w.row), c + next, V, o);
+    const int d0 = min(em - e0, 62), d1 = min(em - e1, 62);
 #pragma unroll
-    for (int j = 0; j < 3; j++) t[j] = cmk((t[j].re >> d0) + (o[j].re >> d1), (t[j].im >> d0) + (o[j].im >> d1));
+    for (int j = 0; j < 3; j++)
+      t[j] = cmk(fx_round_down(t[j].re, d0) + fx_round_down(o[j].re, d1),
+                 fx_round_down(t[j].im, d0) + fx_round_down(o[j].im, d1));
     unit = em - 56;
     e = fx_group_exp(unit, fx_bits_n(t), em > FX_BIG);
   }
@@ -265,7 +267,7 @@ template <bool DAG, int K>
 __device__ __forceinline__ void row_mul_shared(const FxRow& v, const int4 (*m)[32], int lane, cx<i64> o[3]) {
 #pragma unroll
   for (int j = 0; j < 3; j++) {
-    FxSum re = {}, im = {};
+    FxSum re = fx_sum<K>(), im = fx_sum<K>();
 #pragma unroll
     for (int k = 0; k < 3; k++) {
       const int4 x = m[DAG ? 3 * j + k : 3 * k + j][lane];
@@ -373,7 +375,7 @@ __device__ __forceinline__ void hop_force_fx(const Geom& g, const Where& w, int 
       cx<i64> h[6];
       colour(X, n, j, b, s);
       project<MU, -1>(s, h);
-      FxSum re = {0, 1LL << 28}, im = {0, 1LL << 28};
+      FxSum re = fx_sum<2>(), im = fx_sum<2>();
 #pragma unroll
       for (int k = 0; k < 2; k++) {  // (A^dag)_row,b: conj(h_k,b) hw_k,row
         const FxLimb a = limb58(h[3 * k].re, 3), c = limb58(h[3 * k].im, 3);
@@ -386,8 +388,7 @@ __device__ __forceinline__ void hop_force_fx(const Geom& g, const Where& w, int 
       t[b].im += fx_round_down(fx_value<2>(im), dA);
       colour(Y, n, j, b, s);
       project<MU, +1>(s, h);
-      re = {0, 1LL << 28};
-      im = {0, 1LL << 28};
+      re = im = fx_sum<2>();
 #pragma unroll
       for (int k = 0; k < 2; k++) {  // B_row,b: h'_k,row conj(hw'_k,b)
         const FxLimb a = limb58(h[3 * k].re, 3), c = limb58(h[3 * k].im, 3);
@@ -493,14 +494,14 @@ __global__ void __launch_bounds__(96, 4) link_force_fixed_kernel(Geom g, FxScala
       bad = bad || badh || se > FX_BIG;
       // products of the coefficient (units of 2^(se - 59)) and t 2^up, in units of 2^60
       uh = uh - up + se - 59 + 60;
-      const int um = max(unit, uh), d0 = min(um - unit, 63), d1 = min(um - uh, 63);
+      const int um = max(unit, uh), d0 = min(um - unit, 62), d1 = min(um - uh, 62);
 #pragma unroll
       for (int b = 0; b < 3; b++) {
-        FxSum re = {}, im = {};
+        FxSum re = fx_sum<2>(), im = fx_sum<2>();
         fx_mac(re, sv, fx_split_balanced(fx_scaled(t[b].re, up)));
         fx_mac(im, sv, fx_split_balanced(fx_scaled(t[b].im, up)));
-        G[b].re = (G[b].re >> d0) + (fx_value<2>(re) >> d1);
-        G[b].im = (G[b].im >> d0) + (fx_value<2>(im) >> d1);
+        G[b].re = fx_round_down(G[b].re, d0) + fx_round_down(fx_value<2>(re), d1);
+        G[b].im = fx_round_down(G[b].im, d0) + fx_round_down(fx_value<2>(im), d1);
       }
       unit = um;
     }
@@ -580,7 +581,7 @@ __global__ void __launch_bounds__(96) plaquette_fixed_kernel(Geom g, const int4*
                                         fx_link_at(f, mu, 1, nu, 0, nu), Vh);
     const FxRow b = fx_row_times<false>(fx_load_row<false>(fx_link_at(f, mu, 0, nu, 0, nu), Vh, w.row),
                                         fx_link_at(f, mu, 0, nu, 1, mu), Vh);
-    FxSum t = {0, 1LL << 28};
+    FxSum t = fx_sum<2>();
 #pragma unroll
     for (int j = 0; j < 3; j++) {
       fx_mac(t, a.re[j], b.re[j]);

@@ -39,15 +39,16 @@ __device__ __forceinline__ FxRow fx_load_row(const int4* __restrict__ q, size_t 
   return r;
 }
 
-// v M (DAG: v M^dag) in units of 2^(62 - K) of the products (K = 4: again units of 2^-58)
-template <bool DAG, int K = 4>
+// v M (DAG: v M^dag) in units of 2^(62 - K) of the products (K = 4: again units of 2^-58), cut off, or ROUNDed
+// where the results are added up with one sign
+template <bool DAG, int K = 4, bool ROUND = false>
 __device__ __forceinline__ void fx_row_mul(const FxRow& v, const int4* __restrict__ q, size_t stride, cx<i64> o[3]) {
   FxLimb n[3];  // -Im v for M, -Re v for M^dag
 #pragma unroll
   for (int k = 0; k < 3; k++) n[k] = fx_neg(DAG ? v.re[k] : v.im[k]);
 #pragma unroll
   for (int j = 0; j < 3; j++) {
-    FxSum re = {}, im = {};
+    FxSum re = ROUND ? fx_sum<K>() : FxSum{}, im = ROUND ? fx_sum<K>() : FxSum{};
 #pragma unroll
     for (int k = 0; k < 3; k++) {
       const int4 e = __ldg(q + (size_t)(DAG ? 3 * j + k : 3 * k + j) * stride);

@@ -42,3 +42,21 @@ def test_chiral_blocks_of_very_different_size(bits, small):
     (a row sums 6 products, as test_operators states for blocks of like size: 1e-15)."""
     require_gpu()
     assert max(chiral_errors(ratio=2.0 ** -bits, small=small)) < 1e-15
+
+
+def hop_bias(dims=(6, 10, 2, 18), n=8):
+    """(mean signed error of D_eo x over all components, 2^-57 times the mean of a site's bound 2^e)."""
+    U, op = _context(dims)
+    ref = evenodd.SchurOperator(U, KAPPA, CSW, -1.0)
+    x = rand_eo(n, ref.A_ee.shape[0], np.random.default_rng(21))
+    err = to_np(op.dslash(to_dev(x), 0, precision=64)) - np.stack([ref.D_eo(v) for v in x])
+    op.close()
+    bound = 2.0 ** np.ceil(np.log2(np.maximum(np.abs(x.real), np.abs(x.imag)).max(axis=(2, 3)))).mean()
+    return max(abs(err.real.mean()), abs(err.imag.mean())), bound * 2.0 ** -57
+
+
+def test_hops_are_rounded_without_bias():
+    """Values cut off instead of rounded would move every component down by up to 2^-54 of a site's bound."""
+    require_gpu()
+    got, most = hop_bias()
+    assert got < most
