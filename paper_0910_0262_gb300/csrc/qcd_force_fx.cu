@@ -34,6 +34,18 @@ __device__ __forceinline__ int fx_bits_n(const cx<i64> (&t)[N]) {
   return 64 - fx_clz(o);
 }
 
+// Before another term is added to a sum over right-hand sides: a sum that has grown to 2^most units is halved,
+// and *down, the powers of two by which its unit is above the terms', goes up.  (The unit follows the sum's
+// size: one chosen beforehand for n terms of the largest size costs log2(n) bits that sums of random signs do
+// not use, 64 right-hand sides 1.6e-15 of the force against the FP64 kernels' 3.8e-16.)
+template <int N>
+__device__ __forceinline__ void fx_make_room(cx<i64> (&t)[N], int most, int* down) {
+  if (fx_bits_n(t) <= most) return;
+#pragma unroll
+  for (int k = 0; k < N; k++) t[k] = cmk((t[k].re + 1) >> 1, (t[k].im + 1) >> 1);
+  *down += 1;
+}
+
 // t 2^sh, rounded to nearest where sh < 0
 __device__ __forceinline__ i64 fx_scaled(i64 t, int sh) {
   return sh >= 0 ? (i64)((u64)t << (sh < 63 ? sh : 63)) : fx_down_rn(t, -sh);
@@ -88,26 +100,29 @@ struct FieldPair {  // a field on even and odd sites in block fixed point, expon
   const int* e[2];
 };
 
-__global__ void __launch_bounds__(96, 4) clover_coeff_fixed_kernel(Geom g, double f_even, double f_odd, int nrhs, int lg,
+__global__ void __launch_bounds__(96, 4) clover_coeff_fixed_kernel(Geom g, double f_even, double f_odd, int nrhs,
                                                                 FieldPair X, FieldPair Y, double2* Cbuf) {
   __shared__ i64 sm[3][36][32];
+  __shared__ int sd[3][32];
   const Where w = where(g);
   const int Vh = g.Vh;
   const size_t V = 2 * (size_t)Vh;
-  cx<i64> S[6][3] = {};
-  int ex = FX_ZERO;
+  cx<i64> S[18] = {};  // [plane][colour]
+  int ex = FX_ZERO, down = 0;
   if (w.valid) {
     const int *eX = X.e[w.p] + w.h, *eY = Y.e[w.p] + w.h;
     for (int k = 0; k < 2 * nrhs; k++)  // (right-hand side, chiral block)
       ex = max(ex, fx_exp_sum(__ldg(eX + (size_t)k * Vh), __ldg(eY + (size_t)k * Vh)));
 #pragma unroll 1
     for (int r = 0; r < nrhs; r++) {
-      // units of 2^(eX + eY - 56) of a block, brought to the largest and down by lg for the sum over many
+      // units of 2^(eX + eY - 56) of a block, brought to the largest's and the sum's; a term is below 2^59 units of
+      // the former, so the sum stays below 2^60
+      if (r > 0) fx_make_room(S, 59, &down);
       int d[2];
 #pragma unroll
       for (int b = 0; b < 2; b++) {
         const size_t o = eidx(b, Vh, r, 0);
-        d[b] = min(ex - fx_exp_sum(__ldg(eX + o), __ldg(eY + o)) + lg, 62);
+        d[b] = min(ex - fx_exp_sum(__ldg(eX + o), __ldg(eY + o)) + down, 62);
       }
       cx<i64> xs[4];
       load_colour(X.v[w.p], Vh, r, w.h, w.row, xs);
@@ -144,27 +159,29 @@ __global__ void __launch_bounds__(96, 4) clover_coeff_fixed_kernel(Geom g, doubl
           P[b] = t10 + t01;
           Q[b] = times_i(t01 - t10);
         }
-        S[0][c] = S[0][c] + D[0] + D[1];
-        S[1][c] = S[1][c] + Q[0] + Q[1];
-        S[2][c] = S[2][c] + P[1] - P[0];
-        S[3][c] = S[3][c] + P[0] + P[1];
-        S[4][c] = S[4][c] + Q[0] - Q[1];
-        S[5][c] = S[5][c] + D[1] - D[0];
+        S[c] = S[c] + D[0] + D[1];
+        S[3 + c] = S[3 + c] + Q[0] + Q[1];
+        S[6 + c] = S[6 + c] + P[1] - P[0];
+        S[9 + c] = S[9 + c] + P[0] + P[1];
+        S[12 + c] = S[12 + c] + Q[0] - Q[1];
+        S[15 + c] = S[15 + c] + D[1] - D[0];
       }
     }
   }
+  sd[w.row][w.lane] = down;
+  __syncthreads();
+  const int most = max(sd[0][w.lane], max(sd[1][w.lane], sd[2][w.lane]));
 #pragma unroll
-  for (int pl = 0; pl < 6; pl++)
-#pragma unroll
-    for (int c = 0; c < 3; c++) {
-      sm[w.row][6 * pl + 2 * c][w.lane] = S[pl][c].re;
-      sm[w.row][6 * pl + 2 * c + 1][w.lane] = S[pl][c].im;
-    }
+  for (int k = 0; k < 18; k++) {
+    S[k] = cmk(fx_round_down(S[k].re, min(most - down, 62)), fx_round_down(S[k].im, min(most - down, 62)));
+    sm[w.row][2 * k][w.lane] = S[k].re;
+    sm[w.row][2 * k + 1][w.lane] = S[k].im;
+  }
   __syncthreads();
   if (!w.valid) return;
   const double f = w.p ? f_odd : f_even;
   // |X W| < 2^(eX + eY): a product in units of 2^(-58 - 58 + 60)
-  const int e = ex > FX_BIG ? FX_NAN : ex + lg - 56;
+  const int e = ex > FX_BIG ? FX_NAN : ex + most - 56;
 #pragma unroll
   for (int pl = 0; pl < 6; pl++) {
     const i64 tr = sm[0][6 * pl][w.lane] + sm[1][6 * pl + 2][w.lane] + sm[2][6 * pl + 4][w.lane];
@@ -173,10 +190,10 @@ __global__ void __launch_bounds__(96, 4) clover_coeff_fixed_kernel(Geom g, doubl
     for (int c = 0; c < 3; c++) {
       double2 o;
       if (c == w.row) {  // -i f (2 Re S_aa - 2/3 tr)
-        o = make_double2(0.0, -f * (2.0 / 3.0) * fx_to_double(3 * S[pl][c].re - tr, e, 0));
+        o = make_double2(0.0, -f * (2.0 / 3.0) * fx_to_double(3 * S[3 * pl + c].re - tr, e, 0));
       } else {  // H = S_ac + conj(S_ca), -i f H
-        const double hr = fx_to_double(S[pl][c].re + sm[c][6 * pl + 2 * w.row][w.lane], e, 0);
-        const double hi = fx_to_double(S[pl][c].im - sm[c][6 * pl + 2 * w.row + 1][w.lane], e, 0);
+        const double hr = fx_to_double(S[3 * pl + c].re + sm[c][6 * pl + 2 * w.row][w.lane], e, 0);
+        const double hi = fx_to_double(S[3 * pl + c].im - sm[c][6 * pl + 2 * w.row + 1][w.lane], e, 0);
         o = make_double2(f * hi, -f * hr);
       }
       q[(size_t)c * V] = o;
@@ -330,7 +347,7 @@ __device__ __forceinline__ void store_ta(const Geom& g, const Where& w, const in
 // (1 -+ g) is twice a projector, so A = sum_k h_k hw_k^dag over its two rows k with h, hw the projected half
 // spinors of X(y + l) and of Y(y), and likewise B: two outer products each instead of four.
 template <int MU>
-__device__ __forceinline__ void hop_force_fx(const Geom& g, const Where& w, int j, int nrhs, int lg, const FieldPair& X,
+__device__ __forceinline__ void hop_force_fx(const Geom& g, const Where& w, int j, int nrhs, const FieldPair& X,
                                              const FieldPair& Y, cx<i64> t[3], int& unit, bool& bad) {
   const int Vh = g.Vh, p = w.p, n = 1 - w.p;
   // a site's exponent, the larger of its blocks' (the projections add one to the other)
@@ -341,10 +358,12 @@ __device__ __forceinline__ void hop_force_fx(const Geom& g, const Where& w, int 
                      fx_exp_sum(site_exp(X.e[p], r, w.h), site_exp(Y.e[n], r, j))));
 #pragma unroll
   for (int b = 0; b < 3; b++) t[b] = {};
+  int down = 0;
 #pragma unroll 1
   for (int r = 0; r < nrhs; r++) {
-    const int dA = min(em - fx_exp_sum(site_exp(X.e[n], r, j), site_exp(Y.e[p], r, w.h)) + lg, 62);
-    const int dB = min(em - fx_exp_sum(site_exp(X.e[p], r, w.h), site_exp(Y.e[n], r, j)) + lg, 62);
+    if (r > 0) fx_make_room(*reinterpret_cast<cx<i64>(*)[3]>(t), 60, &down);  // a right-hand side's A^dag + B: below 2^59
+    const int dA = min(em - fx_exp_sum(site_exp(X.e[n], r, j), site_exp(Y.e[p], r, w.h)) + down, 62);
+    const int dB = min(em - fx_exp_sum(site_exp(X.e[p], r, w.h), site_exp(Y.e[n], r, j)) + down, 62);
     // colour `row` of the projected Y(y) and X(y)
     cx<i64> s[12] = {}, hy[6], hx[6];
     auto colour = [&](const FieldPair& F, int par, int h, int a, cx<i64> q[12]) {  // in units of the site's exponent
@@ -401,8 +420,8 @@ __device__ __forceinline__ void hop_force_fx(const Geom& g, const Where& w, int 
       t[b].im += fx_round_down(fx_value<2>(im), dB);
     }
   }
-  // |h| < 2^61, brought to 2^58: products in units of 2^(2 (3 - 60) + 60), down by lg
-  unit = em - 54 + lg;
+  // |h| < 2^61, brought to 2^58: products in units of 2^(2 (3 - 60) + 60)
+  unit = em - 54 + down;
   bad = em > FX_BIG;
 }
 
@@ -411,7 +430,7 @@ __device__ __forceinline__ void hop_force_fx(const Geom& g, const Where& w, int 
 //   G += U_o(y) U_l(y+o) E_o(y+l)^dag - E_o(y) U_l(y+o) U_o(y+l)^dag
 //      + U_o(y-o)^dag U_l(y-o) E_o(y-o+l) - E_o(y-o)^dag U_l(y-o) U_o(y-o+l),
 // E_o the insertion into U_o in the plane of l and o.
-__global__ void __launch_bounds__(96, 4) link_force_fixed_kernel(Geom g, FxScalar hop, FxScalar hop_bc, int nrhs, int lg,
+__global__ void __launch_bounds__(96, 4) link_force_fixed_kernel(Geom g, FxScalar hop, FxScalar hop_bc, int nrhs,
                                                               const int4* __restrict__ gfx, FieldPair X, FieldPair Y,
                                                               const int4* __restrict__ Efx, const int* __restrict__ eE,
                                                               double2* out, int gradient) {
@@ -482,10 +501,10 @@ __global__ void __launch_bounds__(96, 4) link_force_fixed_kernel(Geom g, FxScala
       bool badh = false;
       const int j = fx_half_at(f, lam, 1, (lam + 1) & 3, 0);
       switch (lam) {
-        case 0: hop_force_fx<0>(g, w, j, nrhs, lg, X, Y, t, uh, badh); break;
-        case 1: hop_force_fx<1>(g, w, j, nrhs, lg, X, Y, t, uh, badh); break;
-        case 2: hop_force_fx<2>(g, w, j, nrhs, lg, X, Y, t, uh, badh); break;
-        default: hop_force_fx<3>(g, w, j, nrhs, lg, X, Y, t, uh, badh); break;
+        case 0: hop_force_fx<0>(g, w, j, nrhs, X, Y, t, uh, badh); break;
+        case 1: hop_force_fx<1>(g, w, j, nrhs, X, Y, t, uh, badh); break;
+        case 2: hop_force_fx<2>(g, w, j, nrhs, X, Y, t, uh, badh); break;
+        default: hop_force_fx<3>(g, w, j, nrhs, X, Y, t, uh, badh); break;
       }
       const bool edge = lam == 3 && s.t == g.T - 1;
       const FxLimb sv = edge ? hop_bc.v : hop.v;
@@ -601,14 +620,6 @@ FieldPair pair_of(const void* even, const void* odd, const float* even_e, const 
                    {reinterpret_cast<const int*>(even_e), reinterpret_cast<const int*>(odd_e)}};
 }
 
-// powers of two by which the terms of a sum over nrhs right-hand sides (each below 2^59) are brought down, so
-// that it stays below 2^60.6
-int sum_bits(int nrhs) {
-  int l = 0;
-  while ((1 << l) < nrhs) l++;
-  return l > 1 ? l - 1 : 0;
-}
-
 }  // namespace
 
 // bytes of a fixed matrix field set: n fields of V matrices, then their exponents
@@ -619,7 +630,7 @@ void launch_force_coeff_fixed(const Geom& g, double kappa, double csw, int nrhs,
                               const float* yo, double2* Cbuf, cudaStream_t st) {
   g_kernel_launches += 1;
   const double f = kappa * csw / 4.0;
-  clover_coeff_fixed_kernel<<<rows_grid(g, 1), 96, 0, st>>>(g, f, f * kappa * kappa, nrhs, sum_bits(nrhs),
+  clover_coeff_fixed_kernel<<<rows_grid(g, 1), 96, 0, st>>>(g, f, f * kappa * kappa, nrhs,
                                                            pair_of(Xe, Xo, xe, xo), pair_of(Ye, Yo, ye, yo), Cbuf);
 }
 
@@ -639,7 +650,7 @@ void launch_force_links_fixed(const Geom& g, double kappa, int nrhs, const void*
   const int4* e = static_cast<const int4*>(Efx);
   const double hop = 2.0 * kappa * kappa;
   link_force_fixed_kernel<<<rows_grid(g, 4), 96, 0, st>>>(
-      g, fx_scalar(hop), fx_scalar(hop * g.t_bc), nrhs, sum_bits(nrhs), static_cast<const int4*>(gfx),
+      g, fx_scalar(hop), fx_scalar(hop * g.t_bc), nrhs, static_cast<const int4*>(gfx),
       pair_of(Xe, Xo, xe, xo), pair_of(Ye, Yo, ye, yo), e, reinterpret_cast<const int*>(e + 12 * 9 * 2 * (size_t)g.Vh), out,
       gradient ? 1 : 0);
 }
