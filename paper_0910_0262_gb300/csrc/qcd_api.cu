@@ -134,6 +134,8 @@ struct qcd_ctx {
   // the FP64 operators' operands in block fixed point (qcd_fixed.cuh), for near-unitary links: null where
   // they could not be allocated or on t-slabs, which keep the FP64 kernels
   void* gfx = nullptr;
+  unsigned char* far = nullptr;  // in gfx's allocation: [2][4][Vh] links far from one, then weakF, weakG [2][Vh]
+  int weak = 0;                  // bits 0, 1: some site is marked in weakF, weakG
   FxClover cfx{};
   bool fx_links = false;
   // clover
@@ -376,6 +378,13 @@ const int* clover_exps(const qcd_ctx* c, bool inverse) { return inverse ? c->cfx
 // not near-unitary (smeared or scaled ones) and t-slabs keep FP64.
 int fp64_rep(const qcd_ctx* c, bool with_clover) {
   return c->gfx && c->fx_links && (!with_clover || c->cfx.A_even) ? 60 : 64;
+}
+
+// the block fixed-point links for field strength and gauge force (null: not near-unitary, or none kept)
+FxLinks fx_links(const qcd_ctx* c) {
+  if (!c->fx_links) return FxLinks{};
+  const size_t V = 2 * (size_t)c->g.Vh;
+  return FxLinks{c->gfx, c->weak & 1 ? c->far + 4 * V : nullptr, c->weak & 2 ? c->far + 5 * V : nullptr};
 }
 
 DslashArgs base_args(const qcd_ctx* c, int prec, int parity, int nrhs) {
@@ -699,7 +708,8 @@ qcd_status qcd_load_gauge(qcd_ctx* c, const double* U, int on_device, int flags)
     CUDA_TRY(cudaMalloc(&c->g64, canon_bytes));
     CUDA_TRY(cudaMalloc(&c->g32, n_links * 9 * sizeof(float2)));
     CUDA_TRY(cudaMalloc(&c->g16, n_links * 9 * sizeof(uint32_t)));
-    if (!c->slab) try_alloc(&c->gfx, n_links * 9 * sizeof(int4));
+    if (!c->slab && try_alloc(&c->gfx, n_links * 9 * sizeof(int4) + n_links + n_links / 2))
+      c->far = reinterpret_cast<unsigned char*>(static_cast<int4*>(c->gfx) + n_links * 9);
   }
   // a t-slab keeps the whole extended field (its clover build reads it); the slab's own links start
   // two time slices in
@@ -722,11 +732,13 @@ qcd_status qcd_load_gauge(qcd_ctx* c, const double* U, int on_device, int flags)
   // looked for non-finite values took 66 us beside the packing's 186)
   if (c->slab) launch_check_finite(reinterpret_cast<const double*>(src), in_links * 18, c->flags + 1, c->st);
   launch_pack_gauge(g, src + (c->slab ? (size_t)2 * g.XYZ * 4 * 9 : 0), c->g64, c->g32, c->recon, c->g16, c->recon,
-                    c->gfx, c->flags + 2, c->slab ? nullptr : c->flags + 1, c->st);
+                    c->gfx, c->far, c->flags + 2, c->slab ? nullptr : c->flags + 1, c->st);
+  if (c->gfx) launch_weak_sites(g, c->far, c->far + n_links, c->far + n_links + n_links / 4, c->flags + 3, c->st);
   CUDA_TRY(cudaMemcpyAsync(c->h_flags, c->flags, 4 * sizeof(int), cudaMemcpyDeviceToHost, c->st));
   if ((s = sync_and_check(c, "load_gauge"))) return s;
   c->have_clover = false;
   c->fx_links = c->gfx && !c->h_flags[2];
+  c->weak = c->h_flags[3];
   if (c->h_flags[1]) {
     c->have_gauge = false;
     return fail(QCD_ERR_NAN, "gauge field holds a non-finite value");
@@ -768,7 +780,7 @@ qcd_status qcd_clover_build(qcd_ctx* c, double kappa, double csw) {
     // 6 planes x 10 products of 3x3 complex matrices per site (two leaves share a product), plus
     // the two inversions
     ProfScope ps(c, "clover_build", 0, 2.0 * g.Vh * (60 * 216.0 + 2 * 1000.0));
-    launch_clover_build(g, c->g64, c->fx_links ? c->gfx : nullptr, kappa, csw, c->A64, c->Ainv64, c->A32, c->Ainv32, c->A16, c->Ainv16, work,
+    launch_clover_build(g, c->g64, fx_links(c), kappa, csw, c->A64, c->Ainv64, c->A32, c->Ainv32, c->A16, c->Ainv16, work,
                         c->logdet, c->flags, c->fx_links ? c->cfx : FxClover{}, c->st);
   }
   CUDA_TRY(cudaMemcpyAsync(c->h_flags, c->flags, 4 * sizeof(int), cudaMemcpyDeviceToHost, c->st));
@@ -1783,8 +1795,10 @@ qcd_status qcd_gauge_force(qcd_ctx* c, double* F, double beta, int flags) {
     ProfScope ps(c, "gauge_force", 4 * V * (18 * 144.0 + 144.0 * ((flags & QCD_FORCE_ACCUMULATE) ? 2 : 1)),
                  4 * V * 13 * 198.0);
     const bool grad = (flags & QCD_FORCE_GRADIENT) != 0, add = (flags & QCD_FORCE_ACCUMULATE) != 0;
-    if (c->fx_links) launch_gauge_force_fixed(c->g, beta, c->gfx, reinterpret_cast<double2*>(F), grad, add, c->st);
-    else launch_gauge_force(c->g, beta, c->g64, reinterpret_cast<double2*>(F), grad, add, c->st);
+    const FxLinks fl = fx_links(c);
+    double2* out = reinterpret_cast<double2*>(F);
+    if (fl.U) launch_gauge_force_fixed(c->g, beta, fl.U, fl.weakG, out, grad, add, c->st);
+    if (!fl.U || fl.weakG) launch_gauge_force(c->g, beta, c->g64, fl.weakG, out, grad, add, c->st);
   }
   cudaError_t e = cudaGetLastError();
   if (e != cudaSuccess) return fail(QCD_ERR_CUDA, "gauge_force launch: %s", cudaGetErrorString(e));

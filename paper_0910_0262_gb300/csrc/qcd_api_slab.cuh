@@ -59,9 +59,9 @@ qcd_status slab_clover_build(qcd_ctx* c, double kappa, double csw, void* work) {
   }
   {
     ProfScope ps(c, "clover_build", 0, 2.0 * ge.Vh * (60 * 216.0 + 2 * 1000.0));
-    launch_pack_gauge(ge, c->U_ext, c->ext_g64, nullptr, 0, nullptr, 0, nullptr, nullptr, nullptr, c->st);
+    launch_pack_gauge(ge, c->U_ext, c->ext_g64, nullptr, 0, nullptr, 0, nullptr, nullptr, nullptr, nullptr, c->st);
     // every site of the extended lattice (the two outermost slices wrap and are discarded)
-    launch_clover_build(ge, c->ext_g64, nullptr, kappa, csw, c->ext_A64, c->ext_Ainv64, c->ext_A32, c->ext_Ainv32,
+    launch_clover_build(ge, c->ext_g64, FxLinks{}, kappa, csw, c->ext_A64, c->ext_Ainv64, c->ext_A32, c->ext_Ainv32,
                         c->ext_A16, c->ext_Ainv16, work, c->ext_logdet, c->flags, FxClover{}, c->st);
   }
   qcd_status s;

@@ -223,13 +223,16 @@ __device__ __forceinline__ void plane_of(int pl, int& mu, int& nu) {
 // F_{mu nu} from the block fixed-point links (the expressions of field_strength, leaf by leaf along a row:
 // 11 products of a row instead of 10 of matrices).  Three warps per 32 sites of one parity, a row of F each;
 // blockIdx.y is the plane.
-__global__ void __launch_bounds__(96) field_strength_fixed_kernel(Geom g, const int4* __restrict__ gfx, double2* Fbuf) {
+// (6 blocks per SM: 1.6% of a build at 24^3 x 32 over the compiler's own choice, 5 blocks lose 5%)
+__global__ void __launch_bounds__(96, 6) field_strength_fixed_kernel(Geom g, const int4* __restrict__ gfx,
+                                                                     const unsigned char* __restrict__ weak, double2* Fbuf) {
   __shared__ i64 sm[3][6][32];
   const int lane = threadIdx.x & 31, row = threadIdx.x >> 5;
   const int nb = (g.Vh + 31) / 32, p = (int)blockIdx.x / nb, h = ((int)blockIdx.x - p * nb) * 32 + lane;
-  const bool valid = h < g.Vh;
   const int Vh = g.Vh;
   const size_t V = 2 * (size_t)Vh;
+  const bool valid = h < Vh && !(weak && (weak[(size_t)p * Vh + h] >> blockIdx.y & 1));
+  if (weak && __syncthreads_or(valid) == 0) return;
   int mu, nu;
   plane_of(blockIdx.y, mu, nu);
   cx<i64> M[3] = {};
@@ -239,24 +242,26 @@ __global__ void __launch_bounds__(96) field_strength_fixed_kernel(Geom g, const 
     auto at = [&](int sm_, int sn, int dir) { return fx_link_at(f, mu, sm_, nu, sn, dir); };
     cx<i64> t[3];
     {  // U_mu(x) [U_nu(x+mu) U_mu(x+nu)^dag U_nu(x)^dag - U_nu(x+mu-nu)^dag U_mu(x-nu)^dag U_nu(x-nu)]
-      const FxRow r = fx_load_row<false>(at(0, 0, mu), Vh, row);
+      const FxRow r = fx_load_row_fine<false>(at(0, 0, mu), Vh, row);
       fx_row_mul<true>(fx_row_times<true>(fx_row_times<false>(r, at(1, 0, nu), Vh), at(0, 1, mu), Vh), at(0, 0, nu), Vh, M);
       fx_row_mul<false>(fx_row_times<true>(fx_row_times<true>(r, at(1, -1, nu), Vh), at(0, -1, mu), Vh), at(0, -1, nu), Vh,
                         t);
+      // from here on in units of 2^-60
 #pragma unroll
-      for (int j = 0; j < 3; j++) M[j] = M[j] - t[j];
+      for (int j = 0; j < 3; j++) M[j] = cmk((M[j].re - t[j].re) >> 1, (M[j].im - t[j].im) >> 1);
     }
     {  // [U_nu(x) U_mu(x-mu+nu)^dag U_nu(x-mu)^dag - U_nu(x-nu)^dag U_mu(x-mu-nu)^dag U_nu(x-mu-nu)] U_mu(x-mu)
       cx<i64> u[3];
-      fx_row_mul<true>(fx_row_times<true>(fx_load_row<false>(at(0, 0, nu), Vh, row), at(-1, 1, mu), Vh), at(-1, 0, nu), Vh,
+      fx_row_mul<true>(fx_row_times<true>(fx_load_row_fine<false>(at(0, 0, nu), Vh, row), at(-1, 1, mu), Vh), at(-1, 0, nu), Vh,
                        t);
-      fx_row_mul<false>(fx_row_times<true>(fx_load_row<true>(at(0, -1, nu), Vh, row), at(-1, -1, mu), Vh), at(-1, -1, nu),
+      fx_row_mul<false>(fx_row_times<true>(fx_load_row_fine<true>(at(0, -1, nu), Vh, row), at(-1, -1, mu), Vh), at(-1, -1, nu),
                         Vh, u);
 #pragma unroll
-      for (int j = 0; j < 3; j++) t[j] = t[j] - u[j];
+      for (int j = 0; j < 3; j++) t[j] = cmk((t[j].re - u[j].re) >> 1, (t[j].im - u[j].im) >> 1);
       fx_row_mul<false>(fx_row(t), at(-1, 0, mu), Vh, u);
+      // four leaves, entries of magnitude <= 4: in units of 2^-58, so that the sums below stay in range
 #pragma unroll
-      for (int j = 0; j < 3; j++) M[j] = M[j] + u[j];
+      for (int j = 0; j < 3; j++) M[j] = cmk((M[j].re + u[j].re + 2) >> 2, (M[j].im + u[j].im + 2) >> 2);
     }
   }
 #pragma unroll
@@ -273,7 +278,7 @@ __global__ void __launch_bounds__(96) field_strength_fixed_kernel(Geom g, const 
   for (int j = 0; j < 3; j++) {
     double re, im = 0.0;
     if (j == row) {
-      re = fx_to_double_in_range(3 * M[j].im - tr, -FX_LINK - 2) * (1.0 / 3.0);
+      re = fx_to_double_in_range(2 * M[j].im - (tr - M[j].im), -FX_LINK - 2) * (1.0 / 3.0);
     } else {
       re = fx_to_double_in_range(M[j].im + sm[j][2 * row + 1][lane], -FX_LINK - 3);
       im = fx_to_double_in_range(sm[j][2 * row][lane] - M[j].re, -FX_LINK - 3);
@@ -282,8 +287,10 @@ __global__ void __launch_bounds__(96) field_strength_fixed_kernel(Geom g, const 
   }
 }
 
-// the same from the FP64 links (not near-unitary ones, t-slabs), one (site, plane) per thread
-__global__ void __launch_bounds__(128) field_strength_kernel(Geom g, const double2* __restrict__ g64, double2* Fbuf) {
+// the same from the FP64 links (not near-unitary ones, t-slabs; with weak, the (site, plane) pairs marked there), one
+// (site, plane) per thread
+__global__ void __launch_bounds__(128) field_strength_kernel(Geom g, const double2* __restrict__ g64,
+                                                             const unsigned char* __restrict__ weak, double2* Fbuf) {
   const int V = 2 * g.Vh;
   const long long tid = (long long)blockIdx.x * blockDim.x + threadIdx.x;
   if (tid >= 6LL * V) return;
@@ -291,8 +298,9 @@ __global__ void __launch_bounds__(128) field_strength_kernel(Geom g, const doubl
   const int PM[6] = {0, 0, 0, 1, 1, 2}, PN[6] = {1, 2, 3, 2, 3, 3};
   int c[4];
   lattice_coords(g, i, c);
-  const M3 F = field_strength(g, g64, c, PM[pl], PN[pl]);
   const int p = (c[0] + c[1] + c[2] + c[3]) & 1;
+  if (weak && !(weak[(size_t)p * g.Vh + (i >> 1)] >> pl & 1)) return;
+  const M3 F = field_strength(g, g64, c, PM[pl], PN[pl]);
   double2* q = Fbuf + (size_t)pl * 9 * V + (size_t)p * g.Vh + (i >> 1);
 #pragma unroll
   for (int k = 0; k < 9; k++) q[(size_t)k * V] = make_double2(F.e[k].re, F.e[k].im);
@@ -378,20 +386,20 @@ __global__ void clover_apply_kernel(Geom g, const void* clov, const void* in, co
 
 }  // namespace
 
-void launch_clover_build(const Geom& g, const void* g64, const void* gfx, double kappa, double csw, void* A64, void* Ainv64, void* A32,
+void launch_clover_build(const Geom& g, const void* g64, const FxLinks& fl, double kappa, double csw, void* A64, void* Ainv64, void* A32,
                          void* Ainv32, void* A16, void* Ainv16, void* work, double* logdet, int* notposdef,
                          const FxClover& fx, cudaStream_t st) {
   const int B = 128;
   const long long V = 2LL * g.Vh;
   // F per (site, plane), then one chiral block per thread
-  g_kernel_launches += 2;
+  g_kernel_launches += fl.U && fl.weakF ? 3 : 2;
   // (block fixed point against FP64: 24^3 x 32 5.23 -> 1.33 ms, 16^4 805 -> 200 us; 7 or 8 blocks per SM in
   // place of 6 change nothing)
-  if (gfx)
-    field_strength_fixed_kernel<<<dim3(2 * ((g.Vh + 31) / 32), 6), 96, 0, st>>>(g, static_cast<const int4*>(gfx),
+  if (fl.U)
+    field_strength_fixed_kernel<<<dim3(2 * ((g.Vh + 31) / 32), 6), 96, 0, st>>>(g, static_cast<const int4*>(fl.U), fl.weakF,
                                                                                 static_cast<double2*>(work));
-  else
-    field_strength_kernel<<<(int)((6 * V + B - 1) / B), B, 0, st>>>(g, static_cast<const double2*>(g64),
+  if (!fl.U || fl.weakF)
+    field_strength_kernel<<<(int)((6 * V + B - 1) / B), B, 0, st>>>(g, static_cast<const double2*>(g64), fl.weakF,
                                                                       static_cast<double2*>(work));
   clover_assemble_kernel<<<(int)((2 * V + B - 1) / B), B, 0, st>>>(
       g, static_cast<const double2*>(work), kappa, csw, static_cast<double2*>(A64), static_cast<double2*>(Ainv64),

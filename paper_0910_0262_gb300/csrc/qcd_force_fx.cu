@@ -307,13 +307,13 @@ __device__ __forceinline__ void store_ta(const Geom& g, const Where& w, const in
   x.e[w.row][w.lane] = e;
   __syncthreads();
   e = fx_max3(x.e, w.lane);
-  const int sh = e > FX_BIG || e <= FX_ZERO ? -63 : unit - e + 58;
+  const int sh = e > FX_BIG || e <= FX_ZERO ? -63 : unit - e + 61;
 #pragma unroll
   for (int j = 0; j < 3; j++)
     x.m[3 * w.row + j][w.lane] = fx_pack2(fx_split_balanced(fx_scaled(t[j].re, sh)), fx_split_balanced(fx_scaled(t[j].im, sh)));
   __syncthreads();
   cx<i64> M[3] = {};
-  // units of 2^(e - 58 - 58 + 60), |M| < 2^57.4
+  // units of 2^(e - 61 - 58 + 60), |M| < 2^60.4
   if (w.valid) row_mul_shared<DAG, 2>(fx_load_row<false>(u, g.Vh, w.row), x.m, w.lane, M);
 #pragma unroll
   for (int j = 0; j < 3; j++) {
@@ -322,14 +322,14 @@ __device__ __forceinline__ void store_ta(const Geom& g, const Where& w, const in
   }
   __syncthreads();
   if (!w.valid) return;
-  const int em = e > FX_BIG ? FX_NAN : (e <= FX_ZERO ? 0 : e - 56);
+  const int em = e > FX_BIG ? FX_NAN : (e <= FX_ZERO ? 0 : e - 59);
   const i64 tr = x.v[0][1][w.lane] + x.v[1][3][w.lane] + x.v[2][5][w.lane];
   // (M - M^dag) / 2 less its trace / 3
 #pragma unroll
   for (int j = 0; j < 3; j++) {
     double2 o;
     if (j == w.row) {
-      o = make_double2(0.0, f * (1.0 / 3.0) * fx_to_double(3 * M[j].im - tr, em, 0));
+      o = make_double2(0.0, f * (1.0 / 3.0) * fx_to_double(2 * M[j].im - (tr - M[j].im), em, 0));
     } else {
       o.x = 0.5 * f * fx_to_double(M[j].re - x.v[j][2 * w.row][w.lane], em, 0);
       o.y = 0.5 * f * fx_to_double(M[j].im + x.v[j][2 * w.row + 1][w.lane], em, 0);
@@ -541,11 +541,16 @@ __global__ void __launch_bounds__(96, 4) link_force_fixed_kernel(Geom g, FxScala
 //   A = sum_o U_o(y+l) U_l(y+o)^dag U_o(y)^dag + U_o(y+l-o)^dag U_l(y-o)^dag U_o(y-o),
 // G = -(beta/3) A^dag, F = (beta/6) P_TA(U A)
 __global__ void __launch_bounds__(96, 7) gauge_force_fixed_kernel(Geom g, double beta, const int4* __restrict__ gfx,
-                                                               double2* out, int gradient, int accumulate) {
+                                                               const unsigned char* __restrict__ weak, double2* out,
+                                                               int gradient, int accumulate) {
   __shared__ RowsXch xch;
-  const Where w = where(g);
+  Where w = where(g);
   const int Vh = g.Vh, lam = blockIdx.y;
-  cx<i64> A[3] = {};
+  if (weak) {
+    w.valid = w.valid && !(weak[(size_t)w.p * Vh + w.h] >> lam & 1);
+    if (__syncthreads_or(w.valid) == 0) return;
+  }
+  cx<i64> A[3] = {};  // in units of 2^-60
   int i = 0;
   if (w.valid) {
     const Site s = site_of(g, w.p, w.h);
@@ -555,14 +560,17 @@ __global__ void __launch_bounds__(96, 7) gauge_force_fixed_kernel(Geom g, double
     for (int k = 0; k < 3; k++) {
       const int o = k < lam ? k : k + 1;
       cx<i64> t[3], u[3];
-      fx_row_mul<true>(fx_row_times<true>(fx_load_row<false>(fx_link_at(f, lam, 1, o, 0, o), Vh, w.row),
+      fx_row_mul<true>(fx_row_times<true>(fx_load_row_fine<false>(fx_link_at(f, lam, 1, o, 0, o), Vh, w.row),
                                           fx_link_at(f, lam, 0, o, 1, lam), Vh),
                        fx_link_at(f, lam, 0, o, 0, o), Vh, t);
-      fx_row_mul<false>(fx_row_times<true>(fx_load_row<true>(fx_link_at(f, lam, 1, o, -1, o), Vh, w.row),
+      fx_row_mul<false>(fx_row_times<true>(fx_load_row_fine<true>(fx_link_at(f, lam, 1, o, -1, o), Vh, w.row),
                                            fx_link_at(f, lam, 0, o, -1, lam), Vh),
                         fx_link_at(f, lam, 0, o, -1, o), Vh, u);
 #pragma unroll
-      for (int j = 0; j < 3; j++) A[j] = A[j] + t[j] + u[j];  // six terms of 2^58 at most
+      for (int j = 0; j < 3; j++) {  // six terms of 2^60 at most
+        A[j].re += (t[j].re + u[j].re) >> 1;
+        A[j].im += (t[j].im + u[j].im) >> 1;
+      }
     }
   }
   double2* q = out + ((size_t)i * 4 + lam) * 9;
@@ -571,7 +579,7 @@ __global__ void __launch_bounds__(96, 7) gauge_force_fixed_kernel(Geom g, double
     const double f = -beta / 3.0;
 #pragma unroll
     for (int j = 0; j < 3; j++) {  // G_j,row = f conj(A_row,j)
-      double2 o = make_double2(f * fx_to_double_in_range(A[j].re, -FX_LINK), -f * fx_to_double_in_range(A[j].im, -FX_LINK));
+      double2 o = make_double2(f * fx_to_double_in_range(A[j].re, -60), -f * fx_to_double_in_range(A[j].im, -60));
       double2* qq = q + 3 * j + w.row;
       if (accumulate) {
         const double2 was = *qq;
@@ -581,7 +589,7 @@ __global__ void __launch_bounds__(96, 7) gauge_force_fixed_kernel(Geom g, double
     }
     return;
   }
-  store_ta<false>(g, w, gfx + (size_t)(w.p * 4 + lam) * 9 * Vh + w.h, A, -FX_LINK, false, beta / 6.0, xch, q + 3 * w.row,
+  store_ta<false>(g, w, gfx + (size_t)(w.p * 4 + lam) * 9 * Vh + w.h, A, -60, false, beta / 6.0, xch, q + 3 * w.row,
                   accumulate != 0);
 }
 
@@ -660,11 +668,11 @@ void launch_plaquette_fixed(const Geom& g, const void* gfx, const ReduceArgs& re
   plaquette_fixed_kernel<<<rows_grid(g, 6), 96, 0, st>>>(g, static_cast<const int4*>(gfx), red);
 }
 
-void launch_gauge_force_fixed(const Geom& g, double beta, const void* gfx, double2* out, bool gradient, bool accumulate,
-                              cudaStream_t st) {
+void launch_gauge_force_fixed(const Geom& g, double beta, const void* gfx, const unsigned char* weak, double2* out,
+                              bool gradient, bool accumulate, cudaStream_t st) {
   g_kernel_launches += 1;
-  gauge_force_fixed_kernel<<<rows_grid(g, 4), 96, 0, st>>>(g, beta, static_cast<const int4*>(gfx), out, gradient ? 1 : 0,
-                                                           accumulate ? 1 : 0);
+  gauge_force_fixed_kernel<<<rows_grid(g, 4), 96, 0, st>>>(g, beta, static_cast<const int4*>(gfx), weak, out,
+                                                           gradient ? 1 : 0, accumulate ? 1 : 0);
 }
 
 }  // namespace qcd

@@ -63,10 +63,20 @@ cudaError_t launch_cg_persistent(int prec, int recon, const PersistentCGArgs& q,
 cudaError_t launch_barrier_probe(unsigned* count, int* err, cudaStream_t st);
 
 // ---- layout (qcd_layout.cu); prec 60 names block fixed point (qcd_fixed.cuh) with norm its exponents
-// gfx (may be null): the block fixed-point links; *not_unitary is set if a link is not near-unitary,
-// *non_finite (may be null) if one holds a non-finite value
+// the block fixed-point links U ([2][4][9][Vh] int4; null: not kept), and per site ([2][Vh]) the planes (bits of weakF)
+// and directions (of weakG) whose field strength or gauge force comes from links close to one alone: the FP64
+// kernels form these (null: there are none)
+struct FxLinks {
+  void* U;
+  unsigned char *weakF, *weakG;
+};
+// gfx (may be null): the block fixed-point links, and far ([2][4][Vh]) whether a link is not close to one;
+// *not_unitary is set if a link is not near-unitary, *non_finite (may be null) if one holds a non-finite value
 void launch_pack_gauge(const Geom& g, const double2* canon, void* g64, void* g32, int recon32, void* g16,
-                       int recon16, void* gfx, int* not_unitary, int* non_finite, cudaStream_t st);
+                       int recon16, void* gfx, unsigned char* far, int* not_unitary, int* non_finite, cudaStream_t st);
+// weakF, weakG from far; bits 0 and 1 of *any are set if there is one of each
+void launch_weak_sites(const Geom& g, const unsigned char* far, unsigned char* weakF, unsigned char* weakG, int* any,
+                       cudaStream_t st);
 void launch_spinor_to_native(int prec, const Geom& g, const double2* canon, void* nat, float* norm, int nrhs,
                              cudaStream_t st);
 void launch_spinor_to_canon(int prec, const Geom& g, const void* nat, const float* norm, double2* canon, int nrhs,
@@ -83,9 +93,9 @@ struct FxClover {
 // A (even sites) and A^-1 (odd sites) in FP64, FP32 and FP16; flag set if a block is not positive definite.
 // work: 6 * 9 * V double2 for the field strengths (two kernels: F per site and plane, then one chiral
 // block per thread); logdet: [parity][block][Vh] log det of each 6x6 block.
-// gfx (may be null): the near-unitary links in block fixed point, from which F is then formed.  A is stored on
+// fl: the near-unitary links in block fixed point, from which F is then formed (null: from g64).  A is stored on
 // even, A^-1 on odd sites.
-void launch_clover_build(const Geom& g, const void* g64, const void* gfx, double kappa, double csw, void* A64, void* Ainv64,
+void launch_clover_build(const Geom& g, const void* g64, const FxLinks& fl, double kappa, double csw, void* A64, void* Ainv64,
                          void* A32, void* Ainv32, void* A16, void* Ainv16, void* work, double* logdet,
                          int* notposdef, const FxClover& fx, cudaStream_t st);
 // the same for block fixed-point fields and blocks (clover_e: their exponents [2][Vh])
@@ -150,12 +160,12 @@ void launch_finalize(const ReduceArgs& red, const double* totals, int nrhs, cuda
 void launch_norm2(const Geom& g, int nrhs, const double2* v, const ReduceArgs& red, cudaStream_t st);
 // ---- molecular dynamics (qcd_md.cu); canonical link fields [V][4][3][3] complex128
 // Wilson gauge force (or gradient) of beta sum (1 - Re tr P / 3) from the FP64 packed links, written
-// to or added to out
-void launch_gauge_force(const Geom& g, double beta, const void* g64, double2* out, bool gradient, bool accumulate,
-                        cudaStream_t st);
-// the same from the block fixed-point links, and the plaquette sum below
-void launch_gauge_force_fixed(const Geom& g, double beta, const void* gfx, double2* out, bool gradient, bool accumulate,
-                              cudaStream_t st);
+// to or added to out; with weak, the (site, direction) pairs marked there only
+void launch_gauge_force(const Geom& g, double beta, const void* g64, const unsigned char* weak, double2* out, bool gradient,
+                        bool accumulate, cudaStream_t st);
+// the same from the block fixed-point links, those marked in weak left out, and the plaquette sum below
+void launch_gauge_force_fixed(const Geom& g, double beta, const void* gfx, const unsigned char* weak, double2* out,
+                              bool gradient, bool accumulate, cudaStream_t st);
 void launch_plaquette_fixed(const Geom& g, const void* gfx, const ReduceArgs& red, cudaStream_t st);
 // result[0] = sum over sites and planes of Re tr P_{mu nu}(x) / 3 (FIN_STORE)
 void launch_plaquette(const Geom& g, const void* g64, const ReduceArgs& red, cudaStream_t st);

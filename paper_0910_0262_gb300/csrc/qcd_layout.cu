@@ -5,7 +5,7 @@
 // the equivalent goal -- every byte fetched is a byte used -- is met by a
 // component-major, site-minor layout per parity: consecutive threads (sites)
 // read consecutive 8/16-byte words, so no padding is transferred at all.
-#include "qcd_fixed.cuh"
+#include "qcd_fxmat.cuh"
 #include "qcd_kernels.h"
 
 namespace qcd {
@@ -44,11 +44,20 @@ __device__ __forceinline__ bool near_unitary(const float2 v[9]) {
   return worst < 1e-5f;
 }
 
+// whether an entry of U - 1 is 2^-4 or more (the bound of qcd_fxmat.cuh)
+__device__ __forceinline__ bool far_from_one(const float2 v[9]) {
+  float most = 0.f;
+#pragma unroll
+  for (int k = 0; k < 9; k++) most = fmaxf(most, fmaxf(fabsf(k % 4 == 0 ? v[k].x - 1.f : v[k].x), fabsf(v[k].y)));
+  return most >= 0.0625f;
+}
+
 // canonical gauge U[i][mu][3][3] complex128 -> per-parity, per-direction SoA copies.  gfx: the block
-// fixed-point copy, which serves near-unitary links only; *not_unitary is set if one is not.  *non_finite
-// (may be null) is set if a link holds a non-finite value.
+// fixed-point copy, which serves near-unitary links only, with far; *not_unitary is set if one is not.
+// *non_finite (may be null) is set if a link holds a non-finite value.
 __global__ void pack_gauge_kernel(Geom g, const double2* __restrict__ U, double2* g64, void* g32, int recon32,
-                                  void* g16, int recon16, int4* gfx, int* not_unitary, int* non_finite) {
+                                  void* g16, int recon16, int4* gfx, unsigned char* far, int* not_unitary,
+                                  int* non_finite) {
   const int tid = blockIdx.x * blockDim.x + threadIdx.x;
   const int V = 2 * g.Vh;
   if (tid >= V * 4) return;
@@ -74,6 +83,7 @@ __global__ void pack_gauge_kernel(Geom g, const double2* __restrict__ U, double2
   for (int k = 0; k < 9; k++) g64[(base * 9 + k) * g.Vh + h] = u[k];
   if (gfx) {
     fx_store_link(gfx + base * 9 * g.Vh + h, g.Vh, u);
+    far[base * g.Vh + h] = far_from_one(v);
     if (!near_unitary(v)) *not_unitary = 1;
   }
   if (g32) {
@@ -102,6 +112,40 @@ __global__ void pack_gauge_kernel(Geom g, const double2* __restrict__ U, double2
       for (int k = 0; k < 9; k++) q[(base * 9 + k) * g.Vh + h] = f2h(v[k].x, v[k].y);
     }
   }
+}
+
+// Per site the planes and directions all of whose links are close to one: the twelve links of the four leaves of
+// F_{mu nu}(x), the link U_l(x) and the 18 of its staples.
+__global__ void __launch_bounds__(128) weak_sites_kernel(Geom g, const unsigned char* __restrict__ far,
+                                                         unsigned char* weakF, unsigned char* weakG, int* any) {
+  const int tid = blockIdx.x * 128 + threadIdx.x;
+  if (tid >= 2 * g.Vh) return;
+  const int p = tid >= g.Vh, h = tid - p * g.Vh;
+  const Site s = site_of(g, p, h);
+  const FxSites f = {nullptr, g.Vh, g.X, g.Y, g.Z, g.T, {s.x, s.y, s.z, s.t}, p};
+  auto at = [&](int d1, int s1, int d2, int s2, int mu) {
+    return (int)__ldg(far + (size_t)(((p + s1 + s2) & 1) * 4 + mu) * g.Vh + fx_half_at(f, d1, s1, d2, s2));
+  };
+  int wF = 0, force = 0;  // force: directions with a link in their staples that is far from one
+  int pl = 0;
+#pragma unroll
+  for (int m = 0; m < 3; m++)
+#pragma unroll
+    for (int n = m + 1; n < 4; n++) {
+      const int m00 = at(m, 0, n, 0, m), n00 = at(m, 0, n, 0, n);
+      const int n10 = at(m, 1, n, 0, n), m01 = at(m, 0, n, 1, m), n1b = at(m, 1, n, -1, n), m0b = at(m, 0, n, -1, m);
+      const int n0b = at(m, 0, n, -1, n), mb1 = at(m, -1, n, 1, m), nb0 = at(m, -1, n, 0, n);
+      const int mbb = at(m, -1, n, -1, m), nbb = at(m, -1, n, -1, n), mb0 = at(m, -1, n, 0, m);
+      if (!(m00 | n00 | n10 | m01 | n1b | m0b | n0b | mb1 | nb0 | mbb | nbb | mb0)) wF |= 1 << pl;
+      // staples of m through n and of n through m (with the links themselves)
+      if (m00 | n10 | m01 | n00 | n1b | m0b | n0b) force |= 1 << m;
+      if (n00 | m01 | n10 | m00 | mb1 | nb0 | mb0) force |= 1 << n;
+      pl++;
+    }
+  const int wG = ~force & 15;
+  weakF[tid] = (unsigned char)wF;
+  weakG[tid] = (unsigned char)wG;
+  if (wF || wG) atomicOr(any, (wF ? 1 : 0) | (wG ? 2 : 0));
 }
 
 // Canonical sites are 12 consecutive complex128.  Reading them site by site is fine (a site's lines stay in
@@ -237,12 +281,18 @@ inline int nblocks(long long n, int b) { return (int)((n + b - 1) / b); }
 }  // namespace
 
 void launch_pack_gauge(const Geom& g, const double2* canon, void* g64, void* g32, int recon32, void* g16,
-                       int recon16, void* gfx, int* not_unitary, int* non_finite, cudaStream_t st) {
+                       int recon16, void* gfx, unsigned char* far, int* not_unitary, int* non_finite, cudaStream_t st) {
   g_kernel_launches += 1;
   const int B = 128;
   pack_gauge_kernel<<<nblocks(8LL * g.Vh, B), B, 0, st>>>(g, canon, static_cast<double2*>(g64), g32, recon32, g16,
-                                                          recon16, static_cast<int4*>(gfx), not_unitary,
+                                                          recon16, static_cast<int4*>(gfx), far, not_unitary,
                                                           non_finite);
+}
+
+void launch_weak_sites(const Geom& g, const unsigned char* far, unsigned char* weakF, unsigned char* weakG, int* any,
+                       cudaStream_t st) {
+  g_kernel_launches += 1;
+  weak_sites_kernel<<<nblocks(2LL * g.Vh, 128), 128, 0, st>>>(g, far, weakF, weakG, any);
 }
 
 void launch_spinor_to_native(int prec, const Geom& g, const double2* canon, void* nat, float* norm, int nrhs,

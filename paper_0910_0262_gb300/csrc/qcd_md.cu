@@ -55,7 +55,8 @@ __device__ __forceinline__ void store_canon(double2* U, size_t link, const M3& m
 }
 
 // one thread per link (lambda, lexicographic site i): G, or F, into out (canonical), or added to it
-__global__ void __launch_bounds__(MB) gauge_force_kernel(Geom g, double beta, const double2* g64, double2* out,
+__global__ void __launch_bounds__(MB) gauge_force_kernel(Geom g, double beta, const double2* g64,
+                                                         const unsigned char* __restrict__ weak, double2* out,
                                                          int gradient, int accumulate) {
   const int V = 2 * g.Vh;
   const long long tid = (long long)blockIdx.x * MB + threadIdx.x;
@@ -63,6 +64,7 @@ __global__ void __launch_bounds__(MB) gauge_force_kernel(Geom g, double beta, co
   const int lam = (int)(tid / V), i = (int)(tid - (long long)lam * V);
   int c[4];
   lattice_coords(g, i, c);
+  if (weak && !(weak[(size_t)((c[0] + c[1] + c[2] + c[3]) & 1) * g.Vh + (i >> 1)] >> lam & 1)) return;
   auto at = [&](int dl, int dn, int nu, int dir) {
     int q[4] = {c[0], c[1], c[2], c[3]};
     q[lam] += dl;
@@ -289,11 +291,11 @@ __global__ void __launch_bounds__(MB) link_update_kernel(size_t nlinks, double e
 
 }  // namespace
 
-void launch_gauge_force(const Geom& g, double beta, const void* g64, double2* out, bool gradient, bool accumulate,
-                        cudaStream_t st) {
+void launch_gauge_force(const Geom& g, double beta, const void* g64, const unsigned char* weak, double2* out, bool gradient,
+                        bool accumulate, cudaStream_t st) {
   g_kernel_launches += 1;
   const long long n = 8LL * g.Vh;
-  gauge_force_kernel<<<(unsigned)((n + MB - 1) / MB), MB, 0, st>>>(g, beta, static_cast<const double2*>(g64), out,
+  gauge_force_kernel<<<(unsigned)((n + MB - 1) / MB), MB, 0, st>>>(g, beta, static_cast<const double2*>(g64), weak, out,
                                                                    gradient ? 1 : 0, accumulate ? 1 : 0);
 }
 

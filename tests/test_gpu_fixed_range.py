@@ -3,7 +3,9 @@
 import numpy as np
 import pytest
 
-from oracle import evenodd, force as oforce
+from oracle import dirac, evenodd, force as oforce, md as omd
+from oracle.dirac import PLANES, dagger, sigma
+from oracle.lattice import parity
 from paper_0910_0262_gb300 import synth
 from gpu_util import require_gpu, to_dev, to_np, rel_l2, rand_eo
 
@@ -88,3 +90,81 @@ def test_force_of_many_right_hand_sides(n):
     the results' last rounding and the oracle's own (the FP64 kernels: 5.2e-16 for one, 3.1e-16 for 200)."""
     require_gpu()
     assert many_rhs_error(n) < 1e-15
+
+
+def _inverse(A):
+    X = np.linalg.inv(A.astype(complex)).astype(LONG)
+    one = np.eye(A.shape[-1], dtype=LONG)
+    for _ in range(3):
+        X = X @ (2 * one - A @ X)
+    return X
+
+
+def det_force(U):
+    """The force of S_det = -2 sum_{x odd} log det A(x) (oracle.cloverdet) in long double."""
+    U = U.astype(LONG)
+    lat = U.shape[:4]
+    A = np.zeros(lat + (4, 3, 4, 3), dtype=LONG)
+    A += np.einsum('st,ab->satb', np.eye(4), np.eye(3))
+    for mu, nu in PLANES:
+        A -= LONG(KAPPA) * CSW * np.einsum('st,...ab->...satb', sigma(mu, nu), dirac.field_strength(U, mu, nu))
+    inv = _inverse(A.reshape(lat + (12, 12))).reshape(lat + (4, 3, 4, 3))
+    dims = (lat[3], lat[2], lat[1], lat[0])
+    odd = (parity(dims) == 1)[..., None, None]
+    G = np.zeros(U.shape, dtype=LONG)
+    for mu, nu in PLANES:
+        B = np.einsum('...satb,ts->...ab', inv, sigma(mu, nu))
+        B = B - np.trace(B, axis1=-2, axis2=-1)[..., None, None] * np.eye(3) / LONG(3)
+        C = odd * (-1j * (LONG(KAPPA) * CSW / 4) * (B + dagger(B)))
+        for path in dirac.leaf_paths(mu, nu):
+            oforce.insert(G, U, path, C)
+    return oforce.lie_force(U, G)
+
+
+def gauge_force(U, beta):
+    U = U.astype(LONG)
+    G = np.zeros(U.shape, dtype=LONG)
+    C = np.broadcast_to(-LONG(beta) / 3 * np.eye(3, dtype=LONG), U.shape[:4] + (3, 3))
+    for mu, nu in PLANES:
+        oforce.insert(G, U, omd.plaquette_paths(mu, nu), C)
+    return oforce.lie_force(U, G)
+
+
+def weak_errors(eps, dims=(4, 4, 2, 6)):
+    """Relative 2-norm errors on links exp(i eps H) of the gauge force and of the determinant force's off-diagonal
+    colours (its diagonal holds differences of the diagonal of A^-1, close to one, in FP64 kernels too)."""
+    U, op = _context(dims, eps)
+    g = rel(to_np(op.gauge_force(5.6)), gauge_force(U, 5.6))
+    off = 1 - np.eye(3)
+    d = rel(off * to_np(op.fermion_force(None, clover_det=True)[0]), off * det_force(U))
+    op.close()
+    return g, d
+
+
+@pytest.mark.parametrize("eps", [1.0, 0.2, 0.1, 0.05, 1e-2, 1e-3, 1e-6])
+def test_forces_on_weak_fields(eps):
+    """The forces depend on what links differ from one by, which FP64 products keep to their own size: the
+    errors, relative to the force, do not grow as the field gets weak.  (The FP64 kernels give 1.3e-16 and
+    1.0 to 1.2e-15 at every eps, the latter from A^-1.)"""
+    require_gpu()
+    g, d = weak_errors(eps)
+    assert g < 2e-16 and d < 2e-15
+
+
+def test_forces_where_weak_and_strong_links_meet():
+    """One half of the lattice at eps 1e-3, the other at 0.3: each half's force is right to its own size (the
+    links two sites into it, which no strong link reaches)."""
+    require_gpu()
+    dims = (2, 4, 2, 12)
+    U = synth.make_problem(dims, 1e-3, 3)[0]
+    U[6:] = synth.make_problem(dims, 0.3, 4)[0][6:]
+    _, op = _context(dims)
+    op.load_gauge(to_dev(U))
+    op.clover_build(KAPPA, CSW)
+    got = to_np(op.gauge_force(5.6)), to_np(op.fermion_force(None, clover_det=True)[0])
+    op.close()
+    want = gauge_force(U, 5.6), det_force(U)
+    off = 1 - np.eye(3)
+    for part in (slice(2, 4), slice(8, 10)):
+        assert rel(got[0][part], want[0][part]) < 1e-15
+        assert rel(off * got[1][part], off * want[1][part]) < 4e-15
