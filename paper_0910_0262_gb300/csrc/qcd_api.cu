@@ -14,6 +14,7 @@
 #include <cstdio>
 #include <cstdlib>
 #include <cstring>
+#include <initializer_list>
 #include <string>
 #include <vector>
 
@@ -137,7 +138,8 @@ struct qcd_ctx {
   unsigned char* far = nullptr;  // in gfx's allocation: [2][4][Vh] links far from one, then weakF, weakG [2][Vh]
   int weak = 0;                  // bits 0, 1: some site is marked in weakF, weakG
   FxClover cfx{};
-  bool fx_links = false;
+  bool fx_links = false;  // the loaded links are near-unitary
+  bool no_fixed = false, no_fixed_clover = false;  // there was no room for them, or it was given back
   // clover
   void* A64 = nullptr;
   void* Ainv64 = nullptr;
@@ -256,6 +258,49 @@ bool try_alloc(void** p, size_t bytes) {
   return false;
 }
 
+// a context's own buffers: each one that is not there yet
+struct OwnBuffer {
+  void** p;
+  size_t bytes;
+};
+qcd_status own_buffers(std::initializer_list<OwnBuffer> list) {
+  for (const OwnBuffer& b : list)
+    if (!*b.p && !try_alloc(b.p, b.bytes)) return fail(QCD_ERR_NOMEM, "cudaMalloc(%zu bytes) failed", b.bytes);
+  return QCD_OK;
+}
+
+// Gives back the block fixed-point copies and the work space, which their kernels have larger, for good: the
+// context goes on with the FP64 kernels.  False if it held no copies.
+bool give_back_fixed(qcd_ctx* c) {
+  if (!c->gfx) return false;
+  cudaStreamSynchronize(c->st);
+  for (ItGraph* gph : c->graphs) destroy_graph(gph);  // (recorded on those buffers)
+  c->graphs.clear();
+  c->launched.clear();
+  for (void* p : {c->gfx, c->cfx.A_even, c->cfx.Ainv_odd, static_cast<void*>(c->cfx.eA_even), static_cast<void*>(c->cfx.eAinv_odd)})
+    cudaFree(p);
+  c->gfx = nullptr;
+  c->far = nullptr;
+  c->cfx = FxClover{};
+  for (int k = 0; k < S_COUNT; k++) {
+    if (k == S_CANON || k == S_MD_F || k == S_MD_PHI || k == S_PBP) continue;  // (an outer call may hold these)
+    cudaFree(c->ws[k].ptr);
+    c->ws[k] = Buf{};
+  }
+  c->fx_links = false;
+  c->no_fixed = true;
+  return true;
+}
+
+// A call that finds no device memory for a buffer is run again without the fixed-point copies, which the library
+// can do without: a lattice that fits with the FP64 kernels alone is not refused because of them.  body: the call,
+// which may have written its outputs but none of its inputs.
+template <typename F>
+qcd_status with_room(qcd_ctx* c, F body) {
+  const qcd_status s = body();
+  return s == QCD_ERR_NOMEM && give_back_fixed(c) ? body() : s;
+}
+
 // --------------------------------------------------------------- profiling --
 int prof_class(qcd_ctx* c, const std::string& name) {
   for (size_t i = 0; i < c->prof.size(); i++)
@@ -355,19 +400,12 @@ const void* gauge_ptr(const qcd_ctx* c, int prec) {
   return prec == 64 ? c->g64 : (prec == 32 ? c->g32 : c->g16);
 }
 
-// (precision 60 keeps A on even and A^-1 on odd sites only, the parities the operators use)
-const void* clover_ptr(const qcd_ctx* c, int prec, bool inverse, int parity) {
+// A on even or A^-1 on odd sites, the parities that the operators use
+const void* clover_ptr(const qcd_ctx* c, int prec, bool inverse) {
   if (prec == 60) return inverse ? c->cfx.Ainv_odd : c->cfx.A_even;
-  if (prec == 64) {
-    const double2* base = static_cast<const double2*>(inverse ? c->Ainv64 : c->A64);
-    return base + (size_t)parity * 36 * c->g.Vh;
-  }
-  if (prec == 16) {
-    const uint4* base = static_cast<const uint4*>(inverse ? c->Ainv16 : c->A16);
-    return base + (size_t)parity * 9 * c->g.Vh;
-  }
-  const float4* base = static_cast<const float4*>(inverse ? c->Ainv32 : c->A32);
-  return base + (size_t)parity * 18 * c->g.Vh;
+  if (prec == 64) return inverse ? c->Ainv64 : c->A64;
+  if (prec == 16) return inverse ? c->Ainv16 : c->A16;
+  return inverse ? c->Ainv32 : c->A32;
 }
 
 const int* clover_exps(const qcd_ctx* c, bool inverse) { return inverse ? c->cfx.eAinv_odd : c->cfx.eA_even; }
@@ -412,7 +450,7 @@ void run_dslash(qcd_ctx* c, int prec, int epi, const DslashArgs& a) {
 // out = A in (even sites) or A^-1 in (odd sites)
 void run_clover(qcd_ctx* c, int prec, bool inverse, const void* in, const float* in_n, void* out, float* out_n,
                 int nrhs) {
-  const void* cl = clover_ptr(c, prec, inverse, inverse ? 1 : 0);
+  const void* cl = clover_ptr(c, prec, inverse);
   if (prec == 60) launch_clover_apply_fixed(c->g, cl, clover_exps(c, inverse), in, in_n, out, out_n, nrhs, c->st);
   else launch_clover_apply(prec, c->g, cl, in, in_n, out, out_n, nrhs, c->st);
 }
@@ -443,7 +481,7 @@ void apply_mhat(qcd_ctx* c, int prec, int nrhs, bool dagger, const void* in, con
   a.in_norm = in_n;
   a.out = t;
   a.out_norm = t_n;
-  a.clover = clover_ptr(c, prec, true, 1);
+  a.clover = clover_ptr(c, prec, true);
   a.in_g5 = dagger;
   a.halt = halt;
   a.gate = gate;
@@ -455,7 +493,7 @@ void apply_mhat(qcd_ctx* c, int prec, int nrhs, bool dagger, const void* in, con
   b.out_norm = out_n;
   b.x = in;
   b.x_norm = in_n;
-  b.clover = clover_ptr(c, prec, false, 0);
+  b.clover = clover_ptr(c, prec, false);
   b.a = -k2;
   b.x_g5 = dagger;
   b.out_g5 = dagger;
@@ -496,7 +534,7 @@ void apply_mdagm_resid(qcd_ctx* c, int nrhs, const SolverFields& f, const void* 
   a.in_norm = f.y_hi_n;
   a.out = f.t_hi;
   a.out_norm = f.t_hi_n;
-  a.clover = clover_ptr(c, 60, true, 1);
+  a.clover = clover_ptr(c, 60, true);
   a.in_g5 = 1;
   a.gate = gate;
   run_dslash(c, 60, EPI_CLOVER_INV, a);
@@ -505,7 +543,7 @@ void apply_mdagm_resid(qcd_ctx* c, int nrhs, const SolverFields& f, const void* 
   b.in_norm = f.t_hi_n;
   b.x = f.y_hi;
   b.x_norm = f.y_hi_n;
-  b.clover = clover_ptr(c, 60, false, 0);
+  b.clover = clover_ptr(c, 60, false);
   b.a = -c->kappa * c->kappa;
   b.x_g5 = 1;
   b.out_g5 = 1;
@@ -538,8 +576,8 @@ bool ctx_view(const qcd_ctx* c, CtxView* v) {
   v->st = c->st;
   v->device = c->device;
   v->g64 = c->g64;
-  v->A_even64 = c->A64 ? clover_ptr(c, 64, false, 0) : nullptr;
-  v->Ainv_odd64 = c->Ainv64 ? clover_ptr(c, 64, true, 1) : nullptr;
+  v->A_even64 = c->A64 ? clover_ptr(c, 64, false) : nullptr;
+  v->Ainv_odd64 = c->Ainv64 ? clover_ptr(c, 64, true) : nullptr;
   v->kappa = c->kappa;
   v->have_gauge = c->have_gauge;
   v->have_clover = c->have_clover;
@@ -695,21 +733,22 @@ qcd_status qcd_destroy(qcd_ctx* c) {
   return QCD_OK;
 }
 
-qcd_status qcd_load_gauge(qcd_ctx* c, const double* U, int on_device, int flags) {
-  QCD_API_ENTER("qcd_load_gauge", c);
+static qcd_status load_gauge(qcd_ctx* c, const double* U, int on_device, int flags) {
   qcd_status s = QCD_OK;
   if (!U) return fail(QCD_ERR_ARG, "null gauge pointer");
   if (flags & ~QCD_GAUGE_RECON12) return fail(QCD_ERR_ARG, "unknown gauge flags 0x%x", flags);
   const Geom& g = c->g;
   const size_t n_links = (size_t)g.Vh * 2 * 4;
   const size_t canon_bytes = n_links * 9 * sizeof(double2);
-  c->recon = (flags & QCD_GAUGE_RECON12) ? 12 : 18;
-  if (!c->g64) {
-    CUDA_TRY(cudaMalloc(&c->g64, canon_bytes));
-    CUDA_TRY(cudaMalloc(&c->g32, n_links * 9 * sizeof(float2)));
-    CUDA_TRY(cudaMalloc(&c->g16, n_links * 9 * sizeof(uint32_t)));
-    if (!c->slab && try_alloc(&c->gfx, n_links * 9 * sizeof(int4) + n_links + n_links / 2))
+  if ((s = own_buffers({{&c->g64, canon_bytes},
+                        {&c->g32, n_links * 9 * sizeof(float2)},
+                        {&c->g16, n_links * 9 * sizeof(uint32_t)}})))
+    return s;
+  if (!c->slab && !c->no_fixed && !c->gfx) {
+    if (try_alloc(&c->gfx, n_links * 9 * sizeof(int4) + n_links + n_links / 2))
       c->far = reinterpret_cast<unsigned char*>(static_cast<int4*>(c->gfx) + n_links * 9);
+    else
+      c->no_fixed = true;
   }
   // a t-slab keeps the whole extended field (its clover build reads it); the slab's own links start
   // two time slices in
@@ -717,7 +756,7 @@ qcd_status qcd_load_gauge(qcd_ctx* c, const double* U, int on_device, int flags)
   const size_t in_bytes = in_links * 9 * sizeof(double2);
   const double2* src = reinterpret_cast<const double2*>(U);
   if (c->slab) {
-    if (!c->U_ext) CUDA_TRY(cudaMalloc(&c->U_ext, in_bytes));
+    if ((s = own_buffers({{reinterpret_cast<void**>(&c->U_ext), in_bytes}}))) return s;
     CUDA_TRY(cudaMemcpyAsync(c->U_ext, U, in_bytes, on_device ? cudaMemcpyDeviceToDevice : cudaMemcpyHostToDevice,
                              c->st));
     src = c->U_ext;
@@ -727,6 +766,7 @@ qcd_status qcd_load_gauge(qcd_ctx* c, const double* U, int on_device, int flags)
     CUDA_TRY(cudaMemcpyAsync(stage, U, canon_bytes, cudaMemcpyHostToDevice, c->st));
     src = static_cast<const double2*>(stage);
   }
+  c->recon = (flags & QCD_GAUGE_RECON12) ? 12 : 18;
   CUDA_TRY(cudaMemsetAsync(c->flags, 0, 4 * sizeof(int), c->st));
   // (a slab's extended field holds more links than are packed here; 24^3 x 32: the pass over the links that
   // looked for non-finite values took 66 us beside the packing's 186)
@@ -747,28 +787,32 @@ qcd_status qcd_load_gauge(qcd_ctx* c, const double* U, int on_device, int flags)
   return QCD_OK;
 }
 
-qcd_status qcd_clover_build(qcd_ctx* c, double kappa, double csw) {
-  QCD_API_ENTER("qcd_clover_build", c);
+qcd_status qcd_load_gauge(qcd_ctx* c, const double* U, int on_device, int flags) {
+  QCD_API_ENTER("qcd_load_gauge", c);
+  return with_room(c, [&] { return load_gauge(c, U, on_device, flags); });
+}
+
+static qcd_status clover_build(qcd_ctx* c, double kappa, double csw) {
   qcd_status s = QCD_OK;
   if (!c->have_gauge) return fail(QCD_ERR_STATE, "clover_build before load_gauge");
   if (!(kappa == kappa) || !(csw == csw)) return fail(QCD_ERR_ARG, "kappa/csw not finite");
   const Geom& g = c->g;
-  if (!c->A64) {
-    CUDA_TRY(cudaMalloc(&c->A64, (size_t)2 * 36 * g.Vh * sizeof(double2)));
-    CUDA_TRY(cudaMalloc(&c->Ainv64, (size_t)2 * 36 * g.Vh * sizeof(double2)));
-    CUDA_TRY(cudaMalloc(&c->A32, (size_t)2 * 18 * g.Vh * sizeof(float4)));
-    CUDA_TRY(cudaMalloc(&c->Ainv32, (size_t)2 * 18 * g.Vh * sizeof(float4)));
-    CUDA_TRY(cudaMalloc(&c->A16, (size_t)2 * 9 * g.Vh * sizeof(uint4)));
-    CUDA_TRY(cudaMalloc(&c->Ainv16, (size_t)2 * 9 * g.Vh * sizeof(uint4)));
-    CUDA_TRY(cudaMalloc(&c->logdet, (size_t)2 * 2 * g.Vh * sizeof(double)));
-  }
-  if (c->fx_links && !c->cfx.A_even) {
+  if ((s = own_buffers({{&c->A64, (size_t)36 * g.Vh * sizeof(double2)},
+                        {&c->Ainv64, (size_t)36 * g.Vh * sizeof(double2)},
+                        {&c->A32, (size_t)18 * g.Vh * sizeof(float4)},
+                        {&c->Ainv32, (size_t)18 * g.Vh * sizeof(float4)},
+                        {&c->A16, (size_t)9 * g.Vh * sizeof(uint4)},
+                        {&c->Ainv16, (size_t)9 * g.Vh * sizeof(uint4)},
+                        {reinterpret_cast<void**>(&c->logdet), (size_t)2 * 2 * g.Vh * sizeof(double)}})))
+    return s;
+  if (c->fx_links && !c->cfx.A_even && !c->no_fixed_clover) {
     void *a = nullptr, *b = nullptr, *ea = nullptr, *eb = nullptr;
     const size_t blocks = (size_t)36 * g.Vh * sizeof(int4), exps = (size_t)2 * g.Vh * sizeof(int);
     if (try_alloc(&a, blocks) && try_alloc(&b, blocks) && try_alloc(&ea, exps) && try_alloc(&eb, exps)) {
       c->cfx = FxClover{a, b, static_cast<int*>(ea), static_cast<int*>(eb)};
     } else {
       for (void* p : {a, b, ea, eb}) cudaFree(p);
+      c->no_fixed_clover = true;
     }
   }
   void* work;
@@ -796,8 +840,12 @@ qcd_status qcd_clover_build(qcd_ctx* c, double kappa, double csw) {
   return QCD_OK;
 }
 
-qcd_status qcd_dslash(qcd_ctx* c, double* out, const double* in, int op, int dagger, int prec, int nrhs) {
-  QCD_API_ENTER("qcd_dslash", c);
+qcd_status qcd_clover_build(qcd_ctx* c, double kappa, double csw) {
+  QCD_API_ENTER("qcd_clover_build", c);
+  return with_room(c, [&] { return clover_build(c, kappa, csw); });
+}
+
+static qcd_status dslash(qcd_ctx* c, double* out, const double* in, int op, int dagger, int prec, int nrhs) {
   if (qcd_status rs = slab_refuse(c, "qcd_dslash", true)) return rs;
   qcd_status s = QCD_OK;
   if (!out || !in) return fail(QCD_ERR_ARG, "null field pointer");
@@ -860,6 +908,11 @@ qcd_status qcd_dslash(qcd_ctx* c, double* out, const double* in, int op, int dag
   cudaError_t e = cudaGetLastError();
   if (e != cudaSuccess) return fail(QCD_ERR_CUDA, "dslash launch: %s", cudaGetErrorString(e));
   return QCD_OK;
+}
+
+qcd_status qcd_dslash(qcd_ctx* c, double* out, const double* in, int op, int dagger, int prec, int nrhs) {
+  QCD_API_ENTER("qcd_dslash", c);
+  return with_room(c, [&] { return dslash(c, out, in, op, dagger, prec, nrhs); });
 }
 
 }  // extern "C"
@@ -934,7 +987,7 @@ void enqueue_iteration(qcd_ctx* c, const SolverFields& f, int nrhs) {
   a.in_norm = f.y_n;
   a.out = f.t;
   a.out_norm = f.t_n;
-  a.clover = clover_ptr(c, f.pp, true, 1);
+  a.clover = clover_ptr(c, f.pp, true);
   a.in_g5 = 1;
   a.halt = halt;
   run_dslash(c, f.pp, EPI_CLOVER_INV, a);
@@ -945,7 +998,7 @@ void enqueue_iteration(qcd_ctx* c, const SolverFields& f, int nrhs) {
   b.in_norm = f.t_n;
   b.x = f.y;
   b.x_norm = f.y_n;
-  b.clover = clover_ptr(c, f.pp, false, 0);
+  b.clover = clover_ptr(c, f.pp, false);
   b.a = -c->kappa * c->kappa;
   b.x_g5 = 1;
   b.out_g5 = 1;
@@ -1141,8 +1194,8 @@ qcd_status launch_persistent(qcd_ctx* c, const SolverFields& f, int iter_limit, 
   memset(&q, 0, sizeof q);
   q.g = g;
   q.gauge = gauge_ptr(c, f.pp);
-  q.clover_inv_odd = clover_ptr(c, f.pp, true, 1);
-  q.clover_even = clover_ptr(c, f.pp, false, 0);
+  q.clover_inv_odd = clover_ptr(c, f.pp, true);
+  q.clover_even = clover_ptr(c, f.pp, false);
   q.p = f.p;
   q.t = f.t;
   q.y = f.y;
@@ -1426,19 +1479,19 @@ qcd_status check_params(const qcd_solver_params* p) {
 namespace {
 
 // The force or gradient from the solutions X (canonical, nrhs of them, may be 0 with det) on block fixed-point
-// fields.  *ran = false (and QCD_OK): there was no memory for its work space, and nothing was done.
-qcd_status force_fixed(qcd_ctx* c, double2* F, const double2* X, int nrhs, bool gradient, bool det, bool* ran) {
+// fields
+qcd_status force_fixed(qcd_ctx* c, double2* F, const double2* X, int nrhs, bool gradient, bool det) {
   const Geom& g = c->g;
   qcd_status s = QCD_OK;
   void *xf = nullptr, *yf = nullptr, *xn = nullptr, *yn = nullptr, *clf, *cxf, *ef;
   const size_t half = (size_t)nrhs * 12 * g.Vh, hn = (size_t)nrhs * 2 * g.Vh;
-  *ran = false;
-  if ((nrhs > 0 && (ws_get(c, S_F_X, 2 * half * sizeof(double2), &xf) || ws_get(c, S_F_Y, 2 * half * sizeof(double2), &yf) ||
-                    ws_get(c, S_F_XN, 2 * hn * sizeof(int), &xn) || ws_get(c, S_F_YN, 2 * hn * sizeof(int), &yn))) ||
-      ws_get(c, S_F_CL, force_clover_bytes(g), &clf) || ws_get(c, S_F_CX, fixed_matrix_bytes(g, 6), &cxf) ||
-      ws_get(c, S_F_E, fixed_matrix_bytes(g, 12), &ef))
-    return QCD_OK;
-  *ran = true;
+  if (nrhs > 0 &&
+      ((s = ws_get(c, S_F_X, 2 * half * sizeof(double2), &xf)) || (s = ws_get(c, S_F_Y, 2 * half * sizeof(double2), &yf)) ||
+       (s = ws_get(c, S_F_XN, 2 * hn * sizeof(int), &xn)) || (s = ws_get(c, S_F_YN, 2 * hn * sizeof(int), &yn))))
+    return s;
+  if ((s = ws_get(c, S_F_CL, force_clover_bytes(g), &clf)) || (s = ws_get(c, S_F_CX, fixed_matrix_bytes(g, 6), &cxf)) ||
+      (s = ws_get(c, S_F_E, fixed_matrix_bytes(g, 12), &ef)))
+    return s;
   double2 *Xe = static_cast<double2*>(xf), *Xo = Xe + half, *Ye = static_cast<double2*>(yf), *Yo = Ye + half;
   float *xe = static_cast<float*>(xn), *xo = xe + hn, *ye = static_cast<float*>(yn), *yo = ye + hn;
   double2* C = static_cast<double2*>(clf);
@@ -1454,7 +1507,7 @@ qcd_status force_fixed(qcd_ctx* c, double2* F, const double2* X, int nrhs, bool 
     a.in_norm = ye + on;
     a.out = Yo + off;
     a.out_norm = yo + on;
-    a.clover = clover_ptr(c, 60, true, 1);
+    a.clover = clover_ptr(c, 60, true);
     a.in_g5 = 1;
     a.out_g5 = 1;
     run_dslash(c, 60, EPI_CLOVER_INV, a);
@@ -1469,7 +1522,7 @@ qcd_status force_fixed(qcd_ctx* c, double2* F, const double2* X, int nrhs, bool 
   }
   if (det) {
     ProfScope ps(c, "force_det_coeff", g.Vh * (72 * 16.0) + V * 6 * 144.0 * 2, 0.0);
-    launch_force_det_coeff(g, c->kappa, c->csw, static_cast<const double2*>(clover_ptr(c, 64, true, 1)), C, true, c->st);
+    launch_force_det_coeff(g, c->kappa, c->csw, static_cast<const double2*>(clover_ptr(c, 64, true)), C, true, c->st);
   }
   {
     ProfScope ps(c, "force_edges", V * (6 + 4 + 12) * 144.0, V * force_edge_flops());
@@ -1486,9 +1539,8 @@ qcd_status force_fixed(qcd_ctx* c, double2* F, const double2* X, int nrhs, bool 
 
 extern "C" {
 
-qcd_status qcd_cg_solve(qcd_ctx* c, double* x, const double* b, int nrhs, const qcd_solver_params* prm,
-                        qcd_solver_stats* stats) {
-  QCD_API_ENTER("qcd_cg_solve", c);
+static qcd_status cg_solve(qcd_ctx* c, double* x, const double* b, int nrhs, const qcd_solver_params* prm,
+                           qcd_solver_stats* stats) {
   if (qcd_status rs = slab_refuse(c, "qcd_cg_solve", true)) return rs;
   qcd_status s = QCD_OK;
   if (!x || !b) return fail(QCD_ERR_ARG, "null field pointer");
@@ -1513,9 +1565,14 @@ qcd_status qcd_cg_solve(qcd_ctx* c, double* x, const double* b, int nrhs, const 
   return worst;
 }
 
-qcd_status qcd_fermion_force(qcd_ctx* c, double* F, const double* phi_or_x, int nrhs, int flags,
-                             const qcd_solver_params* prm, qcd_solver_stats* stats) {
-  QCD_API_ENTER("qcd_fermion_force", c);
+qcd_status qcd_cg_solve(qcd_ctx* c, double* x, const double* b, int nrhs, const qcd_solver_params* prm,
+                        qcd_solver_stats* stats) {
+  QCD_API_ENTER("qcd_cg_solve", c);
+  return with_room(c, [&] { return cg_solve(c, x, b, nrhs, prm, stats); });
+}
+
+static qcd_status fermion_force(qcd_ctx* c, double* F, const double* phi_or_x, int nrhs, int flags,
+                                const qcd_solver_params* prm, qcd_solver_stats* stats) {
   if (qcd_status rs = slab_refuse(c, "qcd_fermion_force", false)) return rs;
   qcd_status s = QCD_OK;
   const bool det = (flags & QCD_FORCE_CLOVER_DET) != 0;
@@ -1539,11 +1596,8 @@ qcd_status qcd_fermion_force(qcd_ctx* c, double* F, const double* phi_or_x, int 
     if (s && s != QCD_ERR_NOT_CONVERGED) return s;
     X = static_cast<const double2*>(v);
   }
-  if (fp64_rep(c, true) == 60) {
-    bool ran = false;
-    if ((s = force_fixed(c, reinterpret_cast<double2*>(F), X, nrhs, (flags & QCD_FORCE_GRADIENT) != 0, det, &ran)) || ran)
-      return s;
-  }
+  if (fp64_rep(c, true) == 60)
+    return force_fixed(c, reinterpret_cast<double2*>(F), X, nrhs, (flags & QCD_FORCE_GRADIENT) != 0, det);
   if (nrhs == 0) {
     // the determinant term alone: its coefficients into a zeroed buffer, then the leaves
     void* clf;
@@ -1552,7 +1606,7 @@ qcd_status qcd_fermion_force(qcd_ctx* c, double* F, const double* phi_or_x, int 
     const double V = 2.0 * g.Vh;
     {
       ProfScope ps(c, "force_det_coeff", g.Vh * (72 * 16.0) + V * 6 * 144.0 * 2, 0.0);
-      launch_force_det_coeff(g, c->kappa, c->csw, static_cast<const double2*>(clover_ptr(c, 64, true, 1)),
+      launch_force_det_coeff(g, c->kappa, c->csw, static_cast<const double2*>(clover_ptr(c, 64, true)),
                              static_cast<double2*>(clf), false, c->st);
     }
     void* ef;
@@ -1595,7 +1649,7 @@ qcd_status qcd_fermion_force(qcd_ctx* c, double* F, const double* phi_or_x, int 
     DslashArgs a = base_args(c, 64, 1, nb);
     a.in = Ye + off;
     a.out = Yo + off;
-    a.clover = clover_ptr(c, 64, true, 1);
+    a.clover = clover_ptr(c, 64, true);
     a.in_g5 = 1;
     a.out_g5 = 1;
     run_dslash(c, 64, EPI_CLOVER_INV, a);
@@ -1605,7 +1659,7 @@ qcd_status qcd_fermion_force(qcd_ctx* c, double* F, const double* phi_or_x, int 
   }
   if (det) {
     ProfScope ps(c, "force_det_coeff", g.Vh * (72 * 16.0) + V * 6 * 144.0 * 2, 0.0);
-    launch_force_det_coeff(g, c->kappa, c->csw, static_cast<const double2*>(clover_ptr(c, 64, true, 1)),
+    launch_force_det_coeff(g, c->kappa, c->csw, static_cast<const double2*>(clover_ptr(c, 64, true)),
                            static_cast<double2*>(clf), false, c->st);
   }
   {
@@ -1625,6 +1679,12 @@ qcd_status qcd_fermion_force(qcd_ctx* c, double* F, const double* phi_or_x, int 
                        (flags & QCD_FORCE_GRADIENT) != 0, k == 0, k > 0, c->st);
   }
   return sync_and_check(c, "fermion_force");
+}
+
+qcd_status qcd_fermion_force(qcd_ctx* c, double* F, const double* phi_or_x, int nrhs, int flags,
+                             const qcd_solver_params* prm, qcd_solver_stats* stats) {
+  QCD_API_ENTER("qcd_fermion_force", c);
+  return with_room(c, [&] { return fermion_force(c, F, phi_or_x, nrhs, flags, prm, stats); });
 }
 
 qcd_status qcd_selftest_barrier_timeout(qcd_ctx* c) {
@@ -1702,8 +1762,7 @@ static qcd_status eo_check(qcd_ctx* c, const void* out, const void* in1, const v
   return QCD_OK;
 }
 
-qcd_status qcd_prepare_source(qcd_ctx* c, double* bhat_e, const double* b_e, const double* b_o, int nrhs) {
-  QCD_API_ENTER("qcd_prepare_source", c);
+static qcd_status prepare_source(qcd_ctx* c, double* bhat_e, const double* b_e, const double* b_o, int nrhs) {
   if (qcd_status rs = slab_refuse(c, "qcd_prepare_source", false)) return rs;
   qcd_status s = eo_check(c, bhat_e, b_e, b_o, nrhs);
   if (s) return s;
@@ -1740,8 +1799,12 @@ qcd_status qcd_prepare_source(qcd_ctx* c, double* bhat_e, const double* b_e, con
   return QCD_OK;
 }
 
-qcd_status qcd_reconstruct_odd(qcd_ctx* c, double* x_o, const double* x_e, const double* b_o, int nrhs) {
-  QCD_API_ENTER("qcd_reconstruct_odd", c);
+qcd_status qcd_prepare_source(qcd_ctx* c, double* bhat_e, const double* b_e, const double* b_o, int nrhs) {
+  QCD_API_ENTER("qcd_prepare_source", c);
+  return with_room(c, [&] { return prepare_source(c, bhat_e, b_e, b_o, nrhs); });
+}
+
+static qcd_status reconstruct_odd(qcd_ctx* c, double* x_o, const double* x_e, const double* b_o, int nrhs) {
   if (qcd_status rs = slab_refuse(c, "qcd_reconstruct_odd", false)) return rs;
   qcd_status s = eo_check(c, x_o, x_e, b_o, nrhs);
   if (s) return s;
@@ -1761,7 +1824,7 @@ qcd_status qcd_reconstruct_odd(qcd_ctx* c, double* x_o, const double* x_e, const
     a.in_norm = (float*)un;
     a.out = t;
     a.out_norm = (float*)tn;
-    a.clover = clover_ptr(c, rep, true, 1);
+    a.clover = clover_ptr(c, rep, true);
     run_dslash(c, rep, EPI_CLOVER_INV, a);
     double2* cout = reinterpret_cast<double2*>(x_o) + done * n;
     launch_spinor_to_canon(rep, g, t, (float*)tn, cout, nb, c->st);
@@ -1781,6 +1844,11 @@ qcd_status qcd_reconstruct_odd(qcd_ctx* c, double* x_o, const double* x_e, const
   cudaError_t e = cudaGetLastError();
   if (e != cudaSuccess) return fail(QCD_ERR_CUDA, "reconstruct_odd launch: %s", cudaGetErrorString(e));
   return QCD_OK;
+}
+
+qcd_status qcd_reconstruct_odd(qcd_ctx* c, double* x_o, const double* x_e, const double* b_o, int nrhs) {
+  QCD_API_ENTER("qcd_reconstruct_odd", c);
+  return with_room(c, [&] { return reconstruct_odd(c, x_o, x_e, b_o, nrhs); });
 }
 
 qcd_status qcd_gauge_force(qcd_ctx* c, double* F, double beta, int flags) {
@@ -1865,8 +1933,12 @@ qcd_status qcd_r_step(qcd_ctx* c, double* U, double* P, const double* eta, int n
   const int gflags = c->recon == 12 ? QCD_GAUGE_RECON12 : 0;
   const size_t nlinks = (size_t)g.Vh * 2 * 4;
   void *fv, *phiv = nullptr;
-  if ((s = ws_get(c, S_MD_F, nlinks * 9 * sizeof(double2), &fv))) return s;
-  if (nrhs > 0 && (s = ws_get(c, S_MD_PHI, (size_t)g.Vh * 12 * sizeof(double2) * nrhs, &phiv))) return s;
+  if ((s = with_room(c, [&] {
+         qcd_status w = ws_get(c, S_MD_F, nlinks * 9 * sizeof(double2), &fv);
+         if (!w && nrhs > 0) w = ws_get(c, S_MD_PHI, (size_t)g.Vh * 12 * sizeof(double2) * nrhs, &phiv);
+         return w;
+       })))
+    return s;
   double* F = static_cast<double*>(fv);
   // half step of the links, then the fields at U'
   if ((s = qcd_update_links(c, U, P, 0.5 * eps))) return s;
@@ -1917,7 +1989,7 @@ qcd_status qcd_pbp(qcd_ctx* c, const double* eta_e, const double* eta_o, int nrh
   const Geom& g = c->g;
   const size_t n = (size_t)g.Vh * 12, fb = n * nrhs * sizeof(double2);
   void* w;
-  if ((s = ws_get(c, S_PBP, 4 * fb, &w))) return s;
+  if ((s = with_room(c, [&] { return ws_get(c, S_PBP, 4 * fb, &w); }))) return s;
   double2* bh = static_cast<double2*>(w);
   double2* rhs = bh + n * nrhs;
   double2* xe = rhs + n * nrhs;

@@ -35,28 +35,28 @@ size_t halo_bytes(const qcd_ctx* c, int prec, int nrhs) {
 
 int recon_of(const qcd_ctx* c, int prec) { return prec == 64 ? 18 : c->recon; }
 
-// the local part of a clover-shaped field [2 parities][rows][Vh_ext] of elements of `elem` bytes: the
-// slab's sites start XYZ half indices into each row of the extended lattice (two time slices)
+// the local part of a clover-shaped field [rows][Vh_ext] of elements of `elem` bytes: the slab's sites start XYZ
+// half indices into each row of the extended lattice (two time slices)
 qcd_status copy_slab_rows(qcd_ctx* c, void* dst, const void* src, int rows, size_t elem) {
   const size_t off = (size_t)c->g.XYZ * elem;
   CUDA_TRY(cudaMemcpy2DAsync(dst, (size_t)c->g.Vh * elem, static_cast<const char*>(src) + off,
-                             (size_t)c->ge.Vh * elem, (size_t)c->g.Vh * elem, (size_t)2 * rows,
+                             (size_t)c->ge.Vh * elem, (size_t)c->g.Vh * elem, (size_t)rows,
                              cudaMemcpyDeviceToDevice, c->st));
   return QCD_OK;
 }
 
 qcd_status slab_clover_build(qcd_ctx* c, double kappa, double csw, void* work) {
   const Geom& ge = c->ge;
-  if (!c->ext_g64) {
-    CUDA_TRY(cudaMalloc(&c->ext_g64, (size_t)2 * 4 * 9 * ge.Vh * sizeof(double2)));
-    CUDA_TRY(cudaMalloc(&c->ext_A64, (size_t)2 * 36 * ge.Vh * sizeof(double2)));
-    CUDA_TRY(cudaMalloc(&c->ext_Ainv64, (size_t)2 * 36 * ge.Vh * sizeof(double2)));
-    CUDA_TRY(cudaMalloc(&c->ext_A32, (size_t)2 * 18 * ge.Vh * sizeof(float4)));
-    CUDA_TRY(cudaMalloc(&c->ext_Ainv32, (size_t)2 * 18 * ge.Vh * sizeof(float4)));
-    CUDA_TRY(cudaMalloc(&c->ext_A16, (size_t)2 * 9 * ge.Vh * sizeof(uint4)));
-    CUDA_TRY(cudaMalloc(&c->ext_Ainv16, (size_t)2 * 9 * ge.Vh * sizeof(uint4)));
-    CUDA_TRY(cudaMalloc(&c->ext_logdet, (size_t)2 * 2 * ge.Vh * sizeof(double)));
-  }
+  qcd_status s;
+  if ((s = own_buffers({{&c->ext_g64, (size_t)2 * 4 * 9 * ge.Vh * sizeof(double2)},
+                        {&c->ext_A64, (size_t)36 * ge.Vh * sizeof(double2)},
+                        {&c->ext_Ainv64, (size_t)36 * ge.Vh * sizeof(double2)},
+                        {&c->ext_A32, (size_t)18 * ge.Vh * sizeof(float4)},
+                        {&c->ext_Ainv32, (size_t)18 * ge.Vh * sizeof(float4)},
+                        {&c->ext_A16, (size_t)9 * ge.Vh * sizeof(uint4)},
+                        {&c->ext_Ainv16, (size_t)9 * ge.Vh * sizeof(uint4)},
+                        {reinterpret_cast<void**>(&c->ext_logdet), (size_t)2 * 2 * ge.Vh * sizeof(double)}})))
+    return s;
   {
     ProfScope ps(c, "clover_build", 0, 2.0 * ge.Vh * (60 * 216.0 + 2 * 1000.0));
     launch_pack_gauge(ge, c->U_ext, c->ext_g64, nullptr, 0, nullptr, 0, nullptr, nullptr, nullptr, nullptr, c->st);
@@ -64,14 +64,13 @@ qcd_status slab_clover_build(qcd_ctx* c, double kappa, double csw, void* work) {
     launch_clover_build(ge, c->ext_g64, FxLinks{}, kappa, csw, c->ext_A64, c->ext_Ainv64, c->ext_A32, c->ext_Ainv32,
                         c->ext_A16, c->ext_Ainv16, work, c->ext_logdet, c->flags, FxClover{}, c->st);
   }
-  qcd_status s;
   if ((s = copy_slab_rows(c, c->A64, c->ext_A64, 36, sizeof(double2))) ||
       (s = copy_slab_rows(c, c->Ainv64, c->ext_Ainv64, 36, sizeof(double2))) ||
       (s = copy_slab_rows(c, c->A32, c->ext_A32, 18, sizeof(float4))) ||
       (s = copy_slab_rows(c, c->Ainv32, c->ext_Ainv32, 18, sizeof(float4))) ||
       (s = copy_slab_rows(c, c->A16, c->ext_A16, 9, sizeof(uint4))) ||
       (s = copy_slab_rows(c, c->Ainv16, c->ext_Ainv16, 9, sizeof(uint4))) ||
-      (s = copy_slab_rows(c, c->logdet, c->ext_logdet, 2, sizeof(double))))
+      (s = copy_slab_rows(c, c->logdet, c->ext_logdet, 4, sizeof(double))))
     return s;
   return QCD_OK;
 }
@@ -122,7 +121,7 @@ qcd_status slab_mhat(qcd_ctx* c, int prec, int nrhs, bool dagger, const void* in
   a.in_norm = in_n;
   a.out = t;
   a.out_norm = t_n;
-  a.clover = clover_ptr(c, prec, true, 1);
+  a.clover = clover_ptr(c, prec, true);
   a.in_g5 = dagger;
   qcd_status s = slab_pass(c, prec, EPI_CLOVER_INV, a, m);
   if (s) return s;
@@ -133,7 +132,7 @@ qcd_status slab_mhat(qcd_ctx* c, int prec, int nrhs, bool dagger, const void* in
   b.out_norm = out_n;
   b.x = in;
   b.x_norm = in_n;
-  b.clover = clover_ptr(c, prec, false, 0);
+  b.clover = clover_ptr(c, prec, false);
   b.a = -c->kappa * c->kappa;
   b.x_g5 = b.out_g5 = dagger;
   if (red) {
@@ -358,10 +357,10 @@ qcd_status qcd_slab_dslash(qcd_ctx* c, double* out, const double* in, int op, in
         s = slab_mdagm(c, prec, nb, vin, fin, vout, fout, vt, ft, vy, fy, m, nullptr);
         break;
       case QCD_OP_CLOVER:
-        launch_clover_apply(prec, g, clover_ptr(c, prec, false, 0), vin, fin, vout, fout, nb, c->st);
+        launch_clover_apply(prec, g, clover_ptr(c, prec, false), vin, fin, vout, fout, nb, c->st);
         break;
       case QCD_OP_CLOVER_INV:
-        launch_clover_apply(prec, g, clover_ptr(c, prec, true, 1), vin, fin, vout, fout, nb, c->st);
+        launch_clover_apply(prec, g, clover_ptr(c, prec, true), vin, fin, vout, fout, nb, c->st);
         break;
     }
     if (s) return s;

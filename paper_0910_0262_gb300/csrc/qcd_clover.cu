@@ -360,9 +360,9 @@ __global__ void __launch_bounds__(128) clover_assemble_kernel(Geom g, const doub
   }
   logdet[((size_t)p * 2 + b) * g.Vh + h] = ld;
   auto store = [&](const double* dd, const C* LL, double2* c64, float4* c32, uint4* c16, void* cfx, int* efx) {
-    store_block64(c64 + (size_t)p * 36 * g.Vh, g.Vh, h, b, dd, LL);
-    store_block32(c32 + (size_t)p * 18 * g.Vh, g.Vh, h, b, dd, LL);
-    store_block16(c16 + (size_t)p * 9 * g.Vh, g.Vh, h, b, dd, LL);
+    store_block64(c64, g.Vh, h, b, dd, LL);
+    store_block32(c32, g.Vh, h, b, dd, LL);
+    store_block16(c16, g.Vh, h, b, dd, LL);
     if (cfx)
       efx[(size_t)b * g.Vh + h] = fx_store_clover(static_cast<int4*>(cfx) + (size_t)b * 18 * g.Vh + h, g.Vh, dd, LL);
   };
