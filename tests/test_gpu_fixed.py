@@ -3,7 +3,9 @@ beside (other links), against the oracle.
 
 Sizes at the edges of the kernels' blocks of 32 sites: 8 and 24 sites per parity (part of one block), 32
 and 96 (whole blocks), 40, 72, 120 and 1080 (a ragged last block), with 1, 2, 3, 4 and 5 right-hand sides
-(pairs of warps per block: 1, 2, 4; batches 2 + 1 and 4 + 1).  Tolerances: a row of an operator sums at most
+(batches 2 + 1 and 4 + 1), where blocks times right-hand sides are no more than the GPU's SMs and the kernel
+with a direction per pair of warps runs; and larger ones (test_operators_of_many_blocks) for the kernel with
+1, 2 or 4 right-hand sides a block.  Tolerances: a row of an operator sums at most
 8 x 6 products of a link and 11 of a clover block, each rounded to 2^-53 in FP64, so 1e-15 in the norm; of
 one hopping term, site by site, 16 x 2^-53 of the neighbours' largest values.
 """
@@ -57,6 +59,64 @@ def test_operators(dims, t_bc, scale):
         for (o, dag), f in table.items():
             got = to_np(op.dslash(to_dev(x), o, dagger=bool(dag), precision=64))
             assert rel_l2(got, np.stack([f(v) for v in x])) < 1e-15, (n, o, dag)
+    op.close()
+
+
+@gpu
+@pytest.mark.parametrize("dims,n", [((6, 10, 2, 18), 8), ((10, 10, 10, 10), 1), ((10, 10, 10, 10), 2), ((10, 10, 10, 10), 4)],
+                         ids=["1080_rhs8", "5000_rhs1", "5000_rhs2", "5000_rhs4"])
+def test_operators_of_many_blocks(dims, n):
+    """34 blocks x 8 right-hand sides (two turns of four, which reuse the block's shared memory) and 157 blocks x 1, 2
+    and 4: more than any GPU's SMs this library runs on (152), each with a ragged last block."""
+    require_gpu()
+    U, op = _context(dims)
+    ref = evenodd.SchurOperator(U, KAPPA, CSW, -1.0)
+    vh = ref.A_ee.shape[0]
+    x = rand_eo(n, vh, np.random.default_rng(23))
+    for o, dag, f in ((0, False, ref.D_eo), (0, True, ref.D_oe_dag), (1, False, ref.D_oe), (2, False, ref.Mhat),
+                      (2, True, ref.Mhat_dag), (3, False, ref.MdagM)):
+        got = to_np(op.dslash(to_dev(x), o, dagger=dag, precision=64))
+        for k in range(n):
+            assert rel_l2(got[k], f(x[k])) < 1e-15, (o, dag, k)
+    for prec in (64, 32):
+        sol, stats, ok = op.cg_solve(to_dev(x), tol=1e-10, inner_prec=prec)
+        assert ok
+        for k, v in enumerate(to_np(sol)):
+            rel = np.linalg.norm(ref.MdagM(v) - x[k]) / np.linalg.norm(x[k])
+            assert rel < 1.001e-10 and abs(rel - stats[k]["true_rel_resid"]) < 1e-13
+    op.close()
+
+
+@gpu
+def test_sums_in_two_steps():
+    """488 blocks of 32 sites (the last one half full) are eight groups of 64, the last one of 40: sums of at least
+    eight groups are formed group by group.  The residuals that the solves report against numpy's sums over the
+    same operator's result (1e-13 of |b| in their rounding: 1e-5 of a residual of 1e-8), the plaquette against the
+    oracle's; every call twice, as the groups' counters have to be left at zero."""
+    require_gpu()
+    from oracle import md as omd
+    dims = (10, 10, 12, 26)
+    U, op = _context(dims)
+    b = rand_eo(4, int(np.prod(dims)) // 2, np.random.default_rng(29))
+    iters = {}
+    for n in (1, 4):
+        for prec in (64, 32, 16):
+            for turn in range(2):
+                x, stats, ok = op.cg_solve(to_dev(b[:n]), tol=1e-8, inner_prec=prec)
+                assert ok
+                r = b[:n] - to_np(op.dslash(x, 3, precision=64))
+                for k in range(n):
+                    rel = np.linalg.norm(r[k]) / np.linalg.norm(b[k])
+                    assert abs(rel - stats[k]["true_rel_resid"]) < 1e-13
+                    iters[n, prec, turn, k] = stats[k]["iters"]
+    for n in (1, 4):  # a wrong alpha or beta would not converge like exact ones
+        for prec in (64, 32, 16):
+            for k in range(n):
+                assert iters[n, prec, 0, k] == iters[n, prec, 1, k]
+                assert iters[n, 32, 0, k] <= iters[n, 64, 0, k] + 3
+    want = omd.mean_plaquette(U)
+    for turn in range(2):
+        assert abs(op.plaquette() - want) < 4e-15
     op.close()
 
 
@@ -136,9 +196,8 @@ def test_fp64_solve(nrhs):
 @pytest.mark.parametrize("nrhs", [1, 2, 5])
 @pytest.mark.parametrize("dims", [(2, 2, 10, 2), (6, 10, 2, 18), (10, 8, 8, 10)], ids=["40", "1080", "3200"])
 def test_solves_on_ragged_blocks(dims, nrhs, prec):
-    """40 and 1080 sites per parity: a ragged last block of 32; 3200: grid sums over two groups of 64 blocks, the
-    second one ragged.  The true residual, formed by the FP64 operator, differs
-    between two evaluations by its rounding, below 1e-13."""
+    """40 and 1080 sites per parity: a ragged last block of 32; 3200: 100 blocks.  The true residual, formed by the
+    FP64 operator, differs between two evaluations by its rounding, below 1e-13."""
     require_gpu()
     U, op = _context(dims)
     b = rand_eo(nrhs, int(np.prod(dims)) // 2, np.random.default_rng(19))
