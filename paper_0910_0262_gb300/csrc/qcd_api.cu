@@ -125,7 +125,7 @@ struct CaptureSink {
 struct qcd_ctx {
   Geom g{};
   cudaStream_t st = nullptr;
-  int device = 0;
+  int device = 0, sms = 0;  // its multiprocessors
   // links
   void* g64 = nullptr;
   void* g32 = nullptr;
@@ -433,6 +433,7 @@ DslashArgs base_args(const qcd_ctx* c, int prec, int parity, int nrhs) {
   a.nrhs = nrhs;
   a.gauge = gauge_ptr(c, prec);
   a.clover_e = clover_exps(c, parity == 1);  // A^-1 on odd, A on even output
+  a.sms = c->sms;
   return a;
 }
 
@@ -673,10 +674,10 @@ static qcd_status create_ctx(qcd_ctx** out, const int dims[4], double t_bc, void
   cudaMemset(c->flags, 0, 4 * sizeof(int));
   cudaMemset(c->ctl, 0, sizeof(CGControl));
   {
-    int sms = 0, coop = 0;
-    cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
+    int coop = 0;
+    cudaDeviceGetAttribute(&c->sms, cudaDevAttrMultiProcessorCount, dev);
     cudaDeviceGetAttribute(&coop, cudaDevAttrCooperativeLaunch, dev);
-    c->pc_slots = sms * 16;  // 16 resident 128-thread blocks per SM at most
+    c->pc_slots = c->sms * 16;  // 16 resident 128-thread blocks per SM at most
     c->persistent = coop != 0;
     const char* e = getenv("QCD_CG_PERSISTENT");
     if (e && e[0] == '0') c->persistent = false;

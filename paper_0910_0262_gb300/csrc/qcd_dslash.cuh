@@ -39,6 +39,7 @@ struct DslashArgs {
   const void* clover;      // clover block field of parity p (A or A^-1)
   const int* clover_e;     // fixed-point kernels: its exponents [2][Vh]
   int out_f64;             // fixed-point kernels: out is an FP64 field (else block fixed point)
+  int sms;                 // fixed-point kernels: the device's SMs, for the launcher's choice of kernel
   double a;                // EPI_XPAY coefficient on the hopping sum
   float af;                // the same in FP32 (set by the launcher of the site kernels)
   int in_g5;               // apply gamma_5 to the input before hopping

@@ -428,8 +428,8 @@ __device__ __forceinline__ double pair_fx(const DslashArgs& A, const FxScalar& s
   return finish_fx<EPI>(A, sc, hh, valid, r, B, v, eh);
 }
 
-// One pair of warps per (32 output sites, RHS); a block holds the pairs of PAIRS RHS of the same sites,
-// which share the staged links.  Bound by instruction issue: 4290 instructions per warp, 1260 of them
+// One pair of warps per (32 output sites, RHS); a block holds the pairs of PAIRS RHS of the same sites (nrhs is
+// a multiple of PAIRS), which share the staged links.  Bound by instruction issue: 4290 instructions per warp, 1260 of them
 // multiply-adds that take two issue slots, 45% of the slots issuing at 16 warps per SM (128 registers);
 // 32^4, 1 RHS: 256 us a pass with the inverse clover block, 57% of DRAM throughput, bytes read once.
 template <int EPI, int PAIRS>
@@ -458,8 +458,8 @@ __global__ void __launch_bounds__(64 * PAIRS, 8 / PAIRS) dslash_fixed_kernel(Dsl
   for (int r0 = 0; r0 < A.nrhs; r0 += PAIRS) {
     const int r = r0 + q;
     if (r0 > 0) __syncthreads();  // the exchange area of the last RHS has been read
-    double nrm = pair_fx<EPI, PAIRS>(A, sc, hh, site && r < A.nrhs, s.t, r, q, w & 1, nbs, fx_ring);
-    if (reduce && r < A.nrhs) {
+    double nrm = pair_fx<EPI, PAIRS>(A, sc, hh, site, s.t, r, q, w & 1, nbs, fx_ring);
+    if (reduce) {
       for (int off = 16; off >= 1; off >>= 1) nrm += __shfl_xor_sync(0xffffffffu, nrm, off);
       if (lane == 0) {
         const long long slot = (long long)r * (2 * gridDim.x) + 2 * blockIdx.x + (w & 1);
@@ -629,21 +629,25 @@ void launch_fx_pairs(const DslashArgs& a, const FxScalar& sc, cudaStream_t st) {
   dslash_fixed_kernel<EPI, PAIRS><<<(a.g.Vh + 31) / 32, 64 * PAIRS, sh, st>>>(a, sc);
 }
 
-// Units (32 sites, RHS) up to which a pass takes the split kernel: one block on each of the 152 SMs (4^3 x 8, 8
-// units: 12.6 -> 10.4 us a pass; 8 x 8 x 16 x 16, 256 units: 14.3 against 14.5 us, 12^3 x 20, 540 units: 18.2
-// against 23.0 us).
-const int FX_SPLIT_UNITS = 152;
-
+// The split kernel where its blocks, one a unit of 32 sites and RHS, are no more than the SMs: a pass of one pair of
+// warps a unit would leave the others idle (4^3 x 8, 8 units, split 10.4 us a pass, pairs 12.6; 8 x 8 x 16 x 16, 256
+// units, 14.5 against 14.3; 12^3 x 20, 540 units, 23.0 against 18.2 us).
+//
+// Otherwise two RHS share a block's links from two RHS on, and four where all blocks of four are resident at once
+// (two an SM), so that the wider block is there to fill the SMs.  Clover-inverse / xpay passes in us with 1, 2 or 4
+// RHS a block, 4 RHS: 128 blocks of sites 38/41, 24/25, 19/20; 300: -, 30/33, 27/29; 473: -, 46/49, 48/54; 1024: 86/94,
+// 75/82, 78/89; 24^3 x 32, 6912: 451/519, 431/476, 472/515.  8 RHS: 128: 71/78, 41/44, 31/33; 300: -, 54/58, 48/51;
+// 6912: 905/1062, 859/946, 927/1002.
 template <int EPI>
 void launch_fx(const DslashArgs& a, const FxScalar& sc, cudaStream_t st) {
   const int nb = (a.g.Vh + 31) / 32;
-  if ((long long)nb * a.nrhs <= FX_SPLIT_UNITS) {
+  if ((long long)nb * a.nrhs <= a.sms) {
     constexpr size_t sh = sizeof(int4) * 32 * fx_stage_rows(1) * 8;
     cudaFuncSetAttribute(dslash_fixed_split_kernel<EPI>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sh);
     dslash_fixed_split_kernel<EPI><<<dim3(nb, a.nrhs), 256, sh, st>>>(a, sc);
     return;
   }
-  if (a.nrhs >= 4) launch_fx_pairs<EPI, 4>(a, sc, st);
+  if (a.nrhs >= 4 && nb <= 2 * a.sms) launch_fx_pairs<EPI, 4>(a, sc, st);
   else if (a.nrhs >= 2) launch_fx_pairs<EPI, 2>(a, sc, st);
   else launch_fx_pairs<EPI, 1>(a, sc, st);
 }
