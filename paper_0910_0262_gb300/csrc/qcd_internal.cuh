@@ -171,6 +171,17 @@ __device__ __forceinline__ float narrow(double x) {
   }
   return m == 0 ? __uint_as_float((unsigned)(b >> 32)) : (float)x;
 }
+// the same in two parts: whether x is zero or its magnitude lies among the normal floats (below their top binade), and
+// the value then, without a branch
+__device__ __forceinline__ bool narrow_common(double x) {
+  const unsigned hi = (unsigned)__double2hiint(x), lo = (unsigned)__double2loint(x);
+  return (hi >> 20 & 0x7ffu) - 897u < 253u || (hi << 1 | lo) == 0u;
+}
+__device__ __forceinline__ float narrow_of_common(double x) {
+  const unsigned long long b = (unsigned long long)__double_as_longlong(x), m = b & 0x7fffffffffffffffULL;
+  const unsigned r = (unsigned)((m + 0x0fffffffULL + ((m >> 29) & 1ULL)) >> 29) - (896u << 23);
+  return __uint_as_float(((unsigned)(b >> 32) & 0x80000000u) | (m == 0 ? 0u : r));
+}
 template <typename R>
 __device__ __forceinline__ R to_real(double x);
 template <>

@@ -47,6 +47,50 @@ def test_chiral_blocks_of_very_different_size(bits, small):
     assert max(chiral_errors(ratio=2.0 ** -bits, small=small)) < 1e-15
 
 
+@pytest.mark.parametrize("value", [np.nan, np.inf])
+def test_non_finite_block_leaves_the_other(value):
+    """A and A^-1 of a site with a non-finite component: its chiral block is non-finite, the other as without it."""
+    require_gpu()
+    U, op = _context((4, 4, 2, 6))
+    x = rand_eo(1, U.size // 72, np.random.default_rng(7))
+    for o in (4, 5):
+        clean = to_np(op.dslash(to_dev(x), o, precision=64))[0]
+        y = x.copy()
+        y[0, 9, 1, 2] = value
+        got = to_np(op.dslash(to_dev(y), o, precision=64))[0]
+        assert not np.isfinite(got[9, :2]).any() and np.array_equal(got[9, 2:], clean[9, 2:])
+        assert np.array_equal(np.delete(got, 9, 0), np.delete(clean, 9, 0))
+    op.close()
+
+
+@pytest.mark.parametrize("dims", [(2, 2, 2, 2), (4, 4, 4, 6)], ids=["8", "192"])
+def test_conversion_to_fp32(dims):
+    """Canonical fields to FP32 as the hardware rounds them (to nearest even), at every end of the range: with c_sw = 0
+    the clover operator is one.  8 and 192 sites: part of a block of 128, and one and a half."""
+    require_gpu()
+    from paper_0910_0262_gb300.qcd import CloverWilson
+    U = synth.make_problem(dims, 0.2, 3)[0]
+    op = CloverWilson(dims, -1.0)
+    op.load_gauge(to_dev(U))
+    op.clover_build(KAPPA, 0.0)
+    vh = int(np.prod(dims)) // 2
+    rng = np.random.default_rng(2)
+    f = np.float32
+    ends = [0.0, -0.0, 1.0, 1 + 2.0 ** -24, 1 + 3 * 2.0 ** -24, 2.0 ** -126, 2.0 ** -126 * (1 - 2.0 ** -25), 2.0 ** -149, 2.0 ** -150,
+            1e-40, 1e-300, 5e-324, float(np.finfo(f).max), 2.0 ** 127, np.nextafter(2.0 ** 128 * (1 - 2.0 ** -25), 0)]
+    x = rng.choice(ends, (1, vh, 4, 3)) * rng.choice([1, -1], (1, vh, 4, 3)) + 1j * rng.standard_normal((1, vh, 4, 3)) * 2.0 ** rng.integers(-30, 30, (1, vh, 4, 3))
+    got = to_np(op.dslash(to_dev(x), 4, precision=32))
+    with np.errstate(over="ignore"):
+        want = x.real.astype(f) + 1j * x.imag.astype(f).astype(float)
+    assert np.array_equal(got.real, want.real.astype(float)) and np.array_equal(got.imag, want.imag)
+    for v in (1e39, -1e300, np.inf, np.nan):  # not in the range
+        y = x.copy()
+        y[0, 1, 0, 0] = v
+        got = to_np(op.dslash(to_dev(y), 4, precision=32))
+        assert not np.isfinite(got[0, 1, 0, 0]) and np.array_equal(np.delete(got, 1, 1), np.delete(want, 1, 1))
+    op.close()
+
+
 def hop_bias(dims=(6, 10, 2, 18), n=8):
     """(mean signed error of D_eo x over all components, 2^-57 times the mean of a site's bound 2^e)."""
     U, op = _context(dims)
