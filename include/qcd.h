@@ -129,7 +129,7 @@ qcd_status qcd_load_gauge(qcd_ctx* ctx, const double* U, int on_device, int flag
 
 /*
  * Build the clover term A from the loaded links and factorise it on every site in
- * FP64 (Cholesky of each 6x6 chiral block); keeps A on even and A^-1 on odd sites,
+ * FP64 (l D l^dag of each 6x6 chiral block); keeps A on even and A^-1 on odd sites,
  * the ones the operators use.  Returns QCD_ERR_STATE without links, QCD_ERR_NOT_POSDEF if a block
  * is not positive definite.
  */
@@ -140,6 +140,12 @@ qcd_status qcd_clover_build(qcd_ctx* ctx, double kappa, double csw);
  * in and out are device complex128 arrays [nrhs][V/2][4][3] on the parities the
  * op names; they must not overlap.  precision (64/32/16) selects the internal
  * storage and arithmetic; the result is returned in FP64.  nrhs >= 1.
+ * precision 64 on links unitary to 1e-5 works in block fixed point: each site's two
+ * chiral blocks (spins 0, 1 and 2, 3) are held to 2^-61 of their largest component, and
+ * a result's error is below 2^-52 of the largest product that goes into its block (for
+ * the hopping term from the neighbours' larger block) -- no more than rounding each
+ * product to 2^-53 gives a block, but a component far smaller than its block's largest
+ * is right to the block's size and not to its own.  Other links take FP64 kernels.
  * Returns QCD_ERR_STATE if the op needs links/clover that are not loaded.
  */
 qcd_status qcd_dslash(qcd_ctx* ctx, double* out, const double* in, int op, int dagger, int precision, int nrhs);
@@ -181,7 +187,7 @@ qcd_status qcd_fermion_force(qcd_ctx* ctx, double* F, const double* phi_or_x, in
  */
 
 /*
- * log det of the clover term from the Cholesky factors of the last qcd_clover_build, summed over
+ * log det of the clover term from the pivots of the last qcd_clover_build, summed over
  * the sites of each parity (both 6x6 chiral blocks): out[0] = sum_{x even} log det A(x),
  * out[1] = sum_{x odd} log det A(x); S_det = -2 out[1].  out: host array of 2.  Synchronises.
  * Returns QCD_ERR_STATE without a clover term.

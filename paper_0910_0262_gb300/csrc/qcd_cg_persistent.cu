@@ -16,10 +16,11 @@
 //   phase 5  p  = r + beta p
 //
 // FP32 forms phase 5 where phases 1 and 2 of the next iteration read p (p = r + beta p from the
-// previous iteration's r, p and beta), so its iteration has four phases; phase 5 runs as a phase only
-// when a launch stops at its iteration cap.  Sums are formed per block over a fixed set of site blocks;
-// the barrier that closes a sum has the last-arriving block add the per-block partials in block order
-// and publish the total, so all blocks hold the same alpha and beta.  Fields written inside
+// previous iteration's r, p and beta), so its iteration has four phases; the first iteration of a launch
+// takes beta from the state, so phase 5 never runs.  Sums are formed per block over a fixed set of site
+// blocks; the barrier that closes a sum has the last-arriving block add the per-block partials as integers
+// (exact in their common unit, so their order does not matter), derive alpha or beta and publish them, so
+// all blocks hold the same ones.  Fields written inside
 // the kernel are read with ordinary loads after the barrier.  Every barrier wait is bounded: a
 // block that has waited too long sets an error word and all blocks return (the host reports
 // QCD_ERR_TIMEOUT).
@@ -95,8 +96,8 @@ __device__ __forceinline__ double grid_total(const double* part);
 
 // Grid-wide barrier that also sums one double per block (`mine`, thread 0's value): every block
 // writes its partial and arrives on the counter with an acquire-release add; the block whose arrival
-// completes the count reads all partials (the add's acquire makes them visible), sums them in block
-// order -- the same bits whichever block arrives last -- derives from the total what every block needs next
+// completes the count reads all partials (the add's acquire makes them visible), sums them -- the same
+// bits whichever block arrives last (grid_total) -- derives from the total what every block needs next
 // (result(total): the step's coefficient and status, by its thread 0 alone), publishes it and releases the
 // others through *flag.  The total comes out of the barrier instead of after it (at 16^4 the separate sum of
 // 512 partials after a barrier took 2.5 us), and its consequences too: a division or comparison in FP64 that
@@ -352,7 +353,6 @@ __global__ void __launch_bounds__(PcShape<P>::THREADS, PcShape<P>::MIN_BLOCKS)
     a1.in_norm = Q.p_n;
     a1.in_g5 = 0;
     a1.lz_r = Q.r;
-    a1.lz_a = 1.f;
     a1.lz_b = beta32;
     run_phase<P, RECON, EPI_CLOVER_INV, LAZY>(a1, part, xch, stage, 0.0);
     if (!grid_barrier(Q.bar_count, bar_target, Q.bar_err)) return;
@@ -365,7 +365,6 @@ __global__ void __launch_bounds__(PcShape<P>::THREADS, PcShape<P>::MIN_BLOCKS)
       a.out_norm = Q.y_n;
       a.do_norm = 1;
       a.lz_r = a1.lz_r;
-      a.lz_a = a1.lz_a;
       a.lz_b = a1.lz_b;
       const double v = block_sum<BLOCK, PAIR>(run_phase<P, RECON, EPI_XPAY, LAZY>(a, part, xch, stage, 0.0));
       auto next = [&](double t) {

@@ -9,8 +9,8 @@
 //   A_b = 1 - kappa c_sw [[ B3, B1 - i B2 ], [ B1 + i B2, -B3 ]]
 //   b = 0: B1 = F_yz - F_xt, B2 = F_xz + F_yt, B3 = F_xy - F_zt
 //   b = 1: B1 = F_yz + F_xt, B2 = F_xz - F_yt, B3 = F_xy + F_zt.
-// The inverse is formed once per gauge field in FP64 by a Cholesky factorisation
-// A_b = L L^dag and A_b^-1 = L^-dag L^-1; a non-positive pivot raises a flag.
+// The inverse is formed once per gauge field in FP64 by the factorisation A_b = l D l^dag (l unit lower
+// triangular, D diagonal) and A_b^-1 = l^-dag D^-1 l^-1; a non-positive pivot raises a flag.
 #include "qcd_fxmat.cuh"
 #include "qcd_kernels.h"
 #include "qcd_su3.cuh"

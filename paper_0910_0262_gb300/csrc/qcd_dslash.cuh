@@ -63,10 +63,10 @@ struct DslashArgs {
   // and signed by the slab that sent it.
   const void* halo_lo;
   const void* halo_hi;
-  // LAZY loads (the persistent FP32 iteration): the input is p' = lz_b p + lz_a r, formed where it is
+  // LAZY loads (the persistent FP32 iteration): the input is p' = r + lz_b p, formed where it is
   // read (p = in, r = lz_r, both FP32), so that the p update needs no pass of its own
   const void* lz_r;
-  float lz_a, lz_b;
+  float lz_b;
 };
 
 // Halo entries: six complex numbers (a projected half spinor) per face site and RHS, FP64 as
@@ -318,8 +318,8 @@ __device__ __forceinline__ typename Real<P>::T load_neighbor(const DslashArgs& A
     SpinorIO<32>::template load<COH>(A.lz_r, nullptr, A.g.Vh, r, nb, rs);
 #pragma unroll
     for (int c = 0; c < 12; c++) {  // the p update's own expression: fma(beta, p, r)
-      sp[c].re = fmaf(A.lz_b, sp[c].re, A.lz_a * rs[c].re);
-      sp[c].im = fmaf(A.lz_b, sp[c].im, A.lz_a * rs[c].im);
+      sp[c].re = fmaf(A.lz_b, sp[c].re, rs[c].re);
+      sp[c].im = fmaf(A.lz_b, sp[c].im, rs[c].im);
     }
     return R(1);
   }
@@ -748,7 +748,7 @@ __device__ __forceinline__ void pair_hops(const DslashArgs& A, const Site& s, cx
 
 // The pair unit on warp B of its pair (B is the chiral block the warp finishes; a compile-time
 // constant, so that the partial sums stay in registers).
-// LAZY (FP32): with EPI_CLOVER_INV the input p' = lz_b p + lz_a r is formed at every neighbour; with
+// LAZY (FP32): with EPI_CLOVER_INV the input p' = r + lz_b p is formed at every neighbour; with
 // EPI_XPAY the local term x = p is replaced by p' (formed from the staged p and r blocks) and p' is
 // written back over p, which completes the p update of the iteration.
 template <int P, int RECON, int EPI, int COH, int B, bool LAZY = false>
@@ -809,8 +809,8 @@ __device__ __forceinline__ float pair_unit_b(const DslashArgs& A, int hh, bool v
         staged_spinor_block<32>(stage + ST::OFF_X + ST::SPBN, lane, b, rs);
 #pragma unroll
         for (int k = 0; k < 6; k++) {
-          xs[k].re = fmaf(A.lz_b, xs[k].re, A.lz_a * rs[k].re);
-          xs[k].im = fmaf(A.lz_b, xs[k].im, A.lz_a * rs[k].im);
+          xs[k].re = fmaf(A.lz_b, xs[k].re, rs[k].re);
+          xs[k].im = fmaf(A.lz_b, xs[k].im, rs[k].im);
         }
         SpinorIO<32>::store_block(const_cast<void*>(A.x), nullptr, Vh, 0, hh, b, xs);
       }

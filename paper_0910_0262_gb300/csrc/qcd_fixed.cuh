@@ -10,9 +10,11 @@
 // For a product both factors are split as v = hi 2^31 + lo, and
 //   a b = (ah bh) 2^62 + (ah bl + al bh) 2^31 + al bl:
 // three multiply-adds into two 64-bit sums, the last term dropped.  The dropped terms are about 2^59 each
-// whatever the factors, so both factors are brought to their full size before they meet; the products of
+// whatever the factors, so both groups are brought to their full size before they meet; the products of
 // a group's largest members (2^116 and more) are then right to 2^-56 or better, where FP64 rounds each of
-// them to 2^-53 (qcd_selftest_fixed measures both against extended precision).
+// them to 2^-53 (qcd_selftest_fixed measures both against extended precision).  Products of smaller members have
+// that same absolute error, where FP64's shrinks with them: a result is as good as FP64's by its group's size
+// (norms over a chiral block, a matrix), not component by component.
 //
 // Bounds (the sums are exact integers, so only their final values have to fit):
 //   half spinor h = s +- s', |h| < 2^61: hi < 2^30, 0 <= lo < 2^31

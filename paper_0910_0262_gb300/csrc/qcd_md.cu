@@ -211,7 +211,7 @@ __device__ M3 expm3(M3 m) {
       nrm *= 0.5f;
       s++;
     }
-  } else if (x > 120) {  // r < 2^(x / 2): halved x / 2 + 2 times, at most 60
+  } else if (x > 120) {  // r > 2^59: 60 halvings, the most that are made; the phases of such an M are lost to rounding
     s = 60;
     nrm = 0.25f;
   }
