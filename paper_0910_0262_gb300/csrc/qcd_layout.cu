@@ -114,14 +114,16 @@ __global__ void pack_gauge_kernel(Geom g, const double2* __restrict__ U, double2
   }
 }
 
-// Per site the planes and directions all of whose links are close to one: the twelve links of the four leaves of
-// F_{mu nu}(x), the link U_l(x) and the 18 of its staples.
+// Per site the planes and directions all of whose links are close to one (the twelve links of the four leaves of
+// F_{mu nu}(x); the link U_l(x) and the 18 of its staples), for a whole block of 32 sites of a parity if for one of
+// them: a block would take the time of both kernels to be shared out between them.
 __global__ void __launch_bounds__(128) weak_sites_kernel(Geom g, const unsigned char* __restrict__ far,
                                                          unsigned char* weakF, unsigned char* weakG, int* any) {
-  const int tid = blockIdx.x * 128 + threadIdx.x;
-  if (tid >= 2 * g.Vh) return;
-  const int p = tid >= g.Vh, h = tid - p * g.Vh;
-  const Site s = site_of(g, p, h);
+  const int nb = (g.Vh + 31) / 32, blk = blockIdx.x * 4 + (threadIdx.x >> 5);
+  if (blk >= 2 * nb) return;
+  const int p = blk >= nb, h = (blk - p * nb) * 32 + (threadIdx.x & 31);
+  const bool valid = h < g.Vh;
+  const Site s = site_of(g, p, valid ? h : 0);
   const FxSites f = {nullptr, g.Vh, g.X, g.Y, g.Z, g.T, {s.x, s.y, s.z, s.t}, p};
   auto at = [&](int d1, int s1, int d2, int s2, int mu) {
     return (int)__ldg(far + (size_t)(((p + s1 + s2) & 1) * 4 + mu) * g.Vh + fx_half_at(f, d1, s1, d2, s2));
@@ -142,10 +144,11 @@ __global__ void __launch_bounds__(128) weak_sites_kernel(Geom g, const unsigned 
       if (n00 | m01 | n10 | m00 | mb1 | nb0 | mb0) force |= 1 << n;
       pl++;
     }
-  const int wG = ~force & 15;
-  weakF[tid] = (unsigned char)wF;
-  weakG[tid] = (unsigned char)wG;
-  if (wF || wG) atomicOr(any, (wF ? 1 : 0) | (wG ? 2 : 0));
+  const int marks = __reduce_or_sync(0xffffffffu, valid ? wF | (~force & 15) << 6 : 0);
+  if (!valid) return;
+  weakF[(size_t)p * g.Vh + h] = (unsigned char)(marks & 63);
+  weakG[(size_t)p * g.Vh + h] = (unsigned char)(marks >> 6);
+  if (marks && (threadIdx.x & 31) == 0) atomicOr(any, (marks & 63 ? 1 : 0) | (marks >> 6 ? 2 : 0));
 }
 
 // Canonical sites are 12 consecutive complex128.  Reading them site by site is fine (a site's lines stay in
@@ -327,7 +330,7 @@ void launch_pack_gauge(const Geom& g, const double2* canon, void* g64, void* g32
 void launch_weak_sites(const Geom& g, const unsigned char* far, unsigned char* weakF, unsigned char* weakG, int* any,
                        cudaStream_t st) {
   g_kernel_launches += 1;
-  weak_sites_kernel<<<nblocks(2LL * g.Vh, 128), 128, 0, st>>>(g, far, weakF, weakG, any);
+  weak_sites_kernel<<<nblocks(2 * ((g.Vh + 31) / 32), 4), 128, 0, st>>>(g, far, weakF, weakG, any);
 }
 
 void launch_spinor_to_native(int prec, const Geom& g, const double2* canon, void* nat, float* norm, int nrhs,
