@@ -393,8 +393,7 @@ void launch_clover_build(const Geom& g, const void* g64, const FxLinks& fl, doub
   const long long V = 2LL * g.Vh;
   // F per (site, plane), then one chiral block per thread
   g_kernel_launches += fl.U && fl.weakF ? 3 : 2;
-  // (block fixed point against FP64: 24^3 x 32 5.23 -> 1.33 ms, 16^4 805 -> 200 us; 7 or 8 blocks per SM in
-  // place of 6 change nothing)
+  // (block fixed point against FP64: 24^3 x 32 5.23 -> 1.39 ms, 16^4 805 -> 211 us)
   if (fl.U)
     field_strength_fixed_kernel<<<dim3(2 * ((g.Vh + 31) / 32), 6), 96, 0, st>>>(g, static_cast<const int4*>(fl.U), fl.weakF,
                                                                                 static_cast<double2*>(work));

@@ -7,8 +7,8 @@
 // exponents [field][V], the site of parity p and half index h at p Vh + h.
 //
 // Against the FP64 kernels, which ran at 82 to 95% of the FP64 pipe (16^4, one pseudofermion): coefficients
-// 169 -> 50 us, insertions 325 -> 115 us (with the coefficients' conversion), links 1521 -> 443 us, gauge force
-// 737 -> 182 us, plaquette 206 -> 63 us.  Bound by instruction issue and the latency of the matrices' loads:
+// 172 -> 56 us, insertions 328 -> 119 us (with the coefficients' conversion), links 1526 -> 429 us, gauge force
+// 741 -> 201 us, plaquette 206 -> 63 us.  Bound by instruction issue and the latency of the matrices' loads:
 // the link kernel runs 4 blocks of 168 registers per SM (3 of 178 without the bound: 668 us; 5 of 128, which
 // spill: 437 us here, but 2469 against 2449 us at 24^4 with two), the gauge force and insertions 7 of 96
 // (6 of 108: 980 against 863 us and 628 against 575 us at 24^4).

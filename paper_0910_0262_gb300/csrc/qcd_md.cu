@@ -187,8 +187,8 @@ __global__ void __launch_bounds__(MB) flat_redot_kernel(size_t n, int nrhs, cons
 //   (a, b, c)_{k+1} = (c_k det M, a_k - c_k c, b_k + c_k tr M),
 // the same sum as the matrix series, for one matrix product (M^2) instead of one per term.  s and n
 // are chosen in FP32 (r rounded up): on the FP64 pipe, two instructions a clock and SM, the norms'
-// comparisons and divisions of the series took as long as its terms (16^4: 458 us with the divisions,
-// 330 with stored reciprocals, 270 as it stands).
+// comparisons and divisions of the series took as long as its terms (16^4, eps 0.01: 460 us with them,
+// 324 as it stands).
 __device__ const double INVERSE_FACTORIAL[21] = {
     1.0, 1.0, 1.0 / 2, 1.0 / 6, 1.0 / 24, 1.0 / 120, 1.0 / 720, 1.0 / 5040, 1.0 / 40320, 1.0 / 362880, 1.0 / 3628800,
     1.0 / 39916800, 1.0 / 479001600, 1.0 / 6227020800.0, 1.0 / 87178291200.0, 1.0 / 1307674368000.0,
