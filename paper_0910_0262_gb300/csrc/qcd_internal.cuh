@@ -161,27 +161,31 @@ __device__ __forceinline__ double widen(float f) {
     return __hiloint2double((int)((u & 0x80000000u) | ((m >> 3) + 0x38000000u)), (int)(u << 29));
   return m == 0 ? __hiloint2double((int)u, 0) : (double)f;
 }
-// rounded to nearest even
-__device__ __forceinline__ float narrow(double x) {
-  const unsigned long long b = (unsigned long long)__double_as_longlong(x), m = b & 0x7fffffffffffffffULL;
-  // magnitudes from the smallest normal float to below the largest one's upper neighbour's half way
-  if (m - 0x3810000000000000ULL < 0x47efffffe0000000ULL - 0x3810000000000000ULL) {
-    const unsigned long long r = (m + 0x0fffffffULL + ((m >> 29) & 1ULL)) >> 29;
-    return __uint_as_float((unsigned)(b >> 32 & 0x80000000u) | (unsigned)(r - (896ULL << 23)));
-  }
-  return m == 0 ? __uint_as_float((unsigned)(b >> 32)) : (float)x;
+// x's words as integers whose origin the compiler does not see: it makes FP64 comparisons of tests on a double's bits
+__device__ __forceinline__ void double_words(double x, unsigned& hi, unsigned& lo) {
+  asm("mov.b64 {%0, %1}, %2;" : "=r"(lo), "=r"(hi) : "d"(x));
 }
-// the same in two parts: whether x is zero or its magnitude lies among the normal floats (below their top binade), and
-// the value then, without a branch
+// (float)x by the conversion instruction, not speculated: it runs where the branch to it is taken
+__device__ __forceinline__ float narrow_rare(double x) {
+  float f;
+  asm("cvt.rn.f32.f64 %0, %1;" : "=f"(f) : "d"(x));
+  return f;
+}
+// whether x is zero or its magnitude lies among the normal floats (below their top binade), and x rounded to
+// nearest even then
 __device__ __forceinline__ bool narrow_common(double x) {
-  const unsigned hi = (unsigned)__double2hiint(x), lo = (unsigned)__double2loint(x);
+  unsigned hi, lo;
+  double_words(x, hi, lo);
   return (hi >> 20 & 0x7ffu) - 897u < 253u || (hi << 1 | lo) == 0u;
 }
 __device__ __forceinline__ float narrow_of_common(double x) {
-  const unsigned long long b = (unsigned long long)__double_as_longlong(x), m = b & 0x7fffffffffffffffULL;
-  const unsigned r = (unsigned)((m + 0x0fffffffULL + ((m >> 29) & 1ULL)) >> 29) - (896u << 23);
-  return __uint_as_float(((unsigned)(b >> 32) & 0x80000000u) | (m == 0 ? 0u : r));
+  unsigned hi, lo;
+  double_words(x, hi, lo);
+  const unsigned long long m = (unsigned long long)(hi & 0x7fffffffu) << 32 | lo;
+  const unsigned r = (unsigned)((m + 0x0fffffffULL + (lo >> 29 & 1u)) >> 29) - (896u << 23);
+  return __uint_as_float((hi & 0x80000000u) | ((hi << 1 | lo) == 0u ? 0u : r));
 }
+__device__ __forceinline__ float narrow(double x) { return narrow_common(x) ? narrow_of_common(x) : narrow_rare(x); }
 template <typename R>
 __device__ __forceinline__ R to_real(double x);
 template <>

@@ -186,9 +186,13 @@ __global__ void __launch_bounds__(3 * LB) spinor_to_native_kernel(Geom g, const 
     bool common = true;
 #pragma unroll
     for (int c = 0; c < 4; c++) common = common && narrow_common(v[c].x) && narrow_common(v[c].y);
+    if (common) {
 #pragma unroll
-    for (int c = 0; c < 4; c++)
-      f[c] = common ? make_float2(narrow_of_common(v[c].x), narrow_of_common(v[c].y)) : make_float2((float)v[c].x, (float)v[c].y);
+      for (int c = 0; c < 4; c++) f[c] = make_float2(narrow_of_common(v[c].x), narrow_of_common(v[c].y));
+    } else {
+#pragma unroll
+      for (int c = 0; c < 4; c++) f[c] = make_float2(narrow_rare(v[c].x), narrow_rare(v[c].y));
+    }
     if constexpr (P == 32) {
       if (!valid || !dbg_spinor(g.Vh, r, h)) return;
 #pragma unroll
