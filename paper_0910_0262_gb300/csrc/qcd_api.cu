@@ -135,7 +135,7 @@ struct qcd_ctx {
   // the FP64 operators' operands in block fixed point (qcd_fixed.cuh), for near-unitary links: null where
   // they could not be allocated or on t-slabs, which keep the FP64 kernels
   void* gfx = nullptr;
-  unsigned char* far = nullptr;  // in gfx's allocation: [2][4][Vh] links far from one, then weakF, weakG [2][Vh]
+  unsigned char* far = nullptr;  // in gfx's allocation: links far from one, then weakF, weakG, [2][Vh] each
   int weak = 0;                  // bits 0, 1: some site is marked in weakF, weakG
   FxClover cfx{};
   bool fx_links = false;  // the loaded links are near-unitary
@@ -422,7 +422,7 @@ int fp64_rep(const qcd_ctx* c, bool with_clover) {
 FxLinks fx_links(const qcd_ctx* c) {
   if (!c->fx_links) return FxLinks{};
   const size_t V = 2 * (size_t)c->g.Vh;
-  return FxLinks{c->gfx, c->weak & 1 ? c->far + 4 * V : nullptr, c->weak & 2 ? c->far + 5 * V : nullptr};
+  return FxLinks{c->gfx, c->weak & 1 ? c->far + V : nullptr, c->weak & 2 ? c->far + 2 * V : nullptr};
 }
 
 DslashArgs base_args(const qcd_ctx* c, int prec, int parity, int nrhs) {
@@ -746,7 +746,7 @@ static qcd_status load_gauge(qcd_ctx* c, const double* U, int on_device, int fla
                         {&c->g16, n_links * 9 * sizeof(uint32_t)}})))
     return s;
   if (!c->slab && !c->no_fixed && !c->gfx) {
-    if (try_alloc(&c->gfx, n_links * 9 * sizeof(int4) + n_links + n_links / 2))
+    if (try_alloc(&c->gfx, n_links * 9 * sizeof(int4) + 3 * (n_links / 4)))
       c->far = reinterpret_cast<unsigned char*>(static_cast<int4*>(c->gfx) + n_links * 9);
     else
       c->no_fixed = true;
@@ -774,7 +774,7 @@ static qcd_status load_gauge(qcd_ctx* c, const double* U, int on_device, int fla
   if (c->slab) launch_check_finite(reinterpret_cast<const double*>(src), in_links * 18, c->flags + 1, c->st);
   launch_pack_gauge(g, src + (c->slab ? (size_t)2 * g.XYZ * 4 * 9 : 0), c->g64, c->g32, c->recon, c->g16, c->recon,
                     c->gfx, c->far, c->flags + 2, c->slab ? nullptr : c->flags + 1, c->st);
-  if (c->gfx) launch_weak_sites(g, c->far, c->far + n_links, c->far + n_links + n_links / 4, c->flags + 3, c->st);
+  if (c->gfx) launch_weak_sites(g, c->far, c->far + n_links / 4, c->far + n_links / 2, c->flags + 3, c->st);
   CUDA_TRY(cudaMemcpyAsync(c->h_flags, c->flags, 4 * sizeof(int), cudaMemcpyDeviceToHost, c->st));
   if ((s = sync_and_check(c, "load_gauge"))) return s;
   c->have_clover = false;

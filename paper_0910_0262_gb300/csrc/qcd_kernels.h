@@ -70,7 +70,7 @@ struct FxLinks {
   void* U;
   unsigned char *weakF, *weakG;
 };
-// gfx (may be null): the block fixed-point links, and far ([2][4][Vh]) whether a link is not close to one;
+// gfx (may be null): the block fixed-point links, and far ([2][Vh], a bit a direction) which are not close to one;
 // *not_unitary is set if a link is not near-unitary, *non_finite (may be null) if one holds a non-finite value
 void launch_pack_gauge(const Geom& g, const double2* canon, void* g64, void* g32, int recon32, void* g16,
                        int recon16, void* gfx, unsigned char* far, int* not_unitary, int* non_finite, cudaStream_t st);

@@ -83,7 +83,9 @@ __global__ void pack_gauge_kernel(Geom g, const double2* __restrict__ U, double2
   for (int k = 0; k < 9; k++) g64[(base * 9 + k) * g.Vh + h] = u[k];
   if (gfx) {
     fx_store_link(gfx + base * 9 * g.Vh + h, g.Vh, u);
-    far[base * g.Vh + h] = far_from_one(v);
+    // (a site's four links lie in neighbouring lanes; V is a multiple of 16, so warps are whole)
+    const unsigned f = __ballot_sync(0xffffffffu, far_from_one(v));
+    if (mu == 0) far[(size_t)p * g.Vh + h] = (unsigned char)(f >> (threadIdx.x & 28) & 15);
     if (!near_unitary(v)) *not_unitary = 1;
   }
   if (g32) {
@@ -125,23 +127,31 @@ __global__ void __launch_bounds__(128) weak_sites_kernel(Geom g, const unsigned 
   const bool valid = h < g.Vh;
   const Site s = site_of(g, p, valid ? h : 0);
   const FxSites f = {nullptr, g.Vh, g.X, g.Y, g.Z, g.T, {s.x, s.y, s.z, s.t}, p};
-  auto at = [&](int d1, int s1, int d2, int s2, int mu) {
-    return (int)__ldg(far + (size_t)(((p + s1 + s2) & 1) * 4 + mu) * g.Vh + fx_half_at(f, d1, s1, d2, s2));
+  // the far links of a site in its directions, a bit each
+  auto at = [&](int d1, int s1, int d2, int s2) {
+    return (int)__ldg(far + (size_t)((p + s1 + s2) & 1) * g.Vh + fx_half_at(f, d1, s1, d2, s2));
   };
+  int fwd[4], bwd[4];
+#pragma unroll
+  for (int m = 0; m < 4; m++) {
+    fwd[m] = at(m, 1, (m + 1) & 3, 0);
+    bwd[m] = at(m, -1, (m + 1) & 3, 0);
+  }
+  const int here = at(0, 0, 1, 0);
   int wF = 0, force = 0;  // force: directions with a link in their staples that is far from one
   int pl = 0;
 #pragma unroll
   for (int m = 0; m < 3; m++)
 #pragma unroll
     for (int n = m + 1; n < 4; n++) {
-      const int m00 = at(m, 0, n, 0, m), n00 = at(m, 0, n, 0, n);
-      const int n10 = at(m, 1, n, 0, n), m01 = at(m, 0, n, 1, m), n1b = at(m, 1, n, -1, n), m0b = at(m, 0, n, -1, m);
-      const int n0b = at(m, 0, n, -1, n), mb1 = at(m, -1, n, 1, m), nb0 = at(m, -1, n, 0, n);
-      const int mbb = at(m, -1, n, -1, m), nbb = at(m, -1, n, -1, n), mb0 = at(m, -1, n, 0, m);
-      if (!(m00 | n00 | n10 | m01 | n1b | m0b | n0b | mb1 | nb0 | mbb | nbb | mb0)) wF |= 1 << pl;
-      // staples of m through n and of n through m (with the links themselves)
-      if (m00 | n10 | m01 | n00 | n1b | m0b | n0b) force |= 1 << m;
-      if (n00 | m01 | n10 | m00 | mb1 | nb0 | mb0) force |= 1 << n;
+      const int M = 1 << m, N = 1 << n, fb = at(m, 1, n, -1), bf = at(m, -1, n, 1), bb = at(m, -1, n, -1);
+      // U_m and U_n here, U_n(x+m), U_m(x+n); with U_n(x+m-n), U_m(x-n), U_n(x-n) the staples of U_m, with
+      // U_m(x-m+n), U_n(x-m), U_m(x-m) those of U_n
+      const int both = (here & (M | N)) | (fwd[m] & N) | (fwd[n] & M);
+      const int of_m = (fb & N) | (bwd[n] & (M | N)), of_n = (bf & M) | (bwd[m] & (M | N));
+      if (!(both | of_m | of_n | (bb & (M | N)))) wF |= 1 << pl;
+      if (both | of_m) force |= M;
+      if (both | of_n) force |= N;
       pl++;
     }
   const int marks = __reduce_or_sync(0xffffffffu, valid ? wF | (~force & 15) << 6 : 0);

@@ -70,7 +70,7 @@ def child(path):
     run(shim)
     want, most, count = run(shim)
     links = int(np.prod(DIMS)) * 4
-    copies = links * (9 * 16) + links * 3 // 2
+    copies = links * (9 * 16) + links // 4 * 3
     # links that are not unitary to 1e-5 take the FP64 kernels: their peak less the copies' room is what these need
     _, far, _ = run(shim, scale=1.0 + 1e-3)
     need = far - copies
