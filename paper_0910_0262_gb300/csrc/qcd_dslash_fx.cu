@@ -579,33 +579,28 @@ __global__ void __launch_bounds__(256, 2) dslash_fixed_split_kernel(DslashArgs A
   }
 }
 
-// out = C in on the sites of one parity, one thread per (site, RHS)
+// out = C in on the sites of one parity, one thread per (site, RHS, chiral block)
 __global__ void __launch_bounds__(128) clover_fixed_kernel(Geom g, const int4* clover, const int* clover_e,
                                                            const longlong2* in, const int* in_e, longlong2* out,
                                                            int* out_e, int nrhs) {
-  const int tid = blockIdx.x * blockDim.x + threadIdx.x, Vh = g.Vh;
-  if (tid >= Vh * nrhs) return;
-  const int r = tid / Vh, h = tid - r * Vh;
-  if (!dbg_spinor(Vh, r, h) || !dbg_clover(Vh, h, 0)) return;
+  const int Vh = g.Vh, n = Vh * nrhs, k = blockIdx.x * blockDim.x + threadIdx.x;
+  if (k >= 2 * n) return;
+  const int b = k >= n, tid = k - b * n, r = tid / Vh, h = tid - r * Vh;
+  if (!dbg_spinor(Vh, r, h) || !dbg_clover(Vh, h, b)) return;
+  const int ex = in_e[eidx(b, Vh, r, h)], ec = clover_e[(size_t)b * Vh + h];
+  cx<i64> x[6], t[6];
 #pragma unroll
-  for (int b = 0; b < 2; b++) {
-    const int ex = in_e[eidx(b, Vh, r, h)];
-    cx<i64> x[6], t[6];
-#pragma unroll
-    for (int k = 0; k < 6; k++) {
-      const longlong2 v = in[sidx<12>(6 * b + k, Vh, r, h)];
-      x[k] = cmk((i64)v.x, (i64)v.y);
-    }
-    const int ec = clover_e[(size_t)b * Vh + h];
-    clover_fx(clover + (size_t)(18 * b) * Vh + h, Vh, x, t);
-    const int unit = ex - FX_SPINOR + ec + 2, bits = fx_bits_of(t);
-    const int e = ex > FX_BIG || ec > FX_BIG ? FX_NAN : (bits ? unit + bits : FX_ZERO);
-    const FxShift f = fx_shift(unit, e);
-#pragma unroll
-    for (int k = 0; k < 6; k++)
-      out[sidx<12>(6 * b + k, Vh, r, h)] = make_longlong2(f(t[k].re), f(t[k].im));
-    out_e[eidx(b, Vh, r, h)] = e;
+  for (int c = 0; c < 6; c++) {
+    const longlong2 v = in[sidx<12>(6 * b + c, Vh, r, h)];
+    x[c] = cmk((i64)v.x, (i64)v.y);
   }
+  clover_fx(clover + (size_t)(18 * b) * Vh + h, Vh, x, t);
+  const int unit = ex - FX_SPINOR + ec + 2, bits = fx_bits_of(t);
+  const int e = ex > FX_BIG || ec > FX_BIG ? FX_NAN : (bits ? unit + bits : FX_ZERO);
+  const FxShift f = fx_shift(unit, e);
+#pragma unroll
+  for (int c = 0; c < 6; c++) out[sidx<12>(6 * b + c, Vh, r, h)] = make_longlong2(f(t[c].re), f(t[c].im));
+  out_e[eidx(b, Vh, r, h)] = e;
 }
 
 }  // namespace
@@ -614,7 +609,7 @@ void launch_clover_apply_fixed(const Geom& g, const void* clover, const int* clo
                                const float* in_e, void* out, float* out_e, int nrhs, cudaStream_t st) {
   g_kernel_launches += 1;
   const int B = 128;
-  clover_fixed_kernel<<<(g.Vh * nrhs + B - 1) / B, B, 0, st>>>(
+  clover_fixed_kernel<<<(2 * g.Vh * nrhs + B - 1) / B, B, 0, st>>>(
       g, static_cast<const int4*>(clover), clover_e, static_cast<const longlong2*>(in),
       reinterpret_cast<const int*>(in_e), static_cast<longlong2*>(out), reinterpret_cast<int*>(out_e), nrhs);
 }
