@@ -75,7 +75,7 @@ __global__ void pack_gauge_kernel(Geom g, const double2* __restrict__ U, double2
 #pragma unroll
   for (int k = 0; k < 9; k++) {
     bad |= !isfinite(u[k].x) || !isfinite(u[k].y);
-    v[k] = make_float2(narrow(u[k].x), narrow(u[k].y));
+    v[k] = make_float2(narrow_many(u[k].x), narrow_many(u[k].y));
   }
   if (bad && non_finite) *non_finite = 1;
   const size_t base = (size_t)(p * 4 + mu);
