@@ -191,7 +191,7 @@ __global__ void __launch_bounds__(3 * LB) spinor_to_native_kernel(Geom g, const 
     for (int c = 0; c < 4; c++) static_cast<double2*>(nat)[sidx<12>(4 * part + c, g.Vh, r, h)] = v[c];
   } else {
     // one branch for a thread's conversions: with one in each of them, loads wait behind the branches before them
-    // (6x4x4x8, Mdag M in FP32, one thread per site and 24 branches: 26.8 us a pass; so 24.8)
+    // (4^3 x 8, Mdag M in FP32, one thread per site and 24 branches: 26.8 us a pass; so 24.7)
     float2 f[4];
     bool common = true;
 #pragma unroll
